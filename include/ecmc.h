@@ -96,21 +96,18 @@ typedef struct ecmc_opts {
   double cell_side;      /* side of the global cell grid (domain); 0 -> 1.05 sigma */
   double tile_side;      /* batch: target tile side when tiles[0] <= 0 (per replica
                             D = floor(L / tile_side), at least 3); 0 -> 4.2 sigma */
-  int32_t schedule;      /* screened domain form with lanes 4, 8 or 16:
-                            0 -> block lockstep: the tiles of a block advance one
-                            event per step together and their FP64 work (candidate
-                            evaluation, move) is packed one tile per thread;
-                            1 -> warp lockstep: each group of `lanes` lanes does
-                            its own tile's FP64 work.  Same events either way. */
-  int32_t block_tiles;   /* block lockstep: tiles per block (a multiple of
-                            32 / lanes, at most 32); 0 -> most tiles per SM */
-  int32_t request_cap;   /* block lockstep: FP64 requests per tile and step in
-                            the block's request list, 1..6; 0 -> 6.  A tile
-                            whose FP32 survivors (or whose list of 24 x cap
-                            screened slots) do not fit is evaluated
-                            exhaustively in FP64 by its own lanes: same
-                            events, slower; small caps exist to exercise that
-                            path (ecmc_obs.exhaustive counts it). */
+  int32_t schedule;      /* 0 or 1: accepted for compatibility; both run the
+                            same kernel (every warp steps its tiles by itself) */
+  int32_t block_tiles;   /* tiles per block (a multiple of 32 / lanes, at most
+                            32); > 0 also keeps `lanes` lanes per tile where few
+                            tiles would get more; 0 -> most tiles per SM */
+  int32_t request_cap;   /* screened form: FP64 evaluations per tile and step,
+                            1..6; 0 -> 6.  Below 6 a tile with more survivors
+                            of the FP32 screen than that (or more than 8 times
+                            as many obstacles in reach) is evaluated
+                            exhaustively in FP64: same events, slower; small
+                            caps exist to exercise that path
+                            (ecmc_obs.exhaustive counts it). */
   double k_spring;       /* > 0: bead-spring chains (Sec. II): every bond is a
                             harmonic spring (k/2)(b - sigma)^2 with k =
                             k_spring in kT/sigma^2 (the paper's melts: 30)
@@ -130,7 +127,7 @@ typedef struct ecmc_opts {
                             bond, so no joint could keep such tiles apart);
                             tether checks are off; swaps (p_swap > 0) and the
                             batch are refused. */
-  double tight_factor;   /* block lockstep: the first launch of a sweep stages
+  double tight_factor;   /* the first launch of a sweep stages
                             tiles with capacities of tight_factor times a
                             melted tile's mean content (more tiles fit per SM);
                             tiles that do not fit run in a second launch with
@@ -171,8 +168,8 @@ typedef struct ecmc_obs {
                                   f, f_b pairs / bonds per unit distance at
                                   contact, each extrapolated linearly from its
                                   two shells */
-  int64_t exhaustive;          /* tile steps of the block-lockstep kernel
-                                  evaluated exhaustively in FP64 */
+  int64_t exhaustive;          /* tile steps of the screened form evaluated
+                                  exhaustively in FP64 (request_cap below 6) */
   double bond_mean;            /* <b> over all bonds of the current state */
 } ecmc_obs;
 

@@ -1,8 +1,8 @@
 // Device helpers shared by the EC kernels (arXiv:1502.06447, Sec. II, II.A,
 // II.C): FP64 comparisons on bit patterns, the minimum image, the contact and
 // tether distances (Eq. 1), the reflection (Fig. 2c), candidate keys and the
-// tie rule, the shared-memory staging of one tile and its local cell grid,
-// and the FP32 screen.  Included by the kernel translation units only.
+// tie rule, the shared-memory staging of one tile with its slab masks, and
+// the FP32 screen.  Included by the kernel translation units only.
 #pragma once
 #include <cuda_runtime.h>
 #include <float.h>
@@ -111,19 +111,6 @@ __device__ __forceinline__ bool better(double x, uint64_t key, double bx, uint64
 }
 
 template <int G>
-__device__ __forceinline__ void group_argmin(double &bx, uint64_t &bkey) {
-#pragma unroll
-  for (int off = G / 2; off > 0; off >>= 1) {
-    const double ox = __shfl_xor_sync(FULL, bx, off);
-    const uint64_t ok = __shfl_xor_sync(FULL, bkey, off);
-    if (better(ox, ok, bx, bkey)) {
-      bx = ox;
-      bkey = ok;
-    }
-  }
-}
-
-template <int G>
 __device__ __forceinline__ float group_minf(float v) {
 #pragma unroll
   for (int off = G / 2; off > 0; off >>= 1) v = fminf(v, __shfl_xor_sync(FULL, v, off));
@@ -136,63 +123,64 @@ __device__ __forceinline__ float wrapf(float d, float L) {
 }
 
 // ---------------------------------------------------------------- staging
-// Shared memory of one group: FP64 positions of the first M64 slots (the
-// warp-lockstep kernel: M64 = the motile capacity in the screened domain
-// form, where joint beads' FP64 positions, static during a sweep, are read
-// from the global array when an evaluation needs them, M64 = S otherwise;
-// the block-lockstep kernel keeps every FP64 position in the global array,
-// M64 = 0); bond-partner words of the first MNB slots (the motile beads);
-// FP32 shadow (12 B) and id (4 B) of all S slots; the local cell grid (16 B
-// per cell: a 32-bit count, then 6 slots of 16 bits); the overflow list of
-// beads whose cell was full; a header.
-constexpr int CELL_CAP = 6;
-constexpr int OVF_CAP = 64;
+// Shared memory of one group: FP32 shadow (tile-local) and id of every
+// staged bead (16 B, one load); FP64 positions of the first M64 slots (M64 =
+// 0: they are read from the global array, where every move is written
+// through); bond-partner words of the first MNB slots (the motile beads);
+// the slab masks; a header.
+//
+// Slab masks.  Every axis of the tile's box is cut into nsl slabs; row k + 1
+// of an axis is the set of obstacle slots in slabs <= k (row 0 is empty), so
+// the obstacles in slabs [a, b] are row[b + 1] & ~row[a], and those in a box
+// the AND over the axes: six loads give the beads a path can reach, where a
+// grid of cells has to visit, count and gather up to 27 of them.  Slot s is
+// bit (s / G) of lane s % G: a lane reads and keeps current its own words and
+// no others, so the masks need no synchronisation.
 constexpr int HDR_BYTES = 32;
-// the overflow list holds max(64, S / 4) slots, rounded up to a multiple of
-// 8 (16 bytes, so that a group's share of shared memory stays a multiple of
-// 16 bytes for any S that is a multiple of 8): clustered inputs (phantom
-// chains before the push-off) fill many cells past CELL_CAP
+
+// The accepted tile sizes count an overflow list of max(64, S / 4) slots per
+// tile, rounded up to a multiple of 8 (staging_budget in ecmc_internal.h).
+constexpr int OVF_CAP = 64;
 __host__ __device__ __forceinline__ int ovf_cap_for(int S) {
   return S / 4 > OVF_CAP ? (S / 4 + 7) / 8 * 8 : OVF_CAP;
 }
 
 struct Stage {
+  float4 *sh;       // [S] x, y, z, id (bits)
   double *px, *py, *pz;  // [M64]
-  unsigned *nb;          // [MNB] bond partner slots, 16 + 16 bits (0xFFFF = none)
-  float *fx, *fy, *fz;   // [S]
-  int *id;               // [S]
-  unsigned short *cell;  // [NC][8]: 32-bit count, then up to 6 slots
-  unsigned short *ovf;   // [ovf_cap]
-  int *hdr;              // [2] staged count, [3] overflow, [4] overflow-list length
-  int ovf_cap;           // ovf_cap_for(S)
+  unsigned *nb;     // [MNB] bond partner slots, 16 + 16 bits (0xFFFF = none)
+  unsigned *mask;   // [3][nsl + 1][W][G]
+  int *hdr;         // [0] hard-sphere joint beads, [1] tether-only joint beads
+                    // placed, [2] joint beads seen, [3] overflow, [4] motile
+                    // beads seen
 #ifdef ECMC_CHECKED
-  int cap;               // S (slots)
-  long long nglob;       // beads of the system (ids), set by the kernel
+  int cap;          // S (slots)
+  long long nglob;  // beads of the system (ids), set by the kernel
   int *status;
 #endif
 };
 
-__host__ __device__ __forceinline__ size_t group_bytes(int S, int M64, int MNB, int NC) {
-  return (size_t)M64 * 24 + (size_t)MNB * 4 + (size_t)S * 16 + (size_t)NC * 16 + (size_t)ovf_cap_for(S) * 2 +
-         HDR_BYTES;
-}  // (16 B per cell: a 32-bit count and 6 slots of 16 bits)
+// 16-byte units of a group's slab masks (G is a multiple of 4)
+__host__ __device__ __forceinline__ int mask_quads(int S, int G, int nsl) {
+  const int W = (S + 32 * G - 1) / (32 * G);
+  return 3 * (nsl + 1) * W * (G / 4);
+}
 
-// S, M64 and MNB are multiples of 8 (capacities are rounded to 8 or 32), so
+// S, M64 and MNB are multiples of 8 and the masks whole 16-byte units, so
 // every array starts 16-byte aligned and group_bytes is a multiple of 16
-__device__ __forceinline__ Stage carve(unsigned char *base, int S, int M64, int MNB, int NC) {
+__host__ __device__ __forceinline__ size_t group_bytes(int S, int M64, int MNB, int MQ) {
+  return (size_t)S * 16 + (size_t)M64 * 24 + (size_t)MNB * 4 + (size_t)MQ * 16 + HDR_BYTES;
+}
+
+__device__ __forceinline__ Stage carve(unsigned char *base, int S, int M64, int MNB, int MQ) {
   Stage s;
-  s.px = (double *)base;
+  s.sh = (float4 *)base;
+  s.px = (double *)(s.sh + S);
   s.py = s.px + M64;
   s.pz = s.py + M64;
   s.nb = (unsigned *)(s.pz + M64);
-  s.fx = (float *)(s.nb + MNB);
-  s.fy = s.fx + S;
-  s.fz = s.fy + S;
-  s.id = (int *)(s.fz + S);
-  s.cell = (unsigned short *)(s.id + S);
-  s.ovf = s.cell + 8 * NC;
-  s.ovf_cap = ovf_cap_for(S);
-  s.hdr = (int *)(s.ovf + s.ovf_cap);
+  s.mask = s.nb + MNB;
+  s.hdr = (int *)(s.mask + 4 * MQ);
 #ifdef ECMC_CHECKED
   s.cap = S;
   s.nglob = 0x7fffffffffffffffll;
@@ -216,13 +204,6 @@ __device__ __forceinline__ int find_id(const int *ids, int lo, int hi, int id) {
     if (v < id) lo = mid + 1;
     else hi = mid;
   }
-  return -1;
-}
-
-// linear search of id in the unsorted range [lo, hi); -1 if absent
-__device__ __forceinline__ int find_id_lin(const int *ids, int lo, int hi, int id) {
-  for (int i = lo; i < hi; ++i)
-    if (ids[i] == id) return i;
   return -1;
 }
 
@@ -251,83 +232,45 @@ __device__ __forceinline__ T chk_index(T i, long long n, int site, int *st) {
 #define CI(i, n, site, st) (i)
 #endif
 
-// ---------------------------------------------------------------- local grid
-struct LGrid {
-  int g0, g1, g2;
-  float org, inv0, inv1, inv2;
+// ---------------------------------------------------------------- slabs
+// Slab of a tile-local coordinate: rint(f inv) - base, clamped to the nsl
+// slabs (domain) or taken modulo nsl (serial, the slabs go around the box).
+// Both steps are monotone in f, so a bead between two coordinates lies in a
+// slab between theirs.  The rounding is the one of adding 1.5 2^23.
+struct Slabs {
+  float inv0, inv1, inv2;
+  int base;  // magic bits + rint(origin inv)
+  int nsl;
 };
-
-__device__ __forceinline__ int lcell(const LGrid &L, float f0, float f1, float f2, int &c0,
-                                     int &c1, int &c2) {
-  c0 = (int)((f0 - L.org) * L.inv0);
-  c1 = (int)((f1 - L.org) * L.inv1);
-  c2 = (int)((f2 - L.org) * L.inv2);
-  c0 = c0 < 0 ? 0 : (c0 >= L.g0 ? L.g0 - 1 : c0);
-  c1 = c1 < 0 ? 0 : (c1 >= L.g1 ? L.g1 - 1 : c1);
-  c2 = c2 < 0 ? 0 : (c2 >= L.g2 ? L.g2 - 1 : c2);
-  return (c2 * L.g1 + c1) * L.g0 + c0;
+constexpr float SLAB_MAGIC = 12582912.f;
+__device__ __forceinline__ int slab_raw(float f, float inv, int base) {
+  return __float_as_int(__fmaf_rn(f, inv, SLAB_MAGIC)) - base;
 }
-
-__device__ __forceinline__ unsigned &cell_count(unsigned short *c) { return *reinterpret_cast<unsigned *>(c); }
-__device__ __forceinline__ int cell_n(const unsigned short *c) {
-  return (int)*reinterpret_cast<const unsigned *>(c);
-}
-
-// single-writer updates (one lane of the group)
-__device__ __forceinline__ bool lcell_insert(const Stage &st, int ci, int slot) {
-  unsigned short *c = st.cell + 8 * ci;
-  const int n = cell_n(c);
-  if (n < CELL_CAP) {
-    c[2 + n] = (unsigned short)slot;
-    cell_count(c) = (unsigned)(n + 1);
-    return true;
-  }
-  const int k = st.hdr[4];
-  if (k >= st.ovf_cap) return false;
-  st.ovf[k] = (unsigned short)slot;
-  st.hdr[4] = k + 1;
-  return true;
-}
-
-__device__ __forceinline__ void lcell_remove(const Stage &st, int ci, int slot) {
-  unsigned short *c = st.cell + 8 * ci;
-  const int n = cell_n(c);
-  for (int i = 2; i < 2 + n; ++i) {
-    if (c[i] == slot) {
-      c[i] = c[1 + n];
-      cell_count(c) = (unsigned)(n - 1);
-      return;
-    }
-  }
-  const int k = st.hdr[4];
-  for (int i = 0; i < k; ++i) {
-    if (st.ovf[i] == slot) {
-      st.ovf[i] = st.ovf[k - 1];
-      st.hdr[4] = k - 1;
-      return;
-    }
-  }
+template <bool DOM>
+__device__ __forceinline__ int slab_of(float f, float inv, int base, int nsl) {
+  const int k = slab_raw(f, inv, base);
+  if (DOM) return min(max(k, 0), nsl - 1);
+  return k < 0 ? k + nsl : (k >= nsl ? k - nsl : k);
 }
 
 // FP32 screen of one hard-sphere obstacle k for the pivot shadow pf moving
 // along vf: updates the upper bound ubl and keeps the slot when its lower
 // bound can reach it (two kept per lane, more -> ovf)
 struct Screen {
-  float sig2f, eps_v, eps_d, near2;
+  float sig2f, eps_v, eps_d;
 };
 
 __device__ __forceinline__ void screen_hs(const Screen &Z, float d0, float d1, float d2, float vf0,
                                           float vf1, float vf2, int k, float &ubl, int &ks0,
                                           float &kl0, int &ks1, float &kl1, bool &ovf) {
   const float dd = __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, d0 * d0));
-  if (dd > Z.near2) return;
   const float dv = __fmaf_rn(d2, vf2, __fmaf_rn(d1, vf1, d0 * vf0));
   const float disc = Z.sig2f - (dd - dv * dv);
   if (!(dv < Z.eps_v && disc > -Z.eps_d)) return;
-  if (dv < -Z.eps_v && disc > Z.eps_d)
-    ubl = fminf(ubl, fmaxf(0.f, -dv + Z.eps_v - sqrt_lo(disc - Z.eps_d)) + 1e-6f);
   const float lb = -dv - Z.eps_v - sqrt_hi(disc + Z.eps_d);
   if (lb > ubl) return;
+  if (dv < -Z.eps_v && disc > Z.eps_d)
+    ubl = fminf(ubl, fmaxf(0.f, -dv + Z.eps_v - sqrt_lo(disc - Z.eps_d)) + 1e-6f);
   const float INF = __int_as_float(0x7f800000);
   if (kl0 > ubl) {
     ks0 = -1;
@@ -353,51 +296,26 @@ __device__ __forceinline__ float screen_lb(const Screen &Z, float d0, float d1, 
   const float dd = __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, d0 * d0));
   const float dv = __fmaf_rn(d2, vf2, __fmaf_rn(d1, vf1, d0 * vf0));
   const float disc = Z.sig2f - (dd - dv * dv);
-  possible = dd <= Z.near2 && dv < Z.eps_v && disc > -Z.eps_d;
+  possible = dv < Z.eps_v && disc > -Z.eps_d;
   return -dv - Z.eps_v - sqrt_hi(fmaxf(disc + Z.eps_d, 0.f));
 }
 
-// Screen the beads of one local cell (16 bytes: count, then up to 6 slots,
-// read at once) two per round, so that their shadow loads overlap.  The set
-// of candidates a lane keeps or flags does not depend on the order in which
-// it screens them (see screen_hs).
-__device__ __forceinline__ void screen_cell(const Screen &Z, const Stage &st, const unsigned short *rec,
-                                            int p, float a0, float a1, float a2, float w0, float w1,
-                                            float w2, float &ubl, int &ks0, float &kl0, int &ks1,
-                                            float &kl1, bool &ovf) {
-  const uint4 c = *reinterpret_cast<const uint4 *>(rec);
-  const int n = (int)c.x;
-  const int sl[6] = {(int)(c.y & 0xFFFF), (int)(c.y >> 16), (int)(c.z & 0xFFFF),
-                     (int)(c.z >> 16), (int)(c.w & 0xFFFF), (int)(c.w >> 16)};
-#pragma unroll
-  for (int i = 0; i < 6; i += 2) {
-    if (i >= n) break;
-    const int ka = sl[i];
-    const bool two = i + 1 < n;
-    const int kb = two ? sl[i + 1] : ka;
-    const float ax = st.fx[ka], ay = st.fy[ka], az = st.fz[ka];
-    const float bx = st.fx[kb], by = st.fy[kb], bz = st.fz[kb];
-    if (ka != p) screen_hs(Z, a0 - ax, a1 - ay, a2 - az, w0, w1, w2, ka, ubl, ks0, kl0, ks1, kl1, ovf);
-    if (two && kb != p)
-      screen_hs(Z, a0 - bx, a1 - by, a2 - bz, w0, w1, w2, kb, ubl, ks0, kl0, ks1, kl1, ovf);
-  }
-}
-
-// FP64 position of staged slot k: shared memory for the first M slots,
-// otherwise (a joint bead, static this sweep) the global position array
-__device__ __forceinline__ void pos64(const Stage &st, const double *r, int k, bool in_smem,
-                                      double &x, double &y, double &z) {
+// FP64 position of staged slot k: shared memory for the first M64 slots,
+// otherwise the global position array (a joint bead, static this sweep, or
+// a motile one, written through by every move)
+__device__ __forceinline__ void pos64(const Stage &st, const double *r, int k, int M64, double &x,
+                                      double &y, double &z) {
 #ifdef ECMC_CHECKED
   x = y = z = 0.0;
   if (st.status && !CHK(k, st.cap, 1, st.status)) return;
-  if (!in_smem && st.status && !CHK(st.id[k], st.nglob, 2, st.status)) return;
+  if (k >= M64 && st.status && !CHK(__float_as_int(st.sh[k].w), st.nglob, 2, st.status)) return;
 #endif
-  if (in_smem) {
+  if (k < M64) {
     x = st.px[k];
     y = st.py[k];
     z = st.pz[k];
   } else {
-    const int64_t b = st.id[k];
+    const int64_t b = __float_as_int(st.sh[k].w);
     x = r[3 * b];
     y = r[3 * b + 1];
     z = r[3 * b + 2];
@@ -406,18 +324,17 @@ __device__ __forceinline__ void pos64(const Stage &st, const double *r, int k, b
 
 // ---------------------------------------------------------------- staging
 // Stage one tile (domain) or the whole system (serial) into the group's
-// shared memory: the lanes in `mask` call this together (the whole warp, or
-// one group of G lanes while the warp's other groups do something else).  Returns the motile count m, the
-// hard-sphere joint count j1 and the staged count ns; clears `live` when the
-// tile does not fit its capacity.
+// shared memory: the lanes in `mask` call this together (one group of G
+// lanes, or all groups of a warp that take a tile at the same time).
+// Returns the motile count m, the hard-sphere joint count j1 and the staged
+// count ns; clears `live` when the tile does not fit its capacity.
 #define SYS(f) (BATCH ? rp->f : P.f)
-template <int G, bool F32, bool BATCH>
+template <int G, bool DOM, bool SPRING, bool BATCH>
 __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *rp, const Stage &st,
                                            int gl, bool &live, int unit, double c0, double c1,
                                            double c2, double *Rr, const int32_t *Rstart, int S,
-                                           int M64, int MNB, int NC, const LGrid &LG, int &m,
-                                           int &j1, int &ns, unsigned mask = FULL,
-                                           bool *overflow = nullptr) {
+                                           int M64, int MNB, int W, const Slabs &SL, int &m,
+                                           int &j1, int &ns, unsigned mask, bool *overflow) {
   // a tile that does not fit its capacities sets the device status, or, when
   // the caller passes `overflow`, only that flag (the caller stages the tile
   // again later with larger capacities)
@@ -426,31 +343,21 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
     else if (gl == 0) set_status(P.status, DEV_CAPACITY);
   };
   if (overflow) *overflow = false;
-  if (gl == 0) {
-    st.hdr[0] = 0;
-    st.hdr[1] = 0;
-    st.hdr[2] = 0;
-    st.hdr[3] = 0;
-    st.hdr[4] = 0;
-    st.hdr[5] = 0;
-    st.hdr[6] = 0;
-  }
-  __syncwarp(mask);
+  const int nsl = SL.nsl;
   m = 0;
   j1 = 0;
   ns = 0;
-  if (!P.domain) {
+  if (!DOM) {
     // serial: every bead, slot = id, all motile
     const int n = (int)P.n;
     for (int b = gl; b < n; b += G) {
       const double x = Rr[3 * (int64_t)b], y = Rr[3 * (int64_t)b + 1], z = Rr[3 * (int64_t)b + 2];
-      st.px[b] = x;
-      st.py[b] = y;
-      st.pz[b] = z;
-      st.fx[b] = (float)x;
-      st.fy[b] = (float)y;
-      st.fz[b] = (float)z;
-      st.id[b] = b;
+      if (b < M64) {
+        st.px[b] = x;
+        st.py[b] = y;
+        st.pz[b] = z;
+      }
+      st.sh[b] = make_float4((float)x, (float)y, (float)z, __int_as_float(b));
       const int c = b % SYS(N);
       st.nb[b] = nb_pack(c == 0 ? -1 : b - 1, c == SYS(N) - 1 ? -1 : b + 1);
     }
@@ -458,6 +365,9 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
     j1 = 0;
     ns = n;
   } else {
+    if (gl < 8) st.hdr[gl] = 0;
+    if (G < 8) st.hdr[gl + 4] = 0;
+    __syncwarp(mask);
     const double corner[3] = {c0, c1, c2};
     // cell window covering the tether halo of the tile
     int c_lo[3], c_n[3];
@@ -472,14 +382,15 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
         cnt = SYS(nc)[a];
       }
       c_lo[a] = l;
-      c_n[a] = live ? cnt : 0;
+      c_n[a] = cnt;
     }
-    // pass 1: collect (cell-order index, category|id); the shadow arrays
-    // (12 B per slot) serve as 8 B per slot of scratch until pass 3.  The
-    // cells of one row of the window (consecutive x) are one contiguous
-    // range of the cell-ordered arrays (two when the row wraps around the
-    // box); each lane takes whole rows and loads four beads at a time.
-    int2 *scr = (int2 *)st.fx;
+    // pass 1: collect (cell-order index, category|id), motile beads from the
+    // front, joint beads from the back; the shadow array serves as scratch
+    // until pass 3.  The cells of one row of the window (consecutive x) are
+    // one contiguous range of the cell-ordered arrays (two when the row
+    // wraps around the box); each lane takes whole rows and loads four beads
+    // at a time.
+    int2 *scr = (int2 *)st.sh;
     // halo membership in FP32 from FP32 copies of the positions, widened by
     // 1e-3 sigma plus four FP32 ulps of the box: a superset of the exact
     // sets (an extra obstacle beyond reach is never hit; a bond partner is
@@ -553,110 +464,136 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
             cat = in_hs ? 1 : (in_te ? 2 : -1);
           }
           if (cat >= 0) {
-            const int slot = atomicAdd(&st.hdr[2], 1);
-            if (slot < S) scr[slot] = make_int2(jj[u], (cat << 29) | idv[u]);
-            else st.hdr[3] = 1;
-            if (cat < 2) atomicAdd(&st.hdr[5 + cat], 1);
+            const int q = atomicAdd(&st.hdr[cat == 0 ? 4 : 2], 1);
+            const int slot = cat == 0 ? q : S - 1 - q;
+            if (q < S) scr[slot] = make_int2(jj[u], (cat << 29) | idv[u]);
+            if (cat == 1) atomicAdd(&st.hdr[5], 1);
           }
         }
       }
     }
     __syncwarp(mask);
-    ns = st.hdr[2];
-    if (st.hdr[3]) {
+    m = st.hdr[4];
+    const int nj = st.hdr[2];
+    j1 = st.hdr[5];
+    ns = m + nj;
+    // (a list that ran into the other one holds no valid entries)
+    if (ns > S || m > MNB) {
       capacity();
       live = false;
-      ns = 0;
+      m = j1 = ns = 0;
     }
-    const int ns_max = __reduce_max_sync(mask, ns);
     // pass 2: slots.  Motile beads take their rank by id (the start bead of
     // an EC is the u-th motile bead in id order); joint beads take the next
-    // free slot of their category (their order matters to nothing).
-    m = st.hdr[5];
-    j1 = st.hdr[6];
-    for (int s0 = 0; s0 < ns_max; s0 += G) {
-      const int s = s0 + gl;
-      if (s < ns) {
-        const int2 e = scr[s];
-        const int cat = e.y >> 29;
-        int rank;
-        if (cat == 0) {
-          rank = 0;
-          for (int t = 0; t < ns; ++t) rank += (scr[t].y < e.y);
-        } else {
-          rank = (cat == 1 ? m : m + j1) + atomicAdd(&st.hdr[cat - 1], 1);
-        }
-        const int j = e.x;
-        if (!CHK(rank, S, 3, P.status)) continue;
-        if (rank < M64) {
-          st.px[rank] = P.cr[3 * (int64_t)j];
-          st.py[rank] = P.cr[3 * (int64_t)j + 1];
-          st.pz[rank] = P.cr[3 * (int64_t)j + 2];
-        }
-        st.id[rank] = e.y & ((1 << 29) - 1);
+    // free slot of their category (their order matters to nothing).  The ids
+    // go to the mask area (nsl >= 10 makes it as large as S words).
+    int *idt = (int *)st.mask;
+    for (int s = gl; s < m; s += G) {
+      const int2 e = scr[s];
+      int rank = 0;
+      for (int t = 0; t < m; ++t) rank += (scr[t].y < e.y);
+      if (!CHK(rank, S, 3, P.status)) continue;
+      idt[rank] = e.y;
+      if (rank < M64) {
+        st.px[rank] = P.cr[3 * (int64_t)e.x];
+        st.py[rank] = P.cr[3 * (int64_t)e.x + 1];
+        st.pz[rank] = P.cr[3 * (int64_t)e.x + 2];
+      }
+    }
+    for (int s = gl; s < ns - m; s += G) {
+      const int2 e = scr[S - 1 - s];
+      const int cat = e.y >> 29;
+      const int slot = (cat == 1 ? m : m + j1) + atomicAdd(&st.hdr[cat - 1], 1);
+      if (!CHK(slot, S, 33, P.status)) continue;
+      idt[slot] = e.y & ((1 << 29) - 1);
+      if (slot < M64) {
+        st.px[slot] = P.cr[3 * (int64_t)e.x];
+        st.py[slot] = P.cr[3 * (int64_t)e.x + 1];
+        st.pz[slot] = P.cr[3 * (int64_t)e.x + 2];
       }
     }
     __syncwarp(mask);
-    if (m > MNB) {  // more motile beads than the motile capacity
-      if (live) capacity();
-      live = false;
+    // pass 2b: bond partners of motile beads.  A motile partner is found
+    // among the sorted motile ids; a joint partner announces itself (its
+    // neighbours' tags tell whether one of them is motile here).
+    const int Nc = SYS(N);
+    for (int s = gl; s < m; s += G) {
+      const int id = idt[s], c = id % Nc;
+      const int prev = c != 0 ? find_id(idt, 0, m, id - 1) : -1;
+      const int next = c != Nc - 1 ? find_id(idt, 0, m, id + 1) : -1;
+      st.nb[s] = nb_pack(prev, next);
     }
-    // pass 2b (bead springs): a spring has no longest bond, so the bonded
-    // beads of motile beads are staged wherever they are; one outside the
-    // tether halo (a joint bead, static this sweep) is appended after the
-    // staged beads (two motile beads may append the same bead twice; both
-    // copies are read-only and equal)
-    // (the condition is the same for every lane in `mask`: the groups of a
-    // warp may hold live and dead tiles, and all of them reach the barrier)
-    if (P.k_spring > 0.0) {
-      const int Nc = SYS(N);
-      for (int s = gl; live && s < m; s += G) {
-        const int id = st.id[s];
-        const int c = id % Nc;
+    __syncwarp(mask);
+    const int32_t *const Rtag = P.tag + (BATCH ? rp->bead_off : 0);
+    unsigned short *const nbh = (unsigned short *)st.nb;
+    for (int s = m + gl; s < ns; s += G) {
+      const int id = idt[s], c = id % Nc;
+      const bool up = c != Nc - 1 && Rtag[id + 1] == unit;
+      const bool dn = c != 0 && Rtag[id - 1] == unit;
+      if (up) {
+        const int t = find_id(idt, 0, m, id + 1);
+        if (t >= 0) nbh[2 * t] = (unsigned short)s;
+      }
+      if (dn) {
+        const int t = find_id(idt, 0, m, id - 1);
+        if (t >= 0) nbh[2 * t + 1] = (unsigned short)s;
+      }
+    }
+    __syncwarp(mask);
+    if (gl == 0) st.hdr[6] = ns;
+    __syncwarp(mask);
+    for (int s = gl; s < m; s += G) {
+      const int id = idt[s], c = id % Nc;
 #pragma unroll
-        for (int dir = 0; dir < 2; ++dir) {
-          const int q = dir == 0 ? (c != 0 ? id - 1 : -1) : (c != Nc - 1 ? id + 1 : -1);
-          if (q < 0) continue;
-          if (!CHK(q, BATCH ? rp->n_beads : P.n, 4, P.status)) continue;
-          if (find_id(st.id, 0, m, q) >= 0 || find_id_lin(st.id, m, ns, q) >= 0) continue;
-          const int slot = atomicAdd(&st.hdr[2], 1);
-          if (slot < S) {
-            st.id[slot] = q;
-            if (slot < M64) {
-              st.px[slot] = Rr[3 * (int64_t)q];
-              st.py[slot] = Rr[3 * (int64_t)q + 1];
-              st.pz[slot] = Rr[3 * (int64_t)q + 2];
-            }
-          } else {
-            st.hdr[3] = 1;
+      for (int dir = 0; dir < 2; ++dir) {
+        if (nbh[2 * s + dir] != 0xFFFF) continue;
+        const int q = dir == 0 ? (c != 0 ? id - 1 : -1) : (c != Nc - 1 ? id + 1 : -1);
+        if (q < 0) continue;
+        if (!SPRING) {
+          set_status(P.status, DEV_TILE);
+          continue;
+        }
+        // a spring has no longest bond, so the bonded beads of motile beads
+        // are staged wherever they are; one outside the tether halo (a joint
+        // bead, static this sweep) is appended after the staged beads (two
+        // motile beads may append the same bead twice; both copies are
+        // read-only and equal)
+        if (!CHK(q, BATCH ? rp->n_beads : P.n, 4, P.status)) continue;
+        const int slot = atomicAdd(&st.hdr[6], 1);
+        if (slot < S) {
+          idt[slot] = q;
+          nbh[2 * s + dir] = (unsigned short)slot;
+          if (slot < M64) {
+            st.px[slot] = Rr[3 * (int64_t)q];
+            st.py[slot] = Rr[3 * (int64_t)q + 1];
+            st.pz[slot] = Rr[3 * (int64_t)q + 2];
           }
         }
       }
-      __syncwarp(mask);
-      if (live) {
-        if (st.hdr[3]) {
-          capacity();
-          live = false;
-          ns = 0;
-        } else {
-          ns = st.hdr[2];
-        }
+    }
+    __syncwarp(mask);
+    if (SPRING) {
+      ns = st.hdr[6];
+      if (ns > S) {
+        if (live) capacity();
+        live = false;
+        m = j1 = ns = 0;
       }
     }
-    const int ns_max2 = __reduce_max_sync(mask, ns);
     // pass 3: shadows (FP32 position minus FP32 corner, the form the moved
-    // pivot's shadow takes too) and bond partners of motile beads; empty
-    // cells.  Four slots at a time (independent loads).
-    for (int i = gl; i < NC; i += G) cell_count(st.cell + 8 * i) = 0u;
+    // pivot's shadow takes too).  Four slots at a time (independent loads).
     const float *Rf = P.rf + (BATCH ? 3 * rp->bead_off : 0);
-    for (int s0 = 0; s0 < ns_max2; s0 += 4 * G) {
+    for (int s0 = 0; s0 < ns; s0 += 4 * G) {
       float x[4], y[4], z[4];
+      int idv[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int s = s0 + u * G + gl;
         x[u] = y[u] = z[u] = 0.f;
-        if (s < ns && live && CHK(st.id[s], BATCH ? rp->n_beads : P.n, 5, P.status)) {
-          const int64_t b = st.id[s];
+        idv[u] = 0;
+        if (s < ns) {
+          const int64_t b = CI(idt[s], BATCH ? rp->n_beads : P.n, 5, P.status);
+          idv[u] = (int)b;
           x[u] = Rf[3 * b];
           y[u] = Rf[3 * b + 1];
           z[u] = Rf[3 * b + 2];
@@ -665,65 +602,55 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int s = s0 + u * G + gl;
-        if (!(s < ns && live)) continue;
+        if (s >= ns) continue;
         float f0 = x[u] - cf[0], f1 = y[u] - cf[1], f2 = z[u] - cf[2];
         f0 = f0 > Lhf[0] ? f0 - Lf[0] : (f0 < -Lhf[0] ? f0 + Lf[0] : f0);
         f1 = f1 > Lhf[1] ? f1 - Lf[1] : (f1 < -Lhf[1] ? f1 + Lf[1] : f1);
         f2 = f2 > Lhf[2] ? f2 - Lf[2] : (f2 < -Lhf[2] ? f2 + Lf[2] : f2);
-        st.fx[s] = f0;
-        st.fy[s] = f1;
-        st.fz[s] = f2;
-        int prev = -1, next = -1;
-        if (s < m) {
-          const int id = st.id[s];
-          const int c = id % SYS(N);
-          if (c != 0) {
-            prev = find_id(st.id, 0, m, id - 1);
-            if (prev < 0) prev = find_id_lin(st.id, m, ns, id - 1);
-            if (prev < 0) set_status(P.status, DEV_TILE);
-          }
-          if (c != SYS(N) - 1) {
-            next = find_id(st.id, 0, m, id + 1);
-            if (next < 0) next = find_id_lin(st.id, m, ns, id + 1);
-            if (next < 0) set_status(P.status, DEV_TILE);
-          }
-        }
-        if (s < MNB) st.nb[s] = nb_pack(prev, next);
+        st.sh[s] = make_float4(f0, f1, f2, __int_as_float(idv[u]));
       }
-    }
-    __syncwarp(mask);
-    // pass 4: the hard-sphere slots into the local grid, all lanes at once
-    // (the order inside a cell does not matter to the screen)
-    if (live) {
-      for (int s = gl; s < m + j1; s += G) {
-        int a0, a1, a2;
-        unsigned short *c = st.cell + 8 * lcell(LG, st.fx[s], st.fy[s], st.fz[s], a0, a1, a2);
-        const unsigned old = atomicAdd(&cell_count(c), 1u);
-        if (old < (unsigned)CELL_CAP) {
-          c[2 + old] = (unsigned short)s;
-        } else {
-          const int k = atomicAdd(&st.hdr[4], 1);
-          if (k < st.ovf_cap) st.ovf[k] = (unsigned short)s;
-          else st.hdr[3] = 1;
-        }
-      }
-    }
-    __syncwarp(mask);
-    // counts past a cell's capacity went to the overflow list
-    for (int i = gl; i < NC; i += G) {
-      unsigned &cc = cell_count(st.cell + 8 * i);
-      if (cc > (unsigned)CELL_CAP) cc = CELL_CAP;
-    }
-    __syncwarp(mask);
-    if (st.hdr[3]) {
-      if (live) capacity();
-      live = false;
-      if (gl == 0) st.hdr[4] = 0;
     }
   }
+  __syncwarp(mask);
+  // pass 4: the slab masks of the obstacle slots; every lane builds its own
+  // words: the beads of each slab, then the running union
+  const int nhs = m + j1;
+  const int row = W * G;
+  for (int i = 0; i < 3 * (nsl + 1) * W; ++i) st.mask[i * G + gl] = 0u;
+  for (int s = gl; s < nhs; s += G) {
+    const float4 f = st.sh[s];
+    const int b = s / G;
+    unsigned *const w = st.mask + (b >> 5) * G + gl;
+    const unsigned bit = 1u << (b & 31);
+    w[(slab_of<DOM>(f.x, SL.inv0, SL.base, nsl) + 1) * row] |= bit;
+    w[(nsl + 1 + slab_of<DOM>(f.y, SL.inv1, SL.base, nsl) + 1) * row] |= bit;
+    w[(2 * (nsl + 1) + slab_of<DOM>(f.z, SL.inv2, SL.base, nsl) + 1) * row] |= bit;
+  }
+  for (int a = 0; a < 3; ++a)
+    for (int w = 0; w < W; ++w) {
+      unsigned acc = 0u;
+      unsigned *const q = st.mask + (a * (nsl + 1)) * row + w * G + gl;
+      for (int k = 1; k <= nsl; ++k) {
+        acc |= q[k * row];
+        q[k * row] = acc;
+      }
+    }
+  __syncwarp(mask);
   if (!live) m = 0;
 }
 #undef SYS
+
+// The obstacle in slot k went from slabs (o0, o1, o2) to (n0, n1, n2): its
+// bit flips in the rows between (called by lane k % G alone)
+__device__ __forceinline__ void slab_move(const Stage &st, int G, int W, int nsl, int k, int o0, int o1,
+                                          int o2, int n0, int n1, int n2) {
+  const int gl = k % G, b = k / G, row = W * G;
+  const unsigned bit = 1u << (b & 31);
+  unsigned *const w = st.mask + (b >> 5) * G + gl + row;
+  for (int i = min(o0, n0); i < max(o0, n0); ++i) w[i * row] ^= bit;
+  for (int i = min(o1, n1); i < max(o1, n1); ++i) w[(nsl + 1 + i) * row] ^= bit;
+  for (int i = min(o2, n2); i < max(o2, n2); ++i) w[(2 * (nsl + 1) + i) * row] ^= bit;
+}
 
 }  // namespace
 }  // namespace ecmc

@@ -1,0 +1,1002 @@
+// Event-chain kernel (arXiv:1502.06447, Sec. II: EC move, with hard tethers
+// or harmonic bead springs; Sec. II.A: tile-joint decomposition with
+// reflections; Sec. II.B: push-off; Sec. II.C: swap move).  Included by the
+// translation units that instantiate it.
+//
+// One group of G lanes (G = 32, 16, 8 or 4) runs the ECs of one tile, one
+// event per step; the 32 / G groups of a warp step together, and no warp
+// waits for another: there is no block barrier.  The state of an EC (pivot,
+// direction, what is left of ell) is held by every lane of its group, so a
+// step exchanges no more than the winning candidate.  A group whose tile has
+// run its ECs takes the next unit of the launch from a device counter and
+// stages it while the warp's other groups wait.
+//
+// A step:
+//   A  the obstacles the flight can reach come from the slab masks
+//      (ec_device.cuh), each lane its own words.  In the screened form (F32)
+//      a lane bounds its obstacles, a tether or a wall in FP32 and keeps
+//      those whose lower bound can reach the group's smallest upper bound U;
+//      in the plain form every reachable obstacle is kept;
+//   B  each lane evaluates what it kept in FP64 (exactly the definition's
+//      expressions); the group takes the smallest x under the tie rule;
+//   D  all lanes move the pivot, lift, reflect or swap.
+// A candidate left out by the screen cannot win: the winner's exact x is <= U
+// and every lower bound is <= its candidate's exact x, so both forms produce
+// the same events.
+//
+// What bounds it: the latency of one step.  A tile's events follow one
+// another, and a step is a chain of dependent FP64 operations (55-60 cycles
+// each), shared-memory and L1 round trips.
+#pragma once
+#include "ec_device.cuh"
+
+namespace ecmc {
+
+namespace {
+
+// argmin over the group by (x, key)
+template <int G>
+__device__ __forceinline__ void group_argmin(uint64_t &bx, uint64_t &bkey) {
+#pragma unroll
+  for (int off = G / 2; off > 0; off >>= 1) {
+    const uint64_t ox = __shfl_xor_sync(FULL, bx, off);
+    const uint64_t ok = __shfl_xor_sync(FULL, bkey, off);
+    if (ox < bx || (ox == bx && ok < bkey)) {
+      bx = ox;
+      bkey = ok;
+    }
+  }
+}
+
+#define SYS(f) (BATCH ? rp->f : P.f)
+
+// DOM: domain mode (else serial: one unit, the whole periodic box);
+// SPRING: harmonic bonds; PO: push-off (start beads and overlap rule)
+template <int G, bool F32, bool BATCH, bool DOM, bool SPRING, bool PO>
+__global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  // push-off run from the device: nothing to do once no bead overlaps
+  if (PO && P.po_count && *P.po_count == 0ull) return;
+  const int lane = threadIdx.x & 31;
+  const int gl = lane & (G - 1);
+  const int gbase = lane & ~(G - 1);
+  const unsigned gmask = (G == 32) ? FULL : (((1u << G) - 1) << gbase);
+  const int gib = threadIdx.x / G;
+  const int64_t sweep = P.sweep_dev ? *P.sweep_dev : P.sweep;
+  const int S = P.stage_cap, MNB = P.m_cap, M64 = P.m64, nsl = P.nsl;
+  const int W = (S + 32 * G - 1) / (32 * G);
+  const int row = W * G;
+  const int MQ = mask_quads(S, G, nsl);
+  Stage st = carve(smem + (size_t)gib * group_bytes(S, M64, MNB, MQ), S, M64, MNB, MQ);
+#ifdef ECMC_CHECKED
+  st.status = P.status;
+  st.nglob = P.n;
+#endif
+
+  // ------------------------------------------------------------ tile state
+  enum : int { TILE_NEED = 0, EC_NEED = 1, EC_RUN = 2, TILE_DONE = 3 };
+  int state = TILE_NEED;
+  const RepParams *rp = BATCH ? P.reps : nullptr;
+  int unit = 0, gunit = 0;
+  int m = 0, j1 = 0;
+  double *Rr = P.r;
+  int32_t *Ri = P.img;
+  uint64_t Rkey = P.replica;
+  const Slabs SL{P.sinv[0], P.sinv[1], P.sinv[2], slab_raw(P.sorg, P.sinv[0], 0), nsl};
+  double c0 = 0.0, c1 = 0.0, c2 = 0.0;
+  bool wr0 = true, wr1 = true, wr2 = true;
+  int n_ec = P.ecs_per_tile;
+
+  // ------------------------------------------------------------ EC state
+  int e = 0, p = 0, pid = 0;
+  unsigned nbw = 0xFFFFFFFFu;
+  int oslab = 0;  // slabs of the pivot's stored shadow, 10 bits per axis
+  double q0 = 0.0, q1 = 0.0, q2 = 0.0, v0 = 0.0, v1 = 0.0, v2 = 0.0, xrem = 0.0, lift = 0.0;
+  float pf0 = 0.f, pf1 = 0.f, pf2 = 0.f, vf0 = 0.f, vf1 = 0.f, vf2 = 0.f;
+  int64_t nev = 0;
+  unsigned ncontact = 0, swgo = 0;  // swap proposals of this and the next contacts, one bit each
+  uint64_t h = 0;
+  // springs: the Boltzmann energies of the next G / 2 events, drawn together
+  double dE = 0.0;
+  int dE_at = 0;
+
+  double lift_all = 0.0, refl_all = 0.0;
+  unsigned long long tried = 0, confirmed = 0, nev_all = 0, ecs_done = 0;
+  unsigned exh = 0;
+  // events by outcome: eight 8-bit fields, added to the counters every 255
+  // events and at the end
+  uint64_t ev_pk = 0;
+  unsigned ev_pn = 0;
+  auto flush_outcomes = [&]() {
+#pragma unroll
+    for (int k = 0; k < ECMC_NEV; ++k) {
+      const unsigned c = (unsigned)(ev_pk >> (8 * k)) & 0xFFu;
+      if (c) atomicAdd(&P.counters[k], (unsigned long long)c);
+    }
+    ev_pk = 0;
+    ev_pn = 0;
+  };
+
+  Screen Z;
+  Z.sig2f = (float)P.sig2;
+  Z.eps_v = P.eps_v;
+  Z.eps_d = P.eps_d;
+  const float b2f = (float)P.b2;
+  const float eps_v = P.eps_v, eps_d = P.eps_d;
+  const float reach_hs = (float)P.sigma + 2.f * eps_v;  // per-axis reach of a contact
+  const float INF = __int_as_float(0x7f800000);
+  constexpr int ITEMS = G >= 8 ? 1 : 2;  // special candidates per lane
+  const uint64_t r1 = DOM ? (uint64_t)sweep : 0;
+
+  auto slabs_at = [&](float f0, float f1, float f2) {
+    return slab_of<DOM>(f0, SL.inv0, SL.base, nsl) | (slab_of<DOM>(f1, SL.inv1, SL.base, nsl) << 10) |
+           (slab_of<DOM>(f2, SL.inv2, SL.base, nsl) << 20);
+  };
+  // the FP32 shadow of an FP64 position: FP32 position minus FP32 corner
+  auto shadow = [&](double x, double c, double L, bool wr) {
+    if (!DOM) return (float)x;
+    float f = (float)x - (float)c;
+    if (wr) {
+      const float Lf = (float)L, Lh = 0.5f * Lf;
+      f = f > Lh ? f - Lf : (f < -Lh ? f + Lf : f);
+    }
+    return f;
+  };
+  // The bead in slot k sits at (x, y, z) now: FP64 position (write-through),
+  // shadow and slab masks.  A pivot never screens itself, so its copies are
+  // brought up to date only when it stops being the pivot.
+  auto settle = [&](int k, int id, double x, double y, double z, float f0, float f1, float f2, int os) {
+    if (gl < 3) Rr[3 * (int64_t)id + gl] = gl == 0 ? x : (gl == 1 ? y : z);
+    if (gl == (k & (G - 1))) {
+      if (k < M64) {
+        st.px[k] = x;
+        st.py[k] = y;
+        st.pz[k] = z;
+      }
+      st.sh[k] = make_float4(f0, f1, f2, __int_as_float(id));
+      const int nw = slabs_at(f0, f1, f2);
+      if (nw != os)
+        slab_move(st, G, W, nsl, k, os & 1023, (os >> 10) & 1023, os >> 20, nw & 1023,
+                  (nw >> 10) & 1023, nw >> 20);
+    }
+  };
+
+  // take the next unit and stage it (group-collective); false when none left
+  auto take_tile = [&]() -> bool {
+    int u = 0;
+    if (gl == 0) {
+      u = atomicAdd(P.unit_next, 1);
+      if (P.defer_mode == 2) u = u < *P.n_deferred ? P.deferred[u] : P.n_units;
+    }
+    u = __shfl_sync(gmask, u, gbase);
+    if (u >= P.n_units) return false;
+    gunit = u;
+    unit = u;
+    if (BATCH) {
+      int lo = 0, hi = P.n_reps - 1;
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (P.reps[mid].unit_off <= u) lo = mid;
+        else hi = mid - 1;
+      }
+      rp = P.reps + lo;
+      unit = u - (int)rp->unit_off;
+      Rr = P.r + 3 * rp->bead_off;
+      Ri = P.img + 3 * rp->bead_off;
+      Rkey = rp->replica;
+#ifdef ECMC_CHECKED
+      st.nglob = rp->n_beads;
+#endif
+    }
+    const int32_t *const Rstart = BATCH ? P.cstart + rp->cell_off : P.cstart;
+    if (DOM) {
+      const int tk0 = unit % SYS(D)[0];
+      const int tk1 = (unit / SYS(D)[0]) % SYS(D)[1];
+      const int tk2 = unit / (SYS(D)[0] * SYS(D)[1]);
+      const u64x4 w = philox(TAG_SHIFT, (uint64_t)sweep, 0, 0, P.seed, Rkey);
+      c0 = unit53(w.v[0]) * SYS(T)[0] + (double)tk0 * SYS(T)[0];
+      c1 = unit53(w.v[1]) * SYS(T)[1] + (double)tk1 * SYS(T)[1];
+      c2 = unit53(w.v[2]) * SYS(T)[2] + (double)tk2 * SYS(T)[2];
+      // A tile whose halo lies inside (0, L) on an axis never needs the
+      // minimum image or a wrap on that axis: every position it touches
+      // stays in one periodic image.
+      wr0 = !(c0 - P.halo_te > 0.0 && c0 + SYS(W)[0] + P.halo_te < SYS(L)[0]);
+      wr1 = !(c1 - P.halo_te > 0.0 && c1 + SYS(W)[1] + P.halo_te < SYS(L)[1]);
+      wr2 = !(c2 - P.halo_te > 0.0 && c2 + SYS(W)[2] + P.halo_te < SYS(L)[2]);
+    }
+    bool live = true, over = false;
+    int ns = 0;
+    stage_tile<G, DOM, SPRING, BATCH>(P, rp, st, gl, live, unit, c0, c1, c2, Rr, Rstart, S, M64, MNB, W,
+                                      SL, m, j1, ns, gmask, P.defer_mode == 1 ? &over : nullptr);
+    if (over && gl == 0) {
+      const int at = atomicAdd(P.n_deferred, 1);
+      P.deferred[CI(at, P.n_units, 32, P.status)] = gunit;
+    }
+    if (PO) {
+      // push-off: one EC from every flagged motile bead, in id order
+      int f = 0;
+      for (int s = gl; s < m; s += G) f += P.po_flag[__float_as_int(st.sh[s].w)] ? 1 : 0;
+#pragma unroll
+      for (int off = G / 2; off > 0; off >>= 1) f += __shfl_xor_sync(gmask, f, off);
+      n_ec = f;
+    }
+    e = 0;
+    return true;
+  };
+
+  // start EC e of the tile: start bead and direction (Sec. II, R6)
+  auto start_ec = [&]() {
+    const uint64_t r0 = DOM ? (TAG_START | ((uint64_t)e << 8)) : TAG_START;
+    const uint64_t r2 = DOM ? (uint64_t)unit : (uint64_t)(sweep + e);
+    u64x4 w = philox(r0, r1, r2, 0, P.seed, Rkey);
+    p = (int)scale_below(w.v[0], (uint64_t)m);
+    if (PO) {
+      // the e-th flagged motile slot (slots are in id order)
+      int before = 0;
+      for (int s0 = 0; s0 < m; s0 += G) {
+        const int s = s0 + gl;
+        const bool f = s < m && P.po_flag[__float_as_int(st.sh[s].w)];
+        const unsigned bal = (__ballot_sync(gmask, f) & gmask) >> gbase;
+        const int c = __popc(bal);
+        if (e < before + c) {
+          p = s0 + (int)__fns(bal, 0, e - before + 1);
+          break;
+        }
+        before += c;
+      }
+    }
+    if (P.dir_mode == ECMC_DIR_CART3) {
+      const int ax = (int)scale_below(w.v[1], 3);
+      v0 = ax == 0 ? 1.0 : 0.0;
+      v1 = ax == 1 ? 1.0 : 0.0;
+      v2 = ax == 2 ? 1.0 : 0.0;
+    } else {
+      double a = 2.0 * unit53(w.v[1]) - 1.0;
+      double b = 2.0 * unit53(w.v[2]) - 1.0;
+      double c = 2.0 * unit53(w.v[3]) - 1.0;
+      uint64_t att = 0;
+      double s;
+      for (;;) {
+        s = a * a + b * b + c * c;
+        if (s > 1e-6 && s <= 1.0) break;
+        ++att;
+        w = philox(r0, r1, r2, att, P.seed, Rkey);
+        a = 2.0 * unit53(w.v[0]) - 1.0;
+        b = 2.0 * unit53(w.v[1]) - 1.0;
+        c = 2.0 * unit53(w.v[2]) - 1.0;
+      }
+      // one component per lane
+      const double t = ((gl & 3) == 0 ? a : ((gl & 3) == 1 ? b : c)) / sqrt(s);
+      v0 = __shfl_sync(gmask, t, gbase);
+      v1 = __shfl_sync(gmask, t, gbase + 1);
+      v2 = __shfl_sync(gmask, t, gbase + 2);
+    }
+    p = CI(p, m, 10, P.status);
+    const float4 f = st.sh[p];
+    pid = CI(__float_as_int(f.w), BATCH ? rp->n_beads : P.n, 11, P.status);
+    pos64(st, Rr, p, M64, q0, q1, q2);
+    nbw = st.nb[p];
+    pf0 = f.x;
+    pf1 = f.y;
+    pf2 = f.z;
+    oslab = slabs_at(pf0, pf1, pf2);
+    vf0 = (float)v0;
+    vf1 = (float)v1;
+    vf2 = (float)v2;
+    xrem = P.ell;
+    lift = 0.0;
+    nev = 0;
+    ncontact = 0;
+    if (SPRING) dE_at = G / 2;  // draw at the first event
+    h = 0xCBF29CE484222325ull;
+  };
+
+  // ------------------------------------------------------------ steps
+  for (;;) {
+    if (__any_sync(FULL, state != EC_RUN)) {
+      if (state == TILE_NEED) {
+        // (tiles without motile beads have no ECs and are passed over)
+        for (;;) {
+          if (!take_tile()) {
+            state = TILE_DONE;
+            break;
+          }
+          if (m > 0 && n_ec > 0) {
+            state = EC_NEED;
+            break;
+          }
+        }
+      }
+      if (state == EC_NEED) {
+        start_ec();
+        state = EC_RUN;
+      }
+      __syncwarp();
+      if (!__any_sync(FULL, state == EC_RUN)) break;
+    }
+    const bool act = state == EC_RUN;
+
+    // ---------------------------------------------------------- A: screen
+    // what the flight ends with at the latest
+    const bool pass = dbits(P.s_cap) < dbits(xrem);
+    const float xc = act ? (pass ? P.s_cap_f : __double2float_ru(xrem)) : 0.f;
+    float ubl = xc;
+    uint64_t lx = ~0ull, lkey = ~0ull;  // this lane's best evaluated candidate
+    double ldv = 0.0;
+    int spk[ITEMS], sps[ITEMS];
+    float spl[ITEMS];
+    if (SPRING) {
+      // energies for the next G / 2 events of every group's EC: lane
+      // 2 i + j draws bond j of event nev + i, so that the draw and the
+      // logarithm (some 50 dependent FP64 operations) are paid for once per
+      // G / 2 events.  All groups draw when one has used up its own.
+      if (__any_sync(FULL, act && dE_at == G / 2)) {
+        const uint64_t r2 = DOM ? (uint64_t)unit : (uint64_t)(sweep + e);
+        const u64x4 w = philox(TAG_SPRING | ((uint64_t)(DOM ? e : 0) << 8), r1, r2,
+                               (uint64_t)(nev + (gl >> 1)), P.seed, Rkey);
+        dE = spring_dE((gl & 1) ? w.v[1] : w.v[0]);
+        dE_at = 0;
+      }
+      // lane 1: the bond to the previous bead, lane 2: to the next
+      const double my_dE = __shfl_sync(FULL, dE, gbase + 2 * dE_at + (gl == 2 ? 1 : 0));
+      ++dE_at;
+      if (act && (gl == 1 || gl == 2)) {
+        int t = gl == 1 ? nb_prev(nbw) : nb_next(nbw);
+        if (t >= 0) {
+          t = CI(t, S, 20, P.status);
+          double kx, ky, kz;
+          pos64(st, Rr, t, M64, kx, ky, kz);
+          // (a spring partner may lie beyond the tile's halo, across the
+          // periodic boundary: always the minimum image)
+          const double x =
+              spring_x(wrap_i(q0 - kx, SYS(L)[0], dbits(SYS(half)[0])), wrap_i(q1 - ky, SYS(L)[1], dbits(SYS(half)[1])),
+                       wrap_i(q2 - kz, SYS(L)[2], dbits(SYS(half)[2])), v0, v1, v2, P.sigma, P.k_spring, my_dE, ldv);
+          lx = dbits(x);
+          lkey = make_key(KIND_TETHER, __float_as_int(st.sh[t].w), t);
+          ubl = fminf(ubl, __double2float_ru(x));
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+      spk[r] = -1;
+      sps[r] = 0;
+      spl[r] = 0.f;
+      const int it = gl + r * G;
+      if (!act || it == 0 || it >= 6) continue;
+      if (it <= 2) {
+        if (SPRING) continue;
+        int t = it == 1 ? nb_prev(nbw) : nb_next(nbw);
+        if (t < 0) continue;
+        t = CI(t, S, 20, P.status);
+        if (F32) {
+          const float4 f = st.sh[t];
+          float d0 = pf0 - f.x, d1 = pf1 - f.y, d2 = pf2 - f.z;
+          if (!DOM) {
+            d0 = wrapf(d0, (float)P.L[0]);
+            d1 = wrapf(d1, (float)P.L[1]);
+            d2 = wrapf(d2, (float)P.L[2]);
+          }
+          const float dd = __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, d0 * d0));
+          const float dv = __fmaf_rn(d2, vf2, __fmaf_rn(d1, vf1, d0 * vf0));
+          const float rad = b2f - (dd - dv * dv);
+          const float lo = -dv - eps_v + sqrt_lo(fmaxf(rad - eps_d, 0.f));
+          const float hi = -dv + eps_v + sqrt_hi(fmaxf(rad + eps_d, 0.f));
+          spl[r] = fmaxf(lo, 0.f);
+          ubl = fminf(ubl, fmaxf(hi, 0.f) + 1e-6f);
+        }
+        spk[r] = KIND_TETHER;
+        sps[r] = t;
+      } else if (DOM) {
+        const int a = it - 3;
+        const float vfa = a == 0 ? vf0 : (a == 1 ? vf1 : vf2);
+        const double va = a == 0 ? v0 : (a == 1 ? v1 : v2);
+        if (!nonzero(va)) continue;
+        if (F32) {
+          const float pfa = a == 0 ? pf0 : (a == 1 ? pf1 : pf2);
+          const float dist = signbit(vfa) ? pfa : (float)SYS(W)[a] - pfa;
+          const float av = fabsf(vfa);
+          if (av >= 1e-30f) {
+            spl[r] = div_lo(fmaxf(dist - eps_v, 0.f), av);
+            ubl = fminf(ubl, div_hi(fmaxf(dist, 0.f) + eps_v, av));
+          }  // else |v_a| below FP32 range: evaluate in FP64
+        }
+        spk[r] = KIND_WALL;
+        sps[r] = a;
+      }
+    }
+    // the slabs of the box that holds every obstacle in reach: within sigma
+    // (plus the screen's margin) of the path [pf, pf + xc vf] on every axis
+    const float e0 = xc * vf0, e1 = xc * vf1, e2 = xc * vf2;
+    const unsigned *wa0, *wa1, *wa2, *wb0, *wb1, *wb2;
+    bool fl0 = false, fl1 = false, fl2 = false;  // serial: the range goes around the box
+    {
+      const float l0 = pf0 - reach_hs + fminf(e0, 0.f), h0 = pf0 + reach_hs + fmaxf(e0, 0.f);
+      const float l1 = pf1 - reach_hs + fminf(e1, 0.f), h1 = pf1 + reach_hs + fmaxf(e1, 0.f);
+      const float l2 = pf2 - reach_hs + fminf(e2, 0.f), h2 = pf2 + reach_hs + fmaxf(e2, 0.f);
+      int a0 = slab_raw(l0, SL.inv0, SL.base), b0 = slab_raw(h0, SL.inv0, SL.base);
+      int a1 = slab_raw(l1, SL.inv1, SL.base), b1 = slab_raw(h1, SL.inv1, SL.base);
+      int a2 = slab_raw(l2, SL.inv2, SL.base), b2 = slab_raw(h2, SL.inv2, SL.base);
+      if (DOM) {
+        a0 = min(max(a0, 0), nsl - 1);
+        b0 = min(max(b0, 0), nsl - 1);
+        a1 = min(max(a1, 0), nsl - 1);
+        b1 = min(max(b1, 0), nsl - 1);
+        a2 = min(max(a2, 0), nsl - 1);
+        b2 = min(max(b2, 0), nsl - 1);
+      } else {
+        // the range [a, b] of slabs around the box; nsl or more: all of them
+        auto around = [&](int &a, int &b, bool &fl) {
+          if (b - a >= nsl - 1) {
+            a = 0;
+            b = nsl - 1;
+            return;
+          }
+          if (a < 0) a += nsl;
+          else if (a >= nsl) a -= nsl;
+          if (b < 0) b += nsl;
+          else if (b >= nsl) b -= nsl;
+          fl = a > b;
+        };
+        around(a0, b0, fl0);
+        around(a1, b1, fl1);
+        around(a2, b2, fl2);
+      }
+      const unsigned *const mk = st.mask + gl;
+      wa0 = mk + a0 * row;
+      wb0 = mk + (b0 + 1) * row;
+      wa1 = mk + (nsl + 1 + a1) * row;
+      wb1 = mk + (nsl + 2 + b1) * row;
+      wa2 = mk + (2 * (nsl + 1) + a2) * row;
+      wb2 = mk + (2 * (nsl + 1) + b2 + 1) * row;
+    }
+    // this lane's word w of the obstacles in the box, the pivot left out
+    auto cand_word = [&](int w) -> unsigned {
+      const int o = w * G;
+      unsigned c;
+      if (DOM) {
+        c = (wb0[o] & ~wa0[o]) & (wb1[o] & ~wa1[o]) & (wb2[o] & ~wa2[o]);
+      } else {
+        const unsigned all = st.mask[gl + nsl * row + o];
+        c = (fl0 ? wb0[o] | ~wa0[o] : wb0[o] & ~wa0[o]) & (fl1 ? wb1[o] | ~wa1[o] : wb1[o] & ~wa1[o]) &
+            (fl2 ? wb2[o] | ~wa2[o] : wb2[o] & ~wa2[o]) & all;
+      }
+      if (gl == (p & (G - 1)) && (p / G) >> 5 == w) c &= ~(1u << ((p / G) & 31));
+      return act ? c : 0u;
+    };
+    // exact evaluation of a contact or tether with slot k
+    auto exact = [&](int k, bool te) {
+      double kx, ky, kz, dv;
+      pos64(st, Rr, k, M64, kx, ky, kz);
+      const double x =
+          quad_x(te, wrapc(q0 - kx, SYS(L)[0], dbits(SYS(half)[0]), wr0), wrapc(q1 - ky, SYS(L)[1], dbits(SYS(half)[1]), wr1),
+                 wrapc(q2 - kz, SYS(L)[2], dbits(SYS(half)[2]), wr2), v0, v1, v2, te ? P.b2 : P.sig2, dv, PO);
+      if (F32) ++confirmed;
+      if (neg(x)) return;
+      const uint64_t key = make_key(te ? KIND_TETHER : KIND_HS, __float_as_int(st.sh[k].w), k);
+      const uint64_t xb = dbits(x);
+      if (xb < lx || (xb == lx && key < lkey)) {
+        lx = xb;
+        lkey = key;
+        ldv = dv;
+      }
+    };
+
+    bool all_fp64 = !F32;  // evaluate every obstacle in the box
+    if (F32) {
+      int ks0 = -1, ks1 = -1;
+      float kl0 = INF, kl1 = INF;
+      bool kovf = false;
+      int nscr = 0;
+      for (int w = 0; w < W; ++w) {
+        unsigned c = cand_word(w);
+        nscr += __popc(c);
+        // two obstacles per round, so that their loads overlap
+        while (c) {
+          const int ka = CI(((w << 5) + __ffs(c) - 1) * G + gl, S, 21, P.status);
+          c &= c - 1;
+          const bool two = c != 0;
+          const int kb = two ? CI(((w << 5) + __ffs(c) - 1) * G + gl, S, 21, P.status) : ka;
+          c &= c - 1;
+          const float4 fa = st.sh[ka], fb = st.sh[kb];
+          float a0 = pf0 - fa.x, a1 = pf1 - fa.y, a2 = pf2 - fa.z;
+          float b0 = pf0 - fb.x, b1 = pf1 - fb.y, b2 = pf2 - fb.z;
+          if (!DOM) {
+            a0 = wrapf(a0, (float)P.L[0]);
+            a1 = wrapf(a1, (float)P.L[1]);
+            a2 = wrapf(a2, (float)P.L[2]);
+            b0 = wrapf(b0, (float)P.L[0]);
+            b1 = wrapf(b1, (float)P.L[1]);
+            b2 = wrapf(b2, (float)P.L[2]);
+          }
+          screen_hs(Z, a0, a1, a2, vf0, vf1, vf2, ka, ubl, ks0, kl0, ks1, kl1, kovf);
+          if (two) screen_hs(Z, b0, b1, b2, vf0, vf1, vf2, kb, ubl, ks0, kl0, ks1, kl1, kovf);
+        }
+      }
+      const float U = group_minf<G>(ubl);
+      bool t0 = spk[0] == KIND_TETHER && spl[0] <= U;
+      bool t1 = ITEMS > 1 && spk[ITEMS - 1] == KIND_TETHER && spl[ITEMS - 1] <= U;
+      bool w0 = spk[0] == KIND_WALL && spl[0] <= U;
+      bool w1 = ITEMS > 1 && spk[ITEMS - 1] == KIND_WALL && spl[ITEMS - 1] <= U;
+      bool h0 = ks0 >= 0 && kl0 <= U, h1 = ks1 >= 0 && kl1 <= U;
+      if (P.rq_per_tile < 6) {
+        // a small request_cap sends tiles with more survivors than that (or
+        // more than 8 per request in reach) to the exhaustive evaluation
+        int ns = (t0 || w0) + (t1 || w1) + h0 + h1;
+#pragma unroll
+        for (int off = G / 2; off > 0; off >>= 1) {
+          ns += __shfl_xor_sync(FULL, ns, off);
+          nscr += __shfl_xor_sync(FULL, nscr, off);
+        }
+        all_fp64 = act && (ns > P.rq_per_tile || nscr > 8 * P.rq_per_tile);
+        if (all_fp64) {
+          if (gl == 0) ++exh;
+          h0 = h1 = kovf = false;
+          t0 = spk[0] == KIND_TETHER;
+          t1 = ITEMS > 1 && spk[ITEMS - 1] == KIND_TETHER;
+          w0 = spk[0] == KIND_WALL;
+          w1 = ITEMS > 1 && spk[ITEMS - 1] == KIND_WALL;
+        }
+      }
+      spk[0] = w0 ? KIND_WALL : -1;
+      if (ITEMS > 1) spk[ITEMS - 1] = w1 ? KIND_WALL : -1;
+      // ---------------------------------------------------------- B: FP64
+      // a lane rarely holds more than one survivor
+      while (__any_sync(FULL, t0 || t1 || h0 || h1)) {
+        if (t0 || t1 || h0 || h1) {
+          const bool te = t0 || t1;
+          const int k = t0 ? sps[0] : (t1 ? sps[ITEMS - 1] : (h0 ? ks0 : ks1));
+          if (t0) t0 = false;
+          else if (t1) t1 = false;
+          else if (h0) h0 = false;
+          else h1 = false;
+          exact(k, te);
+        }
+      }
+      if (__any_sync(FULL, kovf)) {
+        if (kovf && act) {
+          // more than two possible winners in this lane: screen its obstacles
+          // again against the group's U and evaluate every one that can reach it
+          for (int w = 0; w < W; ++w) {
+            unsigned c = cand_word(w);
+            while (c) {
+              const int k = CI(((w << 5) + __ffs(c) - 1) * G + gl, S, 22, P.status);
+              c &= c - 1;
+              if (k == ks0 || k == ks1) continue;
+              const float4 f = st.sh[k];
+              float d0 = pf0 - f.x, d1 = pf1 - f.y, d2 = pf2 - f.z;
+              if (!DOM) {
+                d0 = wrapf(d0, (float)P.L[0]);
+                d1 = wrapf(d1, (float)P.L[1]);
+                d2 = wrapf(d2, (float)P.L[2]);
+              }
+              bool possible;
+              const float lb = screen_lb(Z, d0, d1, d2, vf0, vf1, vf2, possible);
+              if (possible && lb <= U) exact(k, false);
+            }
+          }
+        }
+        __syncwarp();
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < ITEMS; ++r)
+        if (spk[r] == KIND_TETHER) exact(sps[r], true);
+    }
+    if (!F32 || P.rq_per_tile < 6) {
+      if (all_fp64) {
+        for (int w = 0; w < W; ++w) {
+          unsigned c = cand_word(w);
+          while (c) {
+            const int k = CI(((w << 5) + __ffs(c) - 1) * G + gl, S, 23, P.status);
+            c &= c - 1;
+            exact(k, false);
+          }
+        }
+      }
+      __syncwarp();
+    }
+    if (DOM) {
+      bool wall = spk[0] == KIND_WALL;
+      if (ITEMS > 1) wall = wall || spk[ITEMS - 1] == KIND_WALL;
+      if (__any_sync(FULL, wall)) {
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) {
+          if (spk[r] != KIND_WALL) continue;
+          const int a = sps[r];
+          const double va = a == 0 ? v0 : (a == 1 ? v1 : v2);
+          const double qa = a == 0 ? q0 : (a == 1 ? q1 : q2);
+          const double ca = a == 0 ? c0 : (a == 1 ? c1 : c2);
+          const double loc = wrapc(qa - ca, SYS(L)[a], dbits(SYS(half)[a]), a == 0 ? wr0 : (a == 1 ? wr1 : wr2));
+          double x = (posv(va) ? SYS(W)[a] - loc : 0.0 - loc) / va;
+          if (neg(x)) x = 0.0;
+          if (F32) ++confirmed;
+          const uint64_t key = make_key(KIND_WALL, a, 0);
+          const uint64_t xb = dbits(x);
+          if (xb < lx || (xb == lx && key < lkey)) {
+            lx = xb;
+            lkey = key;
+          }
+        }
+        __syncwarp();
+      }
+    }
+    // ---------------- winner of the group and its pre-flight d.v
+    const unsigned has = __ballot_sync(FULL, lkey != ~0ull) & gmask;
+    uint64_t wx = lx, wkey = lkey;
+    int src = __ffs(has) - 1;
+    if (src < 0) src = lane;
+    if (__any_sync(FULL, (has & (has - 1)) != 0)) {
+      group_argmin<G>(wx, wkey);
+      const unsigned own = __ballot_sync(FULL, lkey == wkey && lx == wx) & gmask;
+      src = __ffs(own) - 1;
+    } else {
+      wx = __shfl_sync(FULL, lx, src);
+      wkey = __shfl_sync(FULL, lkey, src);
+    }
+    const double wdv = __shfl_sync(FULL, ldv, src);
+
+    // ---------------------------------------------------------- D: move
+    if (act && nev >= P.event_cap) {
+      if (gl == 0) set_status(P.status, DEV_STUCK);
+      settle(p, pid, q0, q1, q2, pf0, pf1, pf2, oslab);
+      state = EC_NEED;
+    }
+    if (state == EC_RUN) {
+      double x = pass ? P.s_cap : xrem;
+      int kind = pass ? KIND_PASS : KIND_END, slot = 0;
+      int64_t partner = -1;
+      if (wx < dbits(x)) {  // (END and PASS win ties)
+        x = __longlong_as_double((long long)wx);
+        kind = key_kind(wkey);
+        slot = key_slot(wkey);
+        partner = key_id(wkey);
+      }
+      const bool bead = kind >= KIND_HS;
+      double k0 = 0.0, k1 = 0.0, k2 = 0.0;
+      if (bead) pos64(st, Rr, CI(slot, S, 30, P.status), M64, k0, k1, k2);
+      int di0 = 0, di1 = 0, di2 = 0;
+      if (wr0) di0 = step_i(q0, x, v0, SYS(L)[0]);
+      else q0 = __fma_rn(x, v0, q0);
+      if (wr1) di1 = step_i(q1, x, v1, SYS(L)[1]);
+      else q1 = __fma_rn(x, v1, q1);
+      if (wr2) di2 = step_i(q2, x, v2, SYS(L)[2]);
+      else q2 = __fma_rn(x, v2, q2);
+      if (gl == 0 && (di0 | di1 | di2)) {
+        if (di0) Ri[3 * (int64_t)pid] += di0;
+        if (di1) Ri[3 * (int64_t)pid + 1] += di1;
+        if (di2) Ri[3 * (int64_t)pid + 2] += di2;
+      }
+      ++nev;
+      int out = kind == KIND_END ? ECMC_EV_END : (kind == KIND_PASS ? ECMC_EV_PASS : ECMC_EV_WALL);
+      int np = p;
+      bool swapped = false;
+      if (kind == KIND_WALL) {
+        // (negation is exact in both precisions)
+        if (partner == 0) {
+          v0 = -v0;
+          vf0 = -vf0;
+        } else if (partner == 1) {
+          v1 = -v1;
+          vf1 = -vf1;
+        } else {
+          v2 = -v2;
+          vf2 = -vf2;
+        }
+      } else if (bead) {
+        // (r_target - r_pivot).v at contact = -(d.v) - x
+        const double proj = -wdv - x;
+        const bool hs = kind == KIND_HS;
+        if (slot >= m) {  // immotile: reflect
+          out = hs ? ECMC_EV_HS_REFLECT : ECMC_EV_TE_REFLECT;
+          refl_all = refl_all + proj;
+          const bool sp = SPRING && !hs;
+          mirror2(v0, v1, v2, wrapc(q0 - k0, SYS(L)[0], dbits(SYS(half)[0]), wr0 || sp),
+                  wrapc(q1 - k1, SYS(L)[1], dbits(SYS(half)[1]), wr1 || sp),
+                  wrapc(q2 - k2, SYS(L)[2], dbits(SYS(half)[2]), wr2 || sp));
+          vf0 = (float)v0;
+          vf1 = (float)v1;
+          vf2 = (float)v2;
+        } else {
+          lift = lift + proj;
+          out = hs ? ECMC_EV_HS_LIFT : ECMC_EV_TE_LIFT;
+          np = slot;
+          if (!SPRING && !PO && hs && P.swap_mode) {
+            bool go = true;
+            if (P.swap_mode != 1) {
+              // the proposals of the next 4 min(G, 8) contacts, drawn
+              // together: lane j draws the four of counter word ncontact/4 + j
+              constexpr int NB = G < 8 ? 16 : 32;
+              if ((ncontact & (NB - 1)) == 0) {
+                const uint64_t r2 = DOM ? (uint64_t)unit : (uint64_t)(sweep + e);
+                const u64x4 w = philox(TAG_SWAP | ((uint64_t)(DOM ? e : 0) << 8), r1, r2,
+                                       (uint64_t)((ncontact >> 2) + (gl & (NB / 4 - 1))), P.seed, Rkey);
+                unsigned g4 = 0;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) g4 |= ((w.v[i] >> 11) < P.swap_thr ? 1u : 0u) << i;
+                swgo = 0;
+#pragma unroll
+                for (int j = 0; j < NB / 4; ++j) swgo |= __shfl_sync(gmask, g4, gbase + j) << (4 * j);
+              }
+              go = (swgo >> (ncontact & (NB - 1))) & 1u;
+              ++ncontact;
+            }
+            if (go) {
+              ++tried;
+              // every bond of both beads, positions exchanged, within b_max
+              bool ok = true;
+              const unsigned nbs = st.nb[slot];
+#pragma unroll
+              for (int side = 0; side < 2; ++side) {
+                const double a0 = side == 0 ? k0 : q0;
+                const double a1 = side == 0 ? k1 : q1;
+                const double a2 = side == 0 ? k2 : q2;
+                const unsigned nbv = side == 0 ? nbw : nbs;
+#pragma unroll
+                for (int dir = 0; dir < 2; ++dir) {
+                  const int b = dir == 0 ? nb_prev(nbv) : nb_next(nbv);
+                  if (b < 0) continue;
+                  double b0, b1, b2;
+                  if (b == p) {
+                    b0 = k0;
+                    b1 = k1;
+                    b2 = k2;
+                  } else if (b == slot) {
+                    b0 = q0;
+                    b1 = q1;
+                    b2 = q2;
+                  } else {
+                    pos64(st, Rr, b, M64, b0, b1, b2);
+                  }
+                  const double f0 = wrapc(a0 - b0, SYS(L)[0], dbits(SYS(half)[0]), wr0);
+                  const double f1 = wrapc(a1 - b1, SYS(L)[1], dbits(SYS(half)[1]), wr1);
+                  const double f2 = wrapc(a2 - b2, SYS(L)[2], dbits(SYS(half)[2]), wr2);
+                  const double dd = __fma_rn(f2, f2, __fma_rn(f1, f1, f0 * f0));
+                  ok = ok && !(dbits(dd) > dbits(P.b2));
+                }
+              }
+              if (ok) {
+                swapped = true;
+                out = ECMC_EV_SWAP;
+                np = p;
+                const float4 f = st.sh[slot];
+                const int kid = __float_as_int(f.w);
+                settle(slot, kid, q0, q1, q2, shadow(q0, c0, SYS(L)[0], wr0), shadow(q1, c1, SYS(L)[1], wr1),
+                       shadow(q2, c2, SYS(L)[2], wr2), slabs_at(f.x, f.y, f.z));
+                if (gl == 0) {
+#pragma unroll
+                  for (int a = 0; a < 3; ++a) {
+                    const int ti = Ri[3 * (int64_t)pid + a];
+                    Ri[3 * (int64_t)pid + a] = Ri[3 * (int64_t)kid + a];
+                    Ri[3 * (int64_t)kid + a] = ti;
+                  }
+                }
+                q0 = k0;
+                q1 = k1;
+                q2 = k2;
+              }
+            }
+          }
+        }
+      }
+      ev_pk += 1ull << (8 * out);
+      if (++ev_pn == 255) {
+        if (gl == 0) flush_outcomes();
+        ev_pk = 0;
+        ev_pn = 0;
+      }
+      pf0 = shadow(q0, c0, SYS(L)[0], wr0);
+      pf1 = shadow(q1, c1, SYS(L)[1], wr1);
+      pf2 = shadow(q2, c2, SYS(L)[2], wr2);
+      if (P.rec_digest) {
+        fnv_mix(h, (uint64_t)pid);
+        fnv_mix(h, ((uint64_t)(uint32_t)out << 32) | (uint64_t)(uint32_t)partner);
+        fnv_mix(h, dbits(x));
+      }
+      if (P.log && gl == 0) {
+        const unsigned long long at = atomicAdd(P.log_n, 1ull);
+        if ((int64_t)at < P.log_cap) {
+          ecmc_event ev;
+          ev.unit = P.rec_offset + (P.sweep_dev ? (sweep - P.rec_sweep0) * P.n_units * P.ecs_per_tile : 0) +
+                    (DOM ? (int64_t)gunit * P.ecs_per_tile + e : (int64_t)e);
+          ev.seq = (int32_t)(nev - 1);
+          ev.pivot = pid;
+          ev.kind = out;
+          ev.pad = 0;
+          ev.partner = partner;
+          ev.x = x;
+          P.log[at] = ev;
+        }
+      }
+      xrem = xrem - x;
+      if (out == ECMC_EV_END || np != p) settle(p, pid, q0, q1, q2, pf0, pf1, pf2, oslab);
+      if (out == ECMC_EV_END) state = EC_NEED;
+      if (np != p) {
+        // lift: the partner (motile, unmoved this event) becomes the pivot
+        p = np;
+        const float4 f = st.sh[p];
+        pid = CI(__float_as_int(f.w), BATCH ? rp->n_beads : P.n, 31, P.status);
+        nbw = st.nb[p];
+        q0 = k0;
+        q1 = k1;
+        q2 = k2;
+        pf0 = f.x;
+        pf1 = f.y;
+        pf2 = f.z;
+        oslab = slabs_at(pf0, pf1, pf2);
+      }
+    }
+    if (act && state == EC_NEED) {
+      // end of an EC: records, then the tile's next EC or a new tile
+      lift_all = lift_all + lift;
+      nev_all += (unsigned long long)nev;
+      ++ecs_done;
+      if (gl == 0 && P.rec_digest) {
+        const int64_t idx = P.rec_offset +
+                            (P.sweep_dev ? (sweep - P.rec_sweep0) * P.n_units * P.ecs_per_tile : 0) +
+                            (DOM ? (int64_t)gunit * P.ecs_per_tile + e : (int64_t)e);
+        if (idx < P.rec_cap) {
+          P.rec_digest[idx] = h;
+          P.rec_lift[idx] = lift;
+          P.rec_events[idx] = nev;
+        }
+      }
+      ++e;
+      if (e >= n_ec) state = TILE_NEED;
+    }
+    __syncwarp();
+  }
+
+  // ------------------------------------------------------------ counters
+  if (F32) {
+#pragma unroll
+    for (int off = G / 2; off > 0; off >>= 1) confirmed += __shfl_xor_sync(FULL, confirmed, off);
+  }
+  if (gl == 0 && ecs_done) {
+    if (ev_pn) flush_outcomes();
+    atomicAdd(&P.counters[CNT_EVENTS], nev_all);
+    if (tried) atomicAdd(&P.counters[CNT_SWAP_TRIED], tried);
+    if (confirmed) atomicAdd(&P.counters[CNT_CONFIRMED], confirmed);
+    if (exh) atomicAdd(&P.counters[CNT_EXHAUSTIVE], (unsigned long long)exh);
+    atomicAdd(&P.counters[CNT_ECS], ecs_done);
+    atomicAdd(&P.sums[SUM_LIFT], lift_all);
+    atomicAdd(&P.sums[SUM_REFL], refl_all);
+    atomicAdd(&P.sums[SUM_DISP], (double)ecs_done * P.ell);  // an EC's flights add up to ell
+  }
+}
+#undef SYS
+
+
+// Shared memory of one tile for G lanes and S staged beads: the slab side is
+// 0.3 sigma (a reach box then holds about 12 obstacles at phi = 0.45, 9 with
+// infinitely thin slabs) and grows while the masks of a tile would take
+// more than `budget` bytes; at least 10 slabs (staging keeps S ids in the
+// masks' area).
+struct SlabPick {
+  float inv;
+  int nsl;
+};
+inline SlabPick pick_slabs(double e_max, double sigma, int S, int G, size_t budget) {
+  SlabPick k{};
+  for (double side = 0.3 * sigma;; side *= 1.1) {
+    k.inv = (float)(1.0 / side);
+    const double ns = floor(e_max / side) + 3.0;
+    k.nsl = ns < 10.0 ? 10 : (ns > 1000.0 ? 1001 : (int)ns);
+    if (k.nsl <= 1000 && (k.nsl == 10 || (size_t)mask_quads(S, G, k.nsl) * 16 <= budget)) return k;
+  }
+}
+
+template <int G, bool F32, bool BATCH, bool DOM, bool SPRING, bool PO>
+cudaError_t launch_ec_t(const ECParams &P0, cudaStream_t s) {
+  auto kern = ec_kernel<G, F32, BATCH, DOM, SPRING, PO>;
+  static thread_local int sms = 0, smem_max = 0;
+  if (!sms) {
+    int dev = 0, n = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+    if (e != cudaSuccess) return e;
+    sms = n;
+  }
+  // tiles per block and resident blocks of the last shapes asked for
+  struct Shape {
+    int S, M64, M, nsl, bt, nt, blocks;
+    float inv;
+    size_t smem;
+  };
+  static thread_local Shape memo[4];
+  static thread_local int memo_at = 0;
+  auto shape = [&](int S, int M, Shape *out) -> cudaError_t {
+    ECParams const &P = P0;
+    const int step = 32 / G;
+    const size_t room = (size_t)smem_max / step;  // one warp's tiles must fit a block
+    SlabPick k{};
+    if (DOM) {
+      k = pick_slabs(P.e_max, P.s_len, S, G, (size_t)(G <= 8 ? 2048 : 192 * G));
+      if (group_bytes(S, 0, M, mask_quads(S, G, k.nsl)) > room)
+        k = pick_slabs(P.e_max, P.s_len, S, G, 0);
+    } else {
+      // the box's own slabs, nsl of them around every axis
+      k.nsl = 30;
+      while (k.nsl > 3 && group_bytes(S, 0, M, mask_quads(S, G, k.nsl)) > room) --k.nsl;
+      k.inv = 1.f;
+    }
+    for (const Shape &h : memo)
+      if (h.nt && h.S == S && h.M == M && h.bt == P.block_tiles && h.nsl == k.nsl && h.inv == k.inv) {
+        *out = h;
+        return cudaSuccess;
+      }
+    Shape w{};
+    w.S = S;
+    w.M = M;
+    w.bt = P.block_tiles;
+    w.nsl = k.nsl;
+    w.inv = k.inv;
+    const int MQ = mask_quads(S, G, w.nsl);
+    // FP64 positions in shared memory: the plain form reads many of them per
+    // event; the screened form one, and gives the room to more tiles instead
+    const int want = F32 ? 0 : S;
+    w.M64 = group_bytes(S, want, M, MQ) <= room ? want : 0;
+    const size_t per = group_bytes(S, w.M64, M, MQ);
+    int best = -1;
+    for (int t = step; t <= 128 / G; t += step) {
+      if (P.block_tiles > 0 && t != P.block_tiles && per * P.block_tiles <= (size_t)smem_max &&
+          P.block_tiles % step == 0 && P.block_tiles <= 128 / G)
+        continue;
+      if (per * t > (size_t)smem_max) break;
+      int blocks = 0;
+      cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, t * G, per * t);
+      if (e != cudaSuccess) return e;
+      if (blocks * t > best) {
+        best = blocks * t;
+        w.nt = t;
+        w.blocks = blocks;
+      }
+    }
+    if (w.nt == 0 || w.blocks < 1) return cudaErrorInvalidValue;
+    w.smem = per * w.nt;
+    memo[memo_at] = w;
+    memo_at = (memo_at + 1) & 3;
+    *out = w;
+    return cudaSuccess;
+  };
+  // persistent groups: as many as stay resident, each taking tiles from the
+  // unit counter until none are left
+  auto run = [&](const Shape &h, int mode) -> cudaError_t {
+    ECParams P = P0;
+    P.stage_cap = h.S;
+    P.m_cap = h.M;
+    P.m64 = h.M64;
+    P.nsl = h.nsl;
+    P.sorg = DOM ? P.lorg : 0.f;
+    for (int a = 0; a < 3; ++a) P.sinv[a] = DOM ? h.inv : (float)(h.nsl / P.L[a]);
+    P.defer_mode = mode;
+    const long long want = (P.n_units + h.nt - 1) / h.nt;
+    const long long room = (long long)h.blocks * sms;
+    const int blocks = (int)(want < room ? want : room);
+    cudaError_t e = cudaMemsetAsync(P.unit_next, 0, sizeof(int32_t), s);
+    if (e != cudaSuccess) return e;
+    if (blocks > 0) kern<<<blocks, h.nt * G, h.smem, s>>>(P);
+    return cudaGetLastError();
+  };
+  Shape full{};
+  cudaError_t e = shape(P0.stage_cap, P0.m_cap, &full);
+  if (e != cudaSuccess) return e;
+  // A first pass with tight capacities keeps more tiles resident; the tiles
+  // that do not fit run in a second one.  When all tiles are resident with
+  // the full capacities anyway, one pass does it.
+  const bool two = P0.stage_tight > 0 && P0.m_tight > 0 && P0.deferred && P0.n_deferred &&
+                   (P0.stage_tight < P0.stage_cap || P0.m_tight < P0.m_cap) &&
+                   (long long)full.blocks * full.nt * sms < P0.n_units;
+  if (!two) return run(full, 0);
+  Shape tight{};
+  e = shape(P0.stage_tight, P0.m_tight, &tight);
+  if (e == cudaSuccess) e = cudaMemsetAsync(P0.n_deferred, 0, sizeof(int32_t), s);
+  if (e == cudaSuccess) e = run(tight, 1);
+  if (e == cudaSuccess) e = run(full, 2);
+  return e;
+}
+
+}  // namespace
+}  // namespace ecmc

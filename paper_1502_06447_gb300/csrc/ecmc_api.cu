@@ -60,15 +60,15 @@ struct ecmc_ctx {
   int64_t ncell = 1;
   int32_t stage_cap = 0;
   int32_t m_cap = 0;
-  int32_t stage_tight = 0, m_tight = 0;  // block-lockstep first pass (0: one pass)
+  int32_t stage_tight = 0, m_tight = 0;  // first pass (0: one pass)
   int32_t *d_deferred = nullptr;         // units left to the second pass
   int64_t deferred_cap = 0;
   int32_t *d_n_deferred = nullptr;
   int32_t lanes = 32;
-  // local cell grid of a tile (domain mode)
-  int32_t lg[3] = {1, 1, 1};
-  float linv[3] = {1, 1, 1};
+  // slabs of a tile (domain mode): origin and extent of its box
   float lorg = 0.f;
+  double e_max = 0.0;
+  int64_t ncl = 0;  // cells counted by staging_budget
   int64_t event_cap = 10000000;
   int32_t ecs_per_tile = 1;
   // stream
@@ -552,23 +552,22 @@ ecmc_status ecmc_configure(ecmc_ctx *c, const ecmc_opts *o) {
   stage = (stage + 31) / 32 * 32;  // keeps the staging layouts 16-byte aligned
   if (stage > 65534) return fail(ECMC_EINVAL, "at most 65534 staged beads per tile (serial: beads)");
   int64_t ncl = 0;
+  double e_max = 0.0, hg = 0.0;
   if (p.mode == ECMC_MODE_DOMAIN) {
-    // local cell grid of a tile over [-h, W + h] with cells no narrower than
-    // one free flight's reach (s_cap + 1.01 sigma) and than b_max
-    const double hg = halo_te + 1e-3 * sig;
+    // a tile's box is [-h, W + h] on every axis; its size is accepted by
+    // staging_budget, which counts cells no narrower than one free flight's
+    // reach (s_cap + 1.01 sigma) and than b_max
+    hg = halo_te + 1e-3 * sig;
     const double reach = s_cap + sig + 0.01 * sig;
     const double bm = c->b_max * (1.0 + 1e-6);
     const double side_min = (reach > bm ? reach : bm) + 2e-3 * sig;
     ncl = 1;
     for (int a = 0; a < 3; ++a) {
       const double E = c->W[a] + 2.0 * hg;
-      int g = (int)floor(E / side_min);
-      if (g < 1) g = 1;
-      c->lg[a] = g;
-      c->linv[a] = (float)(g / E);
-      ncl *= g;
+      const int g = (int)floor(E / side_min);
+      ncl *= g < 1 ? 1 : g;
+      e_max = E > e_max ? E : e_max;
     }
-    c->lorg = (float)(-hg);
   }
   {
     int dev = 0, smem_max = 0;
@@ -576,14 +575,22 @@ ecmc_status ecmc_configure(ecmc_ctx *c, const ecmc_opts *o) {
     CU(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const int gmin = 32 / lanes;
     if (mcap > stage) mcap = stage;
-    const int M = (p.precision == ECMC_PREC_FP32F && p.mode == ECMC_MODE_DOMAIN) ? mcap : stage;
-    const bool lock = p.mode == ECMC_MODE_DOMAIN && p.precision == ECMC_PREC_FP32F && p.schedule == 0 &&
-                      p.k_spring == 0.0 && (lanes == 4 || lanes == 8 || lanes == 16);
-    const int bt = p.block_tiles > 0 ? p.block_tiles : gmin;
-    const size_t need = lock ? lock_smem_bytes(stage, M, (int)ncl, bt) : ec_smem_bytes(stage, M, (int)ncl, gmin);
+    const bool screened = p.precision == ECMC_PREC_FP32F && p.mode == ECMC_MODE_DOMAIN;
+    const bool packed = screened && p.schedule == 0 && p.k_spring == 0.0 && lanes <= 16;
+    const int M = screened ? mcap : stage;
+    const int bt = packed && p.block_tiles > 0 ? p.block_tiles : gmin;
+    const size_t need = packed ? staging_budget(stage, 0, M, ncl, bt) + request_budget(bt)
+                               : staging_budget(stage, M, M, ncl, gmin);
     if ((int64_t)need > smem_max)
       return fail(ECMC_EINVAL, "staging needs %lld bytes of shared memory (max %d)",
                   (long long)need, smem_max);
+    if (screened) {
+      const double E[3] = {c->W[0] + 2.0 * halo_te, c->W[1] + 2.0 * halo_te, c->W[2] + 2.0 * halo_te};
+      const int32_t most = packing_bound(E, sig) + (p.k_spring > 0.0 ? 2 * mcap : 0);
+      if (stage > most) stage = (most + 31) / 32 * 32;
+    } else {
+      mcap = stage;
+    }
   }
   c->opts = p;
   c->s_cap = s_cap;
@@ -594,6 +601,9 @@ ecmc_status ecmc_configure(ecmc_ctx *c, const ecmc_opts *o) {
   c->m_cap = mcap > stage ? stage : mcap;
   c->stage_tight = stage_t;
   c->m_tight = m_t;
+  c->lorg = (float)(-hg);
+  c->e_max = e_max;
+  c->ncl = ncl;
   if (p.mode == ECMC_MODE_DOMAIN) {
     const int64_t ntile = (int64_t)p.tiles[0] * p.tiles[1] * p.tiles[2];
     if (ntile > c->deferred_cap) {
@@ -646,13 +656,6 @@ static ecmc_status reserve_records(ecmc_ctx *c, int64_t units) {
 }
 
 // one EC launch between a pair of events (the pair is reused across runs)
-// the block-lockstep kernel runs the screened domain form with 4, 8 or 16 lanes
-static bool uses_lock(const ecmc_opts &o, int lanes) {
-  // (bead springs run in the warp-lockstep kernel)
-  return o.mode == ECMC_MODE_DOMAIN && o.precision == ECMC_PREC_FP32F && o.schedule == 0 &&
-         o.k_spring == 0.0 && (lanes == 4 || lanes == 8 || lanes == 16);
-}
-
 static cudaError_t timed_ec(ecmc_ctx *c, const ECParams &P, int64_t slot) {
   while ((int64_t)c->kev.size() < slot + 2) {
     cudaEvent_t e;
@@ -662,8 +665,7 @@ static cudaError_t timed_ec(ecmc_ctx *c, const ECParams &P, int64_t slot) {
   }
   cudaError_t err = cudaEventRecord(c->kev[slot], c->stream);
   if (err != cudaSuccess) return err;
-  if (uses_lock(c->opts, c->lanes)) err = launch_ec_lock(P, c->lanes, c->stream);
-  else err = launch_ec(P, c->lanes, c->opts.precision == ECMC_PREC_FP32F, c->stream);
+  err = launch_ec(P, c->lanes, c->opts.precision == ECMC_PREC_FP32F, 0, c->stream);
   if (err != cudaSuccess) return err;
   return cudaEventRecord(c->kev[slot + 1], c->stream);
 }
@@ -722,11 +724,9 @@ static ECParams ec_params(const ecmc_ctx *c, uint64_t seed, double ell) {
     P.eps_d = (float)ed;
     P.eps_x = (float)ev;
   }
-  for (int a = 0; a < 3; ++a) {
-    P.lg[a] = c->lg[a];
-    P.linv[a] = c->linv[a];
-  }
   P.lorg = c->lorg;
+  P.e_max = c->e_max;
+  P.s_len = c->sigma;
   P.r = c->d_r;
   P.img = c->d_img;
   P.cr = c->d_cr;
@@ -734,6 +734,7 @@ static ECParams ec_params(const ecmc_ctx *c, uint64_t seed, double ell) {
   P.rf = c->d_rf;
   P.cid = c->d_cid;
   P.ctag = c->d_ctag;
+  P.tag = c->opts.k_spring > 0.0 && c->d_ftag && c->N > 1 ? c->d_ftag : c->d_tag;
   P.cstart = c->d_start;
   P.counters = c->d_cnt;
   P.sums = c->d_sums;
@@ -1076,8 +1077,7 @@ ecmc_status ecmc_pushoff(ecmc_ctx *c, double f0, int32_t stages, double ell, uin
     int dev = 0, smem_max = 0;
     CU(cudaGetDevice(&dev));
     CU(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    const int ncl = c->lg[0] * c->lg[1] * c->lg[2];
-    if (ec_smem_bytes((int)S, (int)S, ncl, 32 / c->lanes) > (size_t)smem_max)
+    if (staging_budget((int)S, (int)S, (int)S, c->ncl, 32 / c->lanes) > (size_t)smem_max)
       return fail(ECMC_EINVAL, "push-off staging of %lld beads per tile does not fit in shared memory "
                   "(use smaller tiles or more lanes)", (long long)S);
     P.stage_cap = (int32_t)S;
@@ -1112,7 +1112,7 @@ ecmc_status ecmc_pushoff(ecmc_ctx *c, double f0, int32_t stages, double ell, uin
       for (int64_t i = 0; i < n; ++i) {
         CU(launch_cells(C, c->ncell, c->stream));
         CU(launch_po_flags(O, thr, c->d_po_flag, c->d_po_cnt, c->stream));
-        CU(launch_ec(P, c->lanes, 0, c->stream));
+        CU(launch_ec(P, c->lanes, 0, 1, c->stream));
         CU(launch_po_advance(c->d_po_cnt, c->d_po_ctr, c->stream));
       }
       // the overlaps left after the chunk

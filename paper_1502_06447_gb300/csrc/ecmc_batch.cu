@@ -48,7 +48,9 @@ struct ecmc_batch {
   ecmc_opts opts{};
   bool configured = false;
   double s_cap = 0.25, halo_hs = 0, halo_te = 0;
-  int32_t stage_cap = 0, m_cap = 0, ncl_max = 0, lanes = 8, ecs_per_tile = 1;
+  int32_t stage_cap = 0, m_cap = 0, lanes = 8, ecs_per_tile = 1;
+  double e_max = 0.0;  // longest axis of any tile's box
+  float lorg = 0.f;
   int64_t event_cap = 10000000;
   cudaStream_t stream = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -132,10 +134,7 @@ cudaError_t batch_sweep(ecmc_batch *b, const ECParams &P, uint64_t seed) {
   C.ctag = b->d_ctag;
   cudaError_t e = launch_cells_batch(C, b->ncell_total, b->stream);
   if (e != cudaSuccess) return e;
-  const bool lock = b->opts.precision == ECMC_PREC_FP32F && b->opts.schedule == 0 &&
-                    (b->lanes == 4 || b->lanes == 8 || b->lanes == 16);
-  e = lock ? launch_ec_lock_batch(P, b->lanes, b->stream)
-           : launch_ec_batch(P, b->lanes, b->opts.precision == ECMC_PREC_FP32F, b->stream);
+  e = launch_ec(P, b->lanes, b->opts.precision == ECMC_PREC_FP32F, 0, b->stream);
   if (e != cudaSuccess) return e;
   return launch_sweep_advance(b->d_sweep, b->stream);
 }
@@ -185,7 +184,10 @@ ECParams batch_params(ecmc_batch *b, uint64_t seed, double ell) {
   P.status = b->d_status;
   P.reps = b->d_reps;
   P.n_reps = b->R;
-  P.ncl_max = b->ncl_max;
+  P.lorg = b->lorg;
+  P.e_max = b->e_max;
+  P.s_len = b->sigma;
+  P.tag = b->d_tag;
   P.sweep_dev = b->d_sweep;
   P.block_tiles = b->opts.block_tiles;
   P.rq_per_tile = b->opts.request_cap > 0 ? b->opts.request_cap : 6;
@@ -318,7 +320,8 @@ ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *o) {
   const double side_min = (reach > bm ? reach : bm) + 2e-3 * sig;
   const double margin = p.precision == ECMC_PREC_FP32F ? 0.01 * sig : 0.0;
   int64_t cell_off = 0, unit_off = 0;
-  int32_t stage = 0, mcap = 0, nclm = 0, stage_t = 0, m_t = 0;
+  int32_t stage = 0, mcap = 0, nclm = 0, stage_t = 0, m_t = 0, most = 0;
+  double e_max = 0.0;
   std::vector<RepParams> reps = b->reps;
   for (int32_t r = 0; r < b->R; ++r) {
     RepParams &R = reps[r];
@@ -346,18 +349,18 @@ ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *o) {
       const double E = W + 2.0 * hg;
       int g = (int)floor(E / side_min);
       if (g < 1) g = 1;
-      R.lg[a] = g;
-      R.linv[a] = (float)(g / E);
       ncl *= g;
+      e_max = E > e_max ? E : e_max;
       nce *= k;
       nt *= D;
     }
-    R.lorg = (float)(-hg);
     R.cell_off = cell_off;
     R.unit_off = unit_off;
     cell_off += nce;
     unit_off += nt;
     const double E[3] = {R.W[0] + 2.0 * halo_te, R.W[1] + 2.0 * halo_te, R.W[2] + 2.0 * halo_te};
+    const int32_t pk = packing_bound(E, sig);
+    most = pk > most ? pk : most;
     const int32_t st = stage_bound(E, rho);
     const int32_t mc = stage_bound(R.W, rho);
     stage = st > stage ? st : stage;
@@ -385,11 +388,15 @@ ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *o) {
       (p.block_tiles > 0 && p.block_tiles % (32 / lanes)))
     return bfail(ECMC_EINVAL, "block_tiles must be a multiple of 32 / lanes, at most 32 and 128 / lanes");
   if (p.request_cap < 0 || p.request_cap > 6) return bfail(ECMC_EINVAL, "request_cap must be in [0, 6]");
-  const bool lock = p.precision == ECMC_PREC_FP32F && p.schedule == 0 && lanes <= 16;
+  const bool packed = p.precision == ECMC_PREC_FP32F && p.schedule == 0 && lanes <= 16;
   const int bt = p.block_tiles > 0 ? p.block_tiles : 32 / lanes;
-  const size_t need = lock ? lock_smem_bytes(stage, M, nclm, bt) : ec_smem_bytes(stage, M, nclm, 32 / lanes);
+  const size_t need = packed ? staging_budget(stage, 0, M, nclm, bt) + request_budget(bt)
+                             : staging_budget(stage, M, M, nclm, 32 / lanes);
   if ((int64_t)need > smem_max)
     return bfail(ECMC_EINVAL, "staging does not fit in shared memory");
+  if (p.precision != ECMC_PREC_FP32F) mcap = stage;
+  else if (stage > most) stage = (most + 31) / 32 * 32;
+  if (mcap > stage) mcap = stage;
   // (re)allocate the concatenated cell arrays
   if (cell_off != b->ncell_total) {
     cudaFree(b->d_count);
@@ -422,7 +429,8 @@ ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *o) {
     BCU(balloc(&b->d_deferred, unit_off));
     b->deferred_cap = unit_off;
   }
-  b->ncl_max = nclm;
+  b->lorg = (float)(-hg);
+  b->e_max = e_max;
   b->lanes = lanes;
   b->ecs_per_tile = p.ecs_per_tile > 0 ? p.ecs_per_tile : 1;
   b->event_cap = p.event_cap > 0 ? p.event_cap : 10000000;

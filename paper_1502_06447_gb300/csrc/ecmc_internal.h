@@ -48,8 +48,7 @@ inline float round_up_f32(double x) {
 // and its Philox key word.
 struct RepParams {
   double L[3], half[3], T[3], W[3], cs[3];
-  int32_t D[3], nc[3], lg[3];
-  float linv[3], lorg;
+  int32_t D[3], nc[3];
   int32_t N;
   int32_t pad;
   int64_t bead_off;   // first bead in the concatenated position array
@@ -85,7 +84,7 @@ struct ECParams {
   uint64_t swap_thr;    // u53(w) < p_swap  <=>  (w >> 11) < swap_thr = ceil(p_swap 2^53)
   int32_t dir_mode;
   int32_t stage_cap;
-  int32_t m_cap;        // motile slots with FP64 in shared memory (screened domain form)
+  int32_t m_cap;        // motile beads per tile
   int32_t n_units;      // tiles (domain) or 1 (serial)
   // FP32 screen margins (units of sigma, sigma^2)
   float eps_v, eps_d, eps_x;
@@ -99,6 +98,7 @@ struct ECParams {
   const int32_t *cstart;   // cell starts (ncell + 1)
   const float *crf;        // FP32 positions in cell order
   const float *rf;         // FP32 positions by bead
+  const int32_t *tag;      // tiles by bead (with springs: after the motility rule)
   unsigned long long *counters;
   double *sums;
   int *status;
@@ -111,20 +111,22 @@ struct ECParams {
   ecmc_event *log;
   unsigned long long *log_n;
   int64_t log_cap;
-  // batch: replica table (units are the concatenated tiles of all replicas),
-  // the sweep counter on the device (graph replays advance it), and the
-  // largest local grid over the replicas
+  // batch: replica table (units are the concatenated tiles of all replicas)
+  // and the sweep counter on the device (graph replays advance it)
   const RepParams *reps;
   int32_t n_reps;
-  int32_t ncl_max;
   const int64_t *sweep_dev;
   int64_t rec_sweep0;
-  // local cell grid of a tile (domain mode)
-  int32_t lg[3];
-  float linv[3];
-  float lorg;
-  // block-lockstep kernel: tiles per block (0: occupancy choice) and the
-  // device counter its persistent blocks take units from (reset per launch)
+  // slabs of a tile's box [lorg, lorg + e_max] on every axis (e_max: the
+  // longest axis of any tile; lengths in units of s_len = sigma); the
+  // launcher fills in their number, origin and inverse side
+  double e_max, s_len;
+  float lorg, sorg;
+  float sinv[3];
+  int32_t nsl;
+  int32_t m64;          // slots with FP64 positions in shared memory (launcher)
+  // tiles per block (0: occupancy choice) and the device counter the
+  // resident groups take units from (reset per launch)
   int32_t block_tiles;
   int32_t *unit_next;
   // slow push-off (plain FP64 domain kernel): the ECs of a tile start at its
@@ -134,8 +136,11 @@ struct ECParams {
   // push-off run from the device: the launch does nothing when no bead
   // overlaps (the count of the flag pass before it); null otherwise
   const unsigned long long *po_count;
-  int32_t rq_per_tile;  // request list entries per tile of the block (1..6)
-  // block-lockstep kernel: tight capacities for a first pass (0: none); a
+  // screened form: a tile with more survivors of the screen than this (below
+  // 6: or more than 8 times as many obstacles in reach) is evaluated
+  // exhaustively in FP64
+  int32_t rq_per_tile;
+  // tight capacities for a first pass (0: none); a
   // tile that does not fit them is listed in `deferred` and run by a second
   // pass with stage_cap / m_cap (tiles are independent, so the events are
   // the same).  defer_mode: 0 one pass, 1 first pass, 2 second pass.
@@ -152,14 +157,18 @@ struct ECParams {
 // message for ecmc_last_error (ecmc_api.cu)
 void set_last_error(const char *msg);
 
-// launchers (k_ec.cu)
-cudaError_t launch_ec(const ECParams &P, int lanes, int fp32f, cudaStream_t s);
-cudaError_t launch_ec_batch(const ECParams &P, int lanes, int fp32f, cudaStream_t s);
-size_t ec_smem_bytes(int stage_cap, int motile_cap, int ncell, int groups_per_block);
-// block-lockstep kernel of the screened domain form (lanes 4, 8, 16)
-cudaError_t launch_ec_lock(const ECParams &P, int lanes, cudaStream_t s);
-cudaError_t launch_ec_lock_batch(const ECParams &P, int lanes, cudaStream_t s);
-size_t lock_smem_bytes(int stage_cap, int motile_cap, int ncell, int tiles_per_block);
+// launchers (k_ec*.cu): lanes 4, 8, 16 or 32
+cudaError_t launch_ec(const ECParams &P, int lanes, int fp32f, int pushoff, cudaStream_t s);
+cudaError_t launch_ec_screened(const ECParams &P, int lanes, cudaStream_t s);
+cudaError_t launch_ec_fp64(const ECParams &P, int lanes, cudaStream_t s);
+cudaError_t launch_ec_batch_screened(const ECParams &P, int lanes, cudaStream_t s);
+cudaError_t launch_ec_batch_fp64(const ECParams &P, int lanes, cudaStream_t s);
+cudaError_t launch_ec_spring_screened(const ECParams &P, int lanes, cudaStream_t s);
+cudaError_t launch_ec_spring_fp64(const ECParams &P, int lanes, cudaStream_t s);
+cudaError_t launch_ec_pushoff_tether(const ECParams &P, int lanes, cudaStream_t s);
+cudaError_t launch_ec_pushoff_spring(const ECParams &P, int lanes, cudaStream_t s);
+// pick_lanes (k_ec.cu): warps per SM up to which a tile gets more lanes
+constexpr int EC_SPREAD_WARPS = 4;
 
 // cell list and domain tags (k_cells.cu)
 struct CellParams {
@@ -317,7 +326,29 @@ inline int32_t stage_bound(const double E[3], double rho) {
   return (int32_t)((n + 31) / 32 * 32);
 }
 
-// Tight capacities of the block-lockstep kernel's first pass: `factor`
+// The accepted tile sizes: `tiles` tiles of a block, each counted as 24 B
+// per FP64 position, 4 B per motile bead, 16 B per staged bead, 16 B per
+// cell of a local grid with cells no narrower than one flight's reach, an
+// overflow list of max(64, S / 4) slots and a header (screened form with 4,
+// 8 or 16 lanes: the request lists and records of a block as well), have to
+// fit a block's shared memory.  The kernel needs no more than that: where
+// its own layout would, it gives a tile more lanes.
+inline size_t staging_budget(int stage_cap, int motile64, int motile, int64_t ncell, int tiles) {
+  const int ovf = stage_cap / 4 > 64 ? (stage_cap / 4 + 7) / 8 * 8 : 64;
+  return (size_t)tiles * ((size_t)motile64 * 24 + (size_t)motile * 4 + (size_t)stage_cap * 16 +
+                          (size_t)ncell * 16 + (size_t)ovf * 2 + 32);
+}
+inline size_t request_budget(int tiles) { return (size_t)tiles * 544 + 80; }
+// Hard spheres of diameter sigma whose centres lie in a box of sides E take
+// at most the volume of the box widened by sigma: a larger staging capacity
+// is never used.
+inline int32_t packing_bound(const double E[3], double sigma) {
+  const double v = (E[0] + sigma) * (E[1] + sigma) * (E[2] + sigma) / (sigma * sigma * sigma);
+  const double n = v * 1.9098593171027443 + 32.0;
+  return n < 65504.0 ? (int32_t)n / 32 * 32 + 32 : 65504;
+}
+
+// Tight capacities of the EC kernel's first pass: `factor`
 // times the mean occupancy of a melted tile plus a margin, rounded to 8
 // (tiles that exceed them, e.g. at the lattice start, run in the second
 // pass; a smaller factor fits more tiles per SM and defers more of them).
