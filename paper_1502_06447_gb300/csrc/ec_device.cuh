@@ -29,6 +29,10 @@ __device__ __forceinline__ bool ge_pos(double y, double L) {
   return (int64_t)dbits(y) >= (int64_t)dbits(L);
 }
 __device__ __forceinline__ bool nonzero(double x) { return (dbits(x) << 1) != 0; }
+// 2 x, exact (|x| zero or normal and below 2^1022)
+__device__ __forceinline__ double twice(double x) {
+  return nonzero(x) ? __longlong_as_double(__double_as_longlong(x) + (1ll << 52)) : x;
+}
 
 // minimum image, same result as d > h ? d - L : (d < -h ? d + L : d)
 __device__ __forceinline__ double wrap_i(double d, double L, uint64_t hbits) {
@@ -42,9 +46,8 @@ __device__ __forceinline__ double wrapc(double d, double L, uint64_t hbits, bool
   return w ? wrap_i(d, L, hbits) : d;
 }
 
-// r += x v on one axis, back into [0, L); returns the image change
-__device__ __forceinline__ int step_i(double &r, double x, double v, double L) {
-  double y = __fma_rn(x, v, r);
+// y = r + x v on one axis back into [0, L); returns the image change
+__device__ __forceinline__ int wrap_step(double &y, double L) {
   int di = 0;
   if (ge_pos(y, L)) {
     y = y - L;
@@ -57,7 +60,6 @@ __device__ __forceinline__ int step_i(double &r, double x, double v, double L) {
       di = 0;
     }
   }
-  r = y;
   return di;
 }
 
@@ -72,26 +74,16 @@ __device__ __forceinline__ double quad_x(bool tether, double d0, double d1, doub
   dv = __fma_rn(d2, v2, __fma_rn(d1, v1, d0 * v0));
   if (!tether && !neg(dv)) return -1.0;
   const double dd = __fma_rn(d2, d2, __fma_rn(d1, d1, d0 * d0));
-  if (!tether && skip_overlap && dd < R2) return -1.0;
+  if (!tether && skip_overlap && dbits(dd) < dbits(R2)) return -1.0;
   double rad = R2 - __fma_rn(-dv, dv, dd);
   if (tether) {
     if (neg(rad)) rad = 0.0;
   } else if (!posv(rad)) {
     return -1.0;
   }
-  const double x = tether ? -dv + sqrt(rad) : -dv - sqrt(rad);
+  const double q = sqrt_rn(rad);
+  const double x = -dv + (tether ? q : -q);
   return neg(x) ? 0.0 : x;
-}
-
-// v <- v - (2 v.d / d.d) d: reflection at the plane normal to d (Fig. 2c)
-__device__ __forceinline__ void mirror2(double &v0, double &v1, double &v2, double d0, double d1,
-                                        double d2) {
-  const double dd = __fma_rn(d2, d2, __fma_rn(d1, d1, d0 * d0));
-  const double vd = __fma_rn(v2, d2, __fma_rn(v1, d1, v0 * d0));
-  const double t = (2.0 * vd) / dd;
-  v0 = __fma_rn(-t, d0, v0);
-  v1 = __fma_rn(-t, d1, v1);
-  v2 = __fma_rn(-t, d2, v2);
 }
 
 // candidate key: kind (3 bits) | partner id (41 bits) | slot (20 bits).
@@ -147,7 +139,7 @@ __host__ __device__ __forceinline__ int ovf_cap_for(int S) {
 
 struct Stage {
   float4 *sh;       // [S] x, y, z, id (bits)
-  double *px, *py, *pz;  // [M64]
+  double *pos;      // [3][M64]
   unsigned *nb;     // [MNB] bond partner slots, 16 + 16 bits (0xFFFF = none)
   unsigned *mask;   // [3][nsl + 1][W][G]
   int *hdr;         // [0] hard-sphere joint beads, [1] tether-only joint beads
@@ -175,10 +167,8 @@ __host__ __device__ __forceinline__ size_t group_bytes(int S, int M64, int MNB, 
 __device__ __forceinline__ Stage carve(unsigned char *base, int S, int M64, int MNB, int MQ) {
   Stage s;
   s.sh = (float4 *)base;
-  s.px = (double *)(s.sh + S);
-  s.py = s.px + M64;
-  s.pz = s.py + M64;
-  s.nb = (unsigned *)(s.pz + M64);
+  s.pos = (double *)(s.sh + S);
+  s.nb = (unsigned *)(s.pos + 3 * M64);
   s.mask = s.nb + MNB;
   s.hdr = (int *)(s.mask + 4 * MQ);
 #ifdef ECMC_CHECKED
@@ -300,26 +290,16 @@ __device__ __forceinline__ float screen_lb(const Screen &Z, float d0, float d1, 
   return -dv - Z.eps_v - sqrt_hi(fmaxf(disc + Z.eps_d, 0.f));
 }
 
-// FP64 position of staged slot k: shared memory for the first M64 slots,
-// otherwise the global position array (a joint bead, static this sweep, or
-// a motile one, written through by every move)
-__device__ __forceinline__ void pos64(const Stage &st, const double *r, int k, int M64, double &x,
-                                      double &y, double &z) {
+// FP64 position of staged slot k on one axis: shared memory for the first
+// M64 slots, otherwise the global position array (a joint bead, static this
+// sweep, or a motile one, written through by every move)
+__device__ __forceinline__ double pos64(const Stage &st, const double *r, int k, int axis, int M64) {
 #ifdef ECMC_CHECKED
-  x = y = z = 0.0;
-  if (st.status && !CHK(k, st.cap, 1, st.status)) return;
-  if (k >= M64 && st.status && !CHK(__float_as_int(st.sh[k].w), st.nglob, 2, st.status)) return;
+  if (st.status && !CHK(k, st.cap, 1, st.status)) return 0.0;
+  if (k >= M64 && st.status && !CHK(__float_as_int(st.sh[k].w), st.nglob, 2, st.status)) return 0.0;
 #endif
-  if (k < M64) {
-    x = st.px[k];
-    y = st.py[k];
-    z = st.pz[k];
-  } else {
-    const int64_t b = __float_as_int(st.sh[k].w);
-    x = r[3 * b];
-    y = r[3 * b + 1];
-    z = r[3 * b + 2];
-  }
+  if (k < M64) return st.pos[axis * M64 + k];
+  return r[3 * (int64_t)__float_as_int(st.sh[k].w) + axis];
 }
 
 // ---------------------------------------------------------------- staging
@@ -331,8 +311,7 @@ __device__ __forceinline__ void pos64(const Stage &st, const double *r, int k, i
 #define SYS(f) (BATCH ? rp->f : P.f)
 template <int G, bool DOM, bool SPRING, bool BATCH>
 __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *rp, const Stage &st,
-                                           int gl, bool &live, int unit, double c0, double c1,
-                                           double c2, double *Rr, const int32_t *Rstart, int S,
+                                           int gl, bool &live, int unit, double ca, double *Rr, const int32_t *Rstart, int S,
                                            int M64, int MNB, int W, const Slabs &SL, int &m,
                                            int &j1, int &ns, unsigned mask, bool *overflow) {
   // a tile that does not fit its capacities sets the device status, or, when
@@ -343,6 +322,11 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
     else if (gl == 0) set_status(P.status, DEV_CAPACITY);
   };
   if (overflow) *overflow = false;
+  auto put64 = [&](int k, const double *x) {
+    st.pos[k] = x[0];
+    st.pos[M64 + k] = x[1];
+    st.pos[2 * M64 + k] = x[2];
+  };
   const int nsl = SL.nsl;
   m = 0;
   j1 = 0;
@@ -352,12 +336,8 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
     const int n = (int)P.n;
     for (int b = gl; b < n; b += G) {
       const double x = Rr[3 * (int64_t)b], y = Rr[3 * (int64_t)b + 1], z = Rr[3 * (int64_t)b + 2];
-      if (b < M64) {
-        st.px[b] = x;
-        st.py[b] = y;
-        st.pz[b] = z;
-      }
-      st.sh[b] = make_float4((float)x, (float)y, (float)z, __int_as_float(b));
+      if (b < M64) put64(b, Rr + 3 * (int64_t)b);
+      st.sh[b] = make_float4(f32_trunc(x), f32_trunc(y), f32_trunc(z), __int_as_float(b));
       const int c = b % SYS(N);
       st.nb[b] = nb_pack(c == 0 ? -1 : b - 1, c == SYS(N) - 1 ? -1 : b + 1);
     }
@@ -368,21 +348,28 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
     if (gl < 8) st.hdr[gl] = 0;
     if (G < 8) st.hdr[gl + 4] = 0;
     __syncwarp(mask);
-    const double corner[3] = {c0, c1, c2};
-    // cell window covering the tether halo of the tile
+    // cell window covering the tether halo of the tile: lane a works out
+    // axis a (corner ca) and the group shares it
     int c_lo[3], c_n[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const double lo = corner[a] - P.halo_te, hi = corner[a] + SYS(W)[a] + P.halo_te;
-      int l = (int)floor(lo / SYS(cs)[a]);
-      const int h = (int)floor(hi / SYS(cs)[a]);
+    float cf[3];
+    {
+      const int ax = (gl & 3) < 3 ? (gl & 3) : 0;
+      const double lo = ca - P.halo_te, hi = ca + SYS(W)[ax] + P.halo_te;
+      int l = (int)floor(div_rn(lo, SYS(cs)[ax]));
+      const int h = (int)floor(div_rn(hi, SYS(cs)[ax]));
       int cnt = h - l + 1;
-      if (cnt >= SYS(nc)[a]) {
+      if (cnt >= SYS(nc)[ax]) {
         l = 0;
-        cnt = SYS(nc)[a];
+        cnt = SYS(nc)[ax];
       }
-      c_lo[a] = l;
-      c_n[a] = cnt;
+      const float cfa = f32_trunc(ca);
+      const int g0 = (threadIdx.x & 31) & ~(G - 1);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        c_lo[a] = __shfl_sync(mask, l, g0 + a);
+        c_n[a] = __shfl_sync(mask, cnt, g0 + a);
+        cf[a] = __shfl_sync(mask, cfa, g0 + a);
+      }
     }
     // pass 1: collect (cell-order index, category|id), motile beads from the
     // front, joint beads from the back; the shadow array serves as scratch
@@ -395,18 +382,17 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
     // 1e-3 sigma plus four FP32 ulps of the box: a superset of the exact
     // sets (an extra obstacle beyond reach is never hit; a bond partner is
     // always within the tether halo)
-    float cf[3], Lf[3], Lhf[3], Wf[3];
+    float Lf[3], Lhf[3], Wf[3];
     float Lmax = 0.f;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      cf[a] = (float)corner[a];
-      Lf[a] = (float)SYS(L)[a];
+      Lf[a] = SYS(Lf)[a];
       Lhf[a] = 0.5f * Lf[a];
-      Wf[a] = (float)SYS(W)[a];
+      Wf[a] = SYS(Wf)[a];
       Lmax = fmaxf(Lmax, Lf[a]);
     }
-    const float widen = 1e-3f * (float)P.sigma + 4.8e-7f * Lmax;
-    const float hs_f = (float)P.halo_hs + widen, te_f = (float)P.halo_te + widen;
+    const float widen = 1e-3f * P.sigma_f + 4.8e-7f * Lmax;
+    const float hs_f = P.halo_hs_f + widen, te_f = P.halo_te_f + widen;
     const int nc0 = SYS(nc)[0], nc1 = SYS(nc)[1], nc2 = SYS(nc)[2];
     const int nrows = c_n[1] * c_n[2];
     int cx = c_lo[0] % nc0;
@@ -494,11 +480,7 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
       for (int t = 0; t < m; ++t) rank += (scr[t].y < e.y);
       if (!CHK(rank, S, 3, P.status)) continue;
       idt[rank] = e.y;
-      if (rank < M64) {
-        st.px[rank] = P.cr[3 * (int64_t)e.x];
-        st.py[rank] = P.cr[3 * (int64_t)e.x + 1];
-        st.pz[rank] = P.cr[3 * (int64_t)e.x + 2];
-      }
+      if (rank < M64) put64(rank, P.cr + 3 * (int64_t)e.x);
     }
     for (int s = gl; s < ns - m; s += G) {
       const int2 e = scr[S - 1 - s];
@@ -506,11 +488,7 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
       const int slot = (cat == 1 ? m : m + j1) + atomicAdd(&st.hdr[cat - 1], 1);
       if (!CHK(slot, S, 33, P.status)) continue;
       idt[slot] = e.y & ((1 << 29) - 1);
-      if (slot < M64) {
-        st.px[slot] = P.cr[3 * (int64_t)e.x];
-        st.py[slot] = P.cr[3 * (int64_t)e.x + 1];
-        st.pz[slot] = P.cr[3 * (int64_t)e.x + 2];
-      }
+      if (slot < M64) put64(slot, P.cr + 3 * (int64_t)e.x);
     }
     __syncwarp(mask);
     // pass 2b: bond partners of motile beads.  A motile partner is found
@@ -563,11 +541,7 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
         if (slot < S) {
           idt[slot] = q;
           nbh[2 * s + dir] = (unsigned short)slot;
-          if (slot < M64) {
-            st.px[slot] = Rr[3 * (int64_t)q];
-            st.py[slot] = Rr[3 * (int64_t)q + 1];
-            st.pz[slot] = Rr[3 * (int64_t)q + 2];
-          }
+          if (slot < M64) put64(slot, Rr + 3 * (int64_t)q);
         }
       }
     }

@@ -5,11 +5,22 @@
 //
 // One group of G lanes (G = 32, 16, 8 or 4) runs the ECs of one tile, one
 // event per step; the 32 / G groups of a warp step together, and no warp
-// waits for another: there is no block barrier.  The state of an EC (pivot,
-// direction, what is left of ell) is held by every lane of its group, so a
-// step exchanges no more than the winning candidate.  A group whose tile has
-// run its ECs takes the next unit of the launch from a device counter and
-// stages it while the warp's other groups wait.
+// waits for another: there is no block barrier.  A group whose tile has run
+// its ECs takes the next unit of the launch from a device counter and stages
+// it while the warp's other groups wait.
+//
+// What bounds it: FP64 instructions.  GB300's FP64 unit takes a warp
+// instruction every 64 cycles per SM sub-partition whatever its active mask
+// and dependences (conversions and comparisons 80-110), so the number of
+// FP64 instructions of a step sets both a lone tile's latency and the rate
+// of a full chip.  Hence:
+//   - the lanes of a quad hold one axis each (lane 3: what is left of ell),
+//     and the three axes of a difference, a move or a reflection are one
+//     instruction; d.v and d.d are one chain of three on two lanes; the move,
+//     the rest of ell and the projection of a lift come from one multiply-add;
+//   - square roots and quotients are integer code (ecmc_dev.cuh), as are
+//     comparisons, sign changes and conversions to FP32.
+// A step with one contact takes 9 FP64 instructions, a reflection 5 more.
 //
 // A step:
 //   A  the obstacles the flight can reach come from the slab masks
@@ -17,16 +28,14 @@
 //      a lane bounds its obstacles, a tether or a wall in FP32 and keeps
 //      those whose lower bound can reach the group's smallest upper bound U;
 //      in the plain form every reachable obstacle is kept;
-//   B  each lane evaluates what it kept in FP64 (exactly the definition's
-//      expressions); the group takes the smallest x under the tie rule;
-//   D  all lanes move the pivot, lift, reflect or swap.
+//   B  what was kept is evaluated in FP64 (exactly the definition's
+//      expressions), one candidate per quad in the screened form, one per
+//      lane in the plain form; the group takes the smallest x under the tie
+//      rule;
+//   D  the lanes move the pivot, lift, reflect or swap.
 // A candidate left out by the screen cannot win: the winner's exact x is <= U
 // and every lower bound is <= its candidate's exact x, so both forms produce
 // the same events.
-//
-// What bounds it: the latency of one step.  A tile's events follow one
-// another, and a step is a chain of dependent FP64 operations (55-60 cycles
-// each), shared-memory and L1 round trips.
 #pragma once
 #include "ec_device.cuh"
 
@@ -60,6 +69,14 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
   const int lane = threadIdx.x & 31;
   const int gl = lane & (G - 1);
   const int gbase = lane & ~(G - 1);
+  const int qbase = lane & ~3;
+  const int ax = lane & 3;            // this lane's axis; 3: what is left of ell
+  const int axc = ax < 3 ? ax : 0;
+  constexpr int NQ = G / 4;           // quads of the group
+  const int qd = gl >> 2;             // this lane's quad
+  // the lane whose move instruction gives the projection of a lift, and
+  // whose lift and reflection sums count
+  constexpr int AL = G >= 8 ? 7 : 0;
   const unsigned gmask = (G == 32) ? FULL : (((1u << G) - 1) << gbase);
   const int gib = threadIdx.x / G;
   const int64_t sweep = P.sweep_dev ? *P.sweep_dev : P.sweep;
@@ -83,26 +100,33 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
   int32_t *Ri = P.img;
   uint64_t Rkey = P.replica;
   const Slabs SL{P.sinv[0], P.sinv[1], P.sinv[2], slab_raw(P.sorg, P.sinv[0], 0), nsl};
-  double c0 = 0.0, c1 = 0.0, c2 = 0.0;
-  bool wr0 = true, wr1 = true, wr2 = true;
+  // this lane's axis: tile corner (FP64, FP32), tile side, whether positions
+  // of the tile can wrap (a tile whose halo lies inside (0, L) on an axis
+  // never needs the minimum image or a wrap there)
+  double ca = 0.0;
+  float cfa = 0.f, Wfa = 0.f;
+  bool wra = !DOM && ax < 3;
   int n_ec = P.ecs_per_tile;
 
   // ------------------------------------------------------------ EC state
   int e = 0, p = 0, pid = 0;
   unsigned nbw = 0xFFFFFFFFu;
   int oslab = 0;  // slabs of the pivot's stored shadow, 10 bits per axis
-  double q0 = 0.0, q1 = 0.0, q2 = 0.0, v0 = 0.0, v1 = 0.0, v2 = 0.0, xrem = 0.0, lift = 0.0;
+  double qa = 0.0;             // pivot position on this lane's axis; lane 3: what is left of ell
+  double va = 0.0;             // direction on this lane's axis; lane 3: -1
+  double v0 = 0.0, v1 = 0.0, v2 = 0.0, xrem = 0.0;  // the same, on every lane
+  double lift = 0.0, refl_all = 0.0;                // (lane AL)
   float pf0 = 0.f, pf1 = 0.f, pf2 = 0.f, vf0 = 0.f, vf1 = 0.f, vf2 = 0.f;
   int64_t nev = 0;
   unsigned ncontact = 0, swgo = 0;  // swap proposals of this and the next contacts, one bit each
   uint64_t h = 0;
-  // springs: the Boltzmann energies of the next G / 2 events, drawn together
-  double dE = 0.0;
+  // springs: 2 dE / k of the next G / 2 events, drawn together
+  double dEk = 0.0;
   int dE_at = 0;
 
-  double lift_all = 0.0, refl_all = 0.0;
-  unsigned long long tried = 0, confirmed = 0, nev_all = 0, ecs_done = 0;
-  unsigned exh = 0;
+  double lift_all = 0.0;
+  unsigned long long nev_all = 0;
+  unsigned tried = 0, confirmed = 0, ecs_done = 0, exh = 0;
   // events by outcome: eight 8-bit fields, added to the counters every 255
   // events and at the end
   uint64_t ev_pk = 0;
@@ -118,41 +142,57 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
   };
 
   Screen Z;
-  Z.sig2f = (float)P.sig2;
+  Z.sig2f = P.sig2_f;
   Z.eps_v = P.eps_v;
   Z.eps_d = P.eps_d;
-  const float b2f = (float)P.b2;
   const float eps_v = P.eps_v, eps_d = P.eps_d;
-  const float reach_hs = (float)P.sigma + 2.f * eps_v;  // per-axis reach of a contact
+  const float reach_hs = P.sigma_f + 2.f * eps_v;  // per-axis reach of a contact
   const float INF = __int_as_float(0x7f800000);
-  constexpr int ITEMS = G >= 8 ? 1 : 2;  // special candidates per lane
   const uint64_t r1 = DOM ? (uint64_t)sweep : 0;
 
   auto slabs_at = [&](float f0, float f1, float f2) {
     return slab_of<DOM>(f0, SL.inv0, SL.base, nsl) | (slab_of<DOM>(f1, SL.inv1, SL.base, nsl) << 10) |
            (slab_of<DOM>(f2, SL.inv2, SL.base, nsl) << 20);
   };
-  // the FP32 shadow of an FP64 position: FP32 position minus FP32 corner
-  auto shadow = [&](double x, double c, double L, bool wr) {
-    if (!DOM) return (float)x;
-    float f = (float)x - (float)c;
-    if (wr) {
-      const float Lf = (float)L, Lh = 0.5f * Lf;
+  // minimum image on this lane's axis (identity where it cannot be needed)
+  auto wrap_a = [&](double d, bool on) {
+    if (on) d = wrap_i(d, SYS(L)[axc], dbits(SYS(half)[axc]));
+    return d;
+  };
+  // the FP32 shadow of the position x on this lane's axis, for every lane:
+  // FP32 position minus FP32 corner
+  auto shadows = [&](double x, float &f0, float &f1, float &f2) {
+    float f = f32_trunc(x) - cfa;
+    if (DOM && wra) {
+      const float Lf = SYS(Lf)[axc], Lh = 0.5f * Lf;
       f = f > Lh ? f - Lf : (f < -Lh ? f + Lf : f);
     }
-    return f;
+    f0 = __shfl_sync(gmask, f, gbase);
+    f1 = __shfl_sync(gmask, f, gbase + 1);
+    f2 = __shfl_sync(gmask, f, gbase + 2);
   };
-  // The bead in slot k sits at (x, y, z) now: FP64 position (write-through),
-  // shadow and slab masks.  A pivot never screens itself, so its copies are
-  // brought up to date only when it stops being the pivot.
-  auto settle = [&](int k, int id, double x, double y, double z, float f0, float f1, float f2, int os) {
-    if (gl < 3) Rr[3 * (int64_t)id + gl] = gl == 0 ? x : (gl == 1 ? y : z);
+  // d.v and d.d of a separation whose components the quad's lanes hold
+  // (lane 3's is not used): one chain of three FP64 instructions, d.v on the
+  // quad's first lane, d.d on the others
+  auto dots = [&](unsigned mask, double d, double &dv, double &dd) {
+    const double d0 = __shfl_sync(mask, d, qbase), d1 = __shfl_sync(mask, d, qbase + 1),
+                 d2 = __shfl_sync(mask, d, qbase + 2);
+    const bool first = ax == 0;
+    double s = d0 * (first ? v0 : d0);
+    s = __fma_rn(d1, first ? v1 : d1, s);
+    s = __fma_rn(d2, first ? v2 : d2, s);
+    dv = __shfl_sync(mask, s, qbase);
+    dd = __shfl_sync(mask, s, qbase + 1);
+  };
+  // The bead in slot k sits at x (this lane's axis) now: FP64 position
+  // (write-through), shadow and slab masks.  A pivot never screens itself, so
+  // its copies are brought up to date only when it stops being the pivot.
+  auto settle = [&](int k, int id, double x, float f0, float f1, float f2, int os) {
+    if (gl < 3) {
+      Rr[3 * (int64_t)id + gl] = x;
+      if (k < M64) st.pos[gl * M64 + k] = x;
+    }
     if (gl == (k & (G - 1))) {
-      if (k < M64) {
-        st.px[k] = x;
-        st.py[k] = y;
-        st.pz[k] = z;
-      }
       st.sh[k] = make_float4(f0, f1, f2, __int_as_float(id));
       const int nw = slabs_at(f0, f1, f2);
       if (nw != os)
@@ -190,24 +230,19 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
     }
     const int32_t *const Rstart = BATCH ? P.cstart + rp->cell_off : P.cstart;
     if (DOM) {
-      const int tk0 = unit % SYS(D)[0];
-      const int tk1 = (unit / SYS(D)[0]) % SYS(D)[1];
-      const int tk2 = unit / (SYS(D)[0] * SYS(D)[1]);
+      const int D0 = SYS(D)[0], D1 = SYS(D)[1];
+      const int tk = ax == 0 ? unit % D0 : (ax == 1 ? (unit / D0) % D1 : unit / (D0 * D1));
       const u64x4 w = philox(TAG_SHIFT, (uint64_t)sweep, 0, 0, P.seed, Rkey);
-      c0 = unit53(w.v[0]) * SYS(T)[0] + (double)tk0 * SYS(T)[0];
-      c1 = unit53(w.v[1]) * SYS(T)[1] + (double)tk1 * SYS(T)[1];
-      c2 = unit53(w.v[2]) * SYS(T)[2] + (double)tk2 * SYS(T)[2];
-      // A tile whose halo lies inside (0, L) on an axis never needs the
-      // minimum image or a wrap on that axis: every position it touches
-      // stays in one periodic image.
-      wr0 = !(c0 - P.halo_te > 0.0 && c0 + SYS(W)[0] + P.halo_te < SYS(L)[0]);
-      wr1 = !(c1 - P.halo_te > 0.0 && c1 + SYS(W)[1] + P.halo_te < SYS(L)[1]);
-      wr2 = !(c2 - P.halo_te > 0.0 && c2 + SYS(W)[2] + P.halo_te < SYS(L)[2]);
+      const double T = SYS(T)[axc], L = SYS(L)[axc];
+      ca = unit53(ax == 0 ? w.v[0] : (ax == 1 ? w.v[1] : w.v[2])) * T + (double)tk * T;
+      cfa = f32_trunc(ca);
+      Wfa = SYS(Wf)[axc];
+      wra = ax < 3 && !(ca - P.halo_te > 0.0 && ca + SYS(W)[axc] + P.halo_te < L);
     }
     bool live = true, over = false;
     int ns = 0;
-    stage_tile<G, DOM, SPRING, BATCH>(P, rp, st, gl, live, unit, c0, c1, c2, Rr, Rstart, S, M64, MNB, W,
-                                      SL, m, j1, ns, gmask, P.defer_mode == 1 ? &over : nullptr);
+    stage_tile<G, DOM, SPRING, BATCH>(P, rp, st, gl, live, unit, ca, Rr, Rstart, S, M64, MNB, W, SL, m,
+                                      j1, ns, gmask, P.defer_mode == 1 ? &over : nullptr);
     if (over && gl == 0) {
       const int at = atomicAdd(P.n_deferred, 1);
       P.deferred[CI(at, P.n_units, 32, P.status)] = gunit;
@@ -236,54 +271,56 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
       for (int s0 = 0; s0 < m; s0 += G) {
         const int s = s0 + gl;
         const bool f = s < m && P.po_flag[__float_as_int(st.sh[s].w)];
-        const unsigned bal = (__ballot_sync(gmask, f) & gmask) >> gbase;
+        unsigned bal = (__ballot_sync(gmask, f) & gmask) >> gbase;
         const int c = __popc(bal);
         if (e < before + c) {
-          p = s0 + (int)__fns(bal, 0, e - before + 1);
+          for (int i = before; i < e; ++i) bal &= bal - 1;
+          p = s0 + __ffs(bal) - 1;
           break;
         }
         before += c;
       }
     }
     if (P.dir_mode == ECMC_DIR_CART3) {
-      const int ax = (int)scale_below(w.v[1], 3);
-      v0 = ax == 0 ? 1.0 : 0.0;
-      v1 = ax == 1 ? 1.0 : 0.0;
-      v2 = ax == 2 ? 1.0 : 0.0;
+      va = ax == (int)scale_below(w.v[1], 3) ? 1.0 : 0.0;
     } else {
-      double a = 2.0 * unit53(w.v[1]) - 1.0;
-      double b = 2.0 * unit53(w.v[2]) - 1.0;
-      double c = 2.0 * unit53(w.v[3]) - 1.0;
+      // one component per lane
+      double t = 2.0 * unit53(ax == 0 ? w.v[1] : (ax == 1 ? w.v[2] : w.v[3])) - 1.0;
       uint64_t att = 0;
-      double s;
       for (;;) {
-        s = a * a + b * b + c * c;
-        if (s > 1e-6 && s <= 1.0) break;
+        const double t2 = t * t;
+        const double s = __shfl_sync(gmask, t2, gbase) + __shfl_sync(gmask, t2, gbase + 1) +
+                         __shfl_sync(gmask, t2, gbase + 2);
+        // s > 1e-6 && s <= 1
+        if (dbits(s) > dbits(1e-6) && dbits(s) <= dbits(1.0)) {
+          va = div_rn(t, sqrt_rn(s));
+          break;
+        }
         ++att;
         w = philox(r0, r1, r2, att, P.seed, Rkey);
-        a = 2.0 * unit53(w.v[0]) - 1.0;
-        b = 2.0 * unit53(w.v[1]) - 1.0;
-        c = 2.0 * unit53(w.v[2]) - 1.0;
+        t = 2.0 * unit53(ax == 0 ? w.v[0] : (ax == 1 ? w.v[1] : w.v[2])) - 1.0;
       }
-      // one component per lane
-      const double t = ((gl & 3) == 0 ? a : ((gl & 3) == 1 ? b : c)) / sqrt(s);
-      v0 = __shfl_sync(gmask, t, gbase);
-      v1 = __shfl_sync(gmask, t, gbase + 1);
-      v2 = __shfl_sync(gmask, t, gbase + 2);
     }
+    v0 = __shfl_sync(gmask, va, gbase);
+    v1 = __shfl_sync(gmask, va, gbase + 1);
+    v2 = __shfl_sync(gmask, va, gbase + 2);
     p = CI(p, m, 10, P.status);
     const float4 f = st.sh[p];
     pid = CI(__float_as_int(f.w), BATCH ? rp->n_beads : P.n, 11, P.status);
-    pos64(st, Rr, p, M64, q0, q1, q2);
+    qa = pos64(st, Rr, p, axc, M64);
+    if (ax == 3) {
+      qa = P.ell;
+      va = -1.0;
+    }
+    xrem = P.ell;
     nbw = st.nb[p];
     pf0 = f.x;
     pf1 = f.y;
     pf2 = f.z;
     oslab = slabs_at(pf0, pf1, pf2);
-    vf0 = (float)v0;
-    vf1 = (float)v1;
-    vf2 = (float)v2;
-    xrem = P.ell;
+    vf0 = f32_trunc(v0);
+    vf1 = f32_trunc(v1);
+    vf2 = f32_trunc(v2);
     lift = 0.0;
     nev = 0;
     ncontact = 0;
@@ -319,90 +356,89 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
     // ---------------------------------------------------------- A: screen
     // what the flight ends with at the latest
     const bool pass = dbits(P.s_cap) < dbits(xrem);
-    const float xc = act ? (pass ? P.s_cap_f : __double2float_ru(xrem)) : 0.f;
+    const float xc = act ? (pass ? P.s_cap_f : f32_above(xrem)) : 0.f;
     float ubl = xc;
     uint64_t lx = ~0ull, lkey = ~0ull;  // this lane's best evaluated candidate
     double ldv = 0.0;
-    int spk[ITEMS], sps[ITEMS];
-    float spl[ITEMS];
     if (SPRING) {
       // energies for the next G / 2 events of every group's EC: lane
       // 2 i + j draws bond j of event nev + i, so that the draw and the
-      // logarithm (some 50 dependent FP64 operations) are paid for once per
-      // G / 2 events.  All groups draw when one has used up its own.
+      // logarithm (some 50 FP64 instructions) are paid for once per G / 2
+      // events.  All groups draw when one has used up its own.
       if (__any_sync(FULL, act && dE_at == G / 2)) {
         const uint64_t r2 = DOM ? (uint64_t)unit : (uint64_t)(sweep + e);
         const u64x4 w = philox(TAG_SPRING | ((uint64_t)(DOM ? e : 0) << 8), r1, r2,
                                (uint64_t)(nev + (gl >> 1)), P.seed, Rkey);
-        dE = spring_dE((gl & 1) ? w.v[1] : w.v[0]);
+        dEk = div_rn(2.0 * spring_dE((gl & 1) ? w.v[1] : w.v[0]), P.k_spring);
         dE_at = 0;
       }
-      // lane 1: the bond to the previous bead, lane 2: to the next
-      const double my_dE = __shfl_sync(FULL, dE, gbase + 2 * dE_at + (gl == 2 ? 1 : 0));
-      ++dE_at;
-      if (act && (gl == 1 || gl == 2)) {
-        int t = gl == 1 ? nb_prev(nbw) : nb_next(nbw);
+      // quad j evaluates bond j (0: to the previous bead, 1: to the next)
+#pragma unroll
+      for (int j0 = 0; j0 < 2; j0 += NQ) {
+        const int j = j0 + qd;
+        const int t = j >= 2 || !act ? -1 : (j == 0 ? nb_prev(nbw) : nb_next(nbw));
+        const double bE = __shfl_sync(FULL, dEk, gbase + 2 * (dE_at & (G / 2 - 1)) + (j & 1));
+        // (a spring partner may lie beyond the tile's halo, across the
+        // periodic boundary: always the minimum image)
+        double d = 0.0, dv, dd;
+        if (t >= 0 && ax < 3) d = wrap_a(qa - pos64(st, Rr, CI(t, S, 20, P.status), ax, M64), true);
+        dots(FULL, d, dv, dd);
         if (t >= 0) {
-          t = CI(t, S, 20, P.status);
-          double kx, ky, kz;
-          pos64(st, Rr, t, M64, kx, ky, kz);
-          // (a spring partner may lie beyond the tile's halo, across the
-          // periodic boundary: always the minimum image)
-          const double x =
-              spring_x(wrap_i(q0 - kx, SYS(L)[0], dbits(SYS(half)[0])), wrap_i(q1 - ky, SYS(L)[1], dbits(SYS(half)[1])),
-                       wrap_i(q2 - kz, SYS(L)[2], dbits(SYS(half)[2])), v0, v1, v2, P.sigma, P.k_spring, my_dE, ldv);
-          lx = dbits(x);
-          lkey = make_key(KIND_TETHER, __float_as_int(st.sh[t].w), t);
-          ubl = fminf(ubl, __double2float_ru(x));
+          const double x = spring_flight(dv, dd, P.sigma, bE);
+          ubl = fminf(ubl, f32_above(x));
+          const uint64_t xb = dbits(x);
+          const uint64_t key = make_key(KIND_TETHER, __float_as_int(st.sh[t].w), t);
+          if (ax == 0 && (xb < lx || (xb == lx && key < lkey))) {
+            lx = xb;
+            lkey = key;
+            ldv = dv;
+          }
         }
       }
+      ++dE_at;
     }
-#pragma unroll
-    for (int r = 0; r < ITEMS; ++r) {
-      spk[r] = -1;
-      sps[r] = 0;
-      spl[r] = 0.f;
-      const int it = gl + r * G;
-      if (!act || it == 0 || it >= 6) continue;
-      if (it <= 2) {
-        if (SPRING) continue;
-        int t = it == 1 ? nb_prev(nbw) : nb_next(nbw);
-        if (t < 0) continue;
-        t = CI(t, S, 20, P.status);
+    // walls: lane a < 3 of the group, axis a
+    bool sw = false;
+    float wlb = 0.f;
+    if (DOM && gl < 3 && act) {
+      const float vfa = ax == 0 ? vf0 : (ax == 1 ? vf1 : vf2);
+      const float pfa = ax == 0 ? pf0 : (ax == 1 ? pf1 : pf2);
+      const float av = fabsf(vfa);
+      if (F32 && av >= 1e-30f) {
+        sw = true;
+        const float dist = signbit(vfa) ? pfa : Wfa - pfa;
+        wlb = div_lo(fmaxf(dist - eps_v, 0.f), av);
+        ubl = fminf(ubl, div_hi(fmaxf(dist, 0.f) + eps_v, av));
+      } else {
+        sw = nonzero(va);  // (|v_a| below FP32 range: evaluate in FP64)
+      }
+    }
+    // tethers: lanes TL and TL + 1
+    constexpr int TL = G >= 8 ? 4 : 0;
+    bool sth = false;
+    int ts = 0;
+    float tlb = 0.f;
+    if (!SPRING && act && (gl == TL || gl == TL + 1)) {
+      const int t = gl == TL ? nb_prev(nbw) : nb_next(nbw);
+      if (t >= 0) {
+        ts = CI(t, S, 20, P.status);
+        sth = true;
         if (F32) {
-          const float4 f = st.sh[t];
+          const float4 f = st.sh[ts];
           float d0 = pf0 - f.x, d1 = pf1 - f.y, d2 = pf2 - f.z;
           if (!DOM) {
-            d0 = wrapf(d0, (float)P.L[0]);
-            d1 = wrapf(d1, (float)P.L[1]);
-            d2 = wrapf(d2, (float)P.L[2]);
+            d0 = wrapf(d0, P.Lf[0]);
+            d1 = wrapf(d1, P.Lf[1]);
+            d2 = wrapf(d2, P.Lf[2]);
           }
           const float dd = __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, d0 * d0));
           const float dv = __fmaf_rn(d2, vf2, __fmaf_rn(d1, vf1, d0 * vf0));
-          const float rad = b2f - (dd - dv * dv);
+          const float rad = P.b2_f - (dd - dv * dv);
           const float lo = -dv - eps_v + sqrt_lo(fmaxf(rad - eps_d, 0.f));
           const float hi = -dv + eps_v + sqrt_hi(fmaxf(rad + eps_d, 0.f));
-          spl[r] = fmaxf(lo, 0.f);
+          tlb = fmaxf(lo, 0.f);
           ubl = fminf(ubl, fmaxf(hi, 0.f) + 1e-6f);
         }
-        spk[r] = KIND_TETHER;
-        sps[r] = t;
-      } else if (DOM) {
-        const int a = it - 3;
-        const float vfa = a == 0 ? vf0 : (a == 1 ? vf1 : vf2);
-        const double va = a == 0 ? v0 : (a == 1 ? v1 : v2);
-        if (!nonzero(va)) continue;
-        if (F32) {
-          const float pfa = a == 0 ? pf0 : (a == 1 ? pf1 : pf2);
-          const float dist = signbit(vfa) ? pfa : (float)SYS(W)[a] - pfa;
-          const float av = fabsf(vfa);
-          if (av >= 1e-30f) {
-            spl[r] = div_lo(fmaxf(dist - eps_v, 0.f), av);
-            ubl = fminf(ubl, div_hi(fmaxf(dist, 0.f) + eps_v, av));
-          }  // else |v_a| below FP32 range: evaluate in FP64
-        }
-        spk[r] = KIND_WALL;
-        sps[r] = a;
       }
     }
     // the slabs of the box that holds every obstacle in reach: within sigma
@@ -464,22 +500,38 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
       if (gl == (p & (G - 1)) && (p / G) >> 5 == w) c &= ~(1u << ((p / G) & 31));
       return act ? c : 0u;
     };
-    // exact evaluation of a contact or tether with slot k
-    auto exact = [&](int k, bool te) {
-      double kx, ky, kz, dv;
-      pos64(st, Rr, k, M64, kx, ky, kz);
-      const double x =
-          quad_x(te, wrapc(q0 - kx, SYS(L)[0], dbits(SYS(half)[0]), wr0), wrapc(q1 - ky, SYS(L)[1], dbits(SYS(half)[1]), wr1),
-                 wrapc(q2 - kz, SYS(L)[2], dbits(SYS(half)[2]), wr2), v0, v1, v2, te ? P.b2 : P.sig2, dv, PO);
-      if (F32) ++confirmed;
-      if (neg(x)) return;
-      const uint64_t key = make_key(te ? KIND_TETHER : KIND_HS, __float_as_int(st.sh[k].w), k);
+    // lane-wise exact evaluation of a contact or tether with slot k (the
+    // pivot's position on every lane: bq0..2)
+    double bq0 = 0.0, bq1 = 0.0, bq2 = 0.0;
+    auto all_axes = [&]() {
+      bq0 = __shfl_sync(FULL, qa, gbase);
+      bq1 = __shfl_sync(FULL, qa, gbase + 1);
+      bq2 = __shfl_sync(FULL, qa, gbase + 2);
+    };
+    auto keep = [&](double x, uint64_t key, double dv) {
       const uint64_t xb = dbits(x);
       if (xb < lx || (xb == lx && key < lkey)) {
         lx = xb;
         lkey = key;
         ldv = dv;
       }
+    };
+    bool wrg0 = false, wrg1 = false, wrg2 = false;  // wrap flags of the group's axes
+    if (!F32) {
+      const unsigned wb = __ballot_sync(FULL, wra) >> gbase;
+      wrg0 = wb & 1;
+      wrg1 = wb & 2;
+      wrg2 = wb & 4;
+    }
+    auto exact = [&](int k, bool te) {
+      const double k0 = pos64(st, Rr, k, 0, M64), k1 = pos64(st, Rr, k, 1, M64), k2 = pos64(st, Rr, k, 2, M64);
+      double dv;
+      const double x = quad_x(te, wrapc(bq0 - k0, SYS(L)[0], dbits(SYS(half)[0]), wrg0),
+                              wrapc(bq1 - k1, SYS(L)[1], dbits(SYS(half)[1]), wrg1),
+                              wrapc(bq2 - k2, SYS(L)[2], dbits(SYS(half)[2]), wrg2), v0, v1, v2,
+                              te ? P.b2 : P.sig2, dv, PO);
+      if (F32) ++confirmed;
+      if (!neg(x)) keep(x, make_key(te ? KIND_TETHER : KIND_HS, __float_as_int(st.sh[k].w), k), dv);
     };
 
     bool all_fp64 = !F32;  // evaluate every obstacle in the box
@@ -502,27 +554,25 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
           float a0 = pf0 - fa.x, a1 = pf1 - fa.y, a2 = pf2 - fa.z;
           float b0 = pf0 - fb.x, b1 = pf1 - fb.y, b2 = pf2 - fb.z;
           if (!DOM) {
-            a0 = wrapf(a0, (float)P.L[0]);
-            a1 = wrapf(a1, (float)P.L[1]);
-            a2 = wrapf(a2, (float)P.L[2]);
-            b0 = wrapf(b0, (float)P.L[0]);
-            b1 = wrapf(b1, (float)P.L[1]);
-            b2 = wrapf(b2, (float)P.L[2]);
+            a0 = wrapf(a0, P.Lf[0]);
+            a1 = wrapf(a1, P.Lf[1]);
+            a2 = wrapf(a2, P.Lf[2]);
+            b0 = wrapf(b0, P.Lf[0]);
+            b1 = wrapf(b1, P.Lf[1]);
+            b2 = wrapf(b2, P.Lf[2]);
           }
           screen_hs(Z, a0, a1, a2, vf0, vf1, vf2, ka, ubl, ks0, kl0, ks1, kl1, kovf);
           if (two) screen_hs(Z, b0, b1, b2, vf0, vf1, vf2, kb, ubl, ks0, kl0, ks1, kl1, kovf);
         }
       }
       const float U = group_minf<G>(ubl);
-      bool t0 = spk[0] == KIND_TETHER && spl[0] <= U;
-      bool t1 = ITEMS > 1 && spk[ITEMS - 1] == KIND_TETHER && spl[ITEMS - 1] <= U;
-      bool w0 = spk[0] == KIND_WALL && spl[0] <= U;
-      bool w1 = ITEMS > 1 && spk[ITEMS - 1] == KIND_WALL && spl[ITEMS - 1] <= U;
+      sth = sth && tlb <= U;
+      sw = sw && wlb <= U;
       bool h0 = ks0 >= 0 && kl0 <= U, h1 = ks1 >= 0 && kl1 <= U;
       if (P.rq_per_tile < 6) {
         // a small request_cap sends tiles with more survivors than that (or
         // more than 8 per request in reach) to the exhaustive evaluation
-        int ns = (t0 || w0) + (t1 || w1) + h0 + h1;
+        int ns = sth + sw + h0 + h1;
 #pragma unroll
         for (int off = G / 2; off > 0; off >>= 1) {
           ns += __shfl_xor_sync(FULL, ns, off);
@@ -532,91 +582,102 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
         if (all_fp64) {
           if (gl == 0) ++exh;
           h0 = h1 = kovf = false;
-          t0 = spk[0] == KIND_TETHER;
-          t1 = ITEMS > 1 && spk[ITEMS - 1] == KIND_TETHER;
-          w0 = spk[0] == KIND_WALL;
-          w1 = ITEMS > 1 && spk[ITEMS - 1] == KIND_WALL;
+          sth = !SPRING && ((gl == TL && nb_prev(nbw) >= 0) || (gl == TL + 1 && nb_next(nbw) >= 0));
+          sw = DOM && gl < 3 && nonzero(va);
         }
       }
-      spk[0] = w0 ? KIND_WALL : -1;
-      if (ITEMS > 1) spk[ITEMS - 1] = w1 ? KIND_WALL : -1;
       // ---------------------------------------------------------- B: FP64
-      // a lane rarely holds more than one survivor
-      while (__any_sync(FULL, t0 || t1 || h0 || h1)) {
-        if (t0 || t1 || h0 || h1) {
-          const bool te = t0 || t1;
-          const int k = t0 ? sps[0] : (t1 ? sps[ITEMS - 1] : (h0 ? ks0 : ks1));
-          if (t0) t0 = false;
-          else if (t1) t1 = false;
+      // The quads of a group take its survivors, one each per round
+      // (rarely more than one survives).
+      for (;;) {
+        const int code = sth ? ts | (1 << 30) : (h0 ? ks0 : (h1 ? ks1 : -1));
+        const unsigned bal = __ballot_sync(FULL, code >= 0);
+        if (bal == 0u) break;
+        const unsigned mine = (bal & gmask) >> gbase;
+        unsigned left = mine;
+#pragma unroll
+        for (int i = 0; i < NQ - 1; ++i)
+          if (i < qd) left &= left - 1u;
+        const bool on = left != 0u;
+        const int qcode = __shfl_sync(FULL, code, on ? gbase + __ffs(left) - 1 : lane);
+        if (code >= 0 && __popc(mine & ((1u << gl) - 1u)) < NQ) {
+          if (sth) sth = false;
           else if (h0) h0 = false;
           else h1 = false;
-          exact(k, te);
+        }
+        const bool te = on && (qcode >> 30) != 0;
+        const int k = on ? CI(qcode & 0x3FFFFFFF, S, 24, P.status) : 0;
+        double d = 0.0, dv, dd;
+        if (on && ax < 3) d = wrap_a(qa - pos64(st, Rr, k, ax, M64), wra);
+        dots(FULL, d, dv, dd);
+        const double R2 = te ? P.b2 : P.sig2;
+        double rad = R2 - __fma_rn(-dv, dv, dd);
+        bool hit = on && (te || (neg(dv) && posv(rad) && !(PO && dbits(dd) < dbits(R2))));
+        if (te && neg(rad)) rad = 0.0;
+        const double q = sqrt_rn(hit ? rad : 1.0);
+        double x = -dv + (te ? q : -q);
+        if (neg(x)) x = 0.0;
+        if (on && ax == 0) {
+          ++confirmed;
+          if (hit) keep(x, make_key(te ? KIND_TETHER : KIND_HS, __float_as_int(st.sh[k].w), k), dv);
         }
       }
-      if (__any_sync(FULL, kovf)) {
-        if (kovf && act) {
+      if (__any_sync(FULL, kovf || all_fp64)) {
+        const unsigned wb = __ballot_sync(FULL, wra) >> gbase;
+        wrg0 = wb & 1;
+        wrg1 = wb & 2;
+        wrg2 = wb & 4;
+        all_axes();
+        if (act && (kovf || all_fp64)) {
           // more than two possible winners in this lane: screen its obstacles
-          // again against the group's U and evaluate every one that can reach it
+          // again against the group's U and evaluate every one that can reach
+          // it (exhaustive evaluation: all of them)
           for (int w = 0; w < W; ++w) {
             unsigned c = cand_word(w);
             while (c) {
               const int k = CI(((w << 5) + __ffs(c) - 1) * G + gl, S, 22, P.status);
               c &= c - 1;
-              if (k == ks0 || k == ks1) continue;
-              const float4 f = st.sh[k];
-              float d0 = pf0 - f.x, d1 = pf1 - f.y, d2 = pf2 - f.z;
-              if (!DOM) {
-                d0 = wrapf(d0, (float)P.L[0]);
-                d1 = wrapf(d1, (float)P.L[1]);
-                d2 = wrapf(d2, (float)P.L[2]);
+              if (!all_fp64) {
+                if (k == ks0 || k == ks1) continue;
+                const float4 f = st.sh[k];
+                float d0 = pf0 - f.x, d1 = pf1 - f.y, d2 = pf2 - f.z;
+                if (!DOM) {
+                  d0 = wrapf(d0, P.Lf[0]);
+                  d1 = wrapf(d1, P.Lf[1]);
+                  d2 = wrapf(d2, P.Lf[2]);
+                }
+                bool possible;
+                const float lb = screen_lb(Z, d0, d1, d2, vf0, vf1, vf2, possible);
+                if (!possible || lb > U) continue;
               }
-              bool possible;
-              const float lb = screen_lb(Z, d0, d1, d2, vf0, vf1, vf2, possible);
-              if (possible && lb <= U) exact(k, false);
+              exact(k, false);
             }
           }
         }
         __syncwarp();
       }
     } else {
-#pragma unroll
-      for (int r = 0; r < ITEMS; ++r)
-        if (spk[r] == KIND_TETHER) exact(sps[r], true);
-    }
-    if (!F32 || P.rq_per_tile < 6) {
-      if (all_fp64) {
-        for (int w = 0; w < W; ++w) {
-          unsigned c = cand_word(w);
-          while (c) {
-            const int k = CI(((w << 5) + __ffs(c) - 1) * G + gl, S, 23, P.status);
-            c &= c - 1;
-            exact(k, false);
-          }
+      // plain form: the tethers and every obstacle in the box
+      all_axes();
+      if (sth) exact(ts, true);
+      for (int w = 0; w < W; ++w) {
+        unsigned c = cand_word(w);
+        while (c) {
+          const int k = CI(((w << 5) + __ffs(c) - 1) * G + gl, S, 23, P.status);
+          c &= c - 1;
+          exact(k, false);
         }
       }
       __syncwarp();
     }
     if (DOM) {
-      bool wall = spk[0] == KIND_WALL;
-      if (ITEMS > 1) wall = wall || spk[ITEMS - 1] == KIND_WALL;
-      if (__any_sync(FULL, wall)) {
-#pragma unroll
-        for (int r = 0; r < ITEMS; ++r) {
-          if (spk[r] != KIND_WALL) continue;
-          const int a = sps[r];
-          const double va = a == 0 ? v0 : (a == 1 ? v1 : v2);
-          const double qa = a == 0 ? q0 : (a == 1 ? q1 : q2);
-          const double ca = a == 0 ? c0 : (a == 1 ? c1 : c2);
-          const double loc = wrapc(qa - ca, SYS(L)[a], dbits(SYS(half)[a]), a == 0 ? wr0 : (a == 1 ? wr1 : wr2));
-          double x = (posv(va) ? SYS(W)[a] - loc : 0.0 - loc) / va;
+      if (__any_sync(FULL, sw)) {
+        if (sw) {
+          const double loc = wrap_a(qa - ca, wra);
+          double x = div_rn((posv(va) ? SYS(W)[axc] : 0.0) - loc, va);
           if (neg(x)) x = 0.0;
           if (F32) ++confirmed;
-          const uint64_t key = make_key(KIND_WALL, a, 0);
-          const uint64_t xb = dbits(x);
-          if (xb < lx || (xb == lx && key < lkey)) {
-            lx = xb;
-            lkey = key;
-          }
+          keep(x, make_key(KIND_WALL, ax, 0), 0.0);
         }
         __syncwarp();
       }
@@ -639,7 +700,7 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
     // ---------------------------------------------------------- D: move
     if (act && nev >= P.event_cap) {
       if (gl == 0) set_status(P.status, DEV_STUCK);
-      settle(p, pid, q0, q1, q2, pf0, pf1, pf2, oslab);
+      settle(p, pid, qa, pf0, pf1, pf2, oslab);
       state = EC_NEED;
     }
     if (state == EC_RUN) {
@@ -653,53 +714,46 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
         partner = key_id(wkey);
       }
       const bool bead = kind >= KIND_HS;
-      double k0 = 0.0, k1 = 0.0, k2 = 0.0;
-      if (bead) pos64(st, Rr, CI(slot, S, 30, P.status), M64, k0, k1, k2);
-      int di0 = 0, di1 = 0, di2 = 0;
-      if (wr0) di0 = step_i(q0, x, v0, SYS(L)[0]);
-      else q0 = __fma_rn(x, v0, q0);
-      if (wr1) di1 = step_i(q1, x, v1, SYS(L)[1]);
-      else q1 = __fma_rn(x, v1, q1);
-      if (wr2) di2 = step_i(q2, x, v2, SYS(L)[2]);
-      else q2 = __fma_rn(x, v2, q2);
-      if (gl == 0 && (di0 | di1 | di2)) {
-        if (di0) Ri[3 * (int64_t)pid] += di0;
-        if (di1) Ri[3 * (int64_t)pid + 1] += di1;
-        if (di2) Ri[3 * (int64_t)pid + 2] += di2;
+      double ka = 0.0;  // the partner's position on this lane's axis
+      if (bead && ax < 3) ka = pos64(st, Rr, CI(slot, S, 30, P.status), ax, M64);
+      // r + x v on the axes, what is left of ell on lane 3, and on lane AL
+      // (of G >= 8) the projection (r_target - r_pivot).v = -(d.v) - x
+      double y = __fma_rn(x, va, G >= 8 && gl == AL ? -wdv : qa);
+      const double proj = G >= 8 ? y : -wdv - x;
+      if (wra) {
+        const int di = wrap_step(y, SYS(L)[axc]);
+        if (di && gl < 3) Ri[3 * (int64_t)pid + gl] += di;
       }
+      qa = y;
+      xrem = __shfl_sync(gmask, qa, gbase + 3);
+      if (G >= 8 && gl == AL) qa = xrem;
       ++nev;
       int out = kind == KIND_END ? ECMC_EV_END : (kind == KIND_PASS ? ECMC_EV_PASS : ECMC_EV_WALL);
       int np = p;
       bool swapped = false;
-      if (kind == KIND_WALL) {
-        // (negation is exact in both precisions)
-        if (partner == 0) {
-          v0 = -v0;
-          vf0 = -vf0;
-        } else if (partner == 1) {
-          v1 = -v1;
-          vf1 = -vf1;
-        } else {
-          v2 = -v2;
-          vf2 = -vf2;
-        }
-      } else if (bead) {
-        // (r_target - r_pivot).v at contact = -(d.v) - x
-        const double proj = -wdv - x;
+      if (bead) {
         const bool hs = kind == KIND_HS;
-        if (slot >= m) {  // immotile: reflect
-          out = hs ? ECMC_EV_HS_REFLECT : ECMC_EV_TE_REFLECT;
-          refl_all = refl_all + proj;
-          const bool sp = SPRING && !hs;
-          mirror2(v0, v1, v2, wrapc(q0 - k0, SYS(L)[0], dbits(SYS(half)[0]), wr0 || sp),
-                  wrapc(q1 - k1, SYS(L)[1], dbits(SYS(half)[1]), wr1 || sp),
-                  wrapc(q2 - k2, SYS(L)[2], dbits(SYS(half)[2]), wr2 || sp));
-          vf0 = (float)v0;
-          vf1 = (float)v1;
-          vf2 = (float)v2;
+        const bool motile = slot < m;
+        out = hs ? (motile ? ECMC_EV_HS_LIFT : ECMC_EV_HS_REFLECT)
+                 : (motile ? ECMC_EV_TE_LIFT : ECMC_EV_TE_REFLECT);
+        const double acc = (motile ? lift : refl_all) + proj;
+        if (motile) lift = acc;
+        else refl_all = acc;
+        if (!motile) {
+          // v <- v - (2 v.d / d.d) d: reflection at the plane normal to d
+          // (Fig. 2c)
+          double d = 0.0, vd, dd;
+          if (ax < 3) d = wrap_a(qa - ka, wra || (SPRING && !hs));
+          dots(gmask, d, vd, dd);
+          const double t = twice(div_rn(vd, dd));
+          va = __fma_rn(-t, d, va);  // (lane 3: d = 0)
+          v0 = __shfl_sync(gmask, va, gbase);
+          v1 = __shfl_sync(gmask, va, gbase + 1);
+          v2 = __shfl_sync(gmask, va, gbase + 2);
+          vf0 = f32_trunc(v0);
+          vf1 = f32_trunc(v1);
+          vf2 = f32_trunc(v2);
         } else {
-          lift = lift + proj;
-          out = hs ? ECMC_EV_HS_LIFT : ECMC_EV_TE_LIFT;
           np = slot;
           if (!SPRING && !PO && hs && P.swap_mode) {
             bool go = true;
@@ -722,61 +776,59 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
               ++ncontact;
             }
             if (go) {
-              ++tried;
-              // every bond of both beads, positions exchanged, within b_max
+              if (gl == 0) ++tried;
+              // every bond of both beads, positions exchanged, within b_max:
+              // bond j (pivot to previous, next; partner to previous, next)
+              // on quad j
               bool ok = true;
               const unsigned nbs = st.nb[slot];
 #pragma unroll
-              for (int side = 0; side < 2; ++side) {
-                const double a0 = side == 0 ? k0 : q0;
-                const double a1 = side == 0 ? k1 : q1;
-                const double a2 = side == 0 ? k2 : q2;
-                const unsigned nbv = side == 0 ? nbw : nbs;
-#pragma unroll
-                for (int dir = 0; dir < 2; ++dir) {
-                  const int b = dir == 0 ? nb_prev(nbv) : nb_next(nbv);
-                  if (b < 0) continue;
-                  double b0, b1, b2;
-                  if (b == p) {
-                    b0 = k0;
-                    b1 = k1;
-                    b2 = k2;
-                  } else if (b == slot) {
-                    b0 = q0;
-                    b1 = q1;
-                    b2 = q2;
-                  } else {
-                    pos64(st, Rr, b, M64, b0, b1, b2);
-                  }
-                  const double f0 = wrapc(a0 - b0, SYS(L)[0], dbits(SYS(half)[0]), wr0);
-                  const double f1 = wrapc(a1 - b1, SYS(L)[1], dbits(SYS(half)[1]), wr1);
-                  const double f2 = wrapc(a2 - b2, SYS(L)[2], dbits(SYS(half)[2]), wr2);
-                  const double dd = __fma_rn(f2, f2, __fma_rn(f1, f1, f0 * f0));
-                  ok = ok && !(dbits(dd) > dbits(P.b2));
+              for (int j0 = 0; j0 < 4; j0 += NQ) {
+                const int j = j0 + qd;
+                const unsigned nbv = (j & 2) ? nbs : nbw;
+                const int b = j >= 4 ? -1 : ((j & 1) ? nb_next(nbv) : nb_prev(nbv));
+                double d = 0.0, dv, dd;
+                if (b >= 0 && ax < 3) {
+                  const double pa = (j & 2) ? qa : ka;
+                  const double ba = b == p ? ka : (b == slot ? qa : pos64(st, Rr, b, ax, M64));
+                  d = wrap_a(pa - ba, wra);
                 }
+                dots(gmask, d, dv, dd);
+                ok = ok && !(b >= 0 && dbits(dd) > dbits(P.b2));
               }
+              ok = (__ballot_sync(gmask, ok) & gmask) == gmask;
               if (ok) {
                 swapped = true;
                 out = ECMC_EV_SWAP;
                 np = p;
                 const float4 f = st.sh[slot];
                 const int kid = __float_as_int(f.w);
-                settle(slot, kid, q0, q1, q2, shadow(q0, c0, SYS(L)[0], wr0), shadow(q1, c1, SYS(L)[1], wr1),
-                       shadow(q2, c2, SYS(L)[2], wr2), slabs_at(f.x, f.y, f.z));
-                if (gl == 0) {
-#pragma unroll
-                  for (int a = 0; a < 3; ++a) {
-                    const int ti = Ri[3 * (int64_t)pid + a];
-                    Ri[3 * (int64_t)pid + a] = Ri[3 * (int64_t)kid + a];
-                    Ri[3 * (int64_t)kid + a] = ti;
-                  }
+                float g0, g1, g2;
+                shadows(qa, g0, g1, g2);
+                settle(slot, kid, qa, g0, g1, g2, slabs_at(f.x, f.y, f.z));
+                if (gl < 3) {
+                  const int ti = Ri[3 * (int64_t)pid + gl];
+                  Ri[3 * (int64_t)pid + gl] = Ri[3 * (int64_t)kid + gl];
+                  Ri[3 * (int64_t)kid + gl] = ti;
                 }
-                q0 = k0;
-                q1 = k1;
-                q2 = k2;
+                if (ax < 3) qa = ka;
               }
             }
           }
+        }
+      } else if (kind == KIND_WALL) {
+        // (negation is exact in both precisions)
+        const int wa = (int)partner;
+        if (ax == wa) va = -va;
+        if (wa == 0) {
+          v0 = -v0;
+          vf0 = -vf0;
+        } else if (wa == 1) {
+          v1 = -v1;
+          vf1 = -vf1;
+        } else {
+          v2 = -v2;
+          vf2 = -vf2;
         }
       }
       ev_pk += 1ull << (8 * out);
@@ -785,9 +837,8 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
         ev_pk = 0;
         ev_pn = 0;
       }
-      pf0 = shadow(q0, c0, SYS(L)[0], wr0);
-      pf1 = shadow(q1, c1, SYS(L)[1], wr1);
-      pf2 = shadow(q2, c2, SYS(L)[2], wr2);
+      __syncwarp(gmask);
+      shadows(qa, pf0, pf1, pf2);
       if (P.rec_digest) {
         fnv_mix(h, (uint64_t)pid);
         fnv_mix(h, ((uint64_t)(uint32_t)out << 32) | (uint64_t)(uint32_t)partner);
@@ -808,8 +859,7 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
           P.log[at] = ev;
         }
       }
-      xrem = xrem - x;
-      if (out == ECMC_EV_END || np != p) settle(p, pid, q0, q1, q2, pf0, pf1, pf2, oslab);
+      if (out == ECMC_EV_END || np != p) settle(p, pid, qa, pf0, pf1, pf2, oslab);
       if (out == ECMC_EV_END) state = EC_NEED;
       if (np != p) {
         // lift: the partner (motile, unmoved this event) becomes the pivot
@@ -817,9 +867,7 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
         const float4 f = st.sh[p];
         pid = CI(__float_as_int(f.w), BATCH ? rp->n_beads : P.n, 31, P.status);
         nbw = st.nb[p];
-        q0 = k0;
-        q1 = k1;
-        q2 = k2;
+        if (ax < 3) qa = ka;
         pf0 = f.x;
         pf1 = f.y;
         pf2 = f.z;
@@ -831,7 +879,7 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
       lift_all = lift_all + lift;
       nev_all += (unsigned long long)nev;
       ++ecs_done;
-      if (gl == 0 && P.rec_digest) {
+      if (gl == AL && P.rec_digest) {
         const int64_t idx = P.rec_offset +
                             (P.sweep_dev ? (sweep - P.rec_sweep0) * P.n_units * P.ecs_per_tile : 0) +
                             (DOM ? (int64_t)gunit * P.ecs_per_tile + e : (int64_t)e);
@@ -855,13 +903,15 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
   if (gl == 0 && ecs_done) {
     if (ev_pn) flush_outcomes();
     atomicAdd(&P.counters[CNT_EVENTS], nev_all);
-    if (tried) atomicAdd(&P.counters[CNT_SWAP_TRIED], tried);
-    if (confirmed) atomicAdd(&P.counters[CNT_CONFIRMED], confirmed);
+    if (tried) atomicAdd(&P.counters[CNT_SWAP_TRIED], (unsigned long long)tried);
+    if (confirmed) atomicAdd(&P.counters[CNT_CONFIRMED], (unsigned long long)confirmed);
     if (exh) atomicAdd(&P.counters[CNT_EXHAUSTIVE], (unsigned long long)exh);
-    atomicAdd(&P.counters[CNT_ECS], ecs_done);
+    atomicAdd(&P.counters[CNT_ECS], (unsigned long long)ecs_done);
+    atomicAdd(&P.sums[SUM_DISP], (double)ecs_done * P.ell);  // an EC's flights add up to ell
+  }
+  if (gl == AL && ecs_done) {
     atomicAdd(&P.sums[SUM_LIFT], lift_all);
     atomicAdd(&P.sums[SUM_REFL], refl_all);
-    atomicAdd(&P.sums[SUM_DISP], (double)ecs_done * P.ell);  // an EC's flights add up to ell
   }
 }
 #undef SYS
@@ -901,7 +951,7 @@ cudaError_t launch_ec_t(const ECParams &P0, cudaStream_t s) {
   }
   // tiles per block and resident blocks of the last shapes asked for
   struct Shape {
-    int S, M64, M, nsl, bt, nt, blocks;
+    int S, M64, M, nsl, bt, nt, blocks, units;
     float inv;
     size_t smem;
   };
@@ -923,7 +973,8 @@ cudaError_t launch_ec_t(const ECParams &P0, cudaStream_t s) {
       k.inv = 1.f;
     }
     for (const Shape &h : memo)
-      if (h.nt && h.S == S && h.M == M && h.bt == P.block_tiles && h.nsl == k.nsl && h.inv == k.inv) {
+      if (h.nt && h.S == S && h.M == M && h.bt == P.block_tiles && h.nsl == k.nsl && h.inv == k.inv &&
+          h.units == P.n_units) {
         *out = h;
         return cudaSuccess;
       }
@@ -931,14 +982,18 @@ cudaError_t launch_ec_t(const ECParams &P0, cudaStream_t s) {
     w.S = S;
     w.M = M;
     w.bt = P.block_tiles;
+    w.units = P.n_units;
     w.nsl = k.nsl;
     w.inv = k.inv;
     const int MQ = mask_quads(S, G, w.nsl);
     // FP64 positions in shared memory: the plain form reads many of them per
-    // event; the screened form one, and gives the room to more tiles instead
-    const int want = F32 ? 0 : S;
-    w.M64 = group_bytes(S, want, M, MQ) <= room ? want : 0;
-    const size_t per = group_bytes(S, w.M64, M, MQ);
+    // event; the screened form one (an L2 round trip less on every event),
+    // and keeps them there only while all tiles stay resident
+    size_t per = 0;
+    for (int want = S;; want = 0) {
+    w.M64 = want;
+    w.nt = w.blocks = 0;
+    per = group_bytes(S, want, M, MQ);
     int best = -1;
     for (int t = step; t <= 128 / G; t += step) {
       if (P.block_tiles > 0 && t != P.block_tiles && per * P.block_tiles <= (size_t)smem_max &&
@@ -953,6 +1008,8 @@ cudaError_t launch_ec_t(const ECParams &P0, cudaStream_t s) {
         w.nt = t;
         w.blocks = blocks;
       }
+    }
+    if (want == 0 || (w.nt > 0 && (!F32 || (long long)w.blocks * w.nt * sms >= P.n_units))) break;
     }
     if (w.nt == 0 || w.blocks < 1) return cudaErrorInvalidValue;
     w.smem = per * w.nt;
@@ -970,7 +1027,16 @@ cudaError_t launch_ec_t(const ECParams &P0, cudaStream_t s) {
     P.m64 = h.M64;
     P.nsl = h.nsl;
     P.sorg = DOM ? P.lorg : 0.f;
-    for (int a = 0; a < 3; ++a) P.sinv[a] = DOM ? h.inv : (float)(h.nsl / P.L[a]);
+    for (int a = 0; a < 3; ++a) {
+      P.sinv[a] = DOM ? h.inv : (float)(h.nsl / P.L[a]);
+      P.Lf[a] = (float)P.L[a];
+      P.Wf[a] = (float)P.W[a];
+    }
+    P.sigma_f = round_up_f32(P.sigma);
+    P.sig2_f = (float)P.sig2;
+    P.b2_f = (float)P.b2;
+    P.halo_hs_f = round_up_f32(P.halo_hs);
+    P.halo_te_f = round_up_f32(P.halo_te);
     P.defer_mode = mode;
     const long long want = (P.n_units + h.nt - 1) / h.nt;
     const long long room = (long long)h.blocks * sms;

@@ -342,6 +342,8 @@ ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *o) {
       R.D[a] = D;
       R.T[a] = T;
       R.W[a] = W;
+      R.Lf[a] = (float)R.L[a];
+      R.Wf[a] = (float)W;
       int k = (int)floor(R.L[a] / side);
       if (k < 3) return bfail(ECMC_EINVAL, "replica " + std::to_string(r) + ": box too small");
       R.nc[a] = k;

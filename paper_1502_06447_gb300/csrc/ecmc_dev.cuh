@@ -95,14 +95,105 @@ ECMC_HD double wrap_d(double d, double L, double half) {
 // kind, then to the smaller partner id.
 enum : int { KIND_END = 0, KIND_PASS = 1, KIND_WALL = 2, KIND_HS = 3, KIND_TETHER = 4 };
 
+// ---------------------------------------------------------------- sqrt, quotient
+// IEEE double square root and quotient (round to nearest even) in integer
+// arithmetic.  GB300 takes 55-60 cycles for a dependent FP64 operation and
+// the FP64 pipe 16 cycles of an SM for each FP64 warp instruction, so the
+// iterations behind sqrt() (700-900 cycles) and / (650-1450 cycles) were the
+// longest links of an event step; a dependent 32-bit multiply-add takes
+// about 4.  Both functions take a 22-bit estimate from the FP32 hardware
+// approximation, correct it twice by the exact remainder (64-bit wrapping
+// arithmetic: the remainders are known to be small), and settle the last
+// bit by the sign of one more exact remainder, so the result does not depend
+// on the estimate's rounding.
+#ifdef __CUDACC__
+// FP32 value of a double, rounded towards zero, by integer operations (the
+// conversion instruction takes as long as an FP64 operation); magnitudes
+// below 2^-126 give 0, above 2^127 are not used
+__device__ __forceinline__ float f32_trunc(double x) {
+  const uint64_t b = (uint64_t)__double_as_longlong(x);
+  const unsigned hi = (unsigned)(b >> 32);
+  const unsigned f = ((unsigned)(b >> 29) - (384u << 23)) & 0x7FFFFFFFu;
+  return __uint_as_float((hi & 0x80000000u) | ((hi & 0x7FFFFFFFu) < (897u << 20) ? 0u : f));
+}
+// an FP32 value above x >= 0
+__device__ __forceinline__ float f32_above(double x) {
+  return __uint_as_float(__float_as_uint(f32_trunc(x)) + 1u);
+}
+
+// y0 in [1/2, 1) as an integer times 2^-31
+__device__ __forceinline__ uint32_t seed_q31(float y) {
+  y = fminf(fmaxf(y, 0.5f), 0.99999994f);
+  return ((__float_as_uint(y) & 0x7FFFFFu) | 0x800000u) << 7;
+}
+
+// a = M 2^E with M in [2^52, 2^54), E even; m = M 2^-52 in [1, 4).
+// With y0 = (1 + d) / sqrt(m), |d| < 2^-21.5, s0 = m y0 has remainder
+// |m - s0^2| < 2^-18.4; s1 = s0 + (m - s0^2) y0 / 2 errs by less than
+// 2^-40.6, its remainder is below 2^-38.6 (exact in units of 2^-90), and
+// s2 = s1 + (m - s1^2) y0 / 2 errs by less than 2^-59.  The result is then
+// R = floor(s2 2^52) or R + 1: sqrt(M 2^52) > R + 1/2 exactly when
+// M 2^52 > R^2 + R (an integer square root is never half-way).
+__device__ __forceinline__ double sqrt_rn(double a) {
+  const uint64_t b = (uint64_t)__double_as_longlong(a);
+  const unsigned e = (unsigned)(b >> 52);
+  if (e - 1u >= 2046u) return sqrt(a);  // zero, subnormal, negative, inf, nan
+  const unsigned even = ~e & 1u;
+  const uint64_t M = ((b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << even;
+  const float mf = __uint_as_float(((127u + even) << 23) | ((unsigned)(b >> 29) & 0x7FFFFFu));
+  const uint32_t y = seed_q31(rsqrtf(mf));                       // Q31
+  const uint32_t s0 = __umulhi((uint32_t)(M >> 22), y << 1);     // Q30
+  const int64_t r0 = (int64_t)((M << 8) - (uint64_t)s0 * s0);    // Q60, < 2^41.7
+  const int64_t s1 = ((int64_t)((uint64_t)s0 << 32)) + (((int64_t)(int32_t)(r0 >> 12) * (int32_t)y) >> 18);  // Q62
+  const uint64_t t = (uint64_t)s1 >> 17;                         // Q45
+  const int64_t r1 = (int64_t)((M << 38) - t * t);               // Q90, < 2^51.5
+  const int64_t s2 = (int64_t)(t << 17) + (((int64_t)(int32_t)(r1 >> 22) * (int32_t)y) >> 38);  // Q62
+  const uint64_t R = (uint64_t)s2 >> 10;
+  const int64_t d = (int64_t)((M << 52) - R * R - R);
+  const uint64_t out = ((uint64_t)((e + 1023u) >> 1) << 52) + (R - 0x0010000000000000ull) + (d > 0 ? 1u : 0u);
+  return __longlong_as_double((long long)out);
+}
+
+// a / b = rho 2^k with rho = Ma / Mb in [1, 2) (Ma doubled when below Mb).
+// With y0 = (1 + d) / (Mb 2^-52), |d| < 2^-21.9, q0 = Ma y0 (Q28) errs by
+// less than 2^-20.8, q1 = q0 + (rho - q0) by less than 2^-42, q2 by less
+// than 2^-59; the last bit follows from the exact remainder (no quotient of
+// two doubles is half-way).
+__device__ __forceinline__ double div_rn(double a, double b) {
+  const uint64_t ab = (uint64_t)__double_as_longlong(a), bb = (uint64_t)__double_as_longlong(b);
+  const unsigned ea = (unsigned)(ab >> 52) & 0x7FFu, eb = (unsigned)(bb >> 52) & 0x7FFu;
+  uint64_t Ma = (ab & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
+  const uint64_t Mb = (bb & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
+  const unsigned less = Ma < Mb ? 1u : 0u;
+  const int eq = (int)ea - (int)eb + 1023 - (int)less;
+  if (ea - 1u >= 2046u || eb - 1u >= 2046u || eq < 1 || eq > 2045) return a / b;
+  Ma <<= less;
+  const float bf = __uint_as_float(0x3F800000u | ((unsigned)(bb >> 29) & 0x7FFFFFu));
+  const uint32_t y = seed_q31(__frcp_rn(bf));                         // Q31
+  const uint32_t q0 = __umulhi((uint32_t)(Ma >> 22), y) >> 1;         // Q30 Q31 / 2^33 = Q28
+  const int64_t r0 = (int64_t)((Ma << 28) - (uint64_t)q0 * Mb);       // Q80 of (rho - q0) b, < 2^60.3
+  const int64_t q1 = ((int64_t)((uint64_t)q0 << 17)) + (((int64_t)(int32_t)(r0 >> 30) * (int32_t)y) >> 36);  // Q45
+  const int64_t r1 = (int64_t)((Ma << 45) - (uint64_t)q1 * Mb);       // Q97, < 2^56
+  const int64_t q2 = (q1 << 7) + (((int64_t)(int32_t)(r1 >> 26) * (int32_t)y) >> 50);  // Q52
+  const int64_t rem = (int64_t)((Ma << 52) - (uint64_t)q2 * Mb);
+  const uint64_t Q = (uint64_t)q2 + (2 * rem > (int64_t)Mb ? 1ull : (2 * rem < -(int64_t)Mb ? ~0ull : 0ull));
+  const uint64_t out = (((uint64_t)(unsigned)eq) << 52) + (Q - 0x0010000000000000ull);
+  return __longlong_as_double((long long)(out | ((ab ^ bb) & 0x8000000000000000ull)));
+}
+#endif
+
 // ---------------------------------------------------------------- springs
 // Bead-spring chains (Sec. II, ECs with pair potentials): the pieces the EC
 // kernels need for a harmonic bond (k/2)(b - sigma)^2.  Host and device
 // share them, so the host can check them against other implementations.
 #ifdef __CUDA_ARCH__
 #define EC_FMA(a, b, c) __fma_rn(a, b, c)
+#define EC_SQRT(a) sqrt_rn(a)
+#define EC_DIV(a, b) div_rn(a, b)
 #else
 #define EC_FMA(a, b, c) fma(a, b, c)
+#define EC_SQRT(a) sqrt(a)
+#define EC_DIV(a, b) ((a) / (b))
 #endif
 
 // Natural logarithm of u in (0, 1]: u = m 2^e with m in [sqrt(1/2), sqrt(2)),
@@ -121,7 +212,7 @@ ECMC_HD double ec_log(double u) {
     m = m * 0.5;
     e += 1;
   }
-  const double z = (m - 1.0) / (m + 1.0);
+  const double z = EC_DIV(m - 1.0, m + 1.0);
   const double z2 = z * z;
   double s = 1.0 / 29.0;
   for (int n = 13; n >= 0; --n) s = s * z2 + 1.0 / (double)(2 * n + 1);
@@ -138,22 +229,31 @@ ECMC_HD double spring_dE(uint64_t w) { return -ec_log(1.0 - unit53(w)); }
 // path and rises after it (or from the start when d.v >= 0); dE is spent
 // on the rise: b_t = sigma + sqrt((b_s - sigma)^2 + 2 dE / k) with b_s the
 // bond length where the rise starts, x = -d.v + sqrt(b_t^2 - |d_perp|^2).
+// spring_flight: from dv = d.v, dd = d.d and dEk = 2 dE / k (signs are read
+// off the bit patterns: a comparison is an FP64 instruction on the device).
+ECMC_HD bool neg_bits(double x) {
+  int64_t b;
+  memcpy(&b, &x, sizeof(b));
+  return b < 0 && ((uint64_t)b << 1) != 0;
+}
+ECMC_HD double spring_flight(double dv, double dd, double sigma, double dEk) {
+  double perp2 = EC_FMA(-dv, dv, dd);
+  if (neg_bits(perp2)) perp2 = 0.0;
+  const double bs = EC_SQRT(neg_bits(dv) ? perp2 : dd);
+  const double e = bs - sigma;
+  const double bt = sigma + EC_SQRT(e * e + dEk);
+  // b_t >= b_s >= |d_perp| exactly; rounding can leave the radicand a few
+  // ulp below zero when dE ~ 0 and the path grazes the closest approach
+  double rad = bt * bt - perp2;
+  if (neg_bits(rad)) rad = 0.0;
+  const double x = -dv + EC_SQRT(rad);
+  return neg_bits(x) ? 0.0 : x;
+}
 ECMC_HD double spring_x(double d0, double d1, double d2, double v0, double v1, double v2,
                         double sigma, double k, double dE, double &dv) {
   dv = EC_FMA(d2, v2, EC_FMA(d1, v1, d0 * v0));
   const double dd = EC_FMA(d2, d2, EC_FMA(d1, d1, d0 * d0));
-  double perp2 = EC_FMA(-dv, dv, dd);
-  if (perp2 < 0.0) perp2 = 0.0;
-  const double bs = dv < 0.0 ? sqrt(perp2) : sqrt(dd);
-  const double e = bs - sigma;
-  const double bt = sigma + sqrt(e * e + 2.0 * dE / k);
-  // b_t >= b_s >= |d_perp| exactly; rounding can leave the radicand a few
-  // ulp below zero when dE ~ 0 and the path grazes the closest approach
-  double rad = bt * bt - perp2;
-  if (rad < 0.0) rad = 0.0;
-  double x = -dv + sqrt(rad);
-  if (x < 0.0) x = 0.0;
-  return x;
+  return spring_flight(dv, dd, sigma, EC_DIV(2.0 * dE, k));
 }
 
 ECMC_HD void fnv_mix(uint64_t &h, uint64_t w) {

@@ -48,6 +48,7 @@ inline float round_up_f32(double x) {
 // and its Philox key word.
 struct RepParams {
   double L[3], half[3], T[3], W[3], cs[3];
+  float Lf[3], Wf[3];  // FP32 values of L and W
   int32_t D[3], nc[3];
   int32_t N;
   int32_t pad;
@@ -89,6 +90,9 @@ struct ECParams {
   // FP32 screen margins (units of sigma, sigma^2)
   float eps_v, eps_d, eps_x;
   float s_cap_f;  // s_cap rounded up to FP32 (the screen's cap on a free flight)
+  // FP32 values (rounded up where they widen a search): a conversion in the
+  // kernel costs as much as an FP64 operation
+  float Lf[3], Wf[3], sigma_f, sig2_f, b2_f, halo_hs_f, halo_te_f;
   // buffers
   double *r;
   int32_t *img;
