@@ -103,7 +103,7 @@ typedef struct ecmc_opts {
                             tiles would get more; 0 -> most tiles per SM */
   int32_t request_cap;   /* screened form: FP64 evaluations per tile and step,
                             1..6; 0 -> 6.  Below 6 a tile with more survivors
-                            of the FP32 screen than that (or more than 8 times
+                            of the FP32 screen than that (or more than 4 times
                             as many obstacles in reach) is evaluated
                             exhaustively in FP64: same events, slower; small
                             caps exist to exercise that path

@@ -37,7 +37,7 @@ __device__ __forceinline__ double twice(double x) {
 // minimum image, same result as d > h ? d - L : (d < -h ? d + L : d)
 __device__ __forceinline__ double wrap_i(double d, double L, uint64_t hbits) {
   const uint64_t b = dbits(d);
-  if ((b & 0x7FFFFFFFFFFFFFFFull) > hbits) return ((int64_t)b < 0) ? d + L : d - L;
+  if ((b & 0x7FFFFFFFFFFFFFFFull) > hbits) return d + (((int64_t)b < 0) ? L : -L);  // (one FP64 instruction)
   return d;
 }
 
@@ -71,35 +71,16 @@ __device__ __forceinline__ int wrap_step(double &y, double L) {
 __device__ __forceinline__ double quad_x(bool tether, double d0, double d1, double d2, double v0,
                                          double v1, double v2, double R2, double &dv,
                                          bool skip_overlap = false) {
+  // (straight-line: the lanes of a warp hold different candidates, and some
+  // lane needs every instruction as a rule)
   dv = __fma_rn(d2, v2, __fma_rn(d1, v1, d0 * v0));
-  if (!tether && !neg(dv)) return -1.0;
   const double dd = __fma_rn(d2, d2, __fma_rn(d1, d1, d0 * d0));
-  if (!tether && skip_overlap && dbits(dd) < dbits(R2)) return -1.0;
   double rad = R2 - __fma_rn(-dv, dv, dd);
-  if (tether) {
-    if (neg(rad)) rad = 0.0;
-  } else if (!posv(rad)) {
-    return -1.0;
-  }
-  const double q = sqrt_rn(rad);
+  const bool hit = tether || (neg(dv) && posv(rad) && !(skip_overlap && dbits(dd) < dbits(R2)));
+  if (tether && neg(rad)) rad = 0.0;
+  const double q = sqrt_rn(hit ? rad : 1.0);
   const double x = -dv + (tether ? q : -q);
-  return neg(x) ? 0.0 : x;
-}
-
-// candidate key: kind (3 bits) | partner id (41 bits) | slot (20 bits).
-// Key order within equal x = (kind, partner id) order, the tie rule.
-__device__ __forceinline__ uint64_t make_key(int kind, int64_t id, int slot) {
-  return ((uint64_t)kind << 61) | (((uint64_t)id & ((1ull << 41) - 1)) << 20) |
-         (uint64_t)(slot & 0xFFFFF);
-}
-__device__ __forceinline__ int key_kind(uint64_t k) { return (int)(k >> 61); }
-__device__ __forceinline__ int64_t key_id(uint64_t k) { return (int64_t)((k >> 20) & ((1ull << 41) - 1)); }
-__device__ __forceinline__ int key_slot(uint64_t k) { return (int)(k & 0xFFFFF); }
-
-// x >= 0 always, so its bit pattern orders like the value
-__device__ __forceinline__ bool better(double x, uint64_t key, double bx, uint64_t bkey) {
-  const uint64_t a = dbits(x), b = dbits(bx);
-  return a < b || (a == b && key < bkey);
+  return hit ? (neg(x) ? 0.0 : x) : -1.0;
 }
 
 template <int G>
@@ -128,7 +109,8 @@ __device__ __forceinline__ float wrapf(float d, float L) {
 // grid of cells has to visit, count and gather up to 27 of them.  Slot s is
 // bit (s / G) of lane s % G: a lane reads and keeps current its own words and
 // no others, so the masks need no synchronisation.
-constexpr int HDR_BYTES = 32;
+constexpr int LIST_CAP = 32;
+constexpr int HDR_BYTES = 32 + 4 * LIST_CAP;
 
 // The accepted tile sizes count an overflow list of max(64, S / 4) slots per
 // tile, rounded up to a multiple of 8 (staging_budget in ecmc_internal.h).
@@ -140,8 +122,10 @@ __host__ __device__ __forceinline__ int ovf_cap_for(int S) {
 struct Stage {
   float4 *sh;       // [S] x, y, z, id (bits)
   double *pos;      // [3][M64]
-  unsigned *nb;     // [MNB] bond partner slots, 16 + 16 bits (0xFFFF = none)
+  uint2 *nb;        // [MNB] x: bond partner slots, 16 + 16 bits (0xFFFF = none);
+                    // y: slabs of the stored shadow, 10 bits per axis
   unsigned *mask;   // [3][nsl + 1][W][G]
+  int *lst;         // [LIST_CAP] candidates dealt to the lanes
   int *hdr;         // [0] hard-sphere joint beads, [1] tether-only joint beads
                     // placed, [2] joint beads seen, [3] overflow, [4] motile
                     // beads seen
@@ -161,16 +145,17 @@ __host__ __device__ __forceinline__ int mask_quads(int S, int G, int nsl) {
 // S, M64 and MNB are multiples of 8 and the masks whole 16-byte units, so
 // every array starts 16-byte aligned and group_bytes is a multiple of 16
 __host__ __device__ __forceinline__ size_t group_bytes(int S, int M64, int MNB, int MQ) {
-  return (size_t)S * 16 + (size_t)M64 * 24 + (size_t)MNB * 4 + (size_t)MQ * 16 + HDR_BYTES;
+  return (size_t)S * 16 + (size_t)M64 * 24 + (size_t)MNB * 8 + (size_t)MQ * 16 + HDR_BYTES;
 }
 
 __device__ __forceinline__ Stage carve(unsigned char *base, int S, int M64, int MNB, int MQ) {
   Stage s;
   s.sh = (float4 *)base;
   s.pos = (double *)(s.sh + S);
-  s.nb = (unsigned *)(s.pos + 3 * M64);
-  s.mask = s.nb + MNB;
+  s.nb = (uint2 *)(s.pos + 3 * M64);
+  s.mask = (unsigned *)(s.nb + MNB);
   s.hdr = (int *)(s.mask + 4 * MQ);
+  s.lst = s.hdr + 8;
 #ifdef ECMC_CHECKED
   s.cap = S;
   s.nglob = 0x7fffffffffffffffll;
@@ -257,10 +242,16 @@ __device__ __forceinline__ void screen_hs(const Screen &Z, float d0, float d1, f
   const float dv = __fmaf_rn(d2, vf2, __fmaf_rn(d1, vf1, d0 * vf0));
   const float disc = Z.sig2f - (dd - dv * dv);
   if (!(dv < Z.eps_v && disc > -Z.eps_d)) return;
-  const float lb = -dv - Z.eps_v - sqrt_hi(disc + Z.eps_d);
+  // bounds on sqrt(disc +- eps_d) from one reciprocal square root: with
+  // dm = max(disc, eps_d) and s = sqrt(dm), sqrt(dm + eps_d) <= s + eps_d / (2 s)
+  // and, for disc > eps_d, sqrt(disc - eps_d) >= s - eps_d / s
+  const float dm = fmaxf(disc, Z.eps_d);
+  const float rs = rsqrtf(dm);
+  const float q = dm * rs, t = Z.eps_d * rs;
+  const float lb = -dv - Z.eps_v - (q + 0.5f * t) * 1.000001f;
   if (lb > ubl) return;
   if (dv < -Z.eps_v && disc > Z.eps_d)
-    ubl = fminf(ubl, fmaxf(0.f, -dv + Z.eps_v - sqrt_lo(disc - Z.eps_d)) + 1e-6f);
+    ubl = fminf(ubl, fmaxf(0.f, -dv + Z.eps_v - (q - t) * 0.999999f) + 1e-6f);
   const float INF = __int_as_float(0x7f800000);
   if (kl0 > ubl) {
     ks0 = -1;
@@ -287,19 +278,19 @@ __device__ __forceinline__ float screen_lb(const Screen &Z, float d0, float d1, 
   const float dv = __fmaf_rn(d2, vf2, __fmaf_rn(d1, vf1, d0 * vf0));
   const float disc = Z.sig2f - (dd - dv * dv);
   possible = dv < Z.eps_v && disc > -Z.eps_d;
-  return -dv - Z.eps_v - sqrt_hi(fmaxf(disc + Z.eps_d, 0.f));
+  const float dm = fmaxf(disc, Z.eps_d), rs = rsqrtf(dm);
+  return -dv - Z.eps_v - (dm * rs + 0.5f * (Z.eps_d * rs)) * 1.000001f;
 }
 
-// FP64 position of staged slot k on one axis: shared memory for the first
-// M64 slots, otherwise the global position array (a joint bead, static this
-// sweep, or a motile one, written through by every move)
-__device__ __forceinline__ double pos64(const Stage &st, const double *r, int k, int axis, int M64) {
+// FP64 position of staged slot k (bead id) on one axis: shared memory for
+// the first M64 slots, otherwise the global position array (a joint bead,
+// static this sweep, or a motile one, written through by every move)
+__device__ __forceinline__ double pos64(const Stage &st, const double *r, int k, int id, int axis, int M64) {
 #ifdef ECMC_CHECKED
   if (st.status && !CHK(k, st.cap, 1, st.status)) return 0.0;
-  if (k >= M64 && st.status && !CHK(__float_as_int(st.sh[k].w), st.nglob, 2, st.status)) return 0.0;
+  if (k >= M64 && st.status && !CHK(id, st.nglob, 2, st.status)) return 0.0;
 #endif
-  if (k < M64) return st.pos[axis * M64 + k];
-  return r[3 * (int64_t)__float_as_int(st.sh[k].w) + axis];
+  return k < M64 ? st.pos[axis * M64 + k] : r[3 * (int64_t)id + axis];
 }
 
 // ---------------------------------------------------------------- staging
@@ -339,7 +330,7 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
       if (b < M64) put64(b, Rr + 3 * (int64_t)b);
       st.sh[b] = make_float4(f32_trunc(x), f32_trunc(y), f32_trunc(z), __int_as_float(b));
       const int c = b % SYS(N);
-      st.nb[b] = nb_pack(c == 0 ? -1 : b - 1, c == SYS(N) - 1 ? -1 : b + 1);
+      st.nb[b].x = nb_pack(c == 0 ? -1 : b - 1, c == SYS(N) - 1 ? -1 : b + 1);
     }
     m = n;
     j1 = 0;
@@ -499,7 +490,7 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
       const int id = idt[s], c = id % Nc;
       const int prev = c != 0 ? find_id(idt, 0, m, id - 1) : -1;
       const int next = c != Nc - 1 ? find_id(idt, 0, m, id + 1) : -1;
-      st.nb[s] = nb_pack(prev, next);
+      st.nb[s].x = nb_pack(prev, next);
     }
     __syncwarp(mask);
     const int32_t *const Rtag = P.tag + (BATCH ? rp->bead_off : 0);
@@ -510,11 +501,11 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
       const bool dn = c != 0 && Rtag[id - 1] == unit;
       if (up) {
         const int t = find_id(idt, 0, m, id + 1);
-        if (t >= 0) nbh[2 * t] = (unsigned short)s;
+        if (t >= 0) nbh[4 * t] = (unsigned short)s;
       }
       if (dn) {
         const int t = find_id(idt, 0, m, id - 1);
-        if (t >= 0) nbh[2 * t + 1] = (unsigned short)s;
+        if (t >= 0) nbh[4 * t + 1] = (unsigned short)s;
       }
     }
     __syncwarp(mask);
@@ -524,7 +515,7 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
       const int id = idt[s], c = id % Nc;
 #pragma unroll
       for (int dir = 0; dir < 2; ++dir) {
-        if (nbh[2 * s + dir] != 0xFFFF) continue;
+        if (nbh[4 * s + dir] != 0xFFFF) continue;
         const int q = dir == 0 ? (c != 0 ? id - 1 : -1) : (c != Nc - 1 ? id + 1 : -1);
         if (q < 0) continue;
         if (!SPRING) {
@@ -540,7 +531,7 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
         const int slot = atomicAdd(&st.hdr[6], 1);
         if (slot < S) {
           idt[slot] = q;
-          nbh[2 * s + dir] = (unsigned short)slot;
+          nbh[4 * s + dir] = (unsigned short)slot;
           if (slot < M64) put64(slot, Rr + 3 * (int64_t)q);
         }
       }
@@ -596,9 +587,12 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
     const int b = s / G;
     unsigned *const w = st.mask + (b >> 5) * G + gl;
     const unsigned bit = 1u << (b & 31);
-    w[(slab_of<DOM>(f.x, SL.inv0, SL.base, nsl) + 1) * row] |= bit;
-    w[(nsl + 1 + slab_of<DOM>(f.y, SL.inv1, SL.base, nsl) + 1) * row] |= bit;
-    w[(2 * (nsl + 1) + slab_of<DOM>(f.z, SL.inv2, SL.base, nsl) + 1) * row] |= bit;
+    const int k0 = slab_of<DOM>(f.x, SL.inv0, SL.base, nsl), k1 = slab_of<DOM>(f.y, SL.inv1, SL.base, nsl),
+              k2 = slab_of<DOM>(f.z, SL.inv2, SL.base, nsl);
+    if (s < m) st.nb[s].y = (unsigned)(k0 | (k1 << 10) | (k2 << 20));
+    w[(k0 + 1) * row] |= bit;
+    w[(nsl + 1 + k1 + 1) * row] |= bit;
+    w[(2 * (nsl + 1) + k2 + 1) * row] |= bit;
   }
   for (int a = 0; a < 3; ++a)
     for (int w = 0; w < W; ++w) {

@@ -43,19 +43,15 @@ namespace ecmc {
 
 namespace {
 
-// argmin over the group by (x, key)
-template <int G>
-__device__ __forceinline__ void group_argmin(uint64_t &bx, uint64_t &bkey) {
-#pragma unroll
-  for (int off = G / 2; off > 0; off >>= 1) {
-    const uint64_t ox = __shfl_xor_sync(FULL, bx, off);
-    const uint64_t ok = __shfl_xor_sync(FULL, bkey, off);
-    if (ox < bx || (ox == bx && ok < bkey)) {
-      bx = ox;
-      bkey = ok;
-    }
-  }
-}
+// A group's candidates: x (bits), kind << 28 | slot, d.v before the flight and
+// the partner's position on this lane's axis.  In a quad all lanes hold the
+// same x, code and d.v.
+struct Cand {
+  uint64_t x;
+  int code;
+  double dv, pos;
+};
+constexpr int CAND_NONE = -1;
 
 #define SYS(f) (BATCH ? rp->f : P.f)
 
@@ -117,7 +113,9 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
   double v0 = 0.0, v1 = 0.0, v2 = 0.0, xrem = 0.0;  // the same, on every lane
   double lift = 0.0, refl_all = 0.0;                // (lane AL)
   float pf0 = 0.f, pf1 = 0.f, pf2 = 0.f, vf0 = 0.f, vf1 = 0.f, vf2 = 0.f;
-  int64_t nev = 0;
+  float rb0 = 0.f, rb1 = 0.f, rb2 = 0.f;  // per-axis reach of a contact against the direction
+  unsigned nev = 0;
+  unsigned pmask = ~0u;  // this lane's first mask word without the pivot
   unsigned ncontact = 0, swgo = 0;  // swap proposals of this and the next contacts, one bit each
   uint64_t h = 0;
   // springs: 2 dE / k of the next G / 2 events, drawn together
@@ -127,19 +125,10 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
   double lift_all = 0.0;
   unsigned long long nev_all = 0;
   unsigned tried = 0, confirmed = 0, ecs_done = 0, exh = 0;
-  // events by outcome: eight 8-bit fields, added to the counters every 255
-  // events and at the end
-  uint64_t ev_pk = 0;
-  unsigned ev_pn = 0;
-  auto flush_outcomes = [&]() {
-#pragma unroll
-    for (int k = 0; k < ECMC_NEV; ++k) {
-      const unsigned c = (unsigned)(ev_pk >> (8 * k)) & 0xFFu;
-      if (c) atomicAdd(&P.counters[k], (unsigned long long)c);
-    }
-    ev_pk = 0;
-    ev_pn = 0;
-  };
+  // events by outcome: lane k of a group (of 4 lanes: lane k % 4, two counts)
+  // counts outcome k
+  unsigned ev_lo = 0, ev_hi = 0;
+  const unsigned event_cap = P.event_cap < 0xFFFFFFFFll ? (unsigned)P.event_cap : 0xFFFFFFFFu;
 
   Screen Z;
   Z.sig2f = P.sig2_f;
@@ -147,6 +136,19 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
   Z.eps_d = P.eps_d;
   const float eps_v = P.eps_v, eps_d = P.eps_d;
   const float reach_hs = P.sigma_f + 2.f * eps_v;  // per-axis reach of a contact
+  // A contact partner lies ahead, within the half sphere of radius sigma
+  // around v from the path: against the direction of v_a it reaches no more
+  // than sigma sqrt(1 - v_a^2).  The box of a flight holds a third fewer
+  // obstacles than one with sigma on both sides.
+  auto reach_back = [&](float v) { return P.sigma_f * sqrt_hi(fmaxf(1.f - v * v, 0.f) + 1e-6f) + 2.f * eps_v; };
+  auto new_direction = [&]() {
+    vf0 = f32_trunc(v0);
+    vf1 = f32_trunc(v1);
+    vf2 = f32_trunc(v2);
+    rb0 = reach_back(vf0);
+    rb1 = reach_back(vf1);
+    rb2 = reach_back(vf2);
+  };
   const float INF = __int_as_float(0x7f800000);
   const uint64_t r1 = DOM ? (uint64_t)sweep : 0;
 
@@ -195,9 +197,11 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
     if (gl == (k & (G - 1))) {
       st.sh[k] = make_float4(f0, f1, f2, __int_as_float(id));
       const int nw = slabs_at(f0, f1, f2);
-      if (nw != os)
+      if (nw != os) {
+        st.nb[k].y = (unsigned)nw;
         slab_move(st, G, W, nsl, k, os & 1023, (os >> 10) & 1023, os >> 20, nw & 1023,
                   (nw >> 10) & 1023, nw >> 20);
+      }
     }
   };
 
@@ -307,20 +311,20 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
     p = CI(p, m, 10, P.status);
     const float4 f = st.sh[p];
     pid = CI(__float_as_int(f.w), BATCH ? rp->n_beads : P.n, 11, P.status);
-    qa = pos64(st, Rr, p, axc, M64);
+    qa = pos64(st, Rr, p, pid, axc, M64);
     if (ax == 3) {
       qa = P.ell;
       va = -1.0;
     }
     xrem = P.ell;
-    nbw = st.nb[p];
+    const uint2 nb = st.nb[p];
+    nbw = nb.x;
+    oslab = (int)nb.y;
+    pmask = gl == (p & (G - 1)) && p / G < 32 ? ~(1u << ((p / G) & 31)) : ~0u;
     pf0 = f.x;
     pf1 = f.y;
     pf2 = f.z;
-    oslab = slabs_at(pf0, pf1, pf2);
-    vf0 = f32_trunc(v0);
-    vf1 = f32_trunc(v1);
-    vf2 = f32_trunc(v2);
+    new_direction();
     lift = 0.0;
     nev = 0;
     ncontact = 0;
@@ -358,8 +362,18 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
     const bool pass = dbits(P.s_cap) < dbits(xrem);
     const float xc = act ? (pass ? P.s_cap_f : f32_above(xrem)) : 0.f;
     float ubl = xc;
-    uint64_t lx = ~0ull, lkey = ~0ull;  // this lane's best evaluated candidate
-    double ldv = 0.0;
+    Cand best{~0ull, CAND_NONE, 0.0, 0.0};  // this lane's best evaluated candidate
+    // (x, kind, partner id) order: an exact tie in x goes to the smaller kind,
+    // then to the smaller id (wall: axis)
+    auto beats = [&](uint64_t xb, int code) {
+      if (xb != best.x || best.code == CAND_NONE) return xb < best.x;
+      const int k0 = code >> 28, k1 = best.code >> 28;
+      if (k0 != k1 || k0 == KIND_WALL) return code < best.code;
+      return __float_as_int(st.sh[code & 0xFFFFFFF].w) < __float_as_int(st.sh[best.code & 0xFFFFFFF].w);
+    };
+    auto keep = [&](double x, int code, double dv, double pos) {
+      if (beats(dbits(x), code)) best = Cand{dbits(x), code, dv, pos};
+    };
     if (SPRING) {
       // energies for the next G / 2 events of every group's EC: lane
       // 2 i + j draws bond j of event nev + i, so that the draw and the
@@ -380,76 +394,30 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
         const double bE = __shfl_sync(FULL, dEk, gbase + 2 * (dE_at & (G / 2 - 1)) + (j & 1));
         // (a spring partner may lie beyond the tile's halo, across the
         // periodic boundary: always the minimum image)
-        double d = 0.0, dv, dd;
-        if (t >= 0 && ax < 3) d = wrap_a(qa - pos64(st, Rr, CI(t, S, 20, P.status), ax, M64), true);
+        double d = 0.0, dv, dd, pos = 0.0;
+        if (t >= 0 && ax < 3) {
+          pos = pos64(st, Rr, CI(t, S, 20, P.status), __float_as_int(st.sh[t].w), ax, M64);
+          d = wrap_a(qa - pos, true);
+        }
         dots(FULL, d, dv, dd);
         if (t >= 0) {
           const double x = spring_flight(dv, dd, P.sigma, bE);
           ubl = fminf(ubl, f32_above(x));
-          const uint64_t xb = dbits(x);
-          const uint64_t key = make_key(KIND_TETHER, __float_as_int(st.sh[t].w), t);
-          if (ax == 0 && (xb < lx || (xb == lx && key < lkey))) {
-            lx = xb;
-            lkey = key;
-            ldv = dv;
-          }
+          if (F32 || ax == 0) keep(x, (KIND_TETHER << 28) | t, dv, pos);
         }
       }
       ++dE_at;
     }
-    // walls: lane a < 3 of the group, axis a
-    bool sw = false;
-    float wlb = 0.f;
-    if (DOM && gl < 3 && act) {
-      const float vfa = ax == 0 ? vf0 : (ax == 1 ? vf1 : vf2);
-      const float pfa = ax == 0 ? pf0 : (ax == 1 ? pf1 : pf2);
-      const float av = fabsf(vfa);
-      if (F32 && av >= 1e-30f) {
-        sw = true;
-        const float dist = signbit(vfa) ? pfa : Wfa - pfa;
-        wlb = div_lo(fmaxf(dist - eps_v, 0.f), av);
-        ubl = fminf(ubl, div_hi(fmaxf(dist, 0.f) + eps_v, av));
-      } else {
-        sw = nonzero(va);  // (|v_a| below FP32 range: evaluate in FP64)
-      }
-    }
-    // tethers: lanes TL and TL + 1
-    constexpr int TL = G >= 8 ? 4 : 0;
-    bool sth = false;
-    int ts = 0;
-    float tlb = 0.f;
-    if (!SPRING && act && (gl == TL || gl == TL + 1)) {
-      const int t = gl == TL ? nb_prev(nbw) : nb_next(nbw);
-      if (t >= 0) {
-        ts = CI(t, S, 20, P.status);
-        sth = true;
-        if (F32) {
-          const float4 f = st.sh[ts];
-          float d0 = pf0 - f.x, d1 = pf1 - f.y, d2 = pf2 - f.z;
-          if (!DOM) {
-            d0 = wrapf(d0, P.Lf[0]);
-            d1 = wrapf(d1, P.Lf[1]);
-            d2 = wrapf(d2, P.Lf[2]);
-          }
-          const float dd = __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, d0 * d0));
-          const float dv = __fmaf_rn(d2, vf2, __fmaf_rn(d1, vf1, d0 * vf0));
-          const float rad = P.b2_f - (dd - dv * dv);
-          const float lo = -dv - eps_v + sqrt_lo(fmaxf(rad - eps_d, 0.f));
-          const float hi = -dv + eps_v + sqrt_hi(fmaxf(rad + eps_d, 0.f));
-          tlb = fmaxf(lo, 0.f);
-          ubl = fminf(ubl, fmaxf(hi, 0.f) + 1e-6f);
-        }
-      }
-    }
-    // the slabs of the box that holds every obstacle in reach: within sigma
-    // (plus the screen's margin) of the path [pf, pf + xc vf] on every axis
+    // the slabs of the box that holds every obstacle in reach of the path
+    // [pf, pf + xc vf]
     const float e0 = xc * vf0, e1 = xc * vf1, e2 = xc * vf2;
     const unsigned *wa0, *wa1, *wa2, *wb0, *wb1, *wb2;
     bool fl0 = false, fl1 = false, fl2 = false;  // serial: the range goes around the box
     {
-      const float l0 = pf0 - reach_hs + fminf(e0, 0.f), h0 = pf0 + reach_hs + fmaxf(e0, 0.f);
-      const float l1 = pf1 - reach_hs + fminf(e1, 0.f), h1 = pf1 + reach_hs + fmaxf(e1, 0.f);
-      const float l2 = pf2 - reach_hs + fminf(e2, 0.f), h2 = pf2 + reach_hs + fmaxf(e2, 0.f);
+      const bool u0 = signbit(vf0), u1 = signbit(vf1), u2 = signbit(vf2);
+      const float l0 = pf0 + (u0 ? e0 - reach_hs : -rb0), h0 = pf0 + (u0 ? rb0 : e0 + reach_hs);
+      const float l1 = pf1 + (u1 ? e1 - reach_hs : -rb1), h1 = pf1 + (u1 ? rb1 : e1 + reach_hs);
+      const float l2 = pf2 + (u2 ? e2 - reach_hs : -rb2), h2 = pf2 + (u2 ? rb2 : e2 + reach_hs);
       int a0 = slab_raw(l0, SL.inv0, SL.base), b0 = slab_raw(h0, SL.inv0, SL.base);
       int a1 = slab_raw(l1, SL.inv1, SL.base), b1 = slab_raw(h1, SL.inv1, SL.base);
       int a2 = slab_raw(l2, SL.inv2, SL.base), b2 = slab_raw(h2, SL.inv2, SL.base);
@@ -497,7 +465,8 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
         c = (fl0 ? wb0[o] | ~wa0[o] : wb0[o] & ~wa0[o]) & (fl1 ? wb1[o] | ~wa1[o] : wb1[o] & ~wa1[o]) &
             (fl2 ? wb2[o] | ~wa2[o] : wb2[o] & ~wa2[o]) & all;
       }
-      if (gl == (p & (G - 1)) && (p / G) >> 5 == w) c &= ~(1u << ((p / G) & 31));
+      if (w == 0) c &= pmask;
+      else if (gl == (p & (G - 1)) && (p / G) >> 5 == w) c &= ~(1u << ((p / G) & 31));
       return act ? c : 0u;
     };
     // lane-wise exact evaluation of a contact or tether with slot k (the
@@ -508,218 +477,364 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
       bq1 = __shfl_sync(FULL, qa, gbase + 1);
       bq2 = __shfl_sync(FULL, qa, gbase + 2);
     };
-    auto keep = [&](double x, uint64_t key, double dv) {
-      const uint64_t xb = dbits(x);
-      if (xb < lx || (xb == lx && key < lkey)) {
-        lx = xb;
-        lkey = key;
-        ldv = dv;
-      }
-    };
     bool wrg0 = false, wrg1 = false, wrg2 = false;  // wrap flags of the group's axes
-    if (!F32) {
+    auto wrap_flags = [&]() {
       const unsigned wb = __ballot_sync(FULL, wra) >> gbase;
       wrg0 = wb & 1;
       wrg1 = wb & 2;
       wrg2 = wb & 4;
-    }
+    };
     auto exact = [&](int k, bool te) {
-      const double k0 = pos64(st, Rr, k, 0, M64), k1 = pos64(st, Rr, k, 1, M64), k2 = pos64(st, Rr, k, 2, M64);
+      const int kid = __float_as_int(st.sh[k].w);
+      const double k0 = pos64(st, Rr, k, kid, 0, M64), k1 = pos64(st, Rr, k, kid, 1, M64),
+                   k2 = pos64(st, Rr, k, kid, 2, M64);
       double dv;
       const double x = quad_x(te, wrapc(bq0 - k0, SYS(L)[0], dbits(SYS(half)[0]), wrg0),
                               wrapc(bq1 - k1, SYS(L)[1], dbits(SYS(half)[1]), wrg1),
                               wrapc(bq2 - k2, SYS(L)[2], dbits(SYS(half)[2]), wrg2), v0, v1, v2,
                               te ? P.b2 : P.sig2, dv, PO);
       if (F32) ++confirmed;
-      if (!neg(x)) keep(x, make_key(te ? KIND_TETHER : KIND_HS, __float_as_int(st.sh[k].w), k), dv);
+      if (!neg(x)) keep(x, ((te ? KIND_TETHER : KIND_HS) << 28) | k, dv, 0.0);
     };
 
-    bool all_fp64 = !F32;  // evaluate every obstacle in the box
+    // walls: lane a < 3 of the group, axis a; tethers: lanes TL and TL + 1
+    constexpr int TL = G >= 8 ? 4 : 0;
+    bool sw = DOM && gl < 3 && act && nonzero(va);
+    bool sth = false;
+    int ts = 0;
+    if (!SPRING && act && (gl == TL || gl == TL + 1)) {
+      const int t = gl == TL ? nb_prev(nbw) : nb_next(nbw);
+      sth = t >= 0;
+      if (sth) ts = CI(t, S, 20, P.status);
+    }
+    // Which lanes may hold the winner: `quads`, more than one quad of a group;
+    // `lanes`, single lanes (walls, lane-wise evaluation: no Cand::pos)
+    bool quads, lanes = false;
     if (F32) {
       int ks0 = -1, ks1 = -1;
       float kl0 = INF, kl1 = INF;
       bool kovf = false;
       int nscr = 0;
-      for (int w = 0; w < W; ++w) {
-        unsigned c = cand_word(w);
-        nscr += __popc(c);
-        // two obstacles per round, so that their loads overlap
-        while (c) {
-          const int ka = CI(((w << 5) + __ffs(c) - 1) * G + gl, S, 21, P.status);
-          c &= c - 1;
-          const bool two = c != 0;
-          const int kb = two ? CI(((w << 5) + __ffs(c) - 1) * G + gl, S, 21, P.status) : ka;
-          c &= c - 1;
-          const float4 fa = st.sh[ka], fb = st.sh[kb];
-          float a0 = pf0 - fa.x, a1 = pf1 - fa.y, a2 = pf2 - fa.z;
-          float b0 = pf0 - fb.x, b1 = pf1 - fb.y, b2 = pf2 - fb.z;
-          if (!DOM) {
-            a0 = wrapf(a0, P.Lf[0]);
-            a1 = wrapf(a1, P.Lf[1]);
-            a2 = wrapf(a2, P.Lf[2]);
-            b0 = wrapf(b0, P.Lf[0]);
-            b1 = wrapf(b1, P.Lf[1]);
-            b2 = wrapf(b2, P.Lf[2]);
+      // the FP32 numbers of this lane's tether and wall
+      float tdv = 0.f, trad = 0.f;
+      if (sth) {
+        const float4 f = st.sh[ts];
+        float d0 = pf0 - f.x, d1 = pf1 - f.y, d2 = pf2 - f.z;
+        if (!DOM) {
+          d0 = wrapf(d0, P.Lf[0]);
+          d1 = wrapf(d1, P.Lf[1]);
+          d2 = wrapf(d2, P.Lf[2]);
+        }
+        const float dd = __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, d0 * d0));
+        tdv = __fmaf_rn(d2, vf2, __fmaf_rn(d1, vf1, d0 * vf0));
+        trad = P.b2_f - (dd - tdv * tdv) - eps_d;
+      }
+      const float vfa = ax == 0 ? vf0 : (ax == 1 ? vf1 : vf2);
+      const float pfa = ax == 0 ? pf0 : (ax == 1 ? pf1 : pf2);
+      const float wdist = (signbit(vfa) ? pfa : Wfa - pfa) - eps_v, wav = fabsf(vfa) * 1.000002f;
+      // screen up to two obstacles, so that their loads overlap
+      auto screen2 = [&](int ka, int kb, bool two) {
+        const float4 fa = st.sh[ka], fb = st.sh[kb];
+        float a0 = pf0 - fa.x, a1 = pf1 - fa.y, a2 = pf2 - fa.z;
+        float b0 = pf0 - fb.x, b1 = pf1 - fb.y, b2 = pf2 - fb.z;
+        if (!DOM) {
+          a0 = wrapf(a0, P.Lf[0]);
+          a1 = wrapf(a1, P.Lf[1]);
+          a2 = wrapf(a2, P.Lf[2]);
+          b0 = wrapf(b0, P.Lf[0]);
+          b1 = wrapf(b1, P.Lf[1]);
+          b2 = wrapf(b2, P.Lf[2]);
+        }
+        screen_hs(Z, a0, a1, a2, vf0, vf1, vf2, ka, ubl, ks0, kl0, ks1, kl1, kovf);
+        if (two) screen_hs(Z, b0, b1, b2, vf0, vf1, vf2, kb, ubl, ks0, kl0, ks1, kl1, kovf);
+      };
+      bool listed = false;
+      int total = 0;  // obstacles in the list
+      if (G <= 4) {
+        // With few lanes a group's obstacles spread unevenly over them, and
+        // the warp would go round as often as its fullest lane asks: deal
+        // them out through a list.
+        for (int w = 0; w < W; ++w) nscr += __popc(cand_word(w));
+        int incl = nscr;
+#pragma unroll
+        for (int off = 1; off < G; off <<= 1) {
+          const int t = __shfl_up_sync(FULL, incl, off, G);
+          if (gl >= off) incl += t;
+        }
+        total = __shfl_sync(FULL, incl, gbase + G - 1);
+        listed = !__any_sync(FULL, total > LIST_CAP);
+        if (listed) {
+          int at = incl - nscr;
+          for (int w = 0; w < W; ++w) {
+            unsigned c = cand_word(w);
+            while (c) {
+              st.lst[at++] = ((w << 5) + __ffs(c) - 1) * G + gl;
+              c &= c - 1;
+            }
           }
-          screen_hs(Z, a0, a1, a2, vf0, vf1, vf2, ka, ubl, ks0, kl0, ks1, kl1, kovf);
-          if (two) screen_hs(Z, b0, b1, b2, vf0, vf1, vf2, kb, ubl, ks0, kl0, ks1, kl1, kovf);
+          __syncwarp();
+          for (int j = gl; j < total; j += 2 * G) {
+            const bool two = j + G < total;
+            screen2(CI(st.lst[j], S, 21, P.status), CI(st.lst[two ? j + G : j], S, 21, P.status), two);
+          }
+        }
+        nscr = gl == 0 ? total : 0;
+      }
+      if (!listed) {
+        for (int w = 0; w < W; ++w) {
+          unsigned c = cand_word(w);
+          if (G > 4) nscr += __popc(c);
+          while (c) {
+            const int ka = CI(((w << 5) + __ffs(c) - 1) * G + gl, S, 21, P.status);
+            c &= c - 1;
+            const bool two = c != 0;
+            const int kb = two ? CI(((w << 5) + __ffs(c) - 1) * G + gl, S, 21, P.status) : ka;
+            c &= c - 1;
+            screen2(ka, kb, two);
+          }
         }
       }
-      const float U = group_minf<G>(ubl);
-      sth = sth && tlb <= U;
-      sw = sw && wlb <= U;
+      const float U = G == 32 ? __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(ubl))) : group_minf<G>(ubl);
+      // A wall or a tether can win only when its lower bound reaches U:
+      // (dist - eps) / |v| <= U, and -dv - eps + sqrt(rad - eps_d) <= U.
+      sw = sw && wdist <= U * wav;
+      const bool bonded = sth;
+      {
+        const float q = U + tdv + eps_v;
+        sth = sth && q >= 0.f && trad <= q * q * 1.000002f;
+      }
       bool h0 = ks0 >= 0 && kl0 <= U, h1 = ks1 >= 0 && kl1 <= U;
+      bool all_fp64 = false;  // evaluate every obstacle in the box
       if (P.rq_per_tile < 6) {
         // a small request_cap sends tiles with more survivors than that (or
-        // more than 8 per request in reach) to the exhaustive evaluation
+        // more than 4 per request in reach) to the exhaustive evaluation
         int ns = sth + sw + h0 + h1;
 #pragma unroll
         for (int off = G / 2; off > 0; off >>= 1) {
           ns += __shfl_xor_sync(FULL, ns, off);
           nscr += __shfl_xor_sync(FULL, nscr, off);
         }
-        all_fp64 = act && (ns > P.rq_per_tile || nscr > 8 * P.rq_per_tile);
+        all_fp64 = act && (ns > P.rq_per_tile || nscr > 4 * P.rq_per_tile);
         if (all_fp64) {
           if (gl == 0) ++exh;
           h0 = h1 = kovf = false;
-          sth = !SPRING && ((gl == TL && nb_prev(nbw) >= 0) || (gl == TL + 1 && nb_next(nbw) >= 0));
+          sth = bonded;
           sw = DOM && gl < 3 && nonzero(va);
         }
       }
       // ---------------------------------------------------------- B: FP64
       // The quads of a group take its survivors, one each per round
       // (rarely more than one survives).
+      quads = SPRING && NQ > 1;
       for (;;) {
-        const int code = sth ? ts | (1 << 30) : (h0 ? ks0 : (h1 ? ks1 : -1));
-        const unsigned bal = __ballot_sync(FULL, code >= 0);
-        if (bal == 0u) break;
-        const unsigned mine = (bal & gmask) >> gbase;
+        const int code = sth ? (KIND_TETHER << 28) | ts : (h0 ? (KIND_HS << 28) | ks0 : (h1 ? (KIND_HS << 28) | ks1 : 0));
+        const unsigned mine = (__ballot_sync(FULL, code != 0) & gmask) >> gbase;
         unsigned left = mine;
 #pragma unroll
         for (int i = 0; i < NQ - 1; ++i)
           if (i < qd) left &= left - 1u;
+        const int qcode = __shfl_sync(FULL, code, gbase + __ffs(left) - 1);
         const bool on = left != 0u;
-        const int qcode = __shfl_sync(FULL, code, on ? gbase + __ffs(left) - 1 : lane);
-        if (code >= 0 && __popc(mine & ((1u << gl) - 1u)) < NQ) {
-          if (sth) sth = false;
-          else if (h0) h0 = false;
-          else h1 = false;
+        const bool te = (qcode >> 28) == KIND_TETHER;
+        const int k = on ? CI(qcode & 0xFFFFFFF, S, 24, P.status) : 0;
+        const int kid = __float_as_int(st.sh[k].w);
+        double d = 0.0, dv, dd, pos = 0.0;
+        if (on && ax < 3) {
+          pos = pos64(st, Rr, k, kid, ax, M64);
+          d = wrap_a(qa - pos, wra);
         }
-        const bool te = on && (qcode >> 30) != 0;
-        const int k = on ? CI(qcode & 0x3FFFFFFF, S, 24, P.status) : 0;
-        double d = 0.0, dv, dd;
-        if (on && ax < 3) d = wrap_a(qa - pos64(st, Rr, k, ax, M64), wra);
         dots(FULL, d, dv, dd);
         const double R2 = te ? P.b2 : P.sig2;
         double rad = R2 - __fma_rn(-dv, dv, dd);
-        bool hit = on && (te || (neg(dv) && posv(rad) && !(PO && dbits(dd) < dbits(R2))));
+        const bool hit = on && (te || (neg(dv) && posv(rad) && !(PO && dbits(dd) < dbits(R2))));
         if (te && neg(rad)) rad = 0.0;
         const double q = sqrt_rn(hit ? rad : 1.0);
         double x = -dv + (te ? q : -q);
         if (neg(x)) x = 0.0;
-        if (on && ax == 0) {
-          ++confirmed;
-          if (hit) keep(x, make_key(te ? KIND_TETHER : KIND_HS, __float_as_int(st.sh[k].w), k), dv);
+        if (hit) keep(x, qcode, dv, pos);
+        if (on && ax == 0) ++confirmed;
+        // survivors that did not get a quad, or share a lane with one that did
+        bool more = code != 0 && __popc(mine & ((1u << gl) - 1u)) >= NQ;
+        if (code != 0 && !more) {
+          more = sth ? h0 || h1 : h0 && h1;
+          if (sth) sth = false;
+          else if (h0) h0 = false;
+          else h1 = false;
         }
+        quads = quads || (mine & (mine - 1u)) != 0u;
+        if (!__any_sync(FULL, more)) break;
+        quads = true;
       }
-      if (__any_sync(FULL, kovf || all_fp64)) {
-        const unsigned wb = __ballot_sync(FULL, wra) >> gbase;
-        wrg0 = wb & 1;
-        wrg1 = wb & 2;
-        wrg2 = wb & 4;
+      lanes = __any_sync(FULL, kovf || all_fp64 || sw);
+      if (lanes && __any_sync(FULL, kovf || all_fp64)) {
+        wrap_flags();
         all_axes();
         if (act && (kovf || all_fp64)) {
           // more than two possible winners in this lane: screen its obstacles
           // again against the group's U and evaluate every one that can reach
           // it (exhaustive evaluation: all of them)
-          for (int w = 0; w < W; ++w) {
-            unsigned c = cand_word(w);
-            while (c) {
-              const int k = CI(((w << 5) + __ffs(c) - 1) * G + gl, S, 22, P.status);
-              c &= c - 1;
-              if (!all_fp64) {
-                if (k == ks0 || k == ks1) continue;
-                const float4 f = st.sh[k];
-                float d0 = pf0 - f.x, d1 = pf1 - f.y, d2 = pf2 - f.z;
-                if (!DOM) {
-                  d0 = wrapf(d0, P.Lf[0]);
-                  d1 = wrapf(d1, P.Lf[1]);
-                  d2 = wrapf(d2, P.Lf[2]);
-                }
-                bool possible;
-                const float lb = screen_lb(Z, d0, d1, d2, vf0, vf1, vf2, possible);
-                if (!possible || lb > U) continue;
+          auto again = [&](int k) {
+            if (!all_fp64) {
+              if (k == ks0 || k == ks1) return;
+              const float4 f = st.sh[k];
+              float d0 = pf0 - f.x, d1 = pf1 - f.y, d2 = pf2 - f.z;
+              if (!DOM) {
+                d0 = wrapf(d0, P.Lf[0]);
+                d1 = wrapf(d1, P.Lf[1]);
+                d2 = wrapf(d2, P.Lf[2]);
               }
-              exact(k, false);
+              bool possible;
+              const float lb = screen_lb(Z, d0, d1, d2, vf0, vf1, vf2, possible);
+              if (!possible || lb > U) return;
+            }
+            exact(k, false);
+          };
+          if (listed) {  // (the obstacles dealt to this lane)
+            for (int j = gl; j < total; j += G) again(CI(st.lst[j], S, 22, P.status));
+          } else {
+            for (int w = 0; w < W; ++w) {
+              unsigned c = cand_word(w);
+              while (c) {
+                const int k = CI(((w << 5) + __ffs(c) - 1) * G + gl, S, 22, P.status);
+                c &= c - 1;
+                again(k);
+              }
             }
           }
         }
         __syncwarp();
       }
+      quads = __any_sync(FULL, quads || kovf || all_fp64);
     } else {
-      // plain form: the tethers and every obstacle in the box
+      // plain form: the tethers, the walls in reach and every obstacle in the
+      // box.  A lane's words hold an uneven share of them and an evaluation
+      // costs the warp the same for one lane as for all, so they are dealt out
+      // through a list: as a rule one round instead of as many as the fullest
+      // lane would take.
+      wrap_flags();
       all_axes();
-      if (sth) exact(ts, true);
-      for (int w = 0; w < W; ++w) {
-        unsigned c = cand_word(w);
-        while (c) {
-          const int k = CI(((w << 5) + __ffs(c) - 1) * G + gl, S, 23, P.status);
-          c &= c - 1;
-          exact(k, false);
-        }
+      if (sw) {
+        const float vfa = ax == 0 ? vf0 : (ax == 1 ? vf1 : vf2);
+        const float pfa = ax == 0 ? pf0 : (ax == 1 ? pf1 : pf2);
+        sw = (signbit(vfa) ? pfa : Wfa - pfa) - eps_v <= xc * fabsf(vfa) * 1.000002f;
       }
-      __syncwarp();
+      int total = 0;
+      for (int from = 0; from == 0 || __any_sync(FULL, from < total); from += LIST_CAP) {
+        total = 0;
+        auto deal = [&](bool have, int code) {
+          const unsigned b = (__ballot_sync(FULL, have) & gmask) >> gbase;
+          const int at = total + __popc(b & ((1u << gl) - 1u)) - from;
+          if (have && at >= 0 && at < LIST_CAP) st.lst[at] = code;
+          total += __popc(b);
+        };
+        deal(sth, (KIND_TETHER << 28) | ts);
+        for (int w = 0; w < W; ++w) {
+          unsigned c = cand_word(w);
+          while (__any_sync(FULL, c != 0u)) {
+            deal(c != 0u, (KIND_HS << 28) | (((w << 5) + __ffs(c) - 1) * G + gl));
+            c &= c - 1u;
+          }
+        }
+        __syncwarp();
+        const int n = total - from < LIST_CAP ? total - from : LIST_CAP;
+        for (int j = gl; j < n; j += G) {
+          const int code = st.lst[j];
+          exact(CI(code & 0xFFFFFFF, S, 23, P.status), (code >> 28) == KIND_TETHER);
+        }
+        __syncwarp();
+      }
+      lanes = true;
+      quads = NQ > 1;
     }
-    if (DOM) {
+    if (DOM && lanes) {
       if (__any_sync(FULL, sw)) {
         if (sw) {
           const double loc = wrap_a(qa - ca, wra);
           double x = div_rn((posv(va) ? SYS(W)[axc] : 0.0) - loc, va);
           if (neg(x)) x = 0.0;
           if (F32) ++confirmed;
-          keep(x, make_key(KIND_WALL, ax, 0), 0.0);
+          keep(x, (KIND_WALL << 28) | ax, 0.0, 0.0);
         }
         __syncwarp();
       }
     }
     // ---------------- winner of the group and its pre-flight d.v
-    const unsigned has = __ballot_sync(FULL, lkey != ~0ull) & gmask;
-    uint64_t wx = lx, wkey = lkey;
-    int src = __ffs(has) - 1;
-    if (src < 0) src = lane;
-    if (__any_sync(FULL, (has & (has - 1)) != 0)) {
-      group_argmin<G>(wx, wkey);
-      const unsigned own = __ballot_sync(FULL, lkey == wkey && lx == wx) & gmask;
-      src = __ffs(own) - 1;
-    } else {
-      wx = __shfl_sync(FULL, lx, src);
-      wkey = __shfl_sync(FULL, lkey, src);
+    auto exchange = [&](int off) {
+      const uint64_t ox = __shfl_xor_sync(FULL, best.x, off);
+      const int oc = __shfl_xor_sync(FULL, best.code, off);
+      const double odv = __shfl_xor_sync(FULL, best.dv, off);
+      const double op = __shfl_xor_sync(FULL, best.pos, off);
+      if (oc != CAND_NONE && oc != best.code && beats(ox, oc)) {
+        best.x = ox;
+        best.code = oc;
+        best.dv = odv;
+        best.pos = op;
+      }
+    };
+    bool done = false;
+    if (!F32) {
+      // single lanes hold the candidates: the smallest upper half of x settles
+      // it unless two share it
+      const unsigned hi = best.code == CAND_NONE ? ~0u : (unsigned)(best.x >> 32);
+      unsigned mn = hi;
+      if (G == 32) {
+        mn = __reduce_min_sync(FULL, hi);
+      } else {
+#pragma unroll
+        for (int off = G / 2; off > 0; off >>= 1) mn = min(mn, __shfl_xor_sync(FULL, mn, off));
+      }
+      const unsigned own = __ballot_sync(FULL, hi == mn) & gmask;
+      done = !__any_sync(FULL, mn != ~0u && (own & (own - 1u)) != 0u);
+      if (done) {
+        const int src = __ffs(own) - 1;
+        best.x = __shfl_sync(FULL, best.x, src);
+        best.code = __shfl_sync(FULL, best.code, src);
+        best.dv = __shfl_sync(FULL, best.dv, src);
+      }
     }
-    const double wdv = __shfl_sync(FULL, ldv, src);
+    if (lanes && !done) {
+      // (a lane-wise candidate carries no position: it is read again below)
+      exchange(1);
+      exchange(2);
+    }
+    if (done) {
+    } else if (NQ > 1 && quads) {
+#pragma unroll
+      for (int off = 4; off < G; off <<= 1) exchange(off);
+    } else if (NQ > 1) {
+      // one candidate at most, the first quad's
+      best.x = __shfl_sync(FULL, best.x, gbase + ax);
+      best.code = __shfl_sync(FULL, best.code, gbase + ax);
+      best.dv = __shfl_sync(FULL, best.dv, gbase + ax);
+      best.pos = __shfl_sync(FULL, best.pos, gbase + ax);
+    }
 
     // ---------------------------------------------------------- D: move
-    if (act && nev >= P.event_cap) {
+    if (act && nev >= event_cap) {
       if (gl == 0) set_status(P.status, DEV_STUCK);
       settle(p, pid, qa, pf0, pf1, pf2, oslab);
       state = EC_NEED;
     }
     if (state == EC_RUN) {
       double x = pass ? P.s_cap : xrem;
-      int kind = pass ? KIND_PASS : KIND_END, slot = 0;
-      int64_t partner = -1;
-      if (wx < dbits(x)) {  // (END and PASS win ties)
-        x = __longlong_as_double((long long)wx);
-        kind = key_kind(wkey);
-        slot = key_slot(wkey);
-        partner = key_id(wkey);
+      int kind = pass ? KIND_PASS : KIND_END, slot = 0, partner = -1;
+      if (best.x < dbits(x)) {  // (END and PASS win ties)
+        x = __longlong_as_double((long long)best.x);
+        kind = best.code >> 28;
+        slot = best.code & 0xFFFFFFF;
+        partner = slot;
       }
       const bool bead = kind >= KIND_HS;
-      double ka = 0.0;  // the partner's position on this lane's axis
-      if (bead && ax < 3) ka = pos64(st, Rr, CI(slot, S, 30, P.status), ax, M64);
+      double ka = best.pos;  // the partner's position on this lane's axis
+      if (bead) {
+        slot = CI(slot, S, 30, P.status);
+        partner = __float_as_int(st.sh[slot].w);
+        if (lanes && ax < 3) ka = pos64(st, Rr, slot, partner, ax, M64);
+      }
       // r + x v on the axes, what is left of ell on lane 3, and on lane AL
       // (of G >= 8) the projection (r_target - r_pivot).v = -(d.v) - x
-      double y = __fma_rn(x, va, G >= 8 && gl == AL ? -wdv : qa);
-      const double proj = G >= 8 ? y : -wdv - x;
+      double y = __fma_rn(x, va, G >= 8 && gl == AL ? -best.dv : qa);
+      const double proj = G >= 8 ? y : -best.dv - x;
       if (wra) {
         const int di = wrap_step(y, SYS(L)[axc]);
         if (di && gl < 3) Ri[3 * (int64_t)pid + gl] += di;
@@ -750,9 +865,7 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
           v0 = __shfl_sync(gmask, va, gbase);
           v1 = __shfl_sync(gmask, va, gbase + 1);
           v2 = __shfl_sync(gmask, va, gbase + 2);
-          vf0 = f32_trunc(v0);
-          vf1 = f32_trunc(v1);
-          vf2 = f32_trunc(v2);
+          new_direction();
         } else {
           np = slot;
           if (!SPRING && !PO && hs && P.swap_mode) {
@@ -781,7 +894,8 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
               // bond j (pivot to previous, next; partner to previous, next)
               // on quad j
               bool ok = true;
-              const unsigned nbs = st.nb[slot];
+              const uint2 nb2 = st.nb[slot];
+              const unsigned nbs = nb2.x;
 #pragma unroll
               for (int j0 = 0; j0 < 4; j0 += NQ) {
                 const int j = j0 + qd;
@@ -790,7 +904,7 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
                 double d = 0.0, dv, dd;
                 if (b >= 0 && ax < 3) {
                   const double pa = (j & 2) ? qa : ka;
-                  const double ba = b == p ? ka : (b == slot ? qa : pos64(st, Rr, b, ax, M64));
+                  const double ba = b == p ? ka : (b == slot ? qa : pos64(st, Rr, b, __float_as_int(st.sh[b].w), ax, M64));
                   d = wrap_a(pa - ba, wra);
                 }
                 dots(gmask, d, dv, dd);
@@ -801,11 +915,10 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
                 swapped = true;
                 out = ECMC_EV_SWAP;
                 np = p;
-                const float4 f = st.sh[slot];
-                const int kid = __float_as_int(f.w);
+                const int kid = __float_as_int(st.sh[slot].w);
                 float g0, g1, g2;
                 shadows(qa, g0, g1, g2);
-                settle(slot, kid, qa, g0, g1, g2, slabs_at(f.x, f.y, f.z));
+                settle(slot, kid, qa, g0, g1, g2, (int)nb2.y);
                 if (gl < 3) {
                   const int ti = Ri[3 * (int64_t)pid + gl];
                   Ri[3 * (int64_t)pid + gl] = Ri[3 * (int64_t)kid + gl];
@@ -818,7 +931,7 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
         }
       } else if (kind == KIND_WALL) {
         // (negation is exact in both precisions)
-        const int wa = (int)partner;
+        const int wa = partner;
         if (ax == wa) va = -va;
         if (wa == 0) {
           v0 = -v0;
@@ -831,12 +944,8 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
           vf2 = -vf2;
         }
       }
-      ev_pk += 1ull << (8 * out);
-      if (++ev_pn == 255) {
-        if (gl == 0) flush_outcomes();
-        ev_pk = 0;
-        ev_pn = 0;
-      }
+      ev_lo += gl == (G >= 8 ? out : out & 3) && (G >= 8 || out < 4) ? 1u : 0u;
+      if (G < 8) ev_hi += out >= 4 && gl == (out & 3) ? 1u : 0u;
       __syncwarp(gmask);
       shadows(qa, pf0, pf1, pf2);
       if (P.rec_digest) {
@@ -866,12 +975,14 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
         p = np;
         const float4 f = st.sh[p];
         pid = CI(__float_as_int(f.w), BATCH ? rp->n_beads : P.n, 31, P.status);
-        nbw = st.nb[p];
+        const uint2 nb = st.nb[p];
+        nbw = nb.x;
+        oslab = (int)nb.y;
+        pmask = gl == (p & (G - 1)) && p / G < 32 ? ~(1u << ((p / G) & 31)) : ~0u;
         if (ax < 3) qa = ka;
         pf0 = f.x;
         pf1 = f.y;
         pf2 = f.z;
-        oslab = slabs_at(pf0, pf1, pf2);
       }
     }
     if (act && state == EC_NEED) {
@@ -886,7 +997,7 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
         if (idx < P.rec_cap) {
           P.rec_digest[idx] = h;
           P.rec_lift[idx] = lift;
-          P.rec_events[idx] = nev;
+          P.rec_events[idx] = (int64_t)nev;
         }
       }
       ++e;
@@ -901,7 +1012,6 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
     for (int off = G / 2; off > 0; off >>= 1) confirmed += __shfl_xor_sync(FULL, confirmed, off);
   }
   if (gl == 0 && ecs_done) {
-    if (ev_pn) flush_outcomes();
     atomicAdd(&P.counters[CNT_EVENTS], nev_all);
     if (tried) atomicAdd(&P.counters[CNT_SWAP_TRIED], (unsigned long long)tried);
     if (confirmed) atomicAdd(&P.counters[CNT_CONFIRMED], (unsigned long long)confirmed);
@@ -909,6 +1019,8 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
     atomicAdd(&P.counters[CNT_ECS], (unsigned long long)ecs_done);
     atomicAdd(&P.sums[SUM_DISP], (double)ecs_done * P.ell);  // an EC's flights add up to ell
   }
+  if (gl < ECMC_NEV && ev_lo) atomicAdd(&P.counters[gl], (unsigned long long)ev_lo);
+  if (G < 8 && ev_hi) atomicAdd(&P.counters[(gl & 3) + 4], (unsigned long long)ev_hi);
   if (gl == AL && ecs_done) {
     atomicAdd(&P.sums[SUM_LIFT], lift_all);
     atomicAdd(&P.sums[SUM_REFL], refl_all);

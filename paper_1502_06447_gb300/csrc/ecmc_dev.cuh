@@ -107,6 +107,18 @@ enum : int { KIND_END = 0, KIND_PASS = 1, KIND_WALL = 2, KIND_HS = 3, KIND_TETHE
 // bit by the sign of one more exact remainder, so the result does not depend
 // on the estimate's rounding.
 #ifdef __CUDACC__
+// minimum image of one coordinate difference, as wrap_d, with the comparisons
+// on the bit patterns and one addition for both signs
+__device__ __forceinline__ double wrap_bits(double d, double L, double half) {
+  const uint64_t b = (uint64_t)__double_as_longlong(d);
+  if ((b & 0x7FFFFFFFFFFFFFFFull) > (uint64_t)__double_as_longlong(half)) return d + ((int64_t)b < 0 ? L : -L);
+  return d;
+}
+// a < b for doubles >= 0
+__device__ __forceinline__ bool less_pos(double a, double b) {
+  return (uint64_t)__double_as_longlong(a) < (uint64_t)__double_as_longlong(b);
+}
+
 // FP32 value of a double, rounded towards zero, by integer operations (the
 // conversion instruction takes as long as an FP64 operation); magnitudes
 // below 2^-126 give 0, above 2^127 are not used

@@ -141,7 +141,7 @@ struct ECParams {
   // overlaps (the count of the flag pass before it); null otherwise
   const unsigned long long *po_count;
   // screened form: a tile with more survivors of the screen than this (below
-  // 6: or more than 8 times as many obstacles in reach) is evaluated
+  // 6: or more than 4 times as many obstacles in reach) is evaluated
   // exhaustively in FP64
   int32_t rq_per_tile;
   // tight capacities for a first pass (0: none); a
@@ -172,7 +172,7 @@ cudaError_t launch_ec_spring_fp64(const ECParams &P, int lanes, cudaStream_t s);
 cudaError_t launch_ec_pushoff_tether(const ECParams &P, int lanes, cudaStream_t s);
 cudaError_t launch_ec_pushoff_spring(const ECParams &P, int lanes, cudaStream_t s);
 // pick_lanes (k_ec.cu): warps per SM up to which a tile gets more lanes
-constexpr int EC_SPREAD_WARPS = 4;
+constexpr int EC_SPREAD_WARPS = 8;
 
 // cell list and domain tags (k_cells.cu)
 struct CellParams {

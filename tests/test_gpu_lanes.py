@@ -1,7 +1,7 @@
-"""Lane counts on a melt with more tiles than the launch gives extra lanes to
-(2,744 tiles: 4, 8 and 16 lanes per tile stay as asked for), so that every
-instance of the EC kernel runs at its own width with ragged last warps, and
-the first pass with tight capacities defers tiles to the second.  Per-EC
+"""Lane counts on a melt of 2,744 tiles with the tiles per block fixed (the
+launch then gives no tile extra lanes), so that every instance of the EC
+kernel runs at its own width with ragged last warps, and the first pass with
+tight capacities defers tiles to the second.  Per-EC
 digests, positions and images equal the oracle's bit for bit."""
 import numpy as np
 import pytest
@@ -34,7 +34,8 @@ def reference():
 @pytest.mark.parametrize("k_spring", [0.0, 30.0])
 def test_lanes_match_oracle_at_full_width(lanes, prec, k_spring, reference):
     r, img, digest = reference[k_spring]
-    ctx = gpu_context(M, precision=prec, lanes=lanes, tight_factor=0.8, k_spring=k_spring,
+    ctx = gpu_context(M, precision=prec, lanes=lanes, block_tiles=32 // lanes, tight_factor=0.8,
+                      k_spring=k_spring,
                       p_swap=0.0 if k_spring else M.p_swap)
     ctx.run(M.ell, seed=M.seed, n_sweeps=M.sweeps)
     dig, _, _ = ctx.records(len(digest))
