@@ -206,7 +206,9 @@ ObsParams obs_params(const ecmc_ctx *c) {
     O.L[a] = c->L[a];
     O.half[a] = 0.5 * c->L[a];
     O.nc[a] = c->nc[a];
+    O.Lf[a] = (float)c->L[a];
   }
+  O.crf = c->d_crf;
   O.sig2 = c->sigma * c->sigma;
   O.b2 = c->b_max * c->b_max;
   O.r = c->d_r;

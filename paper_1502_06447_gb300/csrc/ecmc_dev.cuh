@@ -107,23 +107,49 @@ enum : int { KIND_END = 0, KIND_PASS = 1, KIND_WALL = 2, KIND_HS = 3, KIND_TETHE
 // bit by the sign of one more exact remainder, so the result does not depend
 // on the estimate's rounding.
 #ifdef __CUDACC__
-// minimum image of one coordinate difference, as wrap_d, with the comparisons
-// on the bit patterns and one addition for both signs
-__device__ __forceinline__ double wrap_bits(double d, double L, double half) {
-  const uint64_t b = (uint64_t)__double_as_longlong(d);
-  if ((b & 0x7FFFFFFFFFFFFFFFull) > (uint64_t)__double_as_longlong(half)) return d + ((int64_t)b < 0 ? L : -L);
+// An FP64 instruction takes its unit 64 cycles, a comparison or conversion
+// more, and the compiler knows several ways to bring back one that the source
+// avoids.  Bits of a double go through an empty-handed move, since it turns
+// sign tests into FP64 comparisons and a flipped sign bit into a subtraction
+// from zero when it sees where they come from.  Operations off the common path
+// are calls: it turns a short branch into predicates, and a predicated FP64
+// instruction takes its 64 cycles even when no lane wants it.
+__device__ __forceinline__ uint64_t bits_of(double x) {
+  uint64_t b;
+  asm("mov.b64 %0, %1;" : "=l"(b) : "d"(x));
+  return b;
+}
+__device__ __forceinline__ double from_bits(uint64_t b) {
+  double x;
+  asm("mov.b64 %0, %1;" : "=d"(x) : "l"(b));
+  return x;
+}
+static __device__ __noinline__ double add_fp64(double a, double b) { return a + b; }
+static __device__ __noinline__ double square_fp64(double d) { return d * d; }
+static __device__ __noinline__ double sqrt_fp64(double a) { return sqrt(a); }
+static __device__ __noinline__ double div_fp64(double a, double b) { return a / b; }
+
+// -x
+__device__ __forceinline__ double flip(double x) { return from_bits(bits_of(x) ^ 0x8000000000000000ull); }
+// |x| with the opposite sign of b's bits
+__device__ __forceinline__ double against(double x, uint64_t b) { return from_bits(bits_of(x) ^ (~b & 0x8000000000000000ull)); }
+
+// minimum image of one coordinate difference, as wrap_d, for L > 0
+__device__ __forceinline__ double wrap_bits(double d, double L, double half, bool on = true) {
+  const uint64_t b = bits_of(d);
+  if (on && (b & 0x7FFFFFFFFFFFFFFFull) > bits_of(half)) d = add_fp64(d, against(L, b));
   return d;
 }
 // a < b for doubles >= 0
 __device__ __forceinline__ bool less_pos(double a, double b) {
-  return (uint64_t)__double_as_longlong(a) < (uint64_t)__double_as_longlong(b);
+  return bits_of(a) < bits_of(b);
 }
 
 // FP32 value of a double, rounded towards zero, by integer operations (the
 // conversion instruction takes as long as an FP64 operation); magnitudes
 // below 2^-126 give 0, above 2^127 are not used
 __device__ __forceinline__ float f32_trunc(double x) {
-  const uint64_t b = (uint64_t)__double_as_longlong(x);
+  const uint64_t b = bits_of(x);
   const unsigned hi = (unsigned)(b >> 32);
   const unsigned f = ((unsigned)(b >> 29) - (384u << 23)) & 0x7FFFFFFFu;
   return __uint_as_float((hi & 0x80000000u) | ((hi & 0x7FFFFFFFu) < (897u << 20) ? 0u : f));
@@ -147,9 +173,9 @@ __device__ __forceinline__ uint32_t seed_q31(float y) {
 // R = floor(s2 2^52) or R + 1: sqrt(M 2^52) > R + 1/2 exactly when
 // M 2^52 > R^2 + R (an integer square root is never half-way).
 __device__ __forceinline__ double sqrt_rn(double a) {
-  const uint64_t b = (uint64_t)__double_as_longlong(a);
+  const uint64_t b = bits_of(a);
   const unsigned e = (unsigned)(b >> 52);
-  if (e - 1u >= 2046u) return sqrt(a);  // zero, subnormal, negative, inf, nan
+  if (e - 1u >= 2046u) return sqrt_fp64(a);  // zero, subnormal, negative, inf, nan
   const unsigned even = ~e & 1u;
   const uint64_t M = ((b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << even;
   const float mf = __uint_as_float(((127u + even) << 23) | ((unsigned)(b >> 29) & 0x7FFFFFu));
@@ -163,7 +189,7 @@ __device__ __forceinline__ double sqrt_rn(double a) {
   const uint64_t R = (uint64_t)s2 >> 10;
   const int64_t d = (int64_t)((M << 52) - R * R - R);
   const uint64_t out = ((uint64_t)((e + 1023u) >> 1) << 52) + (R - 0x0010000000000000ull) + (d > 0 ? 1u : 0u);
-  return __longlong_as_double((long long)out);
+  return from_bits(out);
 }
 
 // a / b = rho 2^k with rho = Ma / Mb in [1, 2) (Ma doubled when below Mb).
@@ -172,16 +198,16 @@ __device__ __forceinline__ double sqrt_rn(double a) {
 // than 2^-59; the last bit follows from the exact remainder (no quotient of
 // two doubles is half-way).
 __device__ __forceinline__ double div_rn(double a, double b) {
-  const uint64_t ab = (uint64_t)__double_as_longlong(a), bb = (uint64_t)__double_as_longlong(b);
+  const uint64_t ab = bits_of(a), bb = bits_of(b);
   const unsigned ea = (unsigned)(ab >> 52) & 0x7FFu, eb = (unsigned)(bb >> 52) & 0x7FFu;
   uint64_t Ma = (ab & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
   const uint64_t Mb = (bb & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
   const unsigned less = Ma < Mb ? 1u : 0u;
   const int eq = (int)ea - (int)eb + 1023 - (int)less;
-  if (ea - 1u >= 2046u || eb - 1u >= 2046u || eq < 1 || eq > 2045) return a / b;
+  if (ea - 1u >= 2046u || eb - 1u >= 2046u || eq < 1 || eq > 2045) return div_fp64(a, b);
   Ma <<= less;
   const float bf = __uint_as_float(0x3F800000u | ((unsigned)(bb >> 29) & 0x7FFFFFu));
-  const uint32_t y = seed_q31(__frcp_rn(bf));                         // Q31
+  const uint32_t y = seed_q31(__fdividef(1.f, bf));                         // Q31
   const uint32_t q0 = __umulhi((uint32_t)(Ma >> 22), y) >> 1;         // Q30 Q31 / 2^33 = Q28
   const int64_t r0 = (int64_t)((Ma << 28) - (uint64_t)q0 * Mb);       // Q80 of (rho - q0) b, < 2^60.3
   const int64_t q1 = ((int64_t)((uint64_t)q0 << 17)) + (((int64_t)(int32_t)(r0 >> 30) * (int32_t)y) >> 36);  // Q45
@@ -190,7 +216,31 @@ __device__ __forceinline__ double div_rn(double a, double b) {
   const int64_t rem = (int64_t)((Ma << 52) - (uint64_t)q2 * Mb);
   const uint64_t Q = (uint64_t)q2 + (2 * rem > (int64_t)Mb ? 1ull : (2 * rem < -(int64_t)Mb ? ~0ull : 0ull));
   const uint64_t out = (((uint64_t)(unsigned)eq) << 52) + (Q - 0x0010000000000000ull);
-  return __longlong_as_double((long long)(out | ((ab ^ bb) & 0x8000000000000000ull)));
+  return from_bits(out | ((ab ^ bb) & 0x8000000000000000ull));
+}
+
+// d * d, for use where the FP64 units are the limit and the integer units can
+// take a share of the work beside them (some 25 instructions).  X = M 2^11 in
+// [2^63, 2^64); the upper 64 bits of X^2 are xh^2 + (2 xh xl + ...) >> 32, of
+// which h falls short by less than 3.  Half an ulp added, the bits below the
+// mantissa tell whether that could matter (three cases in 1024: the FP64
+// multiplication decides).
+__device__ __forceinline__ double square_rn(double d) {
+  const uint64_t b = bits_of(d);
+  const unsigned hi = (unsigned)(b >> 32);
+  const int e = (int)((hi >> 20) & 0x7FFu);
+  const unsigned xh = 0x80000000u | (unsigned)((b << 11) >> 32), xl = (unsigned)b << 11;
+  const uint64_t h = (uint64_t)xh * xh + ((uint64_t)__umulhi(xh, xl) << 1);
+  const unsigned top = (unsigned)(h >> 63);  // 1: X^2 >= 2^127
+  const unsigned sh = 10u + top;
+  const uint64_t g = h + (512ull << top);
+  const unsigned low = (unsigned)g & ((1024u << top) - 1u);
+  // (a carry out of g means the mantissa rounded up to 2^53: left to FP64 too)
+  const bool unsure = low - 1u >= (1024u << top) - 3u || g < h || (unsigned)(e - 520) > 999u;
+  if (unsure) return square_fp64(d);
+  const uint64_t m = g >> sh;  // [2^52, 2^53]: 2^53 carries into the exponent
+  const uint64_t out = ((uint64_t)(unsigned)(2 * e - 1023 + (int)top) << 52) + (m - 0x0010000000000000ull);
+  return from_bits(out);
 }
 #endif
 
@@ -220,7 +270,7 @@ ECMC_HD double ec_log(double u) {
   const uint64_t mb = (b & 0x000FFFFFFFFFFFFFull) | 0x3FF0000000000000ull;
   double m;
   memcpy(&m, &mb, sizeof(m));
-  if (m > 1.4142135623730951) {
+  if (mb > 0x3FF6A09E667F3BCDull) {  // m > sqrt(2) rounded to double; both in [1, 2)
     m = m * 0.5;
     e += 1;
   }
@@ -245,7 +295,11 @@ ECMC_HD double spring_dE(uint64_t w) { return -ec_log(1.0 - unit53(w)); }
 // off the bit patterns: a comparison is an FP64 instruction on the device).
 ECMC_HD bool neg_bits(double x) {
   int64_t b;
+#ifdef __CUDA_ARCH__
+  b = (int64_t)bits_of(x);
+#else
   memcpy(&b, &x, sizeof(b));
+#endif
   return b < 0 && ((uint64_t)b << 1) != 0;
 }
 ECMC_HD double spring_flight(double dv, double dd, double sigma, double dEk) {

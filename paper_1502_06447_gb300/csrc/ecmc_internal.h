@@ -252,6 +252,10 @@ struct ObsParams {
   unsigned long long *out_u;
   // squared shell bounds: pairs [lo, s1), [s1, s2); bonds (t1, t0], (t2, t1]
   double c_lo, c_s1, c_s2, c_t0, c_t1, c_t2;
+  const float *crf;        // FP32 positions in cell order
+  float Lf[3];
+  float f_lo, f_s1, f_s2;  // FP32 values of the pair bounds and the error of
+  float f_err;             // an FP32 squared distance near them (launch_obs)
 };
 cudaError_t launch_obs(const ObsParams &O, cudaStream_t s);
 // positions copied in as given: wrap into [0, L), fold boxes into img

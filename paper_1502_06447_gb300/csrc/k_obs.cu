@@ -21,54 +21,98 @@ __device__ __forceinline__ void atomic_max_pos(double *a, double v) {
 __device__ __forceinline__ void atomic_min_pos(double *a, double v) {
   atomicMin((unsigned long long *)a, (unsigned long long)__double_as_longlong(v));
 }
+__device__ __forceinline__ double warp_sum(double v, int width = 32) {
+  for (int off = width / 2; off > 0; off >>= 1) v = v + __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
 
+// Bonds of every chain: g threads per chain (a power of two up to a warp, or
+// the whole block), one bond per thread and round; sums over threads, then one
+// set of atomics per warp.
+// One thread per chain took 1.75 ms on 1000 chains of 1000 beads (1000
+// threads on the chip, each a chain of dependent loads and FP64 operations);
+// spread over the bonds the FP64 units bound it: 13 instructions per bond,
+// 20 us there.
 // out_d: [0] sum R_e^2, [1] max bond, [2] min bond, [3] sum g1, [4] sum of bond lengths
 // out_u: [0] overlaps, [1] tether violations, [4] [5] bonds in the shells
 // (t1, t0] and (t2, t1] below b_max
-__global__ void k_chains(const ObsParams O) {
-  const int64_t ch = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(128) k_chains(const ObsParams O, int g) {
+  __shared__ double Rs[3][4];
+  const int lane = threadIdx.x & 31, gl = threadIdx.x & (g - 1);
+  const int64_t ch = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / g;
   const int64_t nch = O.n / O.N;
-  if (ch >= nch) return;
-  double R0 = 0.0, R1 = 0.0, R2 = 0.0, bmax = 0.0, bmin = 1e300, bsum = 0.0;
-  unsigned long long viol = 0, tb0 = 0, tb1 = 0;
+  const bool live = ch < nch;
+  double R0 = 0.0, R1 = 0.0, R2 = 0.0, bsum = 0.0;
+  double dmax = 0.0, dmin = 1e300;  // squared bond lengths
+  unsigned viol = 0, tb0 = 0, tb1 = 0;
   const double lim = O.b2 * (1.0 + 1e-10);
-  for (int j = 0; j + 1 < O.N; ++j) {
-    const int64_t b = ch * O.N + j;
-    const double d0 = wrap_d(O.r[3 * (b + 1)] - O.r[3 * b], O.L[0], O.half[0]);
-    const double d1 = wrap_d(O.r[3 * (b + 1) + 1] - O.r[3 * b + 1], O.L[1], O.half[1]);
-    const double d2 = wrap_d(O.r[3 * (b + 1) + 2] - O.r[3 * b + 2], O.L[2], O.half[2]);
+  for (int j = gl; live && j + 1 < O.N; j += g) {
+    const double *q = O.r + 3 * (ch * O.N + j);
+    const double d0 = wrap_bits(q[3] - q[0], O.L[0], O.half[0]);
+    const double d1 = wrap_bits(q[4] - q[1], O.L[1], O.half[1]);
+    const double d2 = wrap_bits(q[5] - q[2], O.L[2], O.half[2]);
     R0 += d0;
     R1 += d1;
     R2 += d2;
     const double dd = d0 * d0 + d1 * d1 + d2 * d2;
-    viol += dd > lim;
-    tb0 += (dd > O.c_t1 && dd <= O.c_t0);
-    tb1 += (dd > O.c_t2 && dd <= O.c_t1);
-    const double bl = sqrt(dd);
-    bmax = fmax(bmax, bl);
-    bmin = fmin(bmin, bl);
-    bsum += bl;
+    viol += less_pos(lim, dd);
+    tb0 += less_pos(O.c_t1, dd) && !less_pos(O.c_t0, dd);
+    tb1 += less_pos(O.c_t2, dd) && !less_pos(O.c_t1, dd);
+    bsum += sqrt_rn(dd);
+    if (less_pos(dmax, dd)) dmax = dd;
+    if (less_pos(dd, dmin)) dmin = dd;
   }
-  atomicAdd(&O.out_d[0], R0 * R0 + R1 * R1 + R2 * R2);
+  const int gw = g < 32 ? g : 32;
+  R0 = warp_sum(R0, gw);
+  R1 = warp_sum(R1, gw);
+  R2 = warp_sum(R2, gw);
+  if (g > 32) {
+    if (lane == 0) {
+      Rs[0][threadIdx.x >> 5] = R0;
+      Rs[1][threadIdx.x >> 5] = R1;
+      Rs[2][threadIdx.x >> 5] = R2;
+    }
+    __syncthreads();
+    R0 = (Rs[0][0] + Rs[0][1]) + (Rs[0][2] + Rs[0][3]);
+    R1 = (Rs[1][0] + Rs[1][1]) + (Rs[1][2] + Rs[1][3]);
+    R2 = (Rs[2][0] + Rs[2][1]) + (Rs[2][2] + Rs[2][3]);
+  }
+  double re2 = 0.0, g1 = 0.0;
+  if (live && gl == 0) {
+    re2 = R0 * R0 + R1 * R1 + R2 * R2;
+    if (O.g1ref) {
+      const int64_t b = ch * O.N + O.N / 2;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const double u = O.r[3 * b + a] + (double)O.img[3 * b + a] * O.L[a];
+        const double d = u - O.g1ref[3 * ch + a];
+        g1 += d * d;
+      }
+    }
+  }
+  re2 = warp_sum(re2);
+  bsum = warp_sum(bsum);
+  if (O.g1ref) g1 = warp_sum(g1);
+  for (int off = 16; off > 0; off >>= 1) {
+    const double a = __shfl_xor_sync(0xffffffffu, dmax, off), b = __shfl_xor_sync(0xffffffffu, dmin, off);
+    if (less_pos(dmax, a)) dmax = a;
+    if (less_pos(b, dmin)) dmin = b;
+  }
+  viol = __reduce_add_sync(0xffffffffu, viol);
+  tb0 = __reduce_add_sync(0xffffffffu, tb0);
+  tb1 = __reduce_add_sync(0xffffffffu, tb1);
+  if (lane != 0 || !live) return;
+  atomicAdd(&O.out_d[0], re2);
   if (O.N > 1) {
     atomicAdd(&O.out_d[4], bsum);
-    atomic_max_pos(&O.out_d[1], bmax);
-    atomic_min_pos(&O.out_d[2], bmin);
+    // (the square root is monotone: the longest bond is that of the largest square)
+    atomic_max_pos(&O.out_d[1], sqrt_rn(dmax));
+    atomic_min_pos(&O.out_d[2], sqrt_rn(dmin));
   }
-  if (viol) atomicAdd(&O.out_u[1], viol);
-  if (tb0) atomicAdd(&O.out_u[4], tb0);
-  if (tb1) atomicAdd(&O.out_u[5], tb1);
-  if (O.g1ref) {
-    const int64_t b = ch * O.N + O.N / 2;
-    double g = 0.0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const double u = O.r[3 * b + a] + (double)O.img[3 * b + a] * O.L[a];
-      const double d = u - O.g1ref[3 * ch + a];
-      g += d * d;
-    }
-    atomicAdd(&O.out_d[3], g);
-  }
+  if (viol) atomicAdd(&O.out_u[1], (unsigned long long)viol);
+  if (tb0) atomicAdd(&O.out_u[4], (unsigned long long)tb0);
+  if (tb1) atomicAdd(&O.out_u[5], (unsigned long long)tb1);
+  if (O.g1ref) atomicAdd(&O.out_d[3], g1);
 }
 
 __global__ void k_snapshot(const ObsParams O, double *ref) {
@@ -80,38 +124,84 @@ __global__ void k_snapshot(const ObsParams O, double *ref) {
   for (int a = 0; a < 3; ++a) ref[3 * ch + a] = O.r[3 * b + a] + (double)O.img[3 * b + a] * O.L[a];
 }
 
-// pairs i < j closer than sigma (1 - 1e-10)^(1/2), and pairs in the shells
+// the beads of the cells x = cx + x0 .. cx + x1 of row (y, z): one or two
+// contiguous ranges of the cell-ordered arrays
+template <class F>
+__device__ __forceinline__ void row_ranges(const ObsParams &O, int cx, int x0, int x1, int y, int z, F f) {
+  const int nx = O.nc[0];
+  const int *const st = O.cstart + (z * O.nc[1] + y) * nx;
+  int a = cx + x0, b = cx + x1;  // inclusive
+  if (a < 0) {
+    f(st[a + nx], st[nx]);
+    a = 0;
+  } else if (b >= nx) {
+    f(st[0], st[b - nx + 1]);
+    b = nx - 1;
+  }
+  f(st[a], st[b + 1]);
+}
+
+// pairs closer than sigma (1 - 1e-10)^(1/2), and pairs in the shells
 // [lo, s1) and [s1, s2) above sigma, through the cell list (cell side >=
-// sqrt(s2), at least 3 cells per axis)
-__global__ void k_overlaps(const ObsParams O) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= O.n) return;
-  const int c = O.cell[i];
-  const int cx = c % O.nc[0], cy = (c / O.nc[0]) % O.nc[1], cz = c / (O.nc[0] * O.nc[1]);
-  const double p0 = O.r[3 * i], p1 = O.r[3 * i + 1], p2 = O.r[3 * i + 2];
-  const double lim = O.sig2 * (1.0 - 1e-10);
-  unsigned long long cnt = 0, cs0 = 0, cs1 = 0;
-  for (int dz = -1; dz <= 1; ++dz)
-    for (int dy = -1; dy <= 1; ++dy)
-      for (int dx = -1; dx <= 1; ++dx) {
-        const int x = (cx + dx + O.nc[0]) % O.nc[0];
-        const int y = (cy + dy + O.nc[1]) % O.nc[1];
-        const int z = (cz + dz + O.nc[2]) % O.nc[2];
-        const int cc = (z * O.nc[1] + y) * O.nc[0] + x;
-        for (int j = O.cstart[cc]; j < O.cstart[cc + 1]; ++j) {
-          if (O.cid[j] <= i) continue;
-          const double d0 = wrap_d(p0 - O.cr[3 * (int64_t)j], O.L[0], O.half[0]);
-          const double d1 = wrap_d(p1 - O.cr[3 * (int64_t)j + 1], O.L[1], O.half[1]);
-          const double d2 = wrap_d(p2 - O.cr[3 * (int64_t)j + 2], O.L[2], O.half[2]);
-          const double dd = d0 * d0 + d1 * d1 + d2 * d2;
-          cnt += dd < lim;
-          cs0 += (dd >= O.c_lo && dd < O.c_s1);
-          cs1 += (dd >= O.c_s1 && dd < O.c_s2);
-        }
+// sqrt(s2), at least 3 cells per axis).  A thread takes a bead in cell order
+// and the half of its neighbourhood ahead of it (its own cell past itself,
+// the next cell, three rows' worth of the rest), so that every pair is seen
+// once.  FP32 positions classify a pair; only one within their error of a
+// bound is measured in FP64.
+__global__ void __launch_bounds__(128) k_overlaps(const ObsParams O) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned cnt = 0, cs0 = 0, cs1 = 0;
+  if (t < O.n) {
+    const int c = O.cell[O.cid[t]];
+    const int cx = c % O.nc[0], cy = (c / O.nc[0]) % O.nc[1], cz = c / (O.nc[0] * O.nc[1]);
+    const float p0 = O.crf[3 * t], p1 = O.crf[3 * t + 1], p2 = O.crf[3 * t + 2];
+    const float L0 = O.Lf[0], L1 = O.Lf[1], L2 = O.Lf[2];
+    const double lim = O.sig2 * (1.0 - 1e-10);
+    auto one = [&](int j) {
+      float d0 = p0 - O.crf[3 * (int64_t)j], d1 = p1 - O.crf[3 * (int64_t)j + 1],
+            d2 = p2 - O.crf[3 * (int64_t)j + 2];
+      d0 = fabsf(d0);
+      d1 = fabsf(d1);
+      d2 = fabsf(d2);
+      d0 = fminf(d0, L0 - d0);
+      d1 = fminf(d1, L1 - d1);
+      d2 = fminf(d2, L2 - d2);
+      const float f = __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, d0 * d0));
+      if (f > O.f_s2 + O.f_err) return;
+      if (fabsf(f - O.f_lo) > O.f_err && fabsf(f - O.f_s1) > O.f_err && fabsf(f - O.f_s2) > O.f_err) {
+        cnt += f < O.f_lo;
+        cs0 += f > O.f_lo && f < O.f_s1;
+        cs1 += f > O.f_s1;
+        return;
       }
-  if (cnt) atomicAdd(&O.out_u[0], cnt);
-  if (cs0) atomicAdd(&O.out_u[2], cs0);
-  if (cs1) atomicAdd(&O.out_u[3], cs1);
+      const double e0 = wrap_bits(O.cr[3 * t] - O.cr[3 * (int64_t)j], O.L[0], O.half[0]);
+      const double e1 = wrap_bits(O.cr[3 * t + 1] - O.cr[3 * (int64_t)j + 1], O.L[1], O.half[1]);
+      const double e2 = wrap_bits(O.cr[3 * t + 2] - O.cr[3 * (int64_t)j + 2], O.L[2], O.half[2]);
+      const double dd = e0 * e0 + e1 * e1 + e2 * e2;
+      cnt += less_pos(dd, lim);
+      cs0 += !less_pos(dd, O.c_lo) && less_pos(dd, O.c_s1);
+      cs1 += !less_pos(dd, O.c_s1) && less_pos(dd, O.c_s2);
+    };
+    auto range = [&](int j0, int j1) {
+      for (int j = j0; j < j1; ++j) one(j);
+    };
+    range((int)t + 1, O.cstart[c + 1]);
+    row_ranges(O, cx, 1, 1, cy, cz, range);
+    const int yn = cy + 1 == O.nc[1] ? 0 : cy + 1;
+    row_ranges(O, cx, -1, 1, yn, cz, range);
+    const int zn = cz + 1 == O.nc[2] ? 0 : cz + 1;
+    const int yp = cy == 0 ? O.nc[1] - 1 : cy - 1;
+    row_ranges(O, cx, -1, 1, yp, zn, range);
+    row_ranges(O, cx, -1, 1, cy, zn, range);
+    row_ranges(O, cx, -1, 1, yn, zn, range);
+  }
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  cs0 = __reduce_add_sync(0xffffffffu, cs0);
+  cs1 = __reduce_add_sync(0xffffffffu, cs1);
+  if ((threadIdx.x & 31) != 0) return;
+  if (cnt) atomicAdd(&O.out_u[0], (unsigned long long)cnt);
+  if (cs0) atomicAdd(&O.out_u[2], (unsigned long long)cs0);
+  if (cs1) atomicAdd(&O.out_u[3], (unsigned long long)cs1);
 }
 
 __global__ void k_lattice(int n0, int n1, int n2, double a, double jitter, uint64_t seed,
@@ -139,34 +229,50 @@ __global__ void k_lattice(int n0, int n1, int n2, double a, double jitter, uint6
 
 // beads that overlap another bead (|d|^2 < thr, minimum image, squared
 // length (d0 d0 + d1 d1) + d2 d2) through the cell list: flag 0/1 per bead
-// and their number (the push-off's start beads, Sec. II.B)
-__global__ void k_po_flags(const ObsParams O, double thr, uint8_t *flag, unsigned long long *count) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= O.n) return;
-  const int c = O.cell[i];
-  const int cx = c % O.nc[0], cy = (c / O.nc[0]) % O.nc[1], cz = c / (O.nc[0] * O.nc[1]);
-  const double p0 = O.r[3 * i], p1 = O.r[3 * i + 1], p2 = O.r[3 * i + 2];
-  uint8_t f = 0;
-  for (int dz = -1; dz <= 1 && !f; ++dz)
-    for (int dy = -1; dy <= 1 && !f; ++dy)
-      for (int dx = -1; dx <= 1 && !f; ++dx) {
-        const int x = (cx + dx + O.nc[0]) % O.nc[0];
-        const int y = (cy + dy + O.nc[1]) % O.nc[1];
-        const int z = (cz + dz + O.nc[2]) % O.nc[2];
-        const int cc = (z * O.nc[1] + y) * O.nc[0] + x;
-        for (int j = O.cstart[cc]; j < O.cstart[cc + 1]; ++j) {
-          if (O.cid[j] == i) continue;
-          const double d0 = wrap_d(p0 - O.cr[3 * (int64_t)j], O.L[0], O.half[0]);
-          const double d1 = wrap_d(p1 - O.cr[3 * (int64_t)j + 1], O.L[1], O.half[1]);
-          const double d2 = wrap_d(p2 - O.cr[3 * (int64_t)j + 2], O.L[2], O.half[2]);
-          if ((d0 * d0 + d1 * d1) + d2 * d2 < thr) {
-            f = 1;
-            break;
-          }
-        }
+// and their number (the push-off's start beads, Sec. II.B).  A warp per
+// bead, one of the 27 cells per lane: a push-off has a few thousand beads, and
+// one thread per bead left most of the chip idle (180 us on 2,400 beads).
+// FP32 positions decide unless the square lies within their error of thr.
+__global__ void __launch_bounds__(128) k_po_flags(const ObsParams O, double thr, float thr_f, float err,
+                                                  uint8_t *flag, unsigned long long *count) {
+  const int lane = threadIdx.x & 31;
+  const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (t >= O.n) return;
+  const int i = O.cid[t];
+  bool f = false;
+  if (lane < 27) {
+    const int c = O.cell[i];
+    int x = c % O.nc[0] + lane % 3 - 1, y = (c / O.nc[0]) % O.nc[1] + (lane / 3) % 3 - 1,
+        z = c / (O.nc[0] * O.nc[1]) + lane / 9 - 1;
+    x += x < 0 ? O.nc[0] : (x >= O.nc[0] ? -O.nc[0] : 0);
+    y += y < 0 ? O.nc[1] : (y >= O.nc[1] ? -O.nc[1] : 0);
+    z += z < 0 ? O.nc[2] : (z >= O.nc[2] ? -O.nc[2] : 0);
+    const int cc = (z * O.nc[1] + y) * O.nc[0] + x;
+    const float p0 = O.crf[3 * t], p1 = O.crf[3 * t + 1], p2 = O.crf[3 * t + 2];
+    for (int j = O.cstart[cc]; j < O.cstart[cc + 1] && !f; ++j) {
+      if (j == (int)t) continue;
+      float d0 = fabsf(p0 - O.crf[3 * (int64_t)j]), d1 = fabsf(p1 - O.crf[3 * (int64_t)j + 1]),
+            d2 = fabsf(p2 - O.crf[3 * (int64_t)j + 2]);
+      d0 = fminf(d0, O.Lf[0] - d0);
+      d1 = fminf(d1, O.Lf[1] - d1);
+      d2 = fminf(d2, O.Lf[2] - d2);
+      const float q = __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, d0 * d0));
+      if (q > thr_f + err) continue;
+      if (q < thr_f - err) {
+        f = true;
+        break;
       }
-  flag[i] = f;
-  if (f) atomicAdd(count, 1ull);
+      const double e0 = wrap_bits(O.cr[3 * t] - O.cr[3 * (int64_t)j], O.L[0], O.half[0]);
+      const double e1 = wrap_bits(O.cr[3 * t + 1] - O.cr[3 * (int64_t)j + 1], O.L[1], O.half[1]);
+      const double e2 = wrap_bits(O.cr[3 * t + 2] - O.cr[3 * (int64_t)j + 2], O.L[2], O.half[2]);
+      f = less_pos((e0 * e0 + e1 * e1) + e2 * e2, thr);
+    }
+  }
+  f = __any_sync(0xffffffffu, f);
+  if (lane == 0) {
+    flag[i] = f ? 1 : 0;
+    if (f) atomicAdd(count, 1ull);
+  }
 }
 
 // Phantom chains (Sec. II.B, first stage of the initial configuration):
@@ -317,11 +423,22 @@ cudaError_t launch_wrap(double *r, int32_t *img, int64_t n, const double L[3],
   return cudaGetLastError();
 }
 
+// Error of a squared separation near r^2 from FP32 positions in [0, L): a
+// coordinate is off by L / 2^24, a difference by twice that and its own
+// rounding, the square by 2 sqrt(3) r times it; the bound keeps a factor of 2.
+static float f32_square_error(const ObsParams &O, double r) {
+  double L = O.L[0] > O.L[1] ? O.L[0] : O.L[1];
+  L = L > O.L[2] ? L : O.L[2];
+  return round_up_f32(16.0 * r * (L + r) / 16777216.0 + 1e-6 * r * r);
+}
+
 cudaError_t launch_po_flags(const ObsParams &O, double thr, uint8_t *flag,
                             unsigned long long *count, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(count, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
-  if (O.n > 0) k_po_flags<<<(unsigned)((O.n + 255) / 256), 256, 0, s>>>(O, thr, flag, count);
+  if (O.n > 0)
+    k_po_flags<<<(unsigned)((O.n + 3) / 4), 128, 0, s>>>(O, thr, (float)thr, f32_square_error(O, sqrt(thr)), flag,
+                                                        count);
   return cudaGetLastError();
 }
 
@@ -331,9 +448,18 @@ cudaError_t launch_phantom(int64_t nch, int N, const double L[3], double bond, d
   return cudaGetLastError();
 }
 
-cudaError_t launch_obs(const ObsParams &O, cudaStream_t s) {
+cudaError_t launch_obs(const ObsParams &O0, cudaStream_t s) {
+  ObsParams O = O0;
   const int64_t nch = O.n / O.N;
-  if (nch > 0) k_chains<<<(unsigned)((nch + 127) / 128), 128, 0, s>>>(O);
+  // a block per chain once it has a few rounds of bonds for one
+  int g = 1;
+  while (g < 32 && g < O.N - 1) g *= 2;
+  if (O.N > 256) g = 128;
+  if (nch > 0) k_chains<<<(unsigned)((nch * g + 127) / 128), 128, 0, s>>>(O, g);
+  O.f_lo = (float)O.c_lo;
+  O.f_s1 = (float)O.c_s1;
+  O.f_s2 = (float)O.c_s2;
+  O.f_err = f32_square_error(O, sqrt(O.c_s2));
   if (O.n > 0 && O.cr) k_overlaps<<<(unsigned)((O.n + 127) / 128), 128, 0, s>>>(O);
   return cudaGetLastError();
 }
