@@ -16,7 +16,7 @@ namespace {
 constexpr unsigned FULL = 0xffffffffu;
 
 // ---------------------------------------------------------------- FP64 bits
-__device__ __forceinline__ uint64_t dbits(double x) { return (uint64_t)__double_as_longlong(x); }
+__device__ __forceinline__ uint64_t dbits(double x) { return bits_of(x); }
 // x < 0.0 (false for -0.0)
 __device__ __forceinline__ bool neg(double x) {
   const uint64_t b = dbits(x);
@@ -30,30 +30,16 @@ __device__ __forceinline__ bool ge_pos(double y, double L) {
 }
 __device__ __forceinline__ bool nonzero(double x) { return (dbits(x) << 1) != 0; }
 // 2 x, exact (|x| zero or normal and below 2^1022)
-__device__ __forceinline__ double twice(double x) {
-  return nonzero(x) ? __longlong_as_double(__double_as_longlong(x) + (1ll << 52)) : x;
-}
-
-// minimum image, same result as d > h ? d - L : (d < -h ? d + L : d)
-__device__ __forceinline__ double wrap_i(double d, double L, uint64_t hbits) {
-  const uint64_t b = dbits(d);
-  if ((b & 0x7FFFFFFFFFFFFFFFull) > hbits) return d + (((int64_t)b < 0) ? L : -L);  // (one FP64 instruction)
-  return d;
-}
-
-// wrap_i on an axis that can need it; identity on an axis that cannot
-__device__ __forceinline__ double wrapc(double d, double L, uint64_t hbits, bool w) {
-  return w ? wrap_i(d, L, hbits) : d;
-}
+__device__ __forceinline__ double twice(double x) { return from_bits(dbits(x) + (nonzero(x) ? 1ull << 52 : 0ull)); }
 
 // y = r + x v on one axis back into [0, L); returns the image change
 __device__ __forceinline__ int wrap_step(double &y, double L) {
   int di = 0;
   if (ge_pos(y, L)) {
-    y = y - L;
+    y = add_fp64(y, flip(L));
     di = 1;
   } else if (neg(y)) {
-    y = y + L;
+    y = add_fp64(y, L);
     di = -1;
     if (ge_pos(y, L)) {
       y = 0.0;
@@ -79,7 +65,7 @@ __device__ __forceinline__ double quad_x(bool tether, double d0, double d1, doub
   const bool hit = tether || (neg(dv) && posv(rad) && !(skip_overlap && dbits(dd) < dbits(R2)));
   if (tether && neg(rad)) rad = 0.0;
   const double q = sqrt_rn(hit ? rad : 1.0);
-  const double x = -dv + (tether ? q : -q);
+  const double x = -dv + (tether ? q : flip(q));
   return hit ? (neg(x) ? 0.0 : x) : -1.0;
 }
 

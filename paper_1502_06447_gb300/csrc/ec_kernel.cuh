@@ -158,8 +158,7 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
   };
   // minimum image on this lane's axis (identity where it cannot be needed)
   auto wrap_a = [&](double d, bool on) {
-    if (on) d = wrap_i(d, SYS(L)[axc], dbits(SYS(half)[axc]));
-    return d;
+    return wrap_bits(d, SYS(L)[axc], SYS(half)[axc], on);
   };
   // the FP32 shadow of the position x on this lane's axis, for every lane:
   // FP32 position minus FP32 corner
@@ -181,8 +180,8 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
                  d2 = __shfl_sync(mask, d, qbase + 2);
     const bool first = ax == 0;
     double s = d0 * (first ? v0 : d0);
-    s = __fma_rn(d1, first ? v1 : d1, s);
-    s = __fma_rn(d2, first ? v2 : d2, s);
+    s = __fma_rn(d1, (first ? v1 : d1), s);
+    s = __fma_rn(d2, (first ? v2 : d2), s);
     dv = __shfl_sync(mask, s, qbase);
     dd = __shfl_sync(mask, s, qbase + 1);
   };
@@ -489,10 +488,10 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
       const double k0 = pos64(st, Rr, k, kid, 0, M64), k1 = pos64(st, Rr, k, kid, 1, M64),
                    k2 = pos64(st, Rr, k, kid, 2, M64);
       double dv;
-      const double x = quad_x(te, wrapc(bq0 - k0, SYS(L)[0], dbits(SYS(half)[0]), wrg0),
-                              wrapc(bq1 - k1, SYS(L)[1], dbits(SYS(half)[1]), wrg1),
-                              wrapc(bq2 - k2, SYS(L)[2], dbits(SYS(half)[2]), wrg2), v0, v1, v2,
-                              te ? P.b2 : P.sig2, dv, PO);
+      const double x = quad_x(te, wrap_bits(bq0 - k0, SYS(L)[0], SYS(half)[0], wrg0),
+                              wrap_bits(bq1 - k1, SYS(L)[1], SYS(half)[1], wrg1),
+                              wrap_bits(bq2 - k2, SYS(L)[2], SYS(half)[2], wrg2), v0, v1, v2,
+                              (te ? P.b2 : P.sig2), dv, PO);
       if (F32) ++confirmed;
       if (!neg(x)) keep(x, ((te ? KIND_TETHER : KIND_HS) << 28) | k, dv, 0.0);
     };
@@ -644,12 +643,12 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
           d = wrap_a(qa - pos, wra);
         }
         dots(FULL, d, dv, dd);
-        const double R2 = te ? P.b2 : P.sig2;
+        const double R2 = (te ? P.b2 : P.sig2);
         double rad = R2 - __fma_rn(-dv, dv, dd);
         const bool hit = on && (te || (neg(dv) && posv(rad) && !(PO && dbits(dd) < dbits(R2))));
         if (te && neg(rad)) rad = 0.0;
         const double q = sqrt_rn(hit ? rad : 1.0);
-        double x = -dv + (te ? q : -q);
+        double x = -dv + (te ? q : flip(q));
         if (neg(x)) x = 0.0;
         if (hit) keep(x, qcode, dv, pos);
         if (on && ax == 0) ++confirmed;
@@ -819,7 +818,7 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
       double x = pass ? P.s_cap : xrem;
       int kind = pass ? KIND_PASS : KIND_END, slot = 0, partner = -1;
       if (best.x < dbits(x)) {  // (END and PASS win ties)
-        x = __longlong_as_double((long long)best.x);
+        x = from_bits(best.x);
         kind = best.code >> 28;
         slot = best.code & 0xFFFFFFF;
         partner = slot;
@@ -833,7 +832,7 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
       }
       // r + x v on the axes, what is left of ell on lane 3, and on lane AL
       // (of G >= 8) the projection (r_target - r_pivot).v = -(d.v) - x
-      double y = __fma_rn(x, va, G >= 8 && gl == AL ? -best.dv : qa);
+      double y = __fma_rn(x, va, (G >= 8 && gl == AL ? flip(best.dv) : qa));
       const double proj = G >= 8 ? y : -best.dv - x;
       if (wra) {
         const int di = wrap_step(y, SYS(L)[axc]);
@@ -932,15 +931,15 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
       } else if (kind == KIND_WALL) {
         // (negation is exact in both precisions)
         const int wa = partner;
-        if (ax == wa) va = -va;
+        if (ax == wa) va = flip(va);
         if (wa == 0) {
-          v0 = -v0;
+          v0 = flip(v0);
           vf0 = -vf0;
         } else if (wa == 1) {
-          v1 = -v1;
+          v1 = flip(v1);
           vf1 = -vf1;
         } else {
-          v2 = -v2;
+          v2 = flip(v2);
           vf2 = -vf2;
         }
       }
