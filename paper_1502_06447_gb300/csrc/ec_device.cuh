@@ -6,6 +6,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <float.h>
+#include <limits.h>
 
 #include "ecmc_dev.cuh"
 #include "ecmc_internal.h"
@@ -112,9 +113,7 @@ struct Stage {
                     // y: slabs of the stored shadow, 10 bits per axis
   unsigned *mask;   // [3][nsl + 1][W][G]
   int *lst;         // [LIST_CAP] candidates dealt to the lanes
-  int *hdr;         // [0] hard-sphere joint beads, [1] tether-only joint beads
-                    // placed, [2] joint beads seen, [3] overflow, [4] motile
-                    // beads seen
+  int *hdr;         // [0] staged beads (springs: with the far partners)
 #ifdef ECMC_CHECKED
   int cap;          // S (slots)
   long long nglob;  // beads of the system (ids), set by the kernel
@@ -299,11 +298,6 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
     else if (gl == 0) set_status(P.status, DEV_CAPACITY);
   };
   if (overflow) *overflow = false;
-  auto put64 = [&](int k, const double *x) {
-    st.pos[k] = x[0];
-    st.pos[M64 + k] = x[1];
-    st.pos[2 * M64 + k] = x[2];
-  };
   const int nsl = SL.nsl;
   m = 0;
   j1 = 0;
@@ -313,7 +307,11 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
     const int n = (int)P.n;
     for (int b = gl; b < n; b += G) {
       const double x = Rr[3 * (int64_t)b], y = Rr[3 * (int64_t)b + 1], z = Rr[3 * (int64_t)b + 2];
-      if (b < M64) put64(b, Rr + 3 * (int64_t)b);
+      if (b < M64) {
+        st.pos[b] = x;
+        st.pos[M64 + b] = y;
+        st.pos[2 * M64 + b] = z;
+      }
       st.sh[b] = make_float4(f32_trunc(x), f32_trunc(y), f32_trunc(z), __int_as_float(b));
       const int c = b % SYS(N);
       st.nb[b].x = nb_pack(c == 0 ? -1 : b - 1, c == SYS(N) - 1 ? -1 : b + 1);
@@ -322,9 +320,6 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
     j1 = 0;
     ns = n;
   } else {
-    if (gl < 8) st.hdr[gl] = 0;
-    if (G < 8) st.hdr[gl + 4] = 0;
-    __syncwarp(mask);
     // cell window covering the tether halo of the tile: lane a works out
     // axis a (corner ca) and the group shares it
     int c_lo[3], c_n[3];
@@ -340,21 +335,14 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
         cnt = SYS(nc)[ax];
       }
       const float cfa = f32_trunc(ca);
-      const int g0 = (threadIdx.x & 31) & ~(G - 1);
+      const int first = (threadIdx.x & 31) & ~(G - 1);
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        c_lo[a] = __shfl_sync(mask, l, g0 + a);
-        c_n[a] = __shfl_sync(mask, cnt, g0 + a);
-        cf[a] = __shfl_sync(mask, cfa, g0 + a);
+        c_lo[a] = __shfl_sync(mask, l, first + a);
+        c_n[a] = __shfl_sync(mask, cnt, first + a);
+        cf[a] = __shfl_sync(mask, cfa, first + a);
       }
     }
-    // pass 1: collect (cell-order index, category|id), motile beads from the
-    // front, joint beads from the back; the shadow array serves as scratch
-    // until pass 3.  The cells of one row of the window (consecutive x) are
-    // one contiguous range of the cell-ordered arrays (two when the row
-    // wraps around the box); each lane takes whole rows and loads four beads
-    // at a time.
-    int2 *scr = (int2 *)st.sh;
     // halo membership in FP32 from FP32 copies of the positions, widened by
     // 1e-3 sigma plus four FP32 ulps of the box: a superset of the exact
     // sets (an extra obstacle beyond reach is never hit; a bond partner is
@@ -375,28 +363,52 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
     int cx = c_lo[0] % nc0;
     if (cx < 0) cx += nc0;
     const int len0 = c_n[0] < nc0 - cx ? c_n[0] : nc0 - cx;
-    for (int r = gl; r < nrows; r += G) {
-      const int qy = r % c_n[1], qz = r / c_n[1];
-      int cy = (c_lo[1] + qy) % nc1;
-      int cz = (c_lo[2] + qz) % nc2;
-      if (cy < 0) cy += nc1;
-      if (cz < 0) cz += nc2;
-      const int base = (cz * nc1 + cy) * nc0;
-      const int a0 = Rstart[base + cx], b0 = Rstart[base + cx + len0];
-      int a1 = 0, b1 = 0;
-      if (len0 < c_n[0]) {
-        a1 = Rstart[base];
-        b1 = Rstart[base + c_n[0] - len0];
+    const unsigned below = (1u << gl) - 1u;
+    const int g0 = (threadIdx.x & 31) & ~(G - 1);
+    auto votes = [&](bool v) {
+      const unsigned b = __ballot_sync(mask, v) >> g0;
+      return G == 32 ? b : b & ((1u << (G & 31)) - 1u);
+    };
+    // pass 1: collect (cell-order index, flag | category | id), motile beads
+    // from the front, joint beads from the back; the shadow array serves as
+    // scratch until pass 3.  Obstacles are the joint beads of the hard-sphere
+    // halo; beyond it, in the tether halo, only the bonded beads of motile
+    // ones are wanted, and the tag of a joint bead tells whose tile those are
+    // in (-1: of several, -2 - k: of tile k, else none).  The cells of one row
+    // of the window (consecutive x) are one contiguous range of the
+    // cell-ordered arrays (two when the row wraps around the box); each lane
+    // takes whole rows and loads four beads at a time; votes give the places.
+    int2 *scr = (int2 *)st.sh;
+    int nj = 0;
+    for (int r0 = 0; r0 < nrows; r0 += G) {
+      const int r = r0 + gl;
+      int a0 = 0, a1 = 0, n0 = 0, nt = 0;
+      if (r < nrows) {
+        const int qy = r % c_n[1], qz = r / c_n[1];
+        int cy = (c_lo[1] + qy) % nc1;
+        int cz = (c_lo[2] + qz) % nc2;
+        if (cy < 0) cy += nc1;
+        if (cz < 0) cz += nc2;
+        const int base = (cz * nc1 + cy) * nc0;
+        a0 = Rstart[base + cx];
+        n0 = Rstart[base + cx + len0] - a0;
+        nt = n0;
+        if (len0 < c_n[0]) {
+          a1 = Rstart[base];
+          nt += Rstart[base + c_n[0] - len0] - a1;
+        }
       }
-      const int n0 = b0 - a0, nt = n0 + (b1 - a1);
-      for (int k0 = 0; k0 < nt; k0 += 4) {
+      int most = nt;
+#pragma unroll
+      for (int off = G / 2; off > 0; off >>= 1) most = max(most, __shfl_xor_sync(mask, most, off));
+      for (int k0 = 0; k0 < most; k0 += 4) {
         int tg[4], jj[4], idv[4];
         float px[4], py[4], pz[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int k = k0 + u;
           jj[u] = k < n0 ? a0 + k : a1 + (k - n0);
-          tg[u] = -2;
+          tg[u] = INT_MAX;
           idv[u] = 0;
           px[u] = py[u] = pz[u] = 0.f;
           if (k < nt) {
@@ -410,11 +422,9 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          if (tg[u] == -2) continue;
-          int cat = -1;
-          if (tg[u] == unit) {
-            cat = 0;
-          } else if (tg[u] < 0) {
+          int cat = tg[u] == unit ? 0 : -1;
+          const bool bonded = tg[u] == -1 || tg[u] == -2 - unit;
+          if (tg[u] < 0) {
             const float pp[3] = {px[u], py[u], pz[u]};
             bool in_hs = true, in_te = true;
 #pragma unroll
@@ -424,78 +434,123 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
               in_hs = in_hs && (sa >= -hs_f) && (sa <= Wf[a] + hs_f);
               in_te = in_te && (sa >= -te_f) && (sa <= Wf[a] + te_f);
             }
-            cat = in_hs ? 1 : (in_te ? 2 : -1);
+            cat = in_hs ? 1 : (in_te && bonded ? 2 : -1);
           }
-          if (cat >= 0) {
-            const int q = atomicAdd(&st.hdr[cat == 0 ? 4 : 2], 1);
-            const int slot = cat == 0 ? q : S - 1 - q;
-            if (q < S) scr[slot] = make_int2(jj[u], (cat << 29) | idv[u]);
-            if (cat == 1) atomicAdd(&st.hdr[5], 1);
-          }
+          const unsigned bm = votes(cat == 0), bj = votes(cat > 0);
+          const int q = cat == 0 ? m + __popc(bm & below) : nj + __popc(bj & below);
+          if (cat >= 0 && q < S)
+            scr[cat == 0 ? q : S - 1 - q] =
+                make_int2(jj[u], (int)((bonded && cat > 0 ? 0x80000000u : 0u) | ((unsigned)cat << 29) | (unsigned)idv[u]));
+          m += __popc(bm);
+          nj += __popc(bj);
+          j1 += __popc(votes(cat == 1));
         }
       }
     }
     __syncwarp(mask);
-    m = st.hdr[4];
-    const int nj = st.hdr[2];
-    j1 = st.hdr[5];
     ns = m + nj;
     // (a list that ran into the other one holds no valid entries)
     if (ns > S || m > MNB) {
       capacity();
       live = false;
-      m = j1 = ns = 0;
+      m = j1 = ns = nj = 0;
     }
     // pass 2: slots.  Motile beads take their rank by id (the start bead of
     // an EC is the u-th motile bead in id order); joint beads take the next
     // free slot of their category (their order matters to nothing).  The ids
-    // go to the mask area (nsl >= 10 makes it as large as S words).
+    // go to the mask area (nsl >= 10 makes it as large as S words), those of
+    // joint beads with the flag of a bonded one.
     int *idt = (int *)st.mask;
     for (int s = gl; s < m; s += G) {
-      const int2 e = scr[s];
+      const int id = scr[s].y;
       int rank = 0;
-      for (int t = 0; t < m; ++t) rank += (scr[t].y < e.y);
-      if (!CHK(rank, S, 3, P.status)) continue;
-      idt[rank] = e.y;
-      if (rank < M64) put64(rank, P.cr + 3 * (int64_t)e.x);
+      for (int t = 0; t < m; ++t) rank += (scr[t].y < id);
+      if (CHK(rank, S, 3, P.status)) idt[rank] = id;
     }
-    for (int s = gl; s < ns - m; s += G) {
-      const int2 e = scr[S - 1 - s];
-      const int cat = e.y >> 29;
-      const int slot = (cat == 1 ? m : m + j1) + atomicAdd(&st.hdr[cat - 1], 1);
-      if (!CHK(slot, S, 33, P.status)) continue;
-      idt[slot] = e.y & ((1 << 29) - 1);
-      if (slot < M64) put64(slot, P.cr + 3 * (int64_t)e.x);
+    {
+      int n1 = 0, n2 = 0;
+      for (int s0 = 0; s0 < nj; s0 += G) {
+        const int s = s0 + gl;
+        const unsigned e = s < nj ? (unsigned)scr[S - 1 - s].y : 0u;
+        const int cat = (int)(e >> 29) & 3;
+        const unsigned b1 = votes(cat == 1), b2 = votes(cat == 2);
+        const int slot = cat == 1 ? m + n1 + __popc(b1 & below) : m + j1 + n2 + __popc(b2 & below);
+        if (cat != 0 && CHK(slot, S, 33, P.status)) idt[slot] = (int)(e & 0x9FFFFFFFu);
+        n1 += __popc(b1);
+        n2 += __popc(b2);
+      }
     }
     __syncwarp(mask);
-    // pass 2b: bond partners of motile beads.  A motile partner is found
-    // among the sorted motile ids; a joint partner announces itself (its
-    // neighbours' tags tell whether one of them is motile here).
+    // pass 2b: bond partners among the motile beads (sorted, so id - 1 can
+    // only be the slot before)
     const int Nc = SYS(N);
     for (int s = gl; s < m; s += G) {
       const int id = idt[s], c = id % Nc;
-      const int prev = c != 0 ? find_id(idt, 0, m, id - 1) : -1;
-      const int next = c != Nc - 1 ? find_id(idt, 0, m, id + 1) : -1;
+      const int prev = c != 0 && s > 0 && idt[s - 1] == id - 1 ? s - 1 : -1;
+      const int next = c != Nc - 1 && s + 1 < m && idt[s + 1] == id + 1 ? s + 1 : -1;
       st.nb[s].x = nb_pack(prev, next);
     }
     __syncwarp(mask);
+    // pass 3: shadows (FP32 position minus FP32 corner, the form the moved
+    // pivot's shadow takes too), FP64 positions, and a bonded joint bead
+    // announces itself to its motile neighbours.  Four slots at a time
+    // (independent loads).
+    const float *const Rf = P.rf + (BATCH ? 3 * rp->bead_off : 0);
     const int32_t *const Rtag = P.tag + (BATCH ? rp->bead_off : 0);
     unsigned short *const nbh = (unsigned short *)st.nb;
-    for (int s = m + gl; s < ns; s += G) {
-      const int id = idt[s], c = id % Nc;
-      const bool up = c != Nc - 1 && Rtag[id + 1] == unit;
-      const bool dn = c != 0 && Rtag[id - 1] == unit;
-      if (up) {
-        const int t = find_id(idt, 0, m, id + 1);
-        if (t >= 0) nbh[4 * t] = (unsigned short)s;
+    auto fill = [&](int from, int to) {
+      for (int s0 = from; s0 < to; s0 += 4 * G) {
+        float x[4], y[4], z[4];
+        int idv[4], up[4], dn[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int s = s0 + u * G + gl;
+          idv[u] = 0;
+          up[u] = dn[u] = -1;
+          if (s < to) {
+            const int e = idt[s];
+            const int64_t b = CI(e & 0x7FFFFFFF, BATCH ? rp->n_beads : P.n, 5, P.status);
+            idv[u] = (int)b;
+            x[u] = Rf[3 * b];
+            y[u] = Rf[3 * b + 1];
+            z[u] = Rf[3 * b + 2];
+            if (e < 0) {
+              const int c = (int)b % Nc;
+              if (c != Nc - 1) up[u] = Rtag[b + 1];
+              if (c != 0) dn[u] = Rtag[b - 1];
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int s = s0 + u * G + gl;
+          if (s >= to) continue;
+          float f0 = x[u] - cf[0], f1 = y[u] - cf[1], f2 = z[u] - cf[2];
+          f0 = f0 > Lhf[0] ? f0 - Lf[0] : (f0 < -Lhf[0] ? f0 + Lf[0] : f0);
+          f1 = f1 > Lhf[1] ? f1 - Lf[1] : (f1 < -Lhf[1] ? f1 + Lf[1] : f1);
+          f2 = f2 > Lhf[2] ? f2 - Lf[2] : (f2 < -Lhf[2] ? f2 + Lf[2] : f2);
+          st.sh[s] = make_float4(f0, f1, f2, __int_as_float(idv[u]));
+          if (up[u] == unit) {
+            const int t = find_id(idt, 0, m, idv[u] + 1);
+            if (t >= 0) nbh[4 * t] = (unsigned short)s;
+          }
+          if (dn[u] == unit) {
+            const int t = find_id(idt, 0, m, idv[u] - 1);
+            if (t >= 0) nbh[4 * t + 1] = (unsigned short)s;
+          }
+        }
       }
-      if (dn) {
-        const int t = find_id(idt, 0, m, id - 1);
-        if (t >= 0) nbh[4 * t + 1] = (unsigned short)s;
+#pragma unroll 3
+      for (int s = from + gl; s < to && s < M64; s += G) {
+        const double *const x = Rr + 3 * (int64_t)CI(idt[s] & 0x7FFFFFFF, BATCH ? rp->n_beads : P.n, 6, P.status);
+        const double X = x[0], Y = x[1], Z = x[2];
+        st.pos[s] = X;
+        st.pos[M64 + s] = Y;
+        st.pos[2 * M64 + s] = Z;
       }
-    }
-    __syncwarp(mask);
-    if (gl == 0) st.hdr[6] = ns;
+    };
+    fill(0, ns);
+    if (gl == 0) st.hdr[0] = ns;
     __syncwarp(mask);
     for (int s = gl; s < m; s += G) {
       const int id = idt[s], c = id % Nc;
@@ -514,51 +569,23 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
         // motile beads may append the same bead twice; both copies are
         // read-only and equal)
         if (!CHK(q, BATCH ? rp->n_beads : P.n, 4, P.status)) continue;
-        const int slot = atomicAdd(&st.hdr[6], 1);
+        const int slot = atomicAdd(&st.hdr[0], 1);
         if (slot < S) {
           idt[slot] = q;
           nbh[4 * s + dir] = (unsigned short)slot;
-          if (slot < M64) put64(slot, Rr + 3 * (int64_t)q);
         }
       }
     }
-    __syncwarp(mask);
     if (SPRING) {
-      ns = st.hdr[6];
-      if (ns > S) {
+      __syncwarp(mask);
+      const int all = st.hdr[0];
+      if (all > S) {
         if (live) capacity();
         live = false;
         m = j1 = ns = 0;
-      }
-    }
-    // pass 3: shadows (FP32 position minus FP32 corner, the form the moved
-    // pivot's shadow takes too).  Four slots at a time (independent loads).
-    const float *Rf = P.rf + (BATCH ? 3 * rp->bead_off : 0);
-    for (int s0 = 0; s0 < ns; s0 += 4 * G) {
-      float x[4], y[4], z[4];
-      int idv[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int s = s0 + u * G + gl;
-        x[u] = y[u] = z[u] = 0.f;
-        idv[u] = 0;
-        if (s < ns) {
-          const int64_t b = CI(idt[s], BATCH ? rp->n_beads : P.n, 5, P.status);
-          idv[u] = (int)b;
-          x[u] = Rf[3 * b];
-          y[u] = Rf[3 * b + 1];
-          z[u] = Rf[3 * b + 2];
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int s = s0 + u * G + gl;
-        if (s >= ns) continue;
-        float f0 = x[u] - cf[0], f1 = y[u] - cf[1], f2 = z[u] - cf[2];
-        f0 = f0 > Lhf[0] ? f0 - Lf[0] : (f0 < -Lhf[0] ? f0 + Lf[0] : f0);
-        f1 = f1 > Lhf[1] ? f1 - Lf[1] : (f1 < -Lhf[1] ? f1 + Lf[1] : f1);
-        f2 = f2 > Lhf[2] ? f2 - Lf[2] : (f2 < -Lhf[2] ? f2 + Lf[2] : f2);
-        st.sh[s] = make_float4(f0, f1, f2, __int_as_float(idv[u]));
+      } else {
+        fill(ns, all);
+        ns = all;
       }
     }
   }
@@ -580,15 +607,18 @@ __device__ __forceinline__ void stage_tile(const ECParams &P, const RepParams *r
     w[(nsl + 1 + k1 + 1) * row] |= bit;
     w[(2 * (nsl + 1) + k2 + 1) * row] |= bit;
   }
-  for (int a = 0; a < 3; ++a)
-    for (int w = 0; w < W; ++w) {
-      unsigned acc = 0u;
-      unsigned *const q = st.mask + (a * (nsl + 1)) * row + w * G + gl;
-      for (int k = 1; k <= nsl; ++k) {
-        acc |= q[k * row];
-        q[k * row] = acc;
-      }
+  for (int w = 0; w < W; ++w) {
+    unsigned *const q = st.mask + w * G + gl;
+    unsigned acc0 = 0u, acc1 = 0u, acc2 = 0u;
+#pragma unroll 4
+    for (int k = 1; k <= nsl; ++k) {
+      unsigned *const p = q + k * row;
+      const unsigned x = p[0], y = p[(nsl + 1) * row], z = p[2 * (nsl + 1) * row];
+      p[0] = acc0 |= x;
+      p[(nsl + 1) * row] = acc1 |= y;
+      p[2 * (nsl + 1) * row] = acc2 |= z;
     }
+  }
   __syncwarp(mask);
   if (!live) m = 0;
 }

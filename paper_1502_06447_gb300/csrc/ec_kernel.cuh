@@ -1152,8 +1152,12 @@ cudaError_t launch_ec_t(const ECParams &P0, cudaStream_t s) {
     const long long want = (P.n_units + h.nt - 1) / h.nt;
     const long long room = (long long)h.blocks * sms;
     const int blocks = (int)(want < room ? want : room);
-    cudaError_t e = cudaMemsetAsync(P.unit_next, 0, sizeof(int32_t), s);
-    if (e != cudaSuccess) return e;
+    // (the cell pass before a domain launch clears the unit counters)
+    if (!DOM) {
+      const cudaError_t e = cudaMemsetAsync(P.unit_next, 0, sizeof(int32_t), s);
+      if (e != cudaSuccess) return e;
+    }
+    if (mode == 2) P.unit_next += 1;
     if (blocks > 0) kern<<<blocks, h.nt * G, h.smem, s>>>(P);
     return cudaGetLastError();
   };
@@ -1169,7 +1173,6 @@ cudaError_t launch_ec_t(const ECParams &P0, cudaStream_t s) {
   if (!two) return run(full, 0);
   Shape tight{};
   e = shape(P0.stage_tight, P0.m_tight, &tight);
-  if (e == cudaSuccess) e = cudaMemsetAsync(P0.n_deferred, 0, sizeof(int32_t), s);
   if (e == cudaSuccess) e = run(tight, 1);
   if (e == cudaSuccess) e = run(full, 2);
   return e;

@@ -63,7 +63,7 @@ struct ecmc_ctx {
   int32_t stage_tight = 0, m_tight = 0;  // first pass (0: one pass)
   int32_t *d_deferred = nullptr;         // units left to the second pass
   int64_t deferred_cap = 0;
-  int32_t *d_n_deferred = nullptr;
+  int32_t *d_n_deferred = nullptr;       // (the third int of d_unit_next)
   int32_t lanes = 32;
   // slabs of a tile (domain mode): origin and extent of its box
   float lorg = 0.f;
@@ -139,6 +139,7 @@ void free_cells(ecmc_ctx *c) {
 ecmc_status alloc_cells(ecmc_ctx *c) {
   free_cells(c);
   CU(dalloc(&c->d_count, c->ncell));
+  CU(cudaMemsetAsync(c->d_count, 0, sizeof(int32_t) * c->ncell, c->stream));
   CU(dalloc(&c->d_start, c->ncell + 1));
   CU(dalloc(&c->d_bsum, cells_scratch_ints(c->ncell)));
   return ECMC_OK;
@@ -195,6 +196,7 @@ CellParams cell_params(const ecmc_ctx *c, bool domain, uint64_t seed, int64_t sw
   C.N = c->N;
   C.spring = (domain && c->configured && c->opts.k_spring > 0.0 && c->N > 1) ? 1 : 0;
   C.ftag = C.spring ? c->d_ftag : nullptr;
+  C.counters = c->d_unit_next;
   return C;
 }
 
@@ -302,8 +304,8 @@ ecmc_status alloc_state(ecmc_ctx *c) {
   CU(cudaMemset(c->d_sums, 0, sizeof(double) * SUM_N));
   CU(dalloc(&c->d_status, 1));
   CU(cudaMemset(c->d_status, 0, sizeof(int)));
-  CU(dalloc(&c->d_unit_next, 1));
-  CU(dalloc(&c->d_n_deferred, 1));
+  CU(dalloc(&c->d_unit_next, 3));
+  c->d_n_deferred = c->d_unit_next + 2;
   CU(dalloc(&c->d_obs_d, 5));
   CU(dalloc(&c->d_obs_u, 8));  // [6]: non-finite inputs of set_positions
   CU(dalloc(&c->d_g1ref, 3 * (c->n / c->N)));
@@ -319,7 +321,7 @@ void destroy(ecmc_ctx *c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
   void *ptrs[] = {c->d_r, c->d_img, c->d_tag, c->d_cell, c->d_rank, c->d_count, c->d_start,
                   c->d_bsum, c->d_cr, c->d_crf, c->d_rf, c->d_cid, c->d_ctag, c->d_cnt, c->d_sums, c->d_status,
-                  c->d_unit_next, c->d_n_deferred, c->d_ftag, c->d_deferred, c->d_obs_d, c->d_obs_u, c->d_g1ref, c->d_rdig, c->d_rlift, c->d_rev,
+                  c->d_unit_next, c->d_ftag, c->d_deferred, c->d_obs_d, c->d_obs_u, c->d_g1ref, c->d_rdig, c->d_rlift, c->d_rev,
                   c->d_log, c->d_log_n, c->d_su, c->d_srec, c->d_spart,
                   c->d_sr2n, c->d_ssum, c->d_g2ref, c->d_shist, c->d_po_flag, c->d_po_cnt, c->d_po_ctr,
                   c->d_g1ring, c->d_g1sum, c->d_g1cnt};
@@ -544,7 +546,9 @@ ecmc_status ecmc_configure(ecmc_ctx *c, const ecmc_opts *o) {
     const bool derived = stage <= 0;
     if (derived) stage = stage_bound(E, rho);
     mcap = stage_bound(c->W, rho);
-    if (derived) tight_caps(E, c->W, rho, stage, mcap, &stage_t, &m_t, p.tight_factor > 0 ? p.tight_factor : 1.08);
+    double Es[3];
+    staged_box(E, c->W, sig, Es);
+    if (derived) tight_caps(Es, c->W, rho, stage, mcap, &stage_t, &m_t, p.tight_factor > 0 ? p.tight_factor : 1.08);
   } else {
     if (p.precision == ECMC_PREC_FP32F)
       for (int a = 0; a < 3; ++a)

@@ -91,7 +91,7 @@ void batch_free(ecmc_batch *b) {
   void *ptrs[] = {b->d_r, b->d_img, b->d_rep_of, b->d_tag, b->d_cell, b->d_rank, b->d_count,
                   b->d_start, b->d_bsum, b->d_cid, b->d_ctag, b->d_cr, b->d_crf, b->d_rf, b->d_reps,
                   b->d_cnt,
-                  b->d_sums, b->d_status, b->d_unit_next, b->d_n_deferred, b->d_deferred, b->d_sweep,
+                  b->d_sums, b->d_status, b->d_unit_next, b->d_deferred, b->d_sweep,
                   b->d_rdig, b->d_rlift,
                   b->d_rev};
   for (void *p : ptrs) cudaFree(p);
@@ -132,6 +132,7 @@ cudaError_t batch_sweep(ecmc_batch *b, const ECParams &P, uint64_t seed) {
   C.rf = b->d_rf;
   C.cid = b->d_cid;
   C.ctag = b->d_ctag;
+  C.counters = b->d_unit_next;
   cudaError_t e = launch_cells_batch(C, b->ncell_total, b->stream);
   if (e != cudaSuccess) return e;
   e = launch_ec(P, b->lanes, b->opts.precision == ECMC_PREC_FP32F, 0, b->stream);
@@ -268,8 +269,8 @@ ecmc_status ecmc_batch_create(const ecmc_replica_spec *specs, int32_t n, double 
   if (e == cudaSuccess) e = balloc(&b->d_cnt, CNT_N);
   if (e == cudaSuccess) e = balloc(&b->d_sums, SUM_N);
   if (e == cudaSuccess) e = balloc(&b->d_status, 1);
-  if (e == cudaSuccess) e = balloc(&b->d_unit_next, 1);
-  if (e == cudaSuccess) e = balloc(&b->d_n_deferred, 1);
+  if (e == cudaSuccess) e = balloc(&b->d_unit_next, 3);
+  if (e == cudaSuccess) b->d_n_deferred = b->d_unit_next + 2;
   if (e == cudaSuccess) e = balloc(&b->d_sweep, 1);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_img, 0, sizeof(int32_t) * 3 * n_total, b->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_cnt, 0, sizeof(unsigned long long) * CNT_N, b->stream);
@@ -368,7 +369,9 @@ ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *o) {
     stage = st > stage ? st : stage;
     mcap = mc > mcap ? mc : mcap;
     int32_t st_t = 0, mc_t = 0;
-    tight_caps(E, R.W, rho, st, mc, &st_t, &mc_t, p.tight_factor > 0 ? p.tight_factor : 1.08);
+    double Es[3];
+    staged_box(E, R.W, sig, Es);
+    tight_caps(Es, R.W, rho, st, mc, &st_t, &mc_t, p.tight_factor > 0 ? p.tight_factor : 1.08);
     stage_t = st_t > stage_t ? st_t : stage_t;
     m_t = mc_t > m_t ? mc_t : m_t;
     nclm = (int32_t)ncl > nclm ? (int32_t)ncl : nclm;
@@ -406,6 +409,7 @@ ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *o) {
     cudaFree(b->d_bsum);
     b->d_count = b->d_start = b->d_bsum = nullptr;
     BCU(balloc(&b->d_count, cell_off));
+    BCU(cudaMemsetAsync(b->d_count, 0, sizeof(int32_t) * cell_off, b->stream));
     BCU(balloc(&b->d_start, cell_off + 1));
     BCU(balloc(&b->d_bsum, cells_scratch_ints(cell_off)));
     b->ncell_total = cell_off;

@@ -98,7 +98,7 @@ struct ECParams {
   int32_t *img;
   const double *cr;        // positions in cell order
   const int32_t *cid;      // ids in cell order
-  const int32_t *ctag;     // tiles in cell order
+  const int32_t *ctag;     // tiles in cell order (joint beads: see joint_tag, k_cells.cu)
   const int32_t *cstart;   // cell starts (ncell + 1)
   const float *crf;        // FP32 positions in cell order
   const float *rf;         // FP32 positions by bead
@@ -132,7 +132,7 @@ struct ECParams {
   // tiles per block (0: occupancy choice) and the device counter the
   // resident groups take units from (reset per launch)
   int32_t block_tiles;
-  int32_t *unit_next;
+  int32_t *unit_next;   // [0] first (or only) pass, [1] second pass
   // slow push-off (plain FP64 domain kernel): the ECs of a tile start at its
   // flagged motile beads, one each in id order, and a pivot ignores the
   // beads it overlaps; null otherwise
@@ -189,7 +189,7 @@ struct CellParams {
   int32_t *tag;
   int32_t *cell;
   int32_t *rank;
-  int32_t *count;     // ncell (zeroed by the launcher)
+  int32_t *count;     // ncell, zero between passes
   int32_t *start;     // ncell + 1
   int32_t *block_sums;
   double *cr;
@@ -204,6 +204,10 @@ struct CellParams {
   int32_t N;
   int32_t spring;
   int32_t *ftag;
+  // unit counters of the EC launches that follow (3 ints, zeroed here; may be null)
+  int32_t *counters;
+  // FP32 values and the error of an FP32 coordinate (launch_cells)
+  float Lf[3], Tf[3], Wf[3], cinv_f[3], tinv_f[3], tol;
 };
 cudaError_t launch_cells(const CellParams &C, int64_t ncell, cudaStream_t s);
 
@@ -227,6 +231,7 @@ struct CellBatch {
   int32_t *ctag;
   float *crf;                // FP32 positions in cell order
   float *rf;                 // FP32 positions by bead (concatenated)
+  int32_t *counters;         // unit counters of the EC launches (3 ints, zeroed here)
 };
 cudaError_t launch_cells_batch(const CellBatch &C, int64_t ncell_total, cudaStream_t s);
 cudaError_t launch_sweep_advance(int64_t *sweep_dev, cudaStream_t s);
@@ -354,6 +359,16 @@ inline int32_t packing_bound(const double E[3], double sigma) {
   const double v = (E[0] + sigma) * (E[1] + sigma) * (E[2] + sigma) / (sigma * sigma * sigma);
   const double n = v * 1.9098593171027443 + 32.0;
   return n < 65504.0 ? (int32_t)n / 32 * 32 + 32 : 65504;
+}
+
+// The box that holds as many beads as a tile stages: all of the hard-sphere
+// halo (W widened by sigma on both sides) and of the rest of the tether halo
+// (E) those bonded to a motile bead, a tenth or so.
+inline void staged_box(const double E[3], const double W[3], double sigma, double out[3]) {
+  const double v = E[0] * E[1] * E[2];
+  const double vs = (W[0] + 2.0 * sigma) * (W[1] + 2.0 * sigma) * (W[2] + 2.0 * sigma);
+  const double f = vs < v ? cbrt((vs + 0.15 * (v - vs)) / v) : 1.0;
+  for (int a = 0; a < 3; ++a) out[a] = f * E[a];
 }
 
 // Tight capacities of the EC kernel's first pass: `factor`

@@ -11,6 +11,7 @@
 // motile in another tile is made immotile too (a spring has no longest
 // bond, so only this keeps tiles apart).
 #include <cuda_runtime.h>
+#include <limits.h>
 
 #include "ecmc_dev.cuh"
 #include "ecmc_internal.h"
@@ -22,44 +23,73 @@ constexpr int SCAN_BLOCK = 1024;
 constexpr int SCAN_ITEMS = 4;  // elements per thread
 constexpr int SCAN_TILE = SCAN_BLOCK * SCAN_ITEMS;
 
-__global__ void k_tag_count(const CellParams C) {
-  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= C.n) return;
-  const double r0 = C.r[3 * b], r1 = C.r[3 * b + 1], r2 = C.r[3 * b + 2];
-  if (C.domain) {
+// Cell and tile of one coordinate.  FP32 decides both unless the coordinate
+// lies within its error (C.tol) of a boundary; those few take the FP64
+// expressions of the definition, so the result is always theirs.  (In FP64
+// alone a bead took some 40 FP64 and conversion instructions: 150 us per
+// sweep of 1e6 beads.)
+__device__ __forceinline__ int cell_axis(const CellParams &C, int a, double r, float rf) {
+  const float q = rf * C.cinv_f[a];
+  int k = (int)q;
+  const float f = q - (float)k, e = C.tol * C.cinv_f[a];
+  if (f < e || f > 1.f - e) k = (int)div_rn(r, C.cs[a]);
+  return k < 0 ? 0 : (k >= C.nc[a] ? C.nc[a] - 1 : k);
+}
+
+// o: the tile shift of the axis; false: in the joint
+__device__ __forceinline__ bool tile_axis(const CellParams &C, int a, double r, float rf, double o, float of, int &k) {
+  const float L = C.Lf[a], T = C.Tf[a], e = C.tol;
+  float u = rf - of;
+  const bool edge = fabsf(u) < e || L - fabsf(u) < e;
+  if (u < 0.f) u += L;
+  k = (int)(u * C.tinv_f[a]);
+  const float loc = u - (float)k * T;
+  if (edge || loc < e || loc > T - e || fabsf(loc - C.Wf[a]) < e) {
+    double v = r - o;
+    if (neg_bits(v)) v = v + C.L[a];
+    if (!less_pos(v, C.L[a])) v = v - C.L[a];
+    k = (int)div_rn(v, C.T[a]);
+    if (k > C.D[a] - 1) k = C.D[a] - 1;
+    return v - (double)k * C.T[a] < C.W[a];
+  }
+  if (k > C.D[a] - 1) k = C.D[a] - 1;
+  return loc < C.Wf[a];
+}
+
+// the sweep's tile shift (threads 0..2 of a block, axis each)
+__device__ __forceinline__ void sweep_shift(const CellParams &C, double *o) {
+  if (threadIdx.x < 3) {
     const int64_t sweep = C.sweep_dev ? *C.sweep_dev : C.sweep;
     const u64x4 w = philox(TAG_SHIFT, (uint64_t)sweep, 0, 0, C.seed, C.replica);
-    const double rr[3] = {r0, r1, r2};
-    int k[3];
-    bool in = true;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const double o = unit53(w.v[a]) * C.T[a];
-      double u = rr[a] - o;
-      if (u < 0.0) u = u + C.L[a];
-      if (u >= C.L[a]) u = u - C.L[a];
-      int t = (int)(u / C.T[a]);
-      if (t > C.D[a] - 1) t = C.D[a] - 1;
-      const double loc = u - (double)t * C.T[a];
-      in = in && (loc < C.W[a]);
-      k[a] = t;
-    }
-    C.tag[b] = in ? (k[2] * C.D[1] + k[1]) * C.D[0] + k[0] : -1;
-  } else {
-    C.tag[b] = 0;
+    o[threadIdx.x] = unit53(threadIdx.x == 0 ? w.v[0] : (threadIdx.x == 1 ? w.v[1] : w.v[2])) * C.T[threadIdx.x];
   }
-  int c[3];
-  const double rr[3] = {r0, r1, r2};
+}
+
+// tag and cell of bead b; returns the cell
+__device__ __forceinline__ int tag_and_cell(const CellParams &C, int64_t b, const double *o) {
+  const double r[3] = {C.r[3 * b], C.r[3 * b + 1], C.r[3 * b + 2]};
+  int c[3], k[3];
+  bool in = true;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    int t = (int)(rr[a] / C.cs[a]);
-    if (t >= C.nc[a]) t = C.nc[a] - 1;
-    if (t < 0) t = 0;
-    c[a] = t;
+    const float rf = f32_trunc(r[a]);
+    c[a] = cell_axis(C, a, r[a], rf);
+    k[a] = 0;
+    if (C.domain) in = tile_axis(C, a, r[a], rf, o[a], f32_trunc(o[a]), k[a]) && in;
   }
+  C.tag[b] = in ? (k[2] * C.D[1] + k[1]) * C.D[0] + k[0] : -1;
   const int cell = (c[2] * C.nc[1] + c[1]) * C.nc[0] + c[0];
   C.cell[b] = cell;
-  C.rank[b] = atomicAdd(&C.count[cell], 1);
+  return cell;
+}
+
+__global__ void k_tag_count(const CellParams C) {
+  __shared__ double o[3];
+  if (C.domain) sweep_shift(C, o);
+  if (C.counters && blockIdx.x == 0 && threadIdx.x < 3) C.counters[threadIdx.x] = 0;
+  __syncthreads();
+  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (b < C.n) C.rank[b] = atomicAdd(&C.count[tag_and_cell(C, b, o)], 1);
 }
 
 // block-wide exclusive scan of SCAN_TILE ints; returns the tile total
@@ -100,8 +130,8 @@ __device__ int block_scan(int (&v)[SCAN_ITEMS], int *sh) {
   return total;
 }
 
-__global__ void __launch_bounds__(SCAN_BLOCK) k_scan_tiles(const int *in, int64_t n, int *out,
-                                                          int *block_sums) {
+// (clears the counts it has read, for the next pass)
+__global__ void __launch_bounds__(SCAN_BLOCK) k_scan_tiles(int *in, int64_t n, int *out, int *block_sums) {
   __shared__ int sh[33];
   const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
   int v[SCAN_ITEMS];
@@ -110,64 +140,107 @@ __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_tiles(const int *in, int64_
   const int total = block_scan(v, sh);
 #pragma unroll
   for (int i = 0; i < SCAN_ITEMS; ++i)
-    if (base + i < n) out[base + i] = v[i];
+    if (base + i < n) {
+      out[base + i] = v[i];
+      in[base + i] = 0;
+    }
   if (threadIdx.x == 0) block_sums[blockIdx.x] = total;
 }
 
-// exclusive scan of the block sums (one block, loops over chunks)
-__global__ void __launch_bounds__(SCAN_BLOCK) k_scan_sums(int *sums, int64_t nb, int *total_out) {
-  __shared__ int sh[33];
-  int carry = 0;
-  for (int64_t c0 = 0; c0 < nb; c0 += SCAN_TILE) {
-    const int64_t base = c0 + (int64_t)threadIdx.x * SCAN_ITEMS;
-    int v[SCAN_ITEMS];
+// adds to every tile of SCAN_TILE starts the sums of the tiles before it
+// (each block adds those up itself: a few hundred at most)
+__global__ void __launch_bounds__(256) k_scan_add(int *out, int64_t n, const int *sums, int64_t tiles) {
+  __shared__ int sh[8];
+  int part = 0;
+  for (int64_t i = threadIdx.x; i < blockIdx.x; i += 256) part += sums[i];
+  part = __reduce_add_sync(0xffffffffu, part);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = part;
+  __syncthreads();
+  int before = 0;
 #pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; ++i) v[i] = (base + i < nb) ? sums[base + i] : 0;
-    const int total = block_scan(v, sh);
-#pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; ++i)
-      if (base + i < nb) sums[base + i] = v[i] + carry;
-    carry += total;
-  }
-  if (threadIdx.x == 0) *total_out = carry;
+  for (int i = 0; i < 8; ++i) before += sh[i];
+  const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
+  for (int64_t i = base + threadIdx.x; i < base + SCAN_TILE && i < n; i += 256) out[i] += before;
+  if (blockIdx.x == tiles - 1 && threadIdx.x == 0) out[n] = before + sums[tiles - 1];
 }
 
-__global__ void k_scan_add(int *out, int64_t n, const int *sums) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] += sums[i / SCAN_TILE];
+// Tag of a joint bead in cell order: whose tile its bonded beads are motile
+// in (staging takes a joint bead beyond the hard-sphere halo only for those):
+// -1 several tiles, -2 - k tile k, INT_MIN none
+__device__ __forceinline__ int32_t joint_tag(int32_t tp, int32_t tn) {
+  if (tp >= 0 && tn >= 0 && tp != tn) return -1;
+  const int32_t k = tp >= 0 ? tp : tn;
+  return k >= 0 ? -2 - k : INT_MIN;
+}
+
+__device__ __forceinline__ void scatter_bead(const CellParams &C, int64_t b, int64_t pos) {
+  const double x = C.r[3 * b], y = C.r[3 * b + 1], z = C.r[3 * b + 2];
+  const float fx = (float)x, fy = (float)y, fz = (float)z;
+  C.cr[3 * pos] = x;
+  C.cr[3 * pos + 1] = y;
+  C.cr[3 * pos + 2] = z;
+  C.crf[3 * pos] = fx;
+  C.crf[3 * pos + 1] = fy;
+  C.crf[3 * pos + 2] = fz;
+  C.rf[3 * b] = fx;
+  C.rf[3 * b + 1] = fy;
+  C.rf[3 * b + 2] = fz;
+  C.cid[pos] = (int32_t)b;
+  int32_t t = C.tag[b];
+  const int64_t c = b % C.N;
+  const int32_t tp = c != 0 ? C.tag[b - 1] : -1;
+  const int32_t tn = c != C.N - 1 ? C.tag[b + 1] : -1;
+  // bead-spring chains: a bead whose bonded bead is motile in another
+  // tile waits for a later sweep (the tags of both are the ones
+  // k_tag_count assigned, before any is dropped)
+  if (C.spring && t >= 0 && ((tp >= 0 && tp != t) || (tn >= 0 && tn != t))) t = -1;
+  C.ctag[pos] = t >= 0 ? t : joint_tag(tp, tn);
+  if (C.ftag) C.ftag[b] = t;
 }
 
 __global__ void k_scatter(const CellParams C) {
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= C.n) return;
-  const int64_t pos = (int64_t)C.start[C.cell[b]] + C.rank[b];
-  const double x = C.r[3 * b], y = C.r[3 * b + 1], z = C.r[3 * b + 2];
-  C.cr[3 * pos] = x;
-  C.cr[3 * pos + 1] = y;
-  C.cr[3 * pos + 2] = z;
-  C.crf[3 * pos] = (float)x;
-  C.crf[3 * pos + 1] = (float)y;
-  C.crf[3 * pos + 2] = (float)z;
-  C.rf[3 * b] = (float)x;
-  C.rf[3 * b + 1] = (float)y;
-  C.rf[3 * b + 2] = (float)z;
-  C.cid[pos] = (int32_t)b;
-  int32_t t = C.tag[b];
-  if (C.spring && t >= 0) {
-    // bead-spring chains: a bead whose bonded bead is motile in another
-    // tile waits for a later sweep (the tags of both are the ones
-    // k_tag_count assigned, before any is dropped)
-    const int64_t c = b % C.N;
-    const int32_t tp = c != 0 ? C.tag[b - 1] : -1;
-    const int32_t tn = c != C.N - 1 ? C.tag[b + 1] : -1;
-    if ((tp >= 0 && tp != t) || (tn >= 0 && tn != t)) t = -1;
+  if (b < C.n) scatter_bead(C, b, (int64_t)C.start[C.cell[b]] + C.rank[b]);
+}
+
+// The whole pass of a small melt in one block, counts in shared memory: a
+// small melt's sweep takes as long as its launches, and four of them become
+// one.
+constexpr int SMALL_BEADS = 8192, SMALL_CELLS = 16 * SCAN_BLOCK;
+__global__ void __launch_bounds__(SCAN_BLOCK) k_cells_small(const CellParams C, int ncell) {
+  extern __shared__ int cnt[];  // [ncell]
+  __shared__ int sh[33];
+  __shared__ double o[3];
+  for (int i = threadIdx.x; i < ncell; i += SCAN_BLOCK) cnt[i] = 0;
+  if (C.domain) sweep_shift(C, o);
+  if (C.counters && threadIdx.x < 3) C.counters[threadIdx.x] = 0;
+  __syncthreads();
+  const int n = (int)C.n;
+  for (int b = threadIdx.x; b < n; b += SCAN_BLOCK) C.rank[b] = atomicAdd(&cnt[tag_and_cell(C, b, o)], 1);
+  __syncthreads();
+  int carry = 0;
+  for (int c0 = 0; c0 < ncell; c0 += SCAN_TILE) {
+    const int base = c0 + threadIdx.x * SCAN_ITEMS;
+    int v[SCAN_ITEMS];
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) v[i] = base + i < ncell ? cnt[base + i] : 0;
+    const int total = block_scan(v, sh);
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i)
+      if (base + i < ncell) {
+        cnt[base + i] = v[i] + carry;
+        C.start[base + i] = v[i] + carry;
+      }
+    carry += total;
   }
-  C.ctag[pos] = t;
-  if (C.ftag) C.ftag[b] = t;
+  if (threadIdx.x == 0) C.start[ncell] = carry;
+  __syncthreads();
+  for (int b = threadIdx.x; b < n; b += SCAN_BLOCK) scatter_bead(C, b, cnt[C.cell[b]] + C.rank[b]);
 }
 
 __global__ void k_tag_count_b(const CellBatch C) {
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (blockIdx.x == 0 && threadIdx.x < 3) C.counters[threadIdx.x] = 0;
   if (b >= C.n) return;
   const RepParams &R = C.reps[C.rep_of[b]];
   const double rr[3] = {C.r[3 * b], C.r[3 * b + 1], C.r[3 * b + 2]};
@@ -210,8 +283,16 @@ __global__ void k_scatter_b(const CellBatch C) {
   C.rf[3 * b] = (float)x;
   C.rf[3 * b + 1] = (float)y;
   C.rf[3 * b + 2] = (float)z;
-  C.cid[pos] = (int32_t)(b - C.reps[C.rep_of[b]].bead_off);
-  C.ctag[pos] = C.tag[b];
+  const RepParams &R = C.reps[C.rep_of[b]];
+  const int64_t id = b - R.bead_off;
+  C.cid[pos] = (int32_t)id;
+  const int32_t t = C.tag[b];
+  if (t >= 0) {
+    C.ctag[pos] = t;
+  } else {
+    const int64_t c = id % R.N;
+    C.ctag[pos] = joint_tag(c != 0 ? C.tag[b - 1] : -1, c != R.N - 1 ? C.tag[b + 1] : -1);
+  }
 }
 
 __global__ void k_sweep_advance(int64_t *sweep) { *sweep += 1; }
@@ -219,15 +300,12 @@ __global__ void k_sweep_advance(int64_t *sweep) { *sweep += 1; }
 }  // namespace
 
 cudaError_t launch_cells_batch(const CellBatch &C, int64_t ncell, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(C.count, 0, sizeof(int32_t) * ncell, s);
-  if (e != cudaSuccess) return e;
   const int T = 256;
   const int64_t nb = (C.n + T - 1) / T;
   if (C.n > 0) k_tag_count_b<<<(unsigned)nb, T, 0, s>>>(C);
   const int64_t tiles = (ncell + SCAN_TILE - 1) / SCAN_TILE;
   k_scan_tiles<<<(unsigned)tiles, SCAN_BLOCK, 0, s>>>(C.count, ncell, C.start, C.block_sums);
-  k_scan_sums<<<1, SCAN_BLOCK, 0, s>>>(C.block_sums, tiles, C.start + ncell);
-  k_scan_add<<<(unsigned)((ncell + 255) / 256), 256, 0, s>>>(C.start, ncell, C.block_sums);
+  k_scan_add<<<(unsigned)tiles, 256, 0, s>>>(C.start, ncell, C.block_sums, tiles);
   if (C.n > 0) k_scatter_b<<<(unsigned)nb, T, 0, s>>>(C);
   return cudaGetLastError();
 }
@@ -239,16 +317,33 @@ cudaError_t launch_sweep_advance(int64_t *sweep_dev, cudaStream_t s) {
 
 size_t cells_scratch_ints(int64_t ncell) { return (size_t)((ncell + SCAN_TILE - 1) / SCAN_TILE) + 1; }
 
-cudaError_t launch_cells(const CellParams &C, int64_t ncell, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(C.count, 0, sizeof(int32_t) * ncell, s);
-  if (e != cudaSuccess) return e;
+cudaError_t launch_cells(const CellParams &C0, int64_t ncell, cudaStream_t s) {
+  CellParams C = C0;
+  float Lmax = 0.f;
+  for (int a = 0; a < 3; ++a) {
+    C.Lf[a] = (float)C.L[a];
+    C.cinv_f[a] = (float)(1.0 / C.cs[a]);
+    C.Tf[a] = (float)C.T[a];
+    C.Wf[a] = (float)C.W[a];
+    C.tinv_f[a] = C.T[a] > 0.0 ? (float)(1.0 / C.T[a]) : 0.f;
+    Lmax = C.Lf[a] > Lmax ? C.Lf[a] : Lmax;
+  }
+  // error of a coordinate (truncated to FP32, less a truncated shift, wrapped,
+  // less k T): below 8 L / 2^23, taken twice
+  C.tol = 16.f * Lmax / 8388608.f;
+  if (C.n > 0 && C.n <= SMALL_BEADS && ncell <= SMALL_CELLS) {
+    const cudaError_t e = cudaFuncSetAttribute(k_cells_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)sizeof(int) * SMALL_CELLS);
+    if (e != cudaSuccess) return e;
+    k_cells_small<<<1, SCAN_BLOCK, sizeof(int) * (size_t)ncell, s>>>(C, (int)ncell);
+    return cudaGetLastError();
+  }
   const int T = 256;
   const int64_t nb = (C.n + T - 1) / T;
   if (C.n > 0) k_tag_count<<<(unsigned)nb, T, 0, s>>>(C);
   const int64_t tiles = (ncell + SCAN_TILE - 1) / SCAN_TILE;
   k_scan_tiles<<<(unsigned)tiles, SCAN_BLOCK, 0, s>>>(C.count, ncell, C.start, C.block_sums);
-  k_scan_sums<<<1, SCAN_BLOCK, 0, s>>>(C.block_sums, tiles, C.start + ncell);
-  k_scan_add<<<(unsigned)((ncell + 255) / 256), 256, 0, s>>>(C.start, ncell, C.block_sums);
+  k_scan_add<<<(unsigned)tiles, 256, 0, s>>>(C.start, ncell, C.block_sums, tiles);
   if (C.n > 0) k_scatter<<<(unsigned)nb, T, 0, s>>>(C);
   return cudaGetLastError();
 }
