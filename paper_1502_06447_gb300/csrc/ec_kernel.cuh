@@ -9,11 +9,13 @@
 // its ECs takes the next unit of the launch from a device counter and stages
 // it while the warp's other groups wait.
 //
-// What bounds it: FP64 instructions.  GB300's FP64 unit takes a warp
-// instruction every 64 cycles per SM sub-partition whatever its active mask
-// and dependences (conversions and comparisons 80-110), so the number of
-// FP64 instructions of a step sets both a lone tile's latency and the rate
-// of a full chip.  Hence:
+// What bounds it: the latency of one step, a chain of dependent instructions
+// (a warp issues one every 6.4 cycles, of which 2.4 are fixed latencies, 1.2
+// shuffles and shared memory, 0.7 branches), with 12 warps per SM to hide it
+// (registers; about 4.7 KB of shared memory per tile).  The dearest of them
+// are FP64 instructions: GB300's FP64 unit takes a warp instruction every 64
+// cycles per SM sub-partition whatever its active mask and dependences
+// (conversions and comparisons 80-110).  Hence:
 //   - the lanes of a quad hold one axis each (lane 3: what is left of ell),
 //     and the three axes of a difference, a move or a reflection are one
 //     instruction; d.v and d.d are one chain of three on two lanes; the move,
@@ -36,6 +38,16 @@
 // A candidate left out by the screen cannot win: the winner's exact x is <= U
 // and every lower bound is <= its candidate's exact x, so both forms produce
 // the same events.
+//
+// Measured (cycles per warp step): 9,700 with 48 tiles of 8 lanes per SM on
+// 1e6 beads, 5,200 for a warp alone with one tile of 32 lanes; the kernel
+// that exchanged requests between the tiles of a block over block barriers
+// took 21,100 and some 14,000.  One sweep of 1e6 beads, eight ECs per tile
+// of 4.2 sigma: 91 -> 41 ms; a serial run of 640 beads in FP64, 400 ECs: 529
+// -> 58 ms (2.4 us per event); 64 replicas, four sweeps: 475 -> 181 ms.  A
+// bound of 128 registers with half the mask bytes (64 tiles per SM) lengthens
+// every step by as much as it adds tiles: 1e6 beads 1 % faster, 64 replicas
+// 11 % and lone warps 4 % slower.
 #pragma once
 #include "ec_device.cuh"
 
@@ -1050,19 +1062,21 @@ inline SlabPick pick_slabs(double e_max, double sigma, int S, int G, size_t budg
 template <int G, bool F32, bool BATCH, bool DOM, bool SPRING, bool PO>
 cudaError_t launch_ec_t(const ECParams &P0, cudaStream_t s) {
   auto kern = ec_kernel<G, F32, BATCH, DOM, SPRING, PO>;
-  static thread_local int sms = 0, smem_max = 0;
-  if (!sms) {
-    int dev = 0, n = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
-    if (e != cudaSuccess) return e;
-    sms = n;
+  // the device's limits, asked again when the thread has changed its device
+  static thread_local int sms = 0, smem_max = 0, device = -1;
+  int dev = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err == cudaSuccess && dev != device) {
+    device = -1;
+    err = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (err == cudaSuccess) device = dev;
   }
+  if (err == cudaSuccess) err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+  if (err != cudaSuccess) return err;
   // tiles per block and resident blocks of the last shapes asked for
   struct Shape {
-    int S, M64, M, nsl, bt, nt, blocks, units;
+    int S, M64, M, nsl, bt, nt, blocks, units, dev;
     float inv;
     size_t smem;
   };
@@ -1085,7 +1099,7 @@ cudaError_t launch_ec_t(const ECParams &P0, cudaStream_t s) {
     }
     for (const Shape &h : memo)
       if (h.nt && h.S == S && h.M == M && h.bt == P.block_tiles && h.nsl == k.nsl && h.inv == k.inv &&
-          h.units == P.n_units) {
+          h.units == P.n_units && h.dev == dev) {
         *out = h;
         return cudaSuccess;
       }
@@ -1094,6 +1108,7 @@ cudaError_t launch_ec_t(const ECParams &P0, cudaStream_t s) {
     w.M = M;
     w.bt = P.block_tiles;
     w.units = P.n_units;
+    w.dev = dev;
     w.nsl = k.nsl;
     w.inv = k.inv;
     const int MQ = mask_quads(S, G, w.nsl);

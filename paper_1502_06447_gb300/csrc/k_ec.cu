@@ -12,14 +12,10 @@ namespace {
 // block's tiles keeps the lanes too.
 int pick_lanes(const ECParams &P, int lanes) {
   if (P.block_tiles > 0) return lanes;
-  static thread_local int sms = 0;
-  if (!sms) {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      return lanes;
-    sms = n;
-  }
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return lanes;
   while (lanes < 32 && (long long)P.n_units * (2 * lanes) <= (long long)EC_SPREAD_WARPS * 32 * sms) lanes *= 2;
   return lanes;
 }
