@@ -171,8 +171,17 @@ cudaError_t launch_ec_spring_screened(const ECParams &P, int lanes, cudaStream_t
 cudaError_t launch_ec_spring_fp64(const ECParams &P, int lanes, cudaStream_t s);
 cudaError_t launch_ec_pushoff_tether(const ECParams &P, int lanes, cudaStream_t s);
 cudaError_t launch_ec_pushoff_spring(const ECParams &P, int lanes, cudaStream_t s);
-// pick_lanes (k_ec.cu): warps per SM up to which a tile gets more lanes
-constexpr int EC_SPREAD_WARPS = 8;
+
+// pick_lanes (k_ec.cu): tiles get twice the lanes as long as all of them then stay resident, at
+// most this many warps per SM (what the EC kernel's registers allow).  A
+// group steps faster with more lanes and with fewer groups in its warp; a
+// second round of tiles costs more than that.  ms per sweep (two ECs per tile
+// of 4.2 sigma, GB300, screened / FP64) with 8, 16, 32 lanes: 1,331 tiles
+// 2.93, 2.71, 2.35 / 3.66, 2.85, 2.33; 1,728 tiles (11.4 warps per SM at 32)
+// 2.95, 2.71, 2.36 / 3.58, 2.88, 2.34; 2,197 (14.5 at 32) 2.93, 2.76, 3.15 /
+// 3.67, 2.92, 3.08; 3,375 (11.1 at 16) 2.97, 2.78, 3.52 / 3.60, 3.30, 3.44;
+// 4,096 (13.5 at 16) 3.61, 4.15, 4.85 / 5.28, 4.44, 4.71.
+constexpr int EC_SPREAD_WARPS = 12;
 
 // cell list and domain tags (k_cells.cu)
 struct CellParams {
@@ -390,7 +399,7 @@ inline void tight_caps(const double E[3], const double Wm[3], double rho, int32_
 // ---------------------------------------------------------------- autotuner
 // One launch setting of the domain sweep.  The search is a coordinate
 // descent: lanes per EC, tile side, global cell side, ECs per tile, and the
-// staging of the block-lockstep kernel (warps per block, the first pass's
+// staging of the screened form (warps per block, the first pass's
 // capacity factor), each axis scanned with the others held at their best so
 // far, in up to two rounds.  The
 // objective is ECs per device-second (each EC displaces by ell, so this is
@@ -401,8 +410,8 @@ struct TunePoint {
   double tile_side;  // in units of sigma
   double cell_side;  // in units of sigma
   int ecs;
-  int warps;         // block lockstep: warps per block (tiles = warps 32 / lanes)
-  double tight;      // block lockstep: first-pass capacity factor
+  int warps;         // screened form: warps per block (tiles = warps 32 / lanes)
+  double tight;      // screened form: first-pass capacity factor
 };
 
 struct TuneScore {
