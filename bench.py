@@ -45,9 +45,9 @@ SWAP_RATE = 0.1
 METRIC = "events/s (EC sweep, 1e6-bead melt, FP32 screen + FP64 confirm)"
 UNIT = "events/s"
 C0 = 1.2  # stencil cell side of the bytes-per-event definition (= b_max)
-# revision of the block-lockstep kernel; DRAM counters in profiles/ are used
+# revision of the EC kernel; DRAM counters in profiles/ are used
 # only when they were taken on the same revision
-KERNEL_REV = 6
+KERNEL_REV = 7
 
 
 def launch_settings(args):
@@ -144,7 +144,7 @@ def measured_counters(kernel, st):
     cycles per FP64 instruction), or None unless it was taken on this
     kernel revision in exactly this launch setting."""
     import re
-    p = os.path.join(ROOT, "profiles", "ec_lock_counters_1e6_melt.md")
+    p = os.path.join(ROOT, "profiles", "ec_kernel_counters_1e6_melt.md")
     try:
         txt = open(p).read()
     except OSError:
@@ -181,7 +181,7 @@ def ceilings(cnt, ec_events_per_s, sm_mhz):
                           "fp64_cycles_per_instr": cnt["fp64_cycles_per_instr"]},
             "sms": sms, "sm_mhz": sm_mhz,
             "note": "events/s of the EC launches against each ceiling; the kernel is latency "
-                    "bound (dependent FP64 chains, barriers, shared-memory round trips) and "
+                    "bound (dependent instructions, shuffles, shared-memory round trips) and "
                     "reaches neither"}
 
 
@@ -402,8 +402,8 @@ def run_gpu(args, rank, world):
     phi = C5.phi
     bpe = bytes_per_event(phi, confirmed / max(events, 1))
     achieved = events * bpe / ec_s / 1e9
-    kname = (f"ec_lock_kernel<{setting['lanes']}, 0>" if args.schedule == 0 and setting["lanes"] in (4, 8, 16)
-             else f"ec_kernel<{setting['lanes']}, 1, 0>")
+    # template arguments: lanes, FP32 screen, batch, domain, springs, push-off
+    kname = f"ec_kernel<{setting['lanes']}, 1, 0, 1, 0, 0>"
     traffic = measured_traffic(kname, setting)
     counters = measured_counters(kname, setting)
     csum = clk.summary()
@@ -454,9 +454,9 @@ def run_gpu(args, rank, world):
                 "ms_per_step": 1e3 * e2e_max / n_e2e, "events": e2e_tot,
                 "h2d_bytes_per_step": int(r_host.nbytes + img_host.nbytes),
                 "d2h_bytes_per_step": int(r_host.nbytes + img_host.nbytes)},
-        # per sweep: 5 cell-list kernels + the EC launch (two passes for the
-        # block-lockstep kernel: tight capacities, then deferred tiles)
-        "gpu_launches": (7 if kname.startswith("ec_lock") else 6) * args.steps,
+        # per sweep: 4 cell-list kernels + the EC launches (tight capacities,
+        # then the tiles that did not fit)
+        "gpu_launches": 6 * args.steps,
         "physics": physics,
         "structure": structure,
         "init": init,
@@ -608,7 +608,7 @@ def precision_run(args, stream, sweeps=5):
            "fp32f_events_per_s": f["events_per_s"], "fp64_events_per_s": g["events_per_s"],
            "fp32f_over_fp64": f["events_per_s"] / g["events_per_s"],
            "confirmed_per_event": f["confirmed_per_event"],
-           "note": "FP32 screen (block-lockstep kernel, 8 lanes) vs plain FP64 kernel (16 lanes), "
+           "note": "FP32 screen (8 lanes) vs plain FP64 kernel (16 lanes), "
                    "same lattice and seed; digests are 64-bit FNV-1a over every event of an EC"}
     state = {"r1": f["r1"], "i1": f["i1"], "d1": f["digests"][:nt]}
     return res, state
@@ -1032,9 +1032,9 @@ def main():
     ap.add_argument("--tiles", type=int, default=0, help="tiles per axis (0: workload default)")
     ap.add_argument("--ecs-per-tile", type=int, default=0, help="0: the pinned setting")
     ap.add_argument("--schedule", type=int, default=0,
-                    help="screened kernel: 0 block lockstep, 1 warp lockstep")
+                    help="0 or 1: same kernel and events")
     ap.add_argument("--block-tiles", type=int, default=-1,
-                    help="block lockstep: tiles per block (-1: the pinned setting, 0: occupancy)")
+                    help="tiles per block (-1: the pinned setting, 0: occupancy)")
     ap.add_argument("--no-tune", dest="tune", action="store_false",
                     help="skip the autotuner (the timed setting is the pinned one anyway)")
     ap.add_argument("--time-tuned", action="store_true",

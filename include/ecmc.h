@@ -430,9 +430,9 @@ ecmc_status ecmc_batch_records(ecmc_batch *b, uint64_t *digest, double *lift,
  * Picks the launch setting of the domain sweep for this machine and system
  * (the paper fixes none: Sec. II.A leaves the tile size open): lanes per EC
  * (4, 8, 16, 32), tile side (3.4, 3.8, 4.2, 4.6, 5, 6, 7 sigma), global cell side (1.05 or 1.4
- * sigma), ECs per tile (1, 2, 4 or 8) and the block-lockstep kernel's staging
+ * sigma), ECs per tile (1, 2, 4 or 8) and the screened form's staging
  * (1, 2 or 4 warps per block; first-pass capacity factor 1.0, 1.08 or 1.16;
- * other kernels take only the defaults), by a coordinate descent (up to two
+ * other forms take only the defaults), by a coordinate descent (up to two
  * rounds) over short timed trials.  Each trial restores the state saved on entry, runs one untimed
  * sweep and `trial_sweeps` timed ones; the score is ECs per device-second.
  * On return the context (batch) is configured with the winner and its
@@ -449,8 +449,8 @@ typedef struct ecmc_tuning {
   double ecs_per_s;       /* score of the winner */
   double events_per_s;
   int32_t n_trials;       /* admissible points timed */
-  int32_t block_tiles;    /* block lockstep: tiles per block (0: not that kernel) */
-  double tight_factor;    /* block lockstep: first-pass capacity factor */
+  int32_t block_tiles;    /* screened form: tiles per block (0: another form) */
+  double tight_factor;    /* screened form: first-pass capacity factor */
 } ecmc_tuning;
 ecmc_status ecmc_autotune(ecmc_ctx *ctx, double ell, uint64_t seed,
                           int32_t trial_sweeps, ecmc_tuning *out);

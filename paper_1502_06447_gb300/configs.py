@@ -75,8 +75,9 @@ CONFIGS = {m.name: m for m in (C1, C2, C3, C5)}
 # committed profiles describe it.  block_tiles 0: the occupancy
 # calculator's choice; 8 tiles of 8 lanes = two warps per block.  Eight ECs
 # per tile: a sweep ends with its longest tile, and more ECs per tile spread
-# that tail over more work (timed on a GB300, 25^3 tiles: 2 / 4 / 8 / 16 ECs
-# per tile gave 3.8 / 4.1 / 4.5-4.8 / 5.0e8 events/s).  This maximises
+# that tail over more work (GB300, 25^3 tiles, an earlier version of the
+# kernel: 2 / 4 / 8 / 16 ECs per tile gave 3.8 / 4.1 / 4.5-4.8 / 5.0e8
+# events/s; eight give 8.6e8 now).  This maximises
 # events/s, not relaxation: with the tiles fixed for eight ECs the middle
 # beads' g1 grows about 22 % slower per device-second than at two ECs per
 # tile, and 22^3 tiles at one or two ECs per tile relax fastest.

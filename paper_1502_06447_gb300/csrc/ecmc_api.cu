@@ -1470,7 +1470,7 @@ ecmc_status ecmc_autotune(ecmc_ctx *c, double ell, uint64_t seed, int32_t trial_
     CU(cudaStreamSynchronize(c->stream));
     return ECMC_OK;
   };
-  // the staging axes apply to the block-lockstep kernel only; elsewhere a
+  // the staging axes apply to the screened form with tethers only; elsewhere a
   // point off their defaults is not admissible (never timed)
   auto lock_point = [&](const TunePoint &pt) {
     return base.mode == ECMC_MODE_DOMAIN && base.precision == ECMC_PREC_FP32F && base.schedule == 0 &&

@@ -616,7 +616,7 @@ ecmc_status ecmc_batch_autotune(ecmc_batch *b, double ell, uint64_t seed, int32_
     b->device_seconds = ds0;
     return ECMC_OK;
   };
-  // the staging axes apply to the block-lockstep kernel only
+  // the staging axes apply to the screened form only
   auto lock_point = [&](const TunePoint &pt) {
     return base.precision == ECMC_PREC_FP32F && base.schedule == 0 &&
            (pt.lanes == 4 || pt.lanes == 8 || pt.lanes == 16);
