@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(128) k_overlaps(const ObsParams O) {
       if (fabsf(f - O.f_lo) > O.f_err && fabsf(f - O.f_s1) > O.f_err && fabsf(f - O.f_s2) > O.f_err) {
         cnt += f < O.f_lo;
         cs0 += f > O.f_lo && f < O.f_s1;
-        cs1 += f > O.f_s1;
+        cs1 += f > O.f_s1 && f < O.f_s2;
         return;
       }
       const double e0 = wrap_bits(O.cr[3 * t] - O.cr[3 * (int64_t)j], O.L[0], O.half[0]);

@@ -72,3 +72,22 @@ def test_pair_counts_match_direct_count(dims):
         s2 += int(((q >= 1.02 * 1.02) & (q < 1.04 * 1.04)).sum())
     assert obs["overlaps"] == 0
     assert tuple(obs["contact_pairs"]) == (s1, s2)
+
+
+def test_pairs_just_beyond_the_outer_shell():
+    """Squared distances next to the bound up to which FP32 leaves a pair to
+    FP64 (outer shell + error of a square): beyond the shell, so none counts."""
+    a, dims = 3.0, (12, 12, 24)
+    L = np.array(dims) * a
+    rng = np.random.default_rng(7)
+    site = np.stack(np.meshgrid(*(np.arange(d) for d in (12, 12, 12)), indexing="ij"), -1).reshape(-1, 3)
+    r0 = (site + 0.5) * np.array([3.0, 3.0, 6.0])
+    s2 = 1.04 ** 2
+    err = 16.0 * 1.04 * (L.max() + 1.04) / 2.0 ** 24 + 1e-6 * s2
+    d2 = s2 + err * rng.uniform(0.5, 1.5, len(r0))
+    v = rng.normal(size=r0.shape)
+    v *= (np.sqrt(d2) / np.linalg.norm(v, axis=1))[:, None]
+    ctx = ecmc.Context.create_lattice(dims, a, 1, b_max=1.2)
+    ctx.set_positions(np.concatenate([r0 - 0.5 * v, r0 + 0.5 * v]))
+    obs = ctx.observables()
+    assert obs["overlaps"] == 0 and tuple(obs["contact_pairs"]) == (0, 0)
