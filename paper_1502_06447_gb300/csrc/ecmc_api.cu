@@ -6,6 +6,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -40,8 +41,38 @@ cudaError_t dalloc(T **p, size_t count) {
   *p = nullptr;
   if (count == 0) count = 1;
   if (alloc_refused(sizeof(T) * count)) return cudaErrorMemoryAllocation;
-  return cudaMalloc((void **)p, sizeof(T) * count);
+  const cudaError_t e = cudaMalloc((void **)p, sizeof(T) * count);
+  if (e != cudaSuccess) (void)cudaGetLastError();  // (a launch check after it would report it again)
+  return e;
 }
+
+// Buffers that are used together: all of them are allocated, or none is (a
+// call that finds the first one takes the others for granted).
+struct Want {
+  void **p;
+  size_t bytes;
+  template <class T>
+  Want(T **q, size_t count) : p((void **)q), bytes(sizeof(T) * (count ? count : 1)) {}
+};
+ecmc_status alloc_all(std::initializer_list<Want> group) {
+  for (const Want &w : group) {
+    const cudaError_t e = dalloc((char **)w.p, w.bytes);
+    if (e == cudaSuccess) continue;
+    for (const Want &v : group) {
+      if (&v == &w) break;
+      cudaFree(*v.p);
+      *v.p = nullptr;
+    }
+    return fail(e == cudaErrorMemoryAllocation ? ECMC_ENOMEM : ECMC_ECUDA, "%lld bytes: %s",
+                (long long)w.bytes, cudaGetErrorString(e));
+  }
+  return ECMC_OK;
+}
+#define TRY(call)                        \
+  do {                                   \
+    const ecmc_status s_ = (call);       \
+    if (s_ != ECMC_OK) return s_;        \
+  } while (0)
 }  // namespace
 
 // What a call reads back from the device, in one piece: a copy of a few bytes
@@ -69,7 +100,7 @@ struct ecmc_ctx {
   double halo_hs = 0, halo_te = 0;
   int32_t nc[3] = {1, 1, 1};
   double cs[3] = {1, 1, 1};
-  int64_t ncell = 1;
+  int64_t ncell = 0;  // 0: no cell arrays
   int32_t stage_cap = 0;
   int32_t m_cap = 0;
   int32_t stage_tight = 0, m_tight = 0;  // first pass (0: one pass)
@@ -148,19 +179,14 @@ void free_cells(ecmc_ctx *c) {
   cudaFree(c->d_start);
   cudaFree(c->d_bsum);
   c->d_count = c->d_start = c->d_bsum = nullptr;
+  c->ncell = 0;
 }
 
-ecmc_status alloc_cells(ecmc_ctx *c) {
-  free_cells(c);
-  CU(dalloc(&c->d_count, c->ncell));
-  CU(cudaMemsetAsync(c->d_count, 0, sizeof(int32_t) * c->ncell, c->stream));
-  CU(dalloc(&c->d_start, c->ncell + 1));
-  CU(dalloc(&c->d_bsum, cells_scratch_ints(c->ncell)));
-  return ECMC_OK;
-}
-
-// global cell grid of side >= cell_side (>= sigma), at least 3 per axis
+// global cell grid of side >= cell_side (>= sigma), at least 3 per axis; a
+// side that is refused leaves the grid as it was, one whose arrays cannot be
+// had leaves none (see need_grid)
 ecmc_status set_grid(ecmc_ctx *c, double side) {
+  int32_t nc[3];
   int64_t ncell = 1;
   for (int a = 0; a < 3; ++a) {
     // bounded in double before the cast; the product stays below 2^31
@@ -168,16 +194,30 @@ ecmc_status set_grid(ecmc_ctx *c, double side) {
     if (!(kd >= 3.0)) return fail(ECMC_EINVAL, "box too small for the cell grid (axis %d)", a);
     if (!(kd <= 1048576.0) || (double)ncell * kd > 2147483647.0)
       return fail(ECMC_EINVAL, "cell grid too fine (axis %d)", a);
-    const int k = (int)kd;
-    c->nc[a] = k;
-    c->cs[a] = c->L[a] / k;
-    ncell *= k;
+    nc[a] = (int32_t)kd;
+    ncell *= nc[a];
   }
-  if (ncell != c->ncell || !c->d_count) {
+  if (ncell != c->ncell) {
+    free_cells(c);
+    TRY(alloc_all({{&c->d_count, (size_t)ncell},
+                  {&c->d_start, (size_t)ncell + 1},
+                  {&c->d_bsum, cells_scratch_ints(ncell)}}));
     c->ncell = ncell;
-    return alloc_cells(c);
+    // (zero between passes: each pass clears the counts it has read)
+    CU(cudaMemsetAsync(c->d_count, 0, sizeof(int32_t) * ncell, c->stream));
+  }
+  for (int a = 0; a < 3; ++a) {
+    c->nc[a] = nc[a];
+    c->cs[a] = c->L[a] / nc[a];
   }
   return ECMC_OK;
+}
+
+// the configured grid again, where a call that asked for another one could not
+// have its memory
+ecmc_status need_grid(ecmc_ctx *c) {
+  if (c->ncell > 0) return ECMC_OK;
+  return set_grid(c, c->opts.cell_side > 0 ? c->opts.cell_side : 1.05 * c->sigma);
 }
 
 CellParams cell_params(const ecmc_ctx *c, bool domain, uint64_t seed, int64_t sweep) {
@@ -653,8 +693,7 @@ ecmc_status ecmc_log_reserve(ecmc_ctx *c, int64_t cap) {
   c->d_log_n = nullptr;
   c->log_cap = 0;
   if (cap > 0) {
-    CU(dalloc(&c->d_log, cap));
-    CU(dalloc(&c->d_log_n, 1));
+    TRY(alloc_all({{&c->d_log, (size_t)cap}, {&c->d_log_n, 1}}));
     c->log_cap = cap;
   }
   return ECMC_OK;
@@ -668,10 +707,8 @@ static ecmc_status reserve_records(ecmc_ctx *c, int64_t units) {
   c->d_rdig = nullptr;
   c->d_rlift = nullptr;
   c->d_rev = nullptr;
-  c->rec_cap = 0;
-  CU(dalloc(&c->d_rdig, units));
-  CU(dalloc(&c->d_rlift, units));
-  CU(dalloc(&c->d_rev, units));
+  c->rec_cap = c->rec_n = 0;
+  TRY(alloc_all({{&c->d_rdig, (size_t)units}, {&c->d_rlift, (size_t)units}, {&c->d_rev, (size_t)units}}));
   c->rec_cap = units;
   return ECMC_OK;
 }
@@ -807,6 +844,7 @@ ecmc_status ecmc_run(ecmc_ctx *c, double ell, int64_t chains_per_sweep, uint64_t
   if (c->pushoff_pending) return fail(ECMC_EOVERLAP, "phantom chains overlap: run ecmc_pushoff first");
   if (!(ell >= 0.0) || !isfinite(ell)) return fail(ECMC_EINVAL, "ell must be finite and >= 0");
   const bool domain = c->opts.mode == ECMC_MODE_DOMAIN;
+  if (domain) TRY(need_grid(c));
   const int64_t ntile = (int64_t)c->opts.tiles[0] * c->opts.tiles[1] * c->opts.tiles[2];
   const int k = domain ? (chains_per_sweep > 0 ? (int)chains_per_sweep : c->ecs_per_tile) : 1;
   int64_t units;
@@ -948,20 +986,18 @@ ecmc_status ecmc_observables(ecmc_ctx *c, ecmc_obs *out) {
 static ecmc_status run_structure(ecmc_ctx *c, bool with_r2n, double dR, int64_t nbins) {
   const int64_t nch = c->n / c->N;
   if (!c->d_su) {
-    CU(dalloc(&c->d_su, 3 * c->n));
-    CU(dalloc(&c->d_srec, STRUCT_REC * nch));
-    CU(dalloc(&c->d_ssum, STRUCT_SUMS));
-    CU(dalloc(&c->d_g2ref, 3 * nch));
+    TRY(alloc_all({{&c->d_su, 3 * (size_t)c->n},
+                  {&c->d_srec, STRUCT_REC * (size_t)nch},
+                  {&c->d_ssum, STRUCT_SUMS},
+                  {&c->d_g2ref, 3 * (size_t)nch}}));
   }
-  if (with_r2n && !c->d_spart) {
-    CU(dalloc(&c->d_spart, nch * c->N));
-    CU(dalloc(&c->d_sr2n, c->N));
-  }
+  if (with_r2n && !c->d_spart)
+    TRY(alloc_all({{&c->d_spart, (size_t)nch * c->N}, {&c->d_sr2n, (size_t)c->N}}));
   if (nbins > c->shist_n) {
     cudaFree(c->d_shist);
     c->d_shist = nullptr;
     c->shist_n = 0;
-    CU(cudaMalloc(&c->d_shist, sizeof(unsigned long long) * (size_t)nbins));
+    CU(dalloc(&c->d_shist, nbins));
     c->shist_n = nbins;
   }
   StructParams S{};
@@ -1068,10 +1104,9 @@ ecmc_status ecmc_pushoff(ecmc_ctx *c, double f0, int32_t stages, double ell, uin
     return fail(ECMC_EINVAL, "push-off needs the domain mode and FP64");
   if (!(f0 > 0.0 && f0 <= 1.0) || stages < 1 || max_sweeps < 1 || !(ell >= 0.0 && ell < INFINITY))
     return fail(ECMC_EINVAL, "need 0 < f0 <= 1, stages >= 1, max_sweeps >= 1, finite ell >= 0");
+  TRY(need_grid(c));
   if (!c->d_po_flag) {
-    CU(dalloc(&c->d_po_flag, c->n));
-    CU(dalloc(&c->d_po_cnt, 1));
-    CU(dalloc(&c->d_po_ctr, 2));
+    TRY(alloc_all({{&c->d_po_flag, (size_t)c->n}, {&c->d_po_cnt, 1}, {&c->d_po_ctr, 2}}));
   }
   CU(cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream));
   ECParams P = ec_params(c, seed, ell);
@@ -1199,8 +1234,7 @@ ecmc_status ecmc_g1_track(ecmc_ctx *c, int32_t P, int32_t K) {
     c->g1ring_n = ring_n;
   }
   if (!c->d_g1sum) {
-    CU(dalloc(&c->d_g1sum, 16 * 63));
-    CU(dalloc(&c->d_g1cnt, 16 * 63));
+    TRY(alloc_all({{&c->d_g1sum, 16 * 63}, {&c->d_g1cnt, 16 * 63}}));
   }
   CU(cudaMemsetAsync(c->d_g1sum, 0, sizeof(double) * nlag, c->stream));
   CU(cudaMemsetAsync(c->d_g1cnt, 0, sizeof(unsigned long long) * nlag, c->stream));
@@ -1312,6 +1346,7 @@ ecmc_status ecmc_domain_tags(ecmc_ctx *c, uint64_t seed, int64_t sweep, int32_t 
   if (!c || !tags) return fail(ECMC_EINVAL, "NULL argument");
   if (!c->configured || c->opts.mode != ECMC_MODE_DOMAIN)
     return fail(ECMC_EINVAL, "configure the domain mode first");
+  TRY(need_grid(c));
   CU(launch_cells(cell_params(c, true, seed, sweep), c->ncell, c->stream));
   CU(cudaMemcpyAsync(tags, (c->opts.k_spring > 0.0 && c->N > 1) ? c->d_ftag : c->d_tag, sizeof(int32_t) * c->n, cudaMemcpyDeviceToHost, c->stream));
   CU(cudaStreamSynchronize(c->stream));

@@ -1,0 +1,67 @@
+"""Calls that run out of device memory half way (the injected limit of
+ECMC_ALLOC_LIMIT lets the first buffer of a group through and refuses a later
+one): they return ENOMEM, launch nothing, and once memory is there again the
+same context gives the oracle's events and the structure of a fresh one."""
+import numpy as np
+import pytest
+
+from paper_1502_06447_gb300 import ecmc
+from paper_1502_06447_gb300.configs import small_domain
+
+from helpers import gpu_context, oracle_system
+
+pytestmark = pytest.mark.gpu
+
+ENOMEM = -2
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _build():
+    from paper_1502_06447_gb300 import build
+    build.build()
+
+
+def refused(monkeypatch, limit, call):
+    with monkeypatch.context() as m:
+        m.setenv("ECMC_ALLOC_LIMIT", str(limit))
+        with pytest.raises(ecmc.EcmcError) as e:
+            call()
+    assert e.value.code == ENOMEM
+
+
+def settings(m, **kw):
+    return dict(dict(mode=ecmc.MODE_DOMAIN, dir_mode=ecmc.DIR_ISO, precision=ecmc.PREC_FP32F,
+                     tiles=m.D, lanes=8, record=1), **kw)
+
+
+def assert_runs_as_oracle(ctx, m, o, sweeps, sweep0=0):
+    ctx.run(m.ell, seed=m.seed, n_sweeps=sweeps)
+    res = o.run_domain(sweeps, m.ell, sweep0=sweep0, digests=True)
+    dig, _, _ = ctx.records(len(res["digest"]))
+    assert len(dig) == len(res["digest"]) and (dig == res["digest"]).all()
+    r, img = ctx.get_positions()
+    assert (r == o.r).all() and (img == o.img).all()
+
+
+def test_cell_arrays_half_allocated(monkeypatch):
+    """The counts fit the limit (4 B per cell), the starts (one more) do not."""
+    m = small_domain()
+    ctx, o = gpu_context(m, precision=ecmc.PREC_FP32F, lanes=8), oracle_system(m)
+    assert_runs_as_oracle(ctx, m, o, 1)
+    side = 1.5
+    limit = 4 * int(np.prod([int(L / side) for L in m.L]))
+    refused(monkeypatch, limit, lambda: ctx.configure(**settings(m, cell_side=side)))
+    assert_runs_as_oracle(ctx, m, o, 1, sweep0=1)
+    assert ctx.observables()["overlaps"] == 0
+
+
+def test_structure_scratch_half_allocated(monkeypatch):
+    """Chains of two: the positions along the chains take 24 B per bead, the
+    records of the chains 52."""
+    m = small_domain(N=2)
+    ctx = gpu_context(m, precision=ecmc.PREC_FP32F, lanes=8)
+    refused(monkeypatch, 24 * ctx.n, lambda: ctx.structure(dR=0.5, nbins=8))
+    refused(monkeypatch, 24 * ctx.n, ctx.g1_reset)
+    got, r2n, hist = ctx.structure(dR=0.5, nbins=8)
+    ref, r2n0, hist0 = gpu_context(m, precision=ecmc.PREC_FP32F, lanes=8).structure(dR=0.5, nbins=8)
+    assert got == ref and (r2n == r2n0).all() and (hist == hist0).all()
