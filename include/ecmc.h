@@ -273,6 +273,7 @@ ecmc_status ecmc_get_info(ecmc_ctx *ctx, double box[3], int64_t *n_beads,
                           int32_t *N);
 
 /* ---- running ------------------------------------------------------------ */
+/* A refused call leaves the settings in force as they were. */
 ecmc_status ecmc_configure(ecmc_ctx *ctx, const ecmc_opts *opts);
 
 /* ecmc_run: serial mode: chains_per_sweep ECs (all of them, n_sweeps is

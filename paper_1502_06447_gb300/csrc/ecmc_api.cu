@@ -583,27 +583,28 @@ ecmc_status ecmc_configure(ecmc_ctx *c, const ecmc_opts *o) {
   int32_t stage = p.stage_cap;
   int32_t mcap = 0;
   int32_t stage_t = 0, m_t = 0;
+  // (a call that is refused leaves the settings in force as they were: all
+  // that changes is committed at the end)
+  double T[3] = {c->T[0], c->T[1], c->T[2]}, W[3] = {c->W[0], c->W[1], c->W[2]};
   if (p.mode == ECMC_MODE_DOMAIN) {
     for (int a = 0; a < 3; ++a) {
       if (p.tiles[a] < 3) return fail(ECMC_EINVAL, "tiles per axis must be >= 3");
-      const double T = c->L[a] / p.tiles[a];
-      const double W = T - w;
-      if (!(W > 0.0)) return fail(ECMC_EINVAL, "tile narrower than the joint");
-      if (!(W + 2.0 * halo_te < 0.5 * c->L[a]))
+      T[a] = c->L[a] / p.tiles[a];
+      W[a] = T[a] - w;
+      if (!(W[a] > 0.0)) return fail(ECMC_EINVAL, "tile narrower than the joint");
+      if (!(W[a] + 2.0 * halo_te < 0.5 * c->L[a]))
         return fail(ECMC_EINVAL, "tile plus halo must be < L/2 (use more tiles)");
-      if (p.precision == ECMC_PREC_FP32F && !(W + 2.0 * halo_te <= 64.0 * sig))
+      if (p.precision == ECMC_PREC_FP32F && !(W[a] + 2.0 * halo_te <= 64.0 * sig))
         return fail(ECMC_EINVAL, "FP32 screen needs tiles of at most 64 sigma");
-      c->T[a] = T;
-      c->W[a] = W;
     }
     const double rho = (double)c->n / (c->L[0] * c->L[1] * c->L[2]);
-    const double E[3] = {c->W[0] + 2.0 * halo_te, c->W[1] + 2.0 * halo_te, c->W[2] + 2.0 * halo_te};
+    const double E[3] = {W[0] + 2.0 * halo_te, W[1] + 2.0 * halo_te, W[2] + 2.0 * halo_te};
     const bool derived = stage <= 0;
     if (derived) stage = stage_bound(E, rho);
-    mcap = stage_bound(c->W, rho);
+    mcap = stage_bound(W, rho);
     double Es[3];
-    staged_box(E, c->W, sig, Es);
-    if (derived) tight_caps(Es, c->W, rho, stage, mcap, &stage_t, &m_t, p.tight_factor > 0 ? p.tight_factor : 1.08);
+    staged_box(E, W, sig, Es);
+    if (derived) tight_caps(Es, W, rho, stage, mcap, &stage_t, &m_t, p.tight_factor > 0 ? p.tight_factor : 1.08);
   } else {
     if (p.precision == ECMC_PREC_FP32F)
       for (int a = 0; a < 3; ++a)
@@ -624,7 +625,7 @@ ecmc_status ecmc_configure(ecmc_ctx *c, const ecmc_opts *o) {
     const double side_min = (reach > bm ? reach : bm) + 2e-3 * sig;
     ncl = 1;
     for (int a = 0; a < 3; ++a) {
-      const double E = c->W[a] + 2.0 * hg;
+      const double E = W[a] + 2.0 * hg;
       const int g = (int)floor(E / side_min);
       ncl *= g < 1 ? 1 : g;
       e_max = E > e_max ? E : e_max;
@@ -646,16 +647,34 @@ ecmc_status ecmc_configure(ecmc_ctx *c, const ecmc_opts *o) {
       return fail(ECMC_EINVAL, "staging needs %lld bytes of shared memory (max %d)",
                   (long long)need, smem_max);
     if (screened) {
-      const double E[3] = {c->W[0] + 2.0 * halo_te, c->W[1] + 2.0 * halo_te, c->W[2] + 2.0 * halo_te};
+      const double E[3] = {W[0] + 2.0 * halo_te, W[1] + 2.0 * halo_te, W[2] + 2.0 * halo_te};
       const int32_t most = packing_bound(E, sig) + (p.k_spring > 0.0 ? 2 * mcap : 0);
       if (stage > most) stage = (most + 31) / 32 * 32;
     } else {
       mcap = stage;
     }
   }
+  const double side = p.cell_side > 0 ? p.cell_side : 1.05 * sig;
+  if (!(side >= sig)) return fail(ECMC_EINVAL, "cell side must be >= sigma");
+  if (p.k_spring > 0.0 && p.mode == ECMC_MODE_DOMAIN && !c->d_ftag) CU(dalloc(&c->d_ftag, c->n));
+  if (p.mode == ECMC_MODE_DOMAIN) {
+    const int64_t ntile = (int64_t)p.tiles[0] * p.tiles[1] * p.tiles[2];
+    if (ntile > c->deferred_cap) {
+      int32_t *list = nullptr;
+      CU(dalloc(&list, ntile));
+      cudaFree(c->d_deferred);
+      c->d_deferred = list;
+      c->deferred_cap = ntile;
+    }
+  }
+  TRY(set_grid(c, side));
   c->opts = p;
   c->s_cap = s_cap;
   c->w = w;
+  for (int a = 0; a < 3; ++a) {
+    c->T[a] = T[a];
+    c->W[a] = W[a];
+  }
   c->halo_hs = halo_hs;
   c->halo_te = halo_te;
   c->stage_cap = stage;
@@ -665,24 +684,11 @@ ecmc_status ecmc_configure(ecmc_ctx *c, const ecmc_opts *o) {
   c->lorg = (float)(-hg);
   c->e_max = e_max;
   c->ncl = ncl;
-  if (p.mode == ECMC_MODE_DOMAIN) {
-    const int64_t ntile = (int64_t)p.tiles[0] * p.tiles[1] * p.tiles[2];
-    if (ntile > c->deferred_cap) {
-      cudaFree(c->d_deferred);
-      c->d_deferred = nullptr;
-      c->deferred_cap = 0;
-      CU(dalloc(&c->d_deferred, ntile));
-      c->deferred_cap = ntile;
-    }
-  }
   c->lanes = lanes;
   c->event_cap = p.event_cap > 0 ? p.event_cap : 10000000;
   c->ecs_per_tile = p.ecs_per_tile > 0 ? p.ecs_per_tile : 1;
   c->configured = true;
-  if (p.k_spring > 0.0 && p.mode == ECMC_MODE_DOMAIN && !c->d_ftag) CU(dalloc(&c->d_ftag, c->n));
-  const double side = p.cell_side > 0 ? p.cell_side : 1.05 * sig;
-  if (!(side >= sig)) return fail(ECMC_EINVAL, "cell side must be >= sigma");
-  return set_grid(c, side);
+  return ECMC_OK;
 }
 
 ecmc_status ecmc_log_reserve(ecmc_ctx *c, int64_t cap) {

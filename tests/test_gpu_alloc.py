@@ -65,3 +65,23 @@ def test_structure_scratch_half_allocated(monkeypatch):
     got, r2n, hist = ctx.structure(dR=0.5, nbins=8)
     ref, r2n0, hist0 = gpu_context(m, precision=ecmc.PREC_FP32F, lanes=8).structure(dR=0.5, nbins=8)
     assert got == ref and (r2n == r2n0).all() and (hist == hist0).all()
+
+
+@pytest.mark.parametrize("kw,limit,code", [
+    (dict(tiles=(4, 4, 2)), 0, -1),                      # the third axis is refused after two others
+    (dict(tiles=(4, 4, 4), cell_side=0.5), 0, -1),
+    (dict(tiles=(3, 4, 5), ecs_per_tile=2, block_tiles=3), 0, -1),
+    (dict(tiles=(5, 5, 5)), 4 * 125 - 1, ENOMEM),        # the list of tiles for a second pass
+    (dict(k_spring=30.0), 4 * 4096 - 1, ENOMEM),         # the springs' tags by bead
+    (dict(tiles=(4, 4, 4), cell_side=1.5), 4 * 11 ** 3, ENOMEM),
+])
+def test_refused_settings_leave_those_in_force(kw, limit, code, monkeypatch):
+    m = small_domain()
+    ctx, o = gpu_context(m, precision=ecmc.PREC_FP32F, lanes=8), oracle_system(m)
+    assert_runs_as_oracle(ctx, m, o, 1)
+    with monkeypatch.context() as env:
+        env.setenv("ECMC_ALLOC_LIMIT", str(limit))
+        with pytest.raises(ecmc.EcmcError) as e:
+            ctx.configure(**settings(m, **kw))
+    assert e.value.code == code
+    assert_runs_as_oracle(ctx, m, o, 2, sweep0=1)
