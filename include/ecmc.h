@@ -407,7 +407,8 @@ ecmc_status ecmc_batch_create(const ecmc_replica_spec *specs, int32_t n,
                               double jitter, uint64_t seed, ecmc_batch **out);
 void ecmc_batch_destroy(ecmc_batch *b);
 /* opts as for ecmc_configure, domain mode only; tiles[0] <= 0 -> per
- * replica tiles from opts.tile_side; lanes 4, 8, 16 or 32 (0 -> 8). */
+ * replica tiles from opts.tile_side; lanes 4, 8, 16 or 32 (0 -> 8).  A
+ * refused call leaves the settings in force as they were. */
 ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *opts);
 /* n_sweeps sweeps of every replica; use_graph = 1 captures one sweep in a
  * CUDA graph (after one uncaptured sweep) and replays it. */

@@ -34,7 +34,9 @@ cudaError_t balloc(T **p, size_t count) {
   *p = nullptr;
   if (count == 0) count = 1;
   if (alloc_refused(sizeof(T) * count)) return cudaErrorMemoryAllocation;
-  return cudaMalloc((void **)p, sizeof(T) * count);
+  const cudaError_t e = cudaMalloc((void **)p, sizeof(T) * count);
+  if (e != cudaSuccess) (void)cudaGetLastError();  // (a launch check after it would report it again)
+  return e;
 }
 }  // namespace
 
@@ -99,6 +101,47 @@ void batch_free(ecmc_batch *b) {
   if (b->ev1) cudaEventDestroy(b->ev1);
   if (b->stream) cudaStreamDestroy(b->stream);
   delete b;
+}
+
+void drop_graph(ecmc_batch *b) {
+  if (b->graph) cudaGraphExecDestroy(b->graph);
+  b->graph = nullptr;
+}
+
+// the concatenated cell arrays for `ncell` cells, all of them or none; the
+// graph holds the old ones
+ecmc_status batch_cells(ecmc_batch *b, int64_t ncell) {
+  if (ncell == b->ncell_total) return ECMC_OK;
+  drop_graph(b);
+  cudaFree(b->d_count);
+  cudaFree(b->d_start);
+  cudaFree(b->d_bsum);
+  b->d_count = b->d_start = b->d_bsum = nullptr;
+  b->ncell_total = 0;
+  int32_t *count = nullptr, *start = nullptr, *bsum = nullptr;
+  cudaError_t e = balloc(&count, ncell);
+  if (e == cudaSuccess) e = balloc(&start, ncell + 1);
+  if (e == cudaSuccess) e = balloc(&bsum, cells_scratch_ints(ncell));
+  // (zero between passes: each pass clears the counts it has read)
+  if (e == cudaSuccess) e = cudaMemsetAsync(count, 0, sizeof(int32_t) * ncell, b->stream);
+  if (e != cudaSuccess) {
+    cudaFree(count);
+    cudaFree(start);
+    cudaFree(bsum);
+    return bfail(e == cudaErrorMemoryAllocation ? ECMC_ENOMEM : ECMC_ECUDA,
+                 std::string("cell arrays: ") + cudaGetErrorString(e));
+  }
+  b->d_count = count;
+  b->d_start = start;
+  b->d_bsum = bsum;
+  b->ncell_total = ncell;
+  return ECMC_OK;
+}
+
+// cells of the configured replicas
+int64_t batch_ncell(const ecmc_batch *b) {
+  const RepParams &R = b->reps.back();
+  return R.cell_off + (int64_t)R.nc[0] * R.nc[1] * R.nc[2];
 }
 
 ecmc_status batch_status(ecmc_batch *b) {
@@ -402,18 +445,21 @@ ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *o) {
   if (p.precision != ECMC_PREC_FP32F) mcap = stage;
   else if (stage > most) stage = (most + 31) / 32 * 32;
   if (mcap > stage) mcap = stage;
-  // (re)allocate the concatenated cell arrays
-  if (cell_off != b->ncell_total) {
-    cudaFree(b->d_count);
-    cudaFree(b->d_start);
-    cudaFree(b->d_bsum);
-    b->d_count = b->d_start = b->d_bsum = nullptr;
-    BCU(balloc(&b->d_count, cell_off));
-    BCU(cudaMemsetAsync(b->d_count, 0, sizeof(int32_t) * cell_off, b->stream));
-    BCU(balloc(&b->d_start, cell_off + 1));
-    BCU(balloc(&b->d_bsum, cells_scratch_ints(cell_off)));
-    b->ncell_total = cell_off;
+  // What is needed is allocated before anything of the settings in force
+  // changes (the cell arrays of those settings come back with the next run
+  // when there is no memory for the new ones).
+  if (unit_off > b->deferred_cap) {
+    int32_t *list = nullptr;
+    BCU(balloc(&list, unit_off));
+    drop_graph(b);
+    cudaFree(b->d_deferred);
+    b->d_deferred = list;
+    b->deferred_cap = unit_off;
   }
+  const ecmc_status cs = batch_cells(b, cell_off);
+  if (cs != ECMC_OK) return cs;
+  drop_graph(b);
+  b->configured = false;
   b->reps = reps;
   BCU(cudaMemcpyAsync(b->d_reps, b->reps.data(), sizeof(RepParams) * b->R, cudaMemcpyHostToDevice,
                       b->stream));
@@ -428,13 +474,6 @@ ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *o) {
   b->m_cap = mcap;
   b->stage_tight = stage_t;
   b->m_tight = m_t;
-  if (unit_off > b->deferred_cap) {
-    cudaFree(b->d_deferred);
-    b->d_deferred = nullptr;
-    b->deferred_cap = 0;
-    BCU(balloc(&b->d_deferred, unit_off));
-    b->deferred_cap = unit_off;
-  }
   b->lorg = (float)(-hg);
   b->e_max = e_max;
   b->lanes = lanes;
@@ -442,10 +481,6 @@ ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *o) {
   b->event_cap = p.event_cap > 0 ? p.event_cap : 10000000;
   b->units_total = unit_off;
   b->configured = true;
-  if (b->graph) {
-    cudaGraphExecDestroy(b->graph);
-    b->graph = nullptr;
-  }
   return ECMC_OK;
 }
 
@@ -454,6 +489,8 @@ ecmc_status ecmc_batch_run(ecmc_batch *b, double ell, uint64_t seed, int64_t n_s
   if (!b) return bfail(ECMC_EINVAL, "batch is NULL");
   if (!b->configured) return bfail(ECMC_EINVAL, "call ecmc_batch_configure first");
   if (!(ell >= 0.0) || !isfinite(ell) || n_sweeps < 0) return bfail(ECMC_EINVAL, "bad ell or n_sweeps");
+  const ecmc_status cs = batch_cells(b, batch_ncell(b));
+  if (cs != ECMC_OK) return cs;
   const bool rec = b->opts.record != 0;
   ECParams P = batch_params(b, seed, ell);
   if (rec) {
@@ -465,7 +502,7 @@ ecmc_status ecmc_batch_run(ecmc_batch *b, double ell, uint64_t seed, int64_t n_s
       b->d_rdig = nullptr;
       b->d_rlift = nullptr;
       b->d_rev = nullptr;
-      b->rec_cap = 0;
+      b->rec_cap = b->rec_n = 0;
       BCU(balloc(&b->d_rdig, units));
       BCU(balloc(&b->d_rlift, units));
       BCU(balloc(&b->d_rev, units));
@@ -489,10 +526,7 @@ ecmc_status ecmc_batch_run(ecmc_batch *b, double ell, uint64_t seed, int64_t n_s
                        b->graph_rec != rec;
     int64_t done = 0;
     if (fresh) {
-      if (b->graph) {
-        cudaGraphExecDestroy(b->graph);
-        b->graph = nullptr;
-      }
+      drop_graph(b);
       // first sweep uncaptured: kernel attributes and block sizes are
       // settled outside the capture
       BCU(batch_sweep(b, P, seed));

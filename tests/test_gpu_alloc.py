@@ -85,3 +85,37 @@ def test_refused_settings_leave_those_in_force(kw, limit, code, monkeypatch):
             ctx.configure(**settings(m, **kw))
     assert e.value.code == code
     assert_runs_as_oracle(ctx, m, o, 2, sweep0=1)
+
+
+BATCH = [dict(dims=(12, 12, 12), spacing=1.05, N=8), dict(dims=(10, 12, 14), spacing=1.12, N=10)]
+SEED = 0xEC0B21
+
+
+def batch_cells(side):
+    return sum(int(np.prod([int(d * s["spacing"] / side) for d in s["dims"]])) for s in BATCH)
+
+
+@pytest.mark.parametrize("kw,limit,code", [
+    (dict(cell_side=1.5), 4 * batch_cells(1.5), ENOMEM),  # the counts fit, the starts do not
+    (dict(tile_side=3.0), 4 * 124 - 1, ENOMEM),           # 4 x 4 x 4 + 3 x 4 x 5 tiles: the second pass's list
+    (dict(request_cap=9, tile_side=3.0), 0, -1),
+])
+def test_refused_batch_settings_leave_those_in_force(kw, limit, code, monkeypatch):
+    """A sweep captured before the refused call and replays after it, against
+    a batch that never saw it."""
+    out = []
+    for refuse in (True, False):
+        b = ecmc.Batch(BATCH, jitter=0.01, seed=SEED)
+        b.configure(dir_mode=ecmc.DIR_ISO, precision=ecmc.PREC_FP32F, lanes=8)
+        b.run(3.0, seed=SEED, n_sweeps=2, graph=True)
+        if refuse:
+            with monkeypatch.context() as env:
+                env.setenv("ECMC_ALLOC_LIMIT", str(limit))
+                with pytest.raises(ecmc.EcmcError) as e:
+                    b.configure(dir_mode=ecmc.DIR_ISO, precision=ecmc.PREC_FP32F, lanes=8, **kw)
+            assert e.value.code == code
+        b.run(3.0, seed=SEED, n_sweeps=3, graph=True)
+        out.append([b.get_positions(r) for r in range(len(BATCH))] + [b.stats()["events_total"]])
+    for (r, img), (r0, img0) in zip(out[0][:-1], out[1][:-1]):
+        assert (r == r0).all() and (img == img0).all()
+    assert out[0][-1] == out[1][-1]
