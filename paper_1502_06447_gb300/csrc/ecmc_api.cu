@@ -658,6 +658,7 @@ ecmc_status ecmc_configure(ecmc_ctx *c, const ecmc_opts *o) {
   if (!(side >= sig)) return fail(ECMC_EINVAL, "cell side must be >= sigma");
   if (p.k_spring > 0.0 && p.mode == ECMC_MODE_DOMAIN && !c->d_ftag) CU(dalloc(&c->d_ftag, c->n));
   if (p.mode == ECMC_MODE_DOMAIN) {
+    if (!((double)p.tiles[0] * p.tiles[1] * p.tiles[2] <= 2147483647.0)) return fail(ECMC_EINVAL, "too many tiles");
     const int64_t ntile = (int64_t)p.tiles[0] * p.tiles[1] * p.tiles[2];
     if (ntile > c->deferred_cap) {
       int32_t *list = nullptr;

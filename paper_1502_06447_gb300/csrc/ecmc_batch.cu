@@ -260,6 +260,9 @@ ecmc_status ecmc_batch_create(const ecmc_replica_spec *specs, int32_t n, double 
       return bfail(ECMC_EINVAL, "all replicas need the same sigma and b_max");
     if (sp.dims[0] < 1 || sp.dims[1] < 1 || sp.dims[2] < 1 || sp.N < 1)
       return bfail(ECMC_EINVAL, "replica " + std::to_string(r) + ": bad dims or N");
+    // (staging keeps three flags beside an id)
+    if (!((double)sp.dims[0] * sp.dims[1] * sp.dims[2] < (double)(1ll << 29)))
+      return bfail(ECMC_EINVAL, "replica " + std::to_string(r) + ": at most 2^29 beads");
     const int64_t nb = (int64_t)sp.dims[0] * sp.dims[1] * sp.dims[2];
     if (nb % sp.N) return bfail(ECMC_EINVAL, "replica " + std::to_string(r) + ": N must divide the sites");
     if (!(sp.spacing >= sigma) || (sp.N > 1 && !(sp.spacing <= b_max)))
@@ -374,7 +377,7 @@ ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *o) {
     for (int a = 0; a < 3; ++a) {
       if (!(s_cap + sig + margin < R.half[a]))
         return bfail(ECMC_EINVAL, "replica " + std::to_string(r) + ": need s_cap + sigma < L/2");
-      int D = p.tiles[a] > 0 ? p.tiles[a] : (int)floor(R.L[a] / tside);
+      int D = p.tiles[a] > 0 ? p.tiles[a] : (int)fmin(floor(R.L[a] / tside), 2147483647.0);
       if (D < 3) D = 3;
       // the tile plus its halo must stay below half the box
       while (D < 1024 && !(R.L[a] / D - w + 2.0 * halo_te < R.half[a])) ++D;
@@ -388,7 +391,13 @@ ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *o) {
       R.W[a] = W;
       R.Lf[a] = (float)R.L[a];
       R.Wf[a] = (float)W;
-      int k = (int)floor(R.L[a] / side);
+      // (bounded in double before the casts; tiles and cells of all replicas
+      // together stay below 2^31)
+      const double kd = floor(R.L[a] / side);
+      if (!((double)cell_off + (double)nce * kd <= 2147483647.0))
+        return bfail(ECMC_EINVAL, "replica " + std::to_string(r) + ": cell grid too fine");
+      if (!((double)unit_off + (double)nt * D <= 2147483647.0)) return bfail(ECMC_EINVAL, "too many tiles");
+      const int k = (int)kd;
       if (k < 3) return bfail(ECMC_EINVAL, "replica " + std::to_string(r) + ": box too small");
       R.nc[a] = k;
       R.cs[a] = R.L[a] / k;
@@ -426,7 +435,6 @@ ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *o) {
   if (m_t > stage_t) m_t = stage_t;
   if (mcap > stage) mcap = stage;
   if (stage > 65534) return bfail(ECMC_EINVAL, "at most 65534 staged beads per tile");
-  if (unit_off >= (1ll << 31)) return bfail(ECMC_EINVAL, "too many tiles");
   int dev = 0, smem_max = 0;
   BCU(cudaGetDevice(&dev));
   BCU(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
