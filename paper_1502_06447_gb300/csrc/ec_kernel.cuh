@@ -764,7 +764,11 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
           double x = div_rn((posv(va) ? SYS(W)[axc] : 0.0) - loc, va);
           if (neg(x)) x = 0.0;
           if (F32) ++confirmed;
-          keep(x, (KIND_WALL << 28) | ax, 0.0, 0.0);
+          // A bead on its tile's lower wall, moving out, meets it after
+          // -0.0: bits that order above every candidate.  It competes as 0;
+          // d.v, which a wall does not have, keeps the zero's sign for the
+          // records.
+          keep(nonzero(x) ? x : 0.0, (KIND_WALL << 28) | ax, x, 0.0);
         }
         __syncwarp();
       }
@@ -959,6 +963,7 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
       if (G < 8) ev_hi += out >= 4 && gl == (out & 3) ? 1u : 0u;
       __syncwarp(gmask);
       shadows(qa, pf0, pf1, pf2);
+      if (kind == KIND_WALL) x = best.dv;
       if (P.rec_digest) {
         fnv_mix(h, (uint64_t)pid);
         fnv_mix(h, ((uint64_t)(uint32_t)out << 32) | (uint64_t)(uint32_t)partner);
