@@ -22,6 +22,11 @@ namespace {
 constexpr int SCAN_BLOCK = 1024;
 constexpr int SCAN_ITEMS = 4;  // elements per thread
 constexpr int SCAN_TILE = SCAN_BLOCK * SCAN_ITEMS;
+// A call of ecmc_observables on 4,096 beads (GB300) whose blocks add the sums
+// up / with k_scan_sums: 4,242 tiles 150 / 152 us, 16,950 447 / 459, 33,934
+// 840 / 850, 68,607 1,753 / 1,647, 271,469 10,850 / 6,313, 442,234 24,038 /
+// 10,249.
+constexpr int64_t SCAN_DIRECT = 32768;
 
 // Cell and tile of one coordinate.  FP32 decides both unless the coordinate
 // lies within its error (C.tol) of a boundary; those few take the FP64
@@ -147,21 +152,53 @@ __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_tiles(int *in, int64_t n, i
   if (threadIdx.x == 0) block_sums[blockIdx.x] = total;
 }
 
-// adds to every tile of SCAN_TILE starts the sums of the tiles before it
-// (each block adds those up itself: a few hundred at most)
-__global__ void __launch_bounds__(256) k_scan_add(int *out, int64_t n, const int *sums, int64_t tiles) {
+// adds to every tile of SCAN_TILE starts the sums of the tiles before it:
+// each block adds those up itself, or, of more than SCAN_DIRECT tiles (what
+// the blocks read grows with their square), takes the one that k_scan_sums left
+__global__ void __launch_bounds__(256) k_scan_add(int *out, int64_t n, const int *sums, int64_t tiles, bool summed) {
   __shared__ int sh[8];
-  int part = 0;
-  for (int64_t i = threadIdx.x; i < blockIdx.x; i += 256) part += sums[i];
-  part = __reduce_add_sync(0xffffffffu, part);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = part;
-  __syncthreads();
   int before = 0;
+  if (summed) {
+    before = sums[blockIdx.x];
+  } else {
+    int part = 0;
+    for (int64_t i = threadIdx.x; i < blockIdx.x; i += 256) part += sums[i];
+    part = __reduce_add_sync(0xffffffffu, part);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = part;
+    __syncthreads();
 #pragma unroll
-  for (int i = 0; i < 8; ++i) before += sh[i];
+    for (int i = 0; i < 8; ++i) before += sh[i];
+    if (blockIdx.x == tiles - 1 && threadIdx.x == 0) out[n] = before + sums[tiles - 1];
+  }
   const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
   for (int64_t i = base + threadIdx.x; i < base + SCAN_TILE && i < n; i += 256) out[i] += before;
-  if (blockIdx.x == tiles - 1 && threadIdx.x == 0) out[n] = before + sums[tiles - 1];
+}
+
+// exclusive scan of the tile sums in place, and the total (one block)
+__global__ void __launch_bounds__(SCAN_BLOCK) k_scan_sums(int *sums, int64_t tiles, int *total) {
+  __shared__ int sh[33];
+  int carry = 0;
+  for (int64_t t0 = 0; t0 < tiles; t0 += SCAN_TILE) {
+    const int64_t base = t0 + (int64_t)threadIdx.x * SCAN_ITEMS;
+    int v[SCAN_ITEMS];
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) v[i] = base + i < tiles ? sums[base + i] : 0;
+    const int chunk = block_scan(v, sh);
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i)
+      if (base + i < tiles) sums[base + i] = v[i] + carry;
+    carry += chunk;
+  }
+  if (threadIdx.x == 0) *total = carry;
+}
+
+// counts -> starts (ncell + 1), the counts cleared
+void launch_scan(int *count, int64_t ncell, int *start, int *sums, cudaStream_t s) {
+  const int64_t tiles = (ncell + SCAN_TILE - 1) / SCAN_TILE;
+  const bool summed = tiles > SCAN_DIRECT;
+  k_scan_tiles<<<(unsigned)tiles, SCAN_BLOCK, 0, s>>>(count, ncell, start, sums);
+  if (summed) k_scan_sums<<<1, SCAN_BLOCK, 0, s>>>(sums, tiles, start + ncell);
+  k_scan_add<<<(unsigned)tiles, 256, 0, s>>>(start, ncell, sums, tiles, summed);
 }
 
 // Tag of a joint bead in cell order: whose tile its bonded beads are motile
@@ -303,9 +340,7 @@ cudaError_t launch_cells_batch(const CellBatch &C, int64_t ncell, cudaStream_t s
   const int T = 256;
   const int64_t nb = (C.n + T - 1) / T;
   if (C.n > 0) k_tag_count_b<<<(unsigned)nb, T, 0, s>>>(C);
-  const int64_t tiles = (ncell + SCAN_TILE - 1) / SCAN_TILE;
-  k_scan_tiles<<<(unsigned)tiles, SCAN_BLOCK, 0, s>>>(C.count, ncell, C.start, C.block_sums);
-  k_scan_add<<<(unsigned)tiles, 256, 0, s>>>(C.start, ncell, C.block_sums, tiles);
+  launch_scan(C.count, ncell, C.start, C.block_sums, s);
   if (C.n > 0) k_scatter_b<<<(unsigned)nb, T, 0, s>>>(C);
   return cudaGetLastError();
 }
@@ -341,9 +376,7 @@ cudaError_t launch_cells(const CellParams &C0, int64_t ncell, cudaStream_t s) {
   const int T = 256;
   const int64_t nb = (C.n + T - 1) / T;
   if (C.n > 0) k_tag_count<<<(unsigned)nb, T, 0, s>>>(C);
-  const int64_t tiles = (ncell + SCAN_TILE - 1) / SCAN_TILE;
-  k_scan_tiles<<<(unsigned)tiles, SCAN_BLOCK, 0, s>>>(C.count, ncell, C.start, C.block_sums);
-  k_scan_add<<<(unsigned)tiles, 256, 0, s>>>(C.start, ncell, C.block_sums, tiles);
+  launch_scan(C.count, ncell, C.start, C.block_sums, s);
   if (C.n > 0) k_scatter<<<(unsigned)nb, T, 0, s>>>(C);
   return cudaGetLastError();
 }
