@@ -90,7 +90,11 @@ typedef struct ecmc_opts {
   int64_t event_cap;     /* events per EC before ECMC_ESTUCK; 0 -> 10^7 */
   double p_swap;         /* swap proposal probability at a motile contact */
   int32_t ecs_per_tile;  /* ECs per tile per sweep (domain); 0 -> 1 */
-  int32_t lanes;         /* lanes per EC: 32, 16, 8 or 4; 0 -> 32 */
+  int32_t lanes;         /* lanes per EC: 32, 16, 8 or 4; 0 -> 32.  At least:
+                            where all tiles stay resident with twice as many
+                            (12 warps per SM: 1,824 tiles of 32 lanes, 3,648
+                            of 16 or 7,296 of 8 on 152 SMs) they get them,
+                            unless block_tiles is given.  Same events. */
   int32_t record;        /* 1: keep per-EC digests / lift sums of the last run */
   int32_t stage_cap;     /* staged beads per tile; 0 -> derived from the tile size */
   double cell_side;      /* side of the global cell grid (domain); 0 -> 1.05 sigma */
@@ -443,7 +447,7 @@ ecmc_status ecmc_batch_records(ecmc_batch *b, uint64_t *digest, double *lift,
  * winner's tiles).  Needs a configured domain-mode context; keeps its mode,
  * direction rule, precision, p_swap, joint, s_cap and record setting. */
 typedef struct ecmc_tuning {
-  int32_t lanes;          /* lanes per EC */
+  int32_t lanes;          /* lanes per EC that the winner ran with */
   double tile_side;       /* target tile side (sigma) */
   double cell_side;       /* global cell side (sigma) */
   int32_t ecs_per_tile;

@@ -1570,7 +1570,11 @@ ecmc_status ecmc_autotune(ecmc_ctx *c, double ell, uint64_t seed, int32_t trial_
   TunePoint best{};
   TuneScore best_s{};
   int n = 0;
-  ecmc_status st = tune_search(start, trial, &best, &best_s, &n);
+  auto ran = [&](const TunePoint &pt) {
+    const ecmc_opts o = point_opts(pt);
+    return tile_lanes((int64_t)o.tiles[0] * o.tiles[1] * o.tiles[2], pt.lanes, o.block_tiles);
+  };
+  ecmc_status st = tune_search(start, trial, &best, &best_s, &n, ran);
   if (st != ECMC_OK) {
     const std::string why = g_err;
     ecmc_configure(c, &base);

@@ -138,6 +138,15 @@ ecmc_status batch_cells(ecmc_batch *b, int64_t ncell) {
   return ECMC_OK;
 }
 
+// tiles of side `side` along an axis of length L with a joint of width w: at
+// least 3, the tile plus its halo below half the box
+int tiles_on_axis(double L, double side, double w, double halo_te, int D) {
+  if (D <= 0) D = (int)fmin(floor(L / side), 2147483647.0);
+  if (D < 3) D = 3;
+  while (D < 1024 && !(L / D - w + 2.0 * halo_te < 0.5 * L)) ++D;
+  return D;
+}
+
 // cells of the configured replicas
 int64_t batch_ncell(const ecmc_batch *b) {
   const RepParams &R = b->reps.back();
@@ -377,10 +386,7 @@ ecmc_status ecmc_batch_configure(ecmc_batch *b, const ecmc_opts *o) {
     for (int a = 0; a < 3; ++a) {
       if (!(s_cap + sig + margin < R.half[a]))
         return bfail(ECMC_EINVAL, "replica " + std::to_string(r) + ": need s_cap + sigma < L/2");
-      int D = p.tiles[a] > 0 ? p.tiles[a] : (int)fmin(floor(R.L[a] / tside), 2147483647.0);
-      if (D < 3) D = 3;
-      // the tile plus its halo must stay below half the box
-      while (D < 1024 && !(R.L[a] / D - w + 2.0 * halo_te < R.half[a])) ++D;
+      const int D = tiles_on_axis(R.L[a], tside, w, halo_te, p.tiles[a]);
       const double T = R.L[a] / D, W = T - w;
       if (!(W > 0.0))
         return bfail(ECMC_EINVAL, "replica " + std::to_string(r) + ": tile narrower than the joint");
@@ -707,7 +713,19 @@ ecmc_status ecmc_batch_autotune(ecmc_batch *b, double ell, uint64_t seed, int32_
   TunePoint best{};
   TuneScore best_s{};
   int n = 0;
-  ecmc_status st = tune_search(start, trial, &best, &best_s, &n);
+  const double w = base.joint > 0 ? base.joint : b->b_max;
+  const double halo_te = (b->b_max > sig ? b->b_max : sig) * (1.0 + 1e-6);
+  auto ran = [&](const TunePoint &pt) {
+    const ecmc_opts o = point_opts(pt);
+    int64_t units = 0;
+    for (const RepParams &R : b->reps) {
+      int64_t nt = 1;
+      for (int a = 0; a < 3; ++a) nt *= tiles_on_axis(R.L[a], o.tile_side, w, halo_te, 0);
+      units += nt;
+    }
+    return tile_lanes(units, pt.lanes, o.block_tiles);
+  };
+  ecmc_status st = tune_search(start, trial, &best, &best_s, &n, ran);
   if (st != ECMC_OK) {
     ecmc_batch_configure(b, &base);
     restore();

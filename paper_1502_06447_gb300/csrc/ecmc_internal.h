@@ -172,9 +172,10 @@ cudaError_t launch_ec_spring_fp64(const ECParams &P, int lanes, cudaStream_t s);
 cudaError_t launch_ec_pushoff_tether(const ECParams &P, int lanes, cudaStream_t s);
 cudaError_t launch_ec_pushoff_spring(const ECParams &P, int lanes, cudaStream_t s);
 
-// pick_lanes (k_ec.cu): tiles get twice the lanes as long as all of them then stay resident, at
-// most this many warps per SM (what the EC kernel's registers allow).  A
-// group steps faster with more lanes and with fewer groups in its warp; a
+// Lanes a tile runs with when `lanes` are asked for (the events do not depend
+// on it): tiles get twice the lanes as long as all of them then stay resident,
+// at most EC_SPREAD_WARPS warps per SM (what the EC kernel's registers allow).
+// A caller who fixes the block's tiles keeps the lanes too.  A group steps faster with more lanes and with fewer groups in its warp; a
 // second round of tiles costs more than that.  ms per sweep (two ECs per tile
 // of 4.2 sigma, GB300, screened / FP64) with 8, 16, 32 lanes: 1,331 tiles
 // 2.93, 2.71, 2.35 / 3.66, 2.85, 2.33; 1,728 tiles (11.4 warps per SM at 32)
@@ -182,6 +183,13 @@ cudaError_t launch_ec_pushoff_spring(const ECParams &P, int lanes, cudaStream_t 
 // 3.67, 2.92, 3.08; 3,375 (11.1 at 16) 2.97, 2.78, 3.52 / 3.60, 3.30, 3.44;
 // 4,096 (13.5 at 16) 3.61, 4.15, 4.85 / 5.28, 4.44, 4.71.
 constexpr int EC_SPREAD_WARPS = 12;
+inline int spread_lanes(int64_t n_units, int lanes, int block_tiles, int sms) {
+  if (block_tiles > 0) return lanes;
+  while (lanes < 32 && n_units * (2 * lanes) <= (int64_t)EC_SPREAD_WARPS * 32 * sms) lanes *= 2;
+  return lanes;
+}
+// the same for the current device (k_ec.cu)
+int tile_lanes(int64_t n_units, int lanes, int block_tiles);
 
 // cell list and domain tags (k_cells.cu)
 struct CellParams {
@@ -420,9 +428,11 @@ struct TuneScore {
 
 // trial(point, &score) -> ECMC_OK (scored), ECMC_EINVAL (point not
 // admissible for this system: skipped) or another status (abort).
-template <class Trial>
+// ran(point) -> the lanes the point runs with: points that differ in the lanes
+// asked for alone are one point, timed and returned under those.
+template <class Trial, class Ran>
 ecmc_status tune_search(TunePoint start, Trial trial, TunePoint *best, TuneScore *best_score,
-                        int *n_trials) {
+                        int *n_trials, Ran ran) {
   static const int lanes_c[] = {4, 8, 16, 32};
   static const double tile_c[] = {3.4, 3.8, 4.2, 4.6, 5.0, 6.0, 7.0};
   static const double cell_c[] = {1.05, 1.4};
@@ -430,6 +440,7 @@ ecmc_status tune_search(TunePoint start, Trial trial, TunePoint *best, TuneScore
   static const int warps_c[] = {1, 2, 4};
   static const double tight_c[] = {1.0, 1.08, 1.16};
   TunePoint cur = start;
+  cur.lanes = ran(start);
   TuneScore cur_s{};
   bool have = false;
   int n = 0;
@@ -437,7 +448,8 @@ ecmc_status tune_search(TunePoint start, Trial trial, TunePoint *best, TuneScore
   constexpr int VMAX = 128;
   TunePoint seen[VMAX];
   int nseen = 0;
-  auto consider = [&](const TunePoint &pt) -> ecmc_status {
+  auto consider = [&](TunePoint pt) -> ecmc_status {
+    pt.lanes = ran(pt);
     for (int i = 0; i < nseen; ++i)
       if (seen[i].lanes == pt.lanes && seen[i].tile_side == pt.tile_side &&
           seen[i].cell_side == pt.cell_side && seen[i].ecs == pt.ecs && seen[i].warps == pt.warps &&
@@ -487,6 +499,11 @@ ecmc_status tune_search(TunePoint start, Trial trial, TunePoint *best, TuneScore
   *best_score = cur_s;
   *n_trials = n;
   return ECMC_OK;
+}
+template <class Trial>
+ecmc_status tune_search(TunePoint start, Trial trial, TunePoint *best, TuneScore *best_score,
+                        int *n_trials) {
+  return tune_search(start, trial, best, best_score, n_trials, [](const TunePoint &pt) { return pt.lanes; });
 }
 
 }  // namespace ecmc

@@ -4,22 +4,13 @@
 
 namespace ecmc {
 
-namespace {
-// Lanes per tile.  `lanes` is what the caller asks for (the events do not
-// depend on it); when the tiles would leave warp schedulers without a warp,
-// each tile gets more lanes: its steps get shorter and the FP64 instructions
-// it does not share cost nothing that is missed.  A caller who fixes the
-// block's tiles keeps the lanes too.
-int pick_lanes(const ECParams &P, int lanes) {
-  if (P.block_tiles > 0) return lanes;
+int tile_lanes(int64_t n_units, int lanes, int block_tiles) {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return lanes;
-  while (lanes < 32 && (long long)P.n_units * (2 * lanes) <= (long long)EC_SPREAD_WARPS * 32 * sms) lanes *= 2;
-  return lanes;
+  return spread_lanes(n_units, lanes, block_tiles, sms);
 }
-}  // namespace
 
 cudaError_t launch_ec(const ECParams &P, int lanes, int fp32f, int pushoff, cudaStream_t s) {
   const bool spring = P.k_spring > 0.0;
@@ -33,7 +24,7 @@ cudaError_t launch_ec(const ECParams &P, int lanes, int fp32f, int pushoff, cuda
   cudaError_t e = cudaErrorInvalidValue;
   // (a tile whose staging does not fit a block 32 / lanes times runs with
   // more lanes)
-  for (int g = pick_lanes(P, lanes); g <= 32 && e == cudaErrorInvalidValue; g *= 2) {
+  for (int g = tile_lanes(P.n_units, lanes, P.block_tiles); g <= 32 && e == cudaErrorInvalidValue; g *= 2) {
     if (P.reps) e = fp32f ? launch_ec_batch_screened(P, g, s) : launch_ec_batch_fp64(P, g, s);
     else if (pushoff) e = spring ? launch_ec_pushoff_spring(P, g, s) : launch_ec_pushoff_tether(P, g, s);
     else if (spring) e = fp32f ? launch_ec_spring_screened(P, g, s) : launch_ec_spring_fp64(P, g, s);
