@@ -1064,6 +1064,13 @@ inline SlabPick pick_slabs(double e_max, double sigma, int S, int G, size_t budg
   }
 }
 
+// the staging capacity, at most S and at least M, that fits `room` bytes with
+// the fewest slabs
+inline int fit_stage(int S, int M, int G, size_t room) {
+  while (S - 32 >= M && group_bytes(S, 0, M, mask_quads(S, G, 10)) > room) S -= 32;
+  return S;
+}
+
 template <int G, bool F32, bool BATCH, bool DOM, bool SPRING, bool PO>
 cudaError_t launch_ec_t(const ECParams &P0, cudaStream_t s) {
   auto kern = ec_kernel<G, F32, BATCH, DOM, SPRING, PO>;
@@ -1092,6 +1099,10 @@ cudaError_t launch_ec_t(const ECParams &P0, cudaStream_t s) {
     const int step = 32 / G;
     const size_t room = (size_t)smem_max / step;  // one warp's tiles must fit a block
     SlabPick k{};
+    // (the capacity counts every bead of the tether halo, with long tethers
+    // many times what is staged: where even one tile of it would not fit, the
+    // tile takes what fits)
+    if (DOM && G == 32) S = fit_stage(S, M, G, room);
     if (DOM) {
       k = pick_slabs(P.e_max, P.s_len, S, G, (size_t)(G <= 8 ? 2048 : 192 * G));
       if (group_bytes(S, 0, M, mask_quads(S, G, k.nsl)) > room)
