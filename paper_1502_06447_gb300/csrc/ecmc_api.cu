@@ -787,14 +787,12 @@ static ECParams ec_params(const ecmc_ctx *c, uint64_t seed, double ell) {
                                                                          : 1e-3 * c->sigma * c->sigma;
     P.eps_v = (float)ev;
     P.eps_d = (float)ed;
-    P.eps_x = (float)ev;
   }
   P.lorg = c->lorg;
   P.e_max = c->e_max;
   P.s_len = c->sigma;
   P.r = c->d_r;
   P.img = c->d_img;
-  P.cr = c->d_cr;
   P.crf = c->d_crf;
   P.rf = c->d_rf;
   P.cid = c->d_cid;

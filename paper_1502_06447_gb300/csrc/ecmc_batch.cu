@@ -60,7 +60,6 @@ struct ecmc_batch {
   int32_t *d_img = nullptr, *d_rep_of = nullptr, *d_tag = nullptr, *d_cell = nullptr,
           *d_rank = nullptr, *d_count = nullptr, *d_start = nullptr, *d_bsum = nullptr,
           *d_cid = nullptr, *d_ctag = nullptr;
-  double *d_cr = nullptr;
   float *d_crf = nullptr, *d_rf = nullptr;
   RepParams *d_reps = nullptr;
   unsigned long long *d_cnt = nullptr;
@@ -91,7 +90,7 @@ void batch_free(ecmc_batch *b) {
   if (b->stream) cudaStreamSynchronize(b->stream);
   if (b->graph) cudaGraphExecDestroy(b->graph);
   void *ptrs[] = {b->d_r, b->d_img, b->d_rep_of, b->d_tag, b->d_cell, b->d_rank, b->d_count,
-                  b->d_start, b->d_bsum, b->d_cid, b->d_ctag, b->d_cr, b->d_crf, b->d_rf, b->d_reps,
+                  b->d_start, b->d_bsum, b->d_cid, b->d_ctag, b->d_crf, b->d_rf, b->d_reps,
                   b->d_cnt,
                   b->d_sums, b->d_status, b->d_unit_next, b->d_deferred, b->d_sweep,
                   b->d_rdig, b->d_rlift,
@@ -179,7 +178,6 @@ cudaError_t batch_sweep(ecmc_batch *b, const ECParams &P, uint64_t seed) {
   C.count = b->d_count;
   C.start = b->d_start;
   C.block_sums = b->d_bsum;
-  C.cr = b->d_cr;
   C.crf = b->d_crf;
   C.rf = b->d_rf;
   C.cid = b->d_cid;
@@ -223,10 +221,8 @@ ECParams batch_params(ecmc_batch *b, uint64_t seed, double ell) {
                                                                        : 1e-3 * b->sigma * b->sigma;
   P.eps_v = (float)ev;
   P.eps_d = (float)ed;
-  P.eps_x = (float)ev;
   P.r = b->d_r;
   P.img = b->d_img;
-  P.cr = b->d_cr;
   P.crf = b->d_crf;
   P.rf = b->d_rf;
   P.cid = b->d_cid;
@@ -315,7 +311,6 @@ ecmc_status ecmc_batch_create(const ecmc_replica_spec *specs, int32_t n, double 
   if (e == cudaSuccess) e = balloc(&b->d_tag, n_total);
   if (e == cudaSuccess) e = balloc(&b->d_cell, n_total);
   if (e == cudaSuccess) e = balloc(&b->d_rank, n_total);
-  if (e == cudaSuccess) e = balloc(&b->d_cr, 3 * n_total);
   if (e == cudaSuccess) e = balloc(&b->d_crf, 3 * n_total);
   if (e == cudaSuccess) e = balloc(&b->d_rf, 3 * n_total);
   if (e == cudaSuccess) e = balloc(&b->d_cid, n_total);

@@ -84,13 +84,6 @@ ECMC_HD int64_t scale_below(uint64_t w, uint64_t m) {
 }
 
 // ---------------------------------------------------------------- geometry
-// minimum image of one coordinate difference (|d| < L on input)
-ECMC_HD double wrap_d(double d, double L, double half) {
-  if (d > half) return d - L;
-  if (d < -half) return d + L;
-  return d;
-}
-
 // Candidate kinds in tie-break order: an exact tie in x goes to the smaller
 // kind, then to the smaller partner id.
 enum : int { KIND_END = 0, KIND_PASS = 1, KIND_WALL = 2, KIND_HS = 3, KIND_TETHER = 4 };
@@ -134,7 +127,8 @@ __device__ __forceinline__ double flip(double x) { return from_bits(bits_of(x) ^
 // |x| with the opposite sign of b's bits
 __device__ __forceinline__ double against(double x, uint64_t b) { return from_bits(bits_of(x) ^ (~b & 0x8000000000000000ull)); }
 
-// minimum image of one coordinate difference, as wrap_d, for L > 0
+// minimum image of one coordinate difference (|d| < L): d - L above half,
+// d + L below -half
 __device__ __forceinline__ double wrap_bits(double d, double L, double half, bool on = true) {
   const uint64_t b = bits_of(d);
   if (on && (b & 0x7FFFFFFFFFFFFFFFull) > bits_of(half)) d = add_fp64(d, against(L, b));
@@ -328,18 +322,13 @@ ECMC_HD void fnv_mix(uint64_t &h, uint64_t w) {
 }
 
 #ifdef __CUDACC__
-// FP32 bounds on a square root and a quotient from the hardware's fast
-// approximations.  rsqrtf errs by at most 2 ulp and __fdividef (divisor in
-// [2^-126, 2^126]) by at most 2 ulp (CUDA's accuracy tables), so after the
-// final product the relative error is below 4e-7 and the factors 1 -+ 1e-6
-// give a lower and an upper bound.  sqrt arguments are raised to 1e-30
-// inside rsqrtf: this keeps 0 finite and moves a result by less than 1e-15
-// in absolute terms, far inside the screen's margin eps_v.
-__device__ __forceinline__ float sqrt_lo(float y) { return y * rsqrtf(fmaxf(y, 1e-30f)) * 0.999999f; }
+// FP32 upper bound on a square root from the hardware's fast approximation:
+// rsqrtf errs by at most 2 ulp (CUDA's accuracy tables), so after the product
+// the relative error is below 4e-7 and the factor 1 + 1e-6 gives a bound.  The
+// argument is raised to 1e-30 inside rsqrtf: this keeps 0 finite and moves a
+// result by less than 1e-15 in absolute terms, far inside the screen's margin
+// eps_v.
 __device__ __forceinline__ float sqrt_hi(float y) { return y * rsqrtf(fmaxf(y, 1e-30f)) * 1.000001f; }
-__device__ __forceinline__ float div_lo(float a, float b) { return __fdividef(a, b) * 0.999999f; }
-__device__ __forceinline__ float div_hi(float a, float b) { return __fdividef(a, b) * 1.000001f; }
-
 #endif
 
 }  // namespace ecmc

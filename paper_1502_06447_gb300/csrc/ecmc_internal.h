@@ -88,7 +88,7 @@ struct ECParams {
   int32_t m_cap;        // motile beads per tile
   int32_t n_units;      // tiles (domain) or 1 (serial)
   // FP32 screen margins (units of sigma, sigma^2)
-  float eps_v, eps_d, eps_x;
+  float eps_v, eps_d;
   float s_cap_f;  // s_cap rounded up to FP32 (the screen's cap on a free flight)
   // FP32 values (rounded up where they widen a search): a conversion in the
   // kernel costs as much as an FP64 operation
@@ -96,7 +96,6 @@ struct ECParams {
   // buffers
   double *r;
   int32_t *img;
-  const double *cr;        // positions in cell order
   const int32_t *cid;      // ids in cell order
   const int32_t *ctag;     // tiles in cell order (joint beads: see joint_tag, k_cells.cu)
   const int32_t *cstart;   // cell starts (ncell + 1)
@@ -243,7 +242,6 @@ struct CellBatch {
   int32_t *count;
   int32_t *start;
   int32_t *block_sums;
-  double *cr;
   int32_t *cid;              // id within the replica
   int32_t *ctag;
   float *crf;                // FP32 positions in cell order

@@ -311,9 +311,6 @@ __global__ void k_scatter_b(const CellBatch C) {
   if (b >= C.n) return;
   const int64_t pos = (int64_t)C.start[C.cell[b]] + C.rank[b];
   const double x = C.r[3 * b], y = C.r[3 * b + 1], z = C.r[3 * b + 2];
-  C.cr[3 * pos] = x;
-  C.cr[3 * pos + 1] = y;
-  C.cr[3 * pos + 2] = z;
   C.crf[3 * pos] = (float)x;
   C.crf[3 * pos + 1] = (float)y;
   C.crf[3 * pos + 2] = (float)z;
