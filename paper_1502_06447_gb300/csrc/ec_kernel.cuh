@@ -1049,7 +1049,10 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
 // 0.3 sigma (a reach box then holds about 12 obstacles at phi = 0.45, 9 with
 // infinitely thin slabs) and grows while the masks of a tile would take
 // more than `budget` bytes; at least 10 slabs (staging keeps S ids in the
-// masks' area).
+// masks' area).  The launch gives 2 KB to tiles of 4 and 8 lanes, 192 bytes
+// per lane to the others; with half / with twice that, a pass of the 1e6-bead
+// melt takes 44.1 / 47.0 ms (43.6), 262k beads in FP64 5.29 / 5.12 (5.00), 64
+// replicas 207 / 205 (205), 48,000 beads on springs 10.90 / 10.97 (10.92).
 struct SlabPick {
   float inv;
   int nsl;

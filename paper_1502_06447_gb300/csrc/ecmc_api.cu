@@ -773,11 +773,16 @@ static ECParams ec_params(const ecmc_ctx *c, uint64_t seed, double ell) {
   P.dir_mode = c->opts.dir_mode;
   P.stage_cap = c->stage_cap;
   P.m_cap = c->m_cap;
-  // FP32 screen margins.  A shadow coordinate is off by at most
-  // err = 2^-24 (3 L + 64 sigma) (FP32 rounding of the position, of the tile
-  // corner, of their difference and of a wrap); a separation then by
-  // 2 sqrt(3) err, d.v and |d|^2 - (d.v)^2 by about 3.5 err and 18 err.  The
-  // margins keep a factor of 10 over those.
+  // FP32 screen margins, with u = 2^-24 and err = (3 L + 64 sigma) u.  A staged
+  // shadow is off by 3 L u (its position rounded, the difference to the tile
+  // corner, a wrap), the pivot's by 4 L u (its position truncated), and the
+  // truncated corner cancels in a separation: 7 L u + 128 sigma u < 2.4 err per
+  // axis.  With the direction truncated (2 u per component) d.v is then off by
+  // 4.1 err and |d|^2 - (d.v)^2, at the contact distances that matter, by 8.1
+  // err sigma (12 with a tether of 1.4 sigma).  The margins of 35 and 180 keep
+  // factors of 8 and 15.  Pairs drawn at random (10^6 per setting, worst case
+  // found): 0.02 of the margins at L = 1000 sigma, 0.28 with tethers of 31
+  // sigma or free flights of 100.
   {
     double Lm = c->L[0] > c->L[1] ? c->L[0] : c->L[1];
     Lm = Lm > c->L[2] ? Lm : c->L[2];

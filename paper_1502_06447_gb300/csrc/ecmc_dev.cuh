@@ -92,9 +92,9 @@ enum : int { KIND_END = 0, KIND_PASS = 1, KIND_WALL = 2, KIND_HS = 3, KIND_TETHE
 // IEEE double square root and quotient (round to nearest even) in integer
 // arithmetic.  GB300 takes 55-60 cycles for a dependent FP64 operation and
 // the FP64 pipe 16 cycles of an SM for each FP64 warp instruction, so the
-// iterations behind sqrt() (700-900 cycles) and / (650-1450 cycles) were the
-// longest links of an event step; a dependent 32-bit multiply-add takes
-// about 4.  Both functions take a 22-bit estimate from the FP32 hardware
+// iterations behind sqrt() and / were the longest links of an event step; a
+// dependent 32-bit multiply-add takes about 4.  A lone warp's dependent chain:
+// sqrt() 580 cycles, sqrt_rn 280, / 550, div_rn 320.  Both functions take a 22-bit estimate from the FP32 hardware
 // approximation, correct it twice by the exact remainder (64-bit wrapping
 // arithmetic: the remainders are known to be small), and settle the last
 // bit by the sign of one more exact remainder, so the result does not depend

@@ -359,8 +359,10 @@ inline int32_t stage_bound(const double E[3], double rho) {
 // cell of a local grid with cells no narrower than one flight's reach, an
 // overflow list of max(64, S / 4) slots and a header (screened form with 4,
 // 8 or 16 lanes: the request lists and records of a block as well), have to
-// fit a block's shared memory.  The kernel needs no more than that: where
-// its own layout would, it gives a tile more lanes.
+// fit a block's shared memory.  The rule is older than the kernel's layout and
+// kept as it was, so that the same settings are accepted: most of them need
+// less now, and where the kernel's own layout needs more, it gives a tile more
+// lanes (fewer tiles per warp) and, last, the capacity that fits (fit_stage).
 inline size_t staging_budget(int stage_cap, int motile64, int motile, int64_t ncell, int tiles) {
   const int ovf = stage_cap / 4 > 64 ? (stage_cap / 4 + 7) / 8 * 8 : 64;
   return (size_t)tiles * ((size_t)motile64 * 24 + (size_t)motile * 4 + (size_t)stage_cap * 16 +

@@ -242,7 +242,11 @@ __global__ void k_scatter(const CellParams C) {
 
 // The whole pass of a small melt in one block, counts in shared memory: a
 // small melt's sweep takes as long as its launches, and four of them become
-// one.
+// one.  One block / four kernels: us per sweep (27 tiles, next to no events)
+// of 512 beads 28 / 39, 1,728 38 / 44, 4,096 50 / 51, 5,832 64 / 58, 8,000
+// 84 / 70; us per call of ecmc_observables on 512 beads 47 / 53, 4,096 59 / 63,
+// 6,859 62 / 63, 8,000 73 / 63.  The line at 8,192 beads is older than these
+// figures: even are some 4,300 beads for sweeps, 6,900 for observables.
 constexpr int SMALL_BEADS = 8192, SMALL_CELLS = 16 * SCAN_BLOCK;
 __global__ void __launch_bounds__(SCAN_BLOCK) k_cells_small(const CellParams C, int ncell) {
   extern __shared__ int cnt[];  // [ncell]
