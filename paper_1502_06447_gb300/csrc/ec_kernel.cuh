@@ -768,7 +768,7 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
           // -0.0: bits that order above every candidate.  It competes as 0;
           // d.v, which a wall does not have, keeps the zero's sign for the
           // records.
-          keep(nonzero(x) ? x : 0.0, (KIND_WALL << 28) | ax, x, 0.0);
+          keep(from_bits(dbits(x) & 0x7FFFFFFFFFFFFFFFull), (KIND_WALL << 28) | ax, x, 0.0);
         }
         __syncwarp();
       }
@@ -963,11 +963,12 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
       if (G < 8) ev_hi += out >= 4 && gl == (out & 3) ? 1u : 0u;
       __syncwarp(gmask);
       shadows(qa, pf0, pf1, pf2);
-      if (kind == KIND_WALL) x = best.dv;
+      // (x as recorded)
+      auto flight = [&]() { return kind == KIND_WALL ? best.dv : x; };
       if (P.rec_digest) {
         fnv_mix(h, (uint64_t)pid);
         fnv_mix(h, ((uint64_t)(uint32_t)out << 32) | (uint64_t)(uint32_t)partner);
-        fnv_mix(h, dbits(x));
+        fnv_mix(h, dbits(flight()));
       }
       if (P.log && gl == 0) {
         const unsigned long long at = atomicAdd(P.log_n, 1ull);
@@ -980,7 +981,7 @@ __global__ void __launch_bounds__(128, 3) ec_kernel(const ECParams P) {
           ev.kind = out;
           ev.pad = 0;
           ev.partner = partner;
-          ev.x = x;
+          ev.x = flight();
           P.log[at] = ev;
         }
       }
