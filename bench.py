@@ -47,7 +47,7 @@ UNIT = "events/s"
 C0 = 1.2  # stencil cell side of the bytes-per-event definition (= b_max)
 # revision of the EC kernel; DRAM counters in profiles/ are used
 # only when they were taken on the same revision
-KERNEL_REV = 7
+KERNEL_REV = 8
 
 
 def launch_settings(args):
